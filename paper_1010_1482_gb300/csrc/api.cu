@@ -423,8 +423,6 @@ int evaluate_uniform_in(gbfmm_ctx *ctx, const gbfmm_params *prm, int64_t n, cons
     float4 *sx = at<float4>(ws, lo.sx), *far = at<float4>(ws, lo.far);
     uint32_t *hist = at<uint32_t>(ws, lo.rs_hist), *scan_tmp = at<uint32_t>(ws, lo.scan_tmp);
     int32_t *begin = at<int32_t>(ws, lo.cell_begin), *end = at<int32_t>(ws, lo.cell_end);
-    uint32_t *p2p_len = at<uint32_t>(ws, lo.p2p_len), *p2p_offs = at<uint32_t>(ws, lo.p2p_offs);
-    int32_t *p2p_ids = at<int32_t>(ws, lo.p2p_ids);
     uint32_t *m2l_len = at<uint32_t>(ws, lo.m2l_len), *m2l_offs = at<uint32_t>(ws, lo.m2l_offs);
     int32_t *m2l_ids = at<int32_t>(ws, lo.m2l_ids);
     uint16_t *m2l_code = at<uint16_t>(ws, lo.m2l_code);
@@ -450,22 +448,18 @@ int evaluate_uniform_in(gbfmm_ctx *ctx, const gbfmm_params *prm, int64_t n, cons
     launch_sort_gather(k0, k1, v0, v1, n, 3 * L, hist, ctx->d_status, x, sx, &skeys, &perm, s);
     mark(2);
     launch_cells(skeys, n, L, begin, end, s);
-    // the block M2L reads no M2L list: then only the P2P rows are built, on the near field's
-    // stream (the M2L rows are built on demand by gbfmm_export_lists)
+    // P2P finds its rows by grid position and the block M2L reads no list: M2L rows are built only
+    // for the M2L forms and the treecode that walk them (gbfmm_export_lists builds what it is asked
+    // for from the last evaluation's cells)
     const bool cores = (prm->flags & GBFMM_FLAG_M2L_CUDA_CORES) != 0;
     const bool gathered = (prm->flags & GBFMM_FLAG_M2L_GATHERED) != 0;
     const bool rot = (prm->flags & GBFMM_FLAG_M2L_ROTATION) != 0;
     const bool blk = L >= 2 && prm->method == GBFMM_METHOD_FMM && !cores && !gathered && !rot;
-    auto p2p_lists = [&](cudaStream_t st) {
-        launch_p2p_list_count(L, begin, end, p2p_len, st);
-        launch_exclusive_scan(p2p_len, p2p_offs, lo.nleaves, scan_tmp, st);
-        launch_p2p_list_fill(L, begin, end, p2p_offs, p2p_ids, st);
-    };
-    if (!blk) {
-        launch_list_count(L, begin, end, p2p_len, m2l_len, s);
-        launch_exclusive_scan(p2p_len, p2p_offs, lo.nleaves, scan_tmp, s);
+    const bool m2l_rows = L >= 2 && !blk;
+    if (m2l_rows) {
+        launch_list_count(L, begin, end, nullptr, m2l_len, s);
         launch_exclusive_scan(m2l_len, m2l_offs, lo.ncells, scan_tmp, s);
-        launch_list_fill(L, begin, end, p2p_offs, p2p_ids, m2l_offs, m2l_ids, m2l_code, s);
+        launch_list_fill(L, begin, end, nullptr, nullptr, m2l_offs, m2l_ids, m2l_code, s);
     }
     mark(3);
     // near field beside the far field (FMM): P2P writes its compensated sums, L2P adds the far
@@ -481,12 +475,10 @@ int evaluate_uniform_in(gbfmm_ctx *ctx, const gbfmm_params *prm, int64_t n, cons
         cudaStreamWaitEvent(ctx->s_near, ctx->ev_fork, 0);
         s = ctx->s_far;
         if (timing) cudaEventRecord(ctx->ev_aux[0], ctx->s_near);
-        if (blk) p2p_lists(ctx->s_near);
-        launch_p2p_near(L, n, sx, begin, end, p2p_offs, p2p_ids, (float)prm->eps2, near, ctx->d_status, ctx->s_near);
+        launch_p2p_near(L, n, sx, begin, end, (float)prm->eps2, near, ctx->d_status, ctx->s_near);
         if (timing) cudaEventRecord(ctx->ev_aux[1], ctx->s_near);
         cudaEventRecord(ctx->ev_near, ctx->s_near);
     }
-    if (blk && !fork) p2p_lists(s);  // serial: the P2P rows now, P2P after the far field
     if (L >= 2) launch_p2m(P, L, geo, sx, begin, end, M, s);
     mark(4);
     if (L >= 2)
@@ -527,7 +519,7 @@ int evaluate_uniform_in(gbfmm_ctx *ctx, const gbfmm_params *prm, int64_t n, cons
             cudaStreamWaitEvent(s, ctx->ev_near, 0);
             if (timing) cudaEventRecord(ctx->ev_aux[2], s);
         } else {
-            launch_p2p_near(L, n, sx, begin, end, p2p_offs, p2p_ids, (float)prm->eps2, near, ctx->d_status, s);
+            launch_p2p_near(L, n, sx, begin, end, (float)prm->eps2, near, ctx->d_status, s);
             mark(8);
         }
         launch_l2p(P, L, geo, n, sx, skeys, Lc, far, s, near, perm, out);
@@ -540,8 +532,7 @@ int evaluate_uniform_in(gbfmm_ctx *ctx, const gbfmm_params *prm, int64_t n, cons
     } else {
         if (L >= 2 && prm->method == GBFMM_METHOD_FMM) launch_l2p(P, L, geo, n, sx, skeys, Lc, far, s);
         mark(8);
-        launch_p2p(L, n, sx, begin, end, p2p_offs, p2p_ids, L >= 2 ? far : nullptr, perm, (float)prm->eps2, out,
-                   ctx->d_status, s);
+        launch_p2p(L, n, sx, begin, end, L >= 2 ? far : nullptr, perm, (float)prm->eps2, out, ctx->d_status, s);
         mark(9);
     }
     e = cudaGetLastError();
@@ -555,7 +546,7 @@ int evaluate_uniform_in(gbfmm_ctx *ctx, const gbfmm_params *prm, int64_t n, cons
     ctx->last_keys = (size_t)(reinterpret_cast<unsigned char *>(skeys) - ctx->last_ws);
     ctx->last_idx = (size_t)(reinterpret_cast<unsigned char *>(perm) - ctx->last_ws);
     ctx->last_method = prm->method;
-    ctx->last_m2l_lists = !blk;
+    ctx->last_lists = false;
     ctx->timed_last = timing;
     ctx->stage_order_last = fork ? 2 : (split ? 1 : 0);
     ctx->ops_built_last = built_now;
@@ -686,8 +677,8 @@ int gbfmm_export_lists(gbfmm_ctx *ctx, int kind, int32_t *offs, int32_t *ids, in
     }
     if (kind != GBFMM_LIST_P2P && kind != GBFMM_LIST_M2L) return fail(ctx, GBFMM_EINVAL, "unknown list kind");
     const Layout &lo = ctx->last;
-    if (kind == GBFMM_LIST_M2L && !ctx->last_m2l_lists && lo.L >= 2) {
-        // the evaluation's block M2L read no list: build the rows now from its cells
+    if (!ctx->last_lists) {
+        // evaluations build at most the M2L rows they walk: build both kinds now from the cells
         unsigned char *w = ctx->last_ws;
         const int32_t *cb = reinterpret_cast<const int32_t *>(w + lo.cell_begin);
         const int32_t *ce = reinterpret_cast<const int32_t *>(w + lo.cell_end);
@@ -700,8 +691,8 @@ int gbfmm_export_lists(gbfmm_ctx *ctx, int kind, int32_t *offs, int32_t *ids, in
         launch_list_fill(lo.L, cb, ce, p2p_offs, reinterpret_cast<int32_t *>(w + lo.p2p_ids), m2l_offs,
                          reinterpret_cast<int32_t *>(w + lo.m2l_ids), reinterpret_cast<uint16_t *>(w + lo.m2l_code), 0);
         e = cudaDeviceSynchronize();
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "M2L list build");
-        ctx->last_m2l_lists = true;
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "list build");
+        ctx->last_lists = true;
     }
     const int64_t rows = kind == GBFMM_LIST_P2P ? lo.nleaves : lo.ncells;
     std::vector<uint32_t> o(rows + 1);

@@ -300,14 +300,12 @@ void launch_sort_gather(uint32_t *k0, uint32_t *k1, uint32_t *v0, uint32_t *v1, 
 void launch_exclusive_scan(const uint32_t *in, uint32_t *out, int64_t n, uint32_t *tmp, cudaStream_t s);
 size_t exclusive_scan_tmp_words(int64_t n);
 void launch_cells(const uint32_t *sorted_leaf_keys, int64_t n, int L, int32_t *begin, int32_t *end, cudaStream_t s);
+// the M2L rows (levels 2..L), and with p2p_* given the leaves' P2P rows too (exports: the P2P
+// kernel finds the uniform tree's rows by grid position)
 void launch_list_count(int L, const int32_t *begin, const int32_t *end, uint32_t *p2p_len, uint32_t *m2l_len,
                        cudaStream_t s);
 void launch_list_fill(int L, const int32_t *begin, const int32_t *end, const uint32_t *p2p_offs, int32_t *p2p_ids,
                       const uint32_t *m2l_offs, int32_t *m2l_ids, uint16_t *m2l_code, cudaStream_t s);
-// the P2P rows alone (the block M2L of the uniform tree reads no M2L list)
-void launch_p2p_list_count(int L, const int32_t *begin, const int32_t *end, uint32_t *p2p_len, cudaStream_t s);
-void launch_p2p_list_fill(int L, const int32_t *begin, const int32_t *end, const uint32_t *p2p_offs, int32_t *p2p_ids,
-                          cudaStream_t s);
 
 // expansions.cu
 void launch_build_operators(int P, float *m2l_ops, float *m2m_ops, float *l2l_ops, cudaStream_t s);
@@ -439,15 +437,13 @@ bool p2p_near_supported();
 // CTA (0: the library's choice; at most kMaxP2PLeavesPerCta); the results do not depend on it
 constexpr int kMaxP2PLeavesPerCta = 64;
 void set_p2p_leaves_per_cta(int leaves);
-void launch_p2p_near(int L, int64_t n, const float4 *sx, const int32_t *begin, const int32_t *end,
-                     const uint32_t *p2p_offs, const int32_t *p2p_ids, float eps2, float4 *near, int *status,
-                     cudaStream_t s);
+void launch_p2p_near(int L, int64_t n, const float4 *sx, const int32_t *begin, const int32_t *end, float eps2,
+                     float4 *near, int *status, cudaStream_t s);
 void launch_p2p_cells_near(const int32_t *leaves, Span lv, int64_t n, const float4 *sx, const int32_t *begin,
                            const int32_t *end, const uint32_t *u_offs, const int32_t *u_ids, float eps2, float4 *near,
                            int *status, cudaStream_t s);
-void launch_p2p(int L, int64_t n, const float4 *sx, const int32_t *begin, const int32_t *end,
-                const uint32_t *p2p_offs, const int32_t *p2p_ids, const float4 *far, const uint32_t *perm, float eps2,
-                float4 *out, int *status, cudaStream_t s);
+void launch_p2p(int L, int64_t n, const float4 *sx, const int32_t *begin, const int32_t *end, const float4 *far,
+                const uint32_t *perm, float eps2, float4 *out, int *status, cudaStream_t s);
 void launch_direct(int64_t n_src, const float4 *src, int64_t n_tgt, const float4 *tgt, float eps2, float4 *out,
                    cudaStream_t s);
 
