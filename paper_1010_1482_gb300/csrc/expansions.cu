@@ -625,6 +625,9 @@ void launch_p2m(int P, int L, const float *geo, const float4 *sx, const int32_t 
 // degrees (rounded to whole k-groups of 4).
 // ------------------------------------------------------------------------------------------
 constexpr int kTrTN = 32, kTrCN = 8;
+// k_m2m_small up to this many CTAs (700 parents at p = 10); beyond, k_translate's operator is staged
+// for more cells (1,040 parents: 20 us either way)
+constexpr int kTransSmallCtas = 4 * 152;
 
 template <int P, bool UP, int TN = kTrTN, int CN = kTrCN>
 struct TransCfg {
@@ -701,11 +704,11 @@ __global__ void __launch_bounds__(TransCfg<P, UP, TN, CN>::NT) k_translate(int l
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    float acc[4][CN];
+    float tot[4][CN];  // M2M: the child positions' sums, added in order (as k_m2m_small adds them)
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < CN; ++j) acc[i][j] = 0.f;
+        for (int j = 0; j < CN; ++j) tot[i][j] = 0.f;
     const int c_first = UP ? 0 : blockIdx.y, c_last = UP ? 7 : blockIdx.y;
     stage(c_first, 0);
     for (int c = c_first; c <= c_last; ++c) {
@@ -720,12 +723,21 @@ __global__ void __launch_bounds__(TransCfg<P, UP, TN, CN>::NT) k_translate(int l
         if (work) {
             const float *Ar = tsm + buf * (Cfg::AF + Cfg::BF) + rg * 4;
             const float *Bc = tsm + buf * (Cfg::AF + Cfg::BF) + Cfg::AF + cg * SB;
+            float acc[4][CN];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < CN; ++j) acc[i][j] = 0.f;
 #pragma unroll 2
             for (int k = kbeg; k < kend; k += 4) {
                 Frag<CN, 4> f;
                 f.load(Ar, Bc, k, PR, NCG * SB);
                 f.fma(acc);
             }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < CN; ++j) tot[i][j] += acc[i][j];
         }
         __syncthreads();  // the buffer is refilled two positions later
     }
@@ -740,16 +752,142 @@ __global__ void __launch_bounds__(TransCfg<P, UP, TN, CN>::NT) k_translate(int l
         if (end[g] <= begin[g]) continue;
         float4 *dst = reinterpret_cast<float4 *>(X + g * PP + r);
         if (UP) {
-            *dst = make_float4(acc[0][j], acc[1][j], acc[2][j], acc[3][j]);
+            *dst = make_float4(tot[0][j], tot[1][j], tot[2][j], tot[3][j]);
         } else {
             float4 v = *dst;
-            v.x += acc[0][j];
-            v.y += acc[1][j];
-            v.z += acc[2][j];
-            v.w += acc[3][j];
+            v.x += tot[0][j];
+            v.y += tot[1][j];
+            v.z += tot[2][j];
+            v.w += tot[3][j];
             *dst = v;
         }
     }
+}
+
+// M2M of small levels.  k_translate takes the 8 child positions one after another, on few CTAs,
+// each position waiting for its p^2 x p^2 operator: 9 / 16 / 22 us a level at p = 4 / 8 / 10 however
+// few its cells.  Here a CTA takes 8 parents and one of SL slices of the output rows, and eight
+// thread groups take the eight child positions at once: all copies (the slices of the eight
+// operators and the columns, cut to the degrees the slice reads) are issued together and waited
+// for once.  The groups' sums are added in child order through shared memory, so every sum is
+// formed as in k_translate and k_translate_cells.  At p = 10 a level of
+// 64 / 512 parents takes 7.5 / 13 us (k_translate 20); beside P2P small CTAs also find room sooner
+// (16 parents and 143 KB a CTA: 10 us, and no gain in the 1M step).  L2L has one position per
+// CTA already: the same form took 10 us there against 7.  `Cells` maps parent ordinals q < np to cells: parent(q),
+// child(q, c), -1: none.
+template <int P>
+struct TransSmall {
+    static constexpr int PP = P * P, PR = ops_rows_padded(P), SB = staged_col_stride(P);
+    static constexpr int TN = 8, CN = 1, NCG = TN / CN, NRG = PR / 4;
+    static constexpr int SL = P == 4 ? 1 : P == 6 ? 3 : P == 8 ? 4 : 7;  // row slices
+    static constexpr int RGS = (NRG + SL - 1) / SL;         // row groups of a slice
+    static constexpr int GT = RGS * NCG, NT = 8 * GT;       // threads of a child position, of the CTA
+    static constexpr int LDA = 4 * RGS;
+    static constexpr size_t kSmem = sizeof(float) * 8 * ((size_t)PP * LDA + (size_t)TN * SB);
+    static_assert(NT * CN * 4 <= 8 * PP * LDA, "the child sums reuse the operators' space");
+};
+
+struct LevelCells {  // uniform tree: parents of level l, children of level l + 1
+    int64_t offp, offc, n;
+    const int32_t *begin, *end;
+    GB_DEV int64_t np() const { return n; }
+    GB_DEV int64_t some(int64_t g) const { return end[g] > begin[g] ? g : -1; }
+    GB_DEV int64_t parent(int64_t q) const { return some(offp + q); }
+    GB_DEV int64_t child(int64_t q, int c) const { return some(offc + 8 * q + c); }
+};
+
+struct SpanCells {  // adaptive tree: a span of cells; leaves among them are no parents
+    Span par;
+    const int32_t *child_of, *nchild;
+    GB_DEV int64_t np() const { return span_count(par); }
+    GB_DEV int64_t parent(int64_t q) const
+    {
+        const int64_t g = span_first(par) + q;
+        return nchild[g] != 0 ? g : -1;
+    }
+    GB_DEV int64_t child(int64_t q, int c) const { return child_of[(span_first(par) + q) * 8 + c]; }
+};
+
+template <int P, class Cells>
+__global__ void __launch_bounds__(TransSmall<P>::NT) k_m2m_small(Cells cells, const float *__restrict__ ops,
+                                                                 float *__restrict__ M)
+{
+    using Cfg = TransSmall<P>;
+    constexpr int PP = Cfg::PP, PR = Cfg::PR, SB = Cfg::SB, NCG = Cfg::NCG, TN = Cfg::TN, CN = Cfg::CN;
+    constexpr int GT = Cfg::GT, LDA = Cfg::LDA, RGS = Cfg::RGS, NRG = Cfg::NRG;
+    extern __shared__ __align__(16) float tsm[];
+    __shared__ int64_t s_par[TN], s_child[8][TN];
+    const int64_t q0 = blockIdx.x * (int64_t)TN, np = cells.np();
+    if (q0 >= np) return;
+    const int tid = threadIdx.x, rg0 = blockIdx.y * RGS, rg1 = min(rg0 + RGS, NRG);
+    // the columns k that rows of degree d read: those of degrees <= d
+    auto k_end = [](int r) { const int d = degree_of(min(r, PP - 1)); return min(PP, ((d + 1) * (d + 1) + 3) / 4 * 4); };
+    const int ke = k_end(4 * rg1 - 1);
+    float *B = tsm + 8 * PP * LDA;
+    for (int e = tid; e < 8 * PP * RGS; e += Cfg::NT) {
+        const int r = e % RGS, k = (e / RGS) % PP, c = e / (RGS * PP);
+        if (k < ke && rg0 + r < rg1)
+            cp_async16_t(tsm + (c * PP + k) * LDA + 4 * r, ops + ((size_t)c * PP + k) * PR + 4 * (rg0 + r), 16u);
+    }
+    for (int e = tid; e < 9 * TN; e += Cfg::NT) {
+        const int i = e % TN, c = e / TN - 1;
+        const int64_t g = q0 + i >= np ? -1 : c < 0 ? cells.parent(q0 + i) : cells.child(q0 + i, c);
+        (c < 0 ? s_par[i] : s_child[c][i]) = g;
+    }
+    __syncthreads();
+    for (int e = tid; e < 8 * TN * (PP / 4); e += Cfg::NT) {
+        const int k = 4 * (e % (PP / 4)), i = (e / (PP / 4)) % TN, c = e / (PP / 4 * TN);
+        const int64_t g = s_child[c][i];
+        if (k < ke) cp_async16_t(B + (c * TN + i) * SB + k, g >= 0 ? M + g * PP + k : M, g >= 0 ? 16u : 0u);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    const int c = tid / GT, t = tid % GT, cg = t % NCG, rl = t / NCG, rg = rg0 + rl;
+    float acc[4][CN];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < CN; ++j) acc[i][j] = 0.f;
+    if (rg < rg1) {
+        const int kn = k_end(4 * rg + 3);
+        const float *Ar = tsm + c * PP * LDA + 4 * rl, *Bc = B + (c * TN + cg) * SB;
+#pragma unroll 2
+        for (int k = 0; k < kn; k += 4) {
+            Frag<CN, 4> f;
+            f.load(Ar, Bc, k, LDA, NCG * SB);
+            f.fma(acc);
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < CN; ++j) tsm[(i * CN + j) * Cfg::NT + tid] = acc[i][j];
+    __syncthreads();
+    for (int e = tid; e < 4 * CN * GT; e += Cfg::NT) {
+        const int i = e % 4, tt = (e / 4) % GT, j = e / (4 * GT);
+        const int r = 4 * (rg0 + tt / NCG) + i;
+        const int64_t g = s_par[tt % NCG + j * NCG];
+        if (g < 0 || rg0 + tt / NCG >= rg1 || r >= PP) continue;
+        float v = 0.f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v += tsm[(i * CN + j) * Cfg::NT + k * GT + tt];
+        M[g * PP + r] = v;
+    }
+}
+
+// false (nothing launched) on levels of more CTAs than kTransSmallCtas
+template <int P, class Cells>
+static bool launch_m2m_small(int64_t np, const Cells &cells, const float *ops, float *M, cudaStream_t s)
+{
+    using Cfg = TransSmall<P>;
+    const int64_t ctas = (np + Cfg::TN - 1) / Cfg::TN;
+    if (ctas * Cfg::SL > kTransSmallCtas) return false;
+    cudaFuncSetAttribute(k_m2m_small<P, Cells>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::kSmem);
+    k_m2m_small<P, Cells><<<dim3((unsigned)ctas, Cfg::SL), Cfg::NT, Cfg::kSmem, s>>>(cells, ops, M);
+    note_launches(1);
+    return true;
 }
 
 template <int P, bool UP, int TN, int CN>
@@ -772,7 +910,10 @@ template <int P, bool UP>
 static void launch_translate_t(int l, const int32_t *begin, const int32_t *end, const float *ops, float *X,
                                cudaStream_t s)
 {
-    const int64_t np = int64_t(1) << (3 * (UP ? l : l - 1));
+    const int lp = UP ? l : l - 1;
+    const int64_t np = int64_t(1) << (3 * lp);
+    if constexpr (UP)
+        if (launch_m2m_small<P>(np, LevelCells{level_offset(lp), level_offset(lp + 1), np, begin, end}, ops, X, s)) return;
     const int64_t ctas32 = (np + 31) / 32 * (UP ? 1 : 8);
     if (ctas32 >= 2 * 152)
         launch_translate_tn<P, UP, 32, 8>(l, begin, end, ops, X, s);
@@ -1426,11 +1567,11 @@ __global__ void __launch_bounds__(TransCfg<P, UP, TN, CN>::NT) k_translate_cells
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    float acc[4][CN];
+    float tot[4][CN];  // M2M: the child positions' sums, added in order (as k_m2m_small adds them)
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < CN; ++j) acc[i][j] = 0.f;
+        for (int j = 0; j < CN; ++j) tot[i][j] = 0.f;
     const int c_first = UP ? 0 : blockIdx.y, c_last = UP ? 7 : blockIdx.y;
     stage(c_first, 0);
     for (int c = c_first; c <= c_last; ++c) {
@@ -1445,12 +1586,21 @@ __global__ void __launch_bounds__(TransCfg<P, UP, TN, CN>::NT) k_translate_cells
         if (work) {
             const float *Ar = tsm + buf * (Cfg::AF + Cfg::BF) + rg * 4;
             const float *Bc = tsm + buf * (Cfg::AF + Cfg::BF) + Cfg::AF + cg * SB;
+            float acc[4][CN];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < CN; ++j) acc[i][j] = 0.f;
 #pragma unroll 2
             for (int k = kbeg; k < kend; k += 4) {
                 Frag<CN, 4> f;
                 f.load(Ar, Bc, k, PR, NCG * SB);
                 f.fma(acc);
             }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < CN; ++j) tot[i][j] += acc[i][j];
         }
         __syncthreads();  // the buffer is refilled two positions later
     }
@@ -1472,13 +1622,13 @@ __global__ void __launch_bounds__(TransCfg<P, UP, TN, CN>::NT) k_translate_cells
         }
         float4 *dst = reinterpret_cast<float4 *>(X + g * PP + r);
         if (UP) {
-            *dst = make_float4(acc[0][j], acc[1][j], acc[2][j], acc[3][j]);
+            *dst = make_float4(tot[0][j], tot[1][j], tot[2][j], tot[3][j]);
         } else {
             float4 v = *dst;
-            v.x += acc[0][j];
-            v.y += acc[1][j];
-            v.z += acc[2][j];
-            v.w += acc[3][j];
+            v.x += tot[0][j];
+            v.y += tot[1][j];
+            v.z += tot[2][j];
+            v.w += tot[3][j];
             *dst = v;
         }
     }
@@ -1549,6 +1699,8 @@ template <int P, bool UP>
 static void translate_cells_t(Span par, const int32_t *child_of, const int32_t *nchild, const float *ops, float *X,
                               cudaStream_t s)
 {
+    if constexpr (UP)
+        if (launch_m2m_small<P>(par.cap, SpanCells{par, child_of, nchild}, ops, X, s)) return;
     const int64_t ctas32 = (par.cap + 31) / 32 * (UP ? 1 : 8), ctas64 = (par.cap + 63) / 64 * (UP ? 1 : 8);
     if constexpr (UP) {  // large levels: 128 (upward) or 64 cells per CTA share each staged operator
         if ((par.cap + 127) / 128 >= 4 * 152) return translate_cells_tn<P, UP, 128, 8>(par, child_of, nchild, ops, X, s);
