@@ -30,6 +30,7 @@ namespace gbfmm {
 constexpr int kAdaptMaxLevel = kAdaptiveMaxLevel;
 constexpr int kListU = 0, kListV = 1, kListW = 2, kListX = 3;
 constexpr int kDescentStack = 256;
+constexpr int64_t kColleagueFindCells = 1 << 17;  // below this many cells one launch finds all colleagues by key
 constexpr int64_t kListWarpCells = 1 << 17;  // below this many cells the U/W/X rows take a warp per cell
 
 // ---- keys ---------------------------------------------------------------------------------
@@ -292,20 +293,33 @@ __global__ void __launch_bounds__(kTreeB) k_tree_cells(int64_t n, const uint64_t
     }
 }
 
+// integer box of a cell at depth 21: anchor x, y, z and log2 of the side
+GB_DEV int4 cell_box(uint64_t key, int l)
+{
+    int x, y, z;
+    demorton63(key, x, y, z);
+    const int sh = kAdaptMaxLevel - l;
+    return make_int4(x << sh, y << sh, z << sh, sh);
+}
+
 // per cell: particle count (end of its key prefix in the sorted keys), the parent of a cell
-// whose parent starts at an earlier particle (key search within the parent level), and the
-// parent's child links
+// whose parent starts at an earlier particle (key search within the parent level), the
+// parent's child links, and the cell's geometry and integer box (launch_cell_geom, k_cell_anchor)
 __global__ void k_tree_links(Span cells, int64_t n, const uint64_t *__restrict__ sk, const int32_t *__restrict__ info,
                              const int32_t *__restrict__ level, const uint64_t *__restrict__ key,
                              const int32_t *__restrict__ begin, int32_t *__restrict__ count, int32_t *__restrict__ end,
                              int32_t *__restrict__ parent, int32_t *__restrict__ child_begin,
-                             int32_t *__restrict__ nchild, int32_t *__restrict__ child_of)
+                             int32_t *__restrict__ nchild, int32_t *__restrict__ child_of,
+                             const Box *__restrict__ box, float4 *__restrict__ geom, int4 *__restrict__ anc)
 {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= span_count(cells)) return;
     const int64_t c = span_first(cells) + i;
     const int l = level[c];
     const uint64_t kk = key[c];
+    const CellGeom g = cell_geom63(*box, l, kk);
+    geom[c] = make_float4(g.cx, g.cy, g.cz, g.inv_h);
+    anc[c] = cell_box(kk, l);
     const int64_t b = begin[c];
     int64_t e = n;
     if (l > 0) {
@@ -340,25 +354,6 @@ __global__ void k_tree_links(Span cells, int64_t n, const uint64_t *__restrict__
         child_of[(int64_t)p * 8 + (int)(kk & 7)] = (int32_t)c;
         atomicAdd(&nchild[p], 1);
         atomicMin(&child_begin[p], (int32_t)c);
-    }
-}
-
-__global__ void k_tree_leaf_of(int64_t n, const int32_t *__restrict__ leaves, int32_t *__restrict__ leaf_of,
-                               const int32_t *__restrict__ abort)
-{
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < n && !(abort && *abort)) leaf_of[i] = leaves[leaf_of[i]];
-}
-
-// list sizes of the four kinds into info[0..3]
-__global__ void k_list_totals(int64_t nc, const uint32_t *o0, const uint32_t *o1, const uint32_t *o2,
-                              const uint32_t *o3, int32_t *info)
-{
-    if (threadIdx.x == 0) {
-        info[0] = (int32_t)o0[nc];
-        info[1] = (int32_t)o1[nc];
-        info[2] = (int32_t)o2[nc];
-        info[3] = (int32_t)o3[nc];
     }
 }
 
@@ -401,6 +396,40 @@ __global__ void k_colleagues(Span lv, int l, const uint64_t *__restrict__ key, c
             }
 }
 
+// The colleagues of every cell in one launch: a warp per cell, a lane per slot, each finding its
+// neighbour's key among the sorted keys of the cell's level, info[l] .. info[l + 1].  k_colleagues
+// needs the parents' rows and so a launch per level, 7-9 us each however few the cells: 1,300
+// cells of 9 levels 66 -> 5.6 us, 24,500 of 10 levels 78 -> 14.4.
+__global__ void __launch_bounds__(256) k_colleagues_find(Span cells, const int32_t *__restrict__ info,
+                                                         const int32_t *__restrict__ level,
+                                                         const uint64_t *__restrict__ key, int32_t *__restrict__ coll)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t w = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (w >= span_count(cells) || lane >= 27) return;
+    const int64_t b = span_first(cells) + w;
+    const int l = level[b], side = 1 << l;
+    int x, y, z;
+    demorton63(key[b], x, y, z);
+    x += lane % 3 - 1;
+    y += (lane / 3) % 3 - 1;
+    z += lane / 9 - 1;
+    int32_t r = -1;
+    if (x >= 0 && y >= 0 && z >= 0 && x < side && y < side && z < side) {
+        const uint64_t k = morton63((uint64_t)x, (uint64_t)y, (uint64_t)z);
+        int32_t lo = info[l], hi = info[l + 1] - 1;
+        while (lo < hi) {
+            const int32_t mid = (lo + hi) >> 1;
+            if (key[mid] < k)
+                lo = mid + 1;
+            else
+                hi = mid;
+        }
+        if (key[lo] == k) r = lo;
+    }
+    coll[b * 27 + lane] = r;
+}
+
 // ---- lists --------------------------------------------------------------------------------
 struct TreeView {
     const int32_t *level, *parent, *nchild, *child_of, *coll;
@@ -415,10 +444,7 @@ __global__ void k_cell_anchor(Span cells, const int32_t *__restrict__ level, con
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= span_count(cells)) return;
     const int64_t c = span_first(cells) + i;
-    int x, y, z;
-    demorton63(key[c], x, y, z);
-    const int sh = kAdaptMaxLevel - level[c];
-    anc[c] = make_int4(x << sh, y << sh, z << sh, sh);
+    anc[c] = cell_box(key[c], level[c]);
 }
 
 // boxes that touch or overlap in all three dimensions
@@ -430,16 +456,16 @@ GB_DEV bool adjacent(const TreeView &t, int32_t a, int32_t b)
              lb.z > la.z + sa);
 }
 
-// Descent below colleague a of leaf b (U and W lists): a leaf colleague is a U entry; below a
-// split colleague, descendants adjacent to b are opened (leaves among them are U entries) and
-// the first non-adjacent ones on each path are W entries.  Calls f(id) for the entries of the
-// list kind; returns false if the stack overflowed.
-template <bool U, class F>
-GB_DEV bool descend(const TreeView &t, int32_t b, int32_t a, F f)
+// Descent below colleague a of leaf b: a leaf colleague is a U entry; below a split colleague,
+// descendants adjacent to b are opened (leaves among them are U entries) and the first
+// non-adjacent ones on each path are W entries.  Calls u(id) and w(id); returns false if the stack
+// overflowed.
+template <class FU, class FW>
+GB_DEV bool descend(const TreeView &t, int32_t b, int32_t a, FU u, FW w)
 {
     if (a < 0) return true;
     if (t.nchild[a] == 0) {
-        if (U) f(a);
+        u(a);
         return true;
     }
     bool ok = true;
@@ -451,21 +477,19 @@ GB_DEV bool descend(const TreeView &t, int32_t b, int32_t a, F f)
     }
     while (sp > 0) {
         const int32_t d = stack[--sp];
-        if (adjacent(t, b, d)) {
-            if (t.nchild[d] == 0) {
-                if (U) f(d);
-            } else {
-                for (int q = 0; q < 8; ++q) {
-                    const int32_t c = t.child_of[(int64_t)d * 8 + q];
-                    if (c < 0) continue;
-                    if (sp < kDescentStack)
-                        stack[sp++] = c;
-                    else
-                        ok = false;
-                }
+        if (!adjacent(t, b, d)) {
+            w(d);
+        } else if (t.nchild[d] == 0) {
+            u(d);
+        } else {
+            for (int q = 0; q < 8; ++q) {
+                const int32_t c = t.child_of[(int64_t)d * 8 + q];
+                if (c < 0) continue;
+                if (sp < kDescentStack)
+                    stack[sp++] = c;
+                else
+                    ok = false;
             }
-        } else if (!U) {
-            f(d);
         }
     }
     return ok;
@@ -483,88 +507,111 @@ GB_DEV uint32_t warp_excl_scan(uint32_t v, int lane, uint32_t &total)
     return x - v;
 }
 
-// U, W and X lists, one warp per cell.  Entries come in the order: colleague slot (lane), the
-// descent below it, then (U, X) ancestors from the parent up, colleague slot within each.  The
-// count pass (FILL = false) writes the row lengths; the fill pass writes the rows at `offs`.
-template <int KIND, bool FILL>
-__global__ void k_alist_warp(Span cells, TreeView t, uint32_t *__restrict__ cnt, const uint32_t *__restrict__ offs,
-                             int32_t *__restrict__ ids, int *status)
+// U, W and X rows of one tree: the row lengths (count pass) or offsets and entries (fill pass).
+// One descent below a leaf's colleagues finds its U and W entries, one walk over the leaf
+// colleagues of its strict ancestors its U (adjacent to the leaf) and X entries (adjacent to its
+// parent but not to it): one launch a pass (1,300 cells: the two take 29 us, one launch
+// a kind and pass 75).
+struct ListRows {
+    uint32_t *u_cnt, *w_cnt, *x_cnt;
+    const uint32_t *u_offs, *w_offs, *x_offs;
+    int32_t *u_ids, *w_ids, *x_ids;
+};
+
+// One warp per cell.  Entries come in the order: colleague slot (lane), the descent below it,
+// then (U, X) ancestors from the parent up, colleague slot within each.  The count pass (FILL =
+// false) writes the row lengths, 0 for rows past the cells; the fill pass writes the rows.
+template <bool FILL>
+__global__ void __launch_bounds__(256) k_alist_warp(Span cells, TreeView t, ListRows r, int *status)
 {
     const int lane = threadIdx.x & 31;
     const int64_t w = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (w >= span_count(cells)) return;
+    if (w >= span_count(cells)) {
+        if (!FILL && w < cells.cap && lane == 0) r.u_cnt[w] = r.w_cnt[w] = r.x_cnt[w] = 0;
+        return;
+    }
     const int64_t bb = span_first(cells) + w;
     const int32_t b = (int32_t)bb;
     const unsigned lt = (1u << lane) - 1u;
-    uint32_t e = FILL ? offs[b] : 0u;
-    if (KIND == kListU || KIND == kListW) {
-        if (t.nchild[b] != 0) {
-            if (!FILL && lane == 0) cnt[b] = 0;
-            return;
-        }
+    const bool leaf = t.nchild[b] == 0;
+    uint32_t eu = FILL ? r.u_offs[b] : 0u, ew = FILL ? r.w_offs[b] : 0u, ex = FILL ? r.x_offs[b] : 0u;
+    if (leaf) {
         const int32_t a = lane < 27 ? t.coll[(int64_t)b * 27 + lane] : -1;
-        uint32_t mine = 0;
-        const bool ok = descend<KIND == kListU>(t, b, a, [&](int32_t) { ++mine; });
+        uint32_t nu = 0, nw = 0;
+        const bool ok = descend(t, b, a, [&](int32_t) { ++nu; }, [&](int32_t) { ++nw; });
         if (!FILL && !ok) atomicOr(status, kStatusTimeout);
-        uint32_t total;
-        const uint32_t excl = warp_excl_scan(mine, lane, total);
+        uint32_t tu, tw;
+        const uint32_t xu = warp_excl_scan(nu, lane, tu), xw = warp_excl_scan(nw, lane, tw);
         if (FILL) {
-            uint32_t w = e + excl;
-            descend<KIND == kListU>(t, b, a, [&](int32_t d) { ids[w++] = d; });
+            uint32_t ku = eu + xu, kw = ew + xw;
+            descend(t, b, a, [&](int32_t d) { r.u_ids[ku++] = d; }, [&](int32_t d) { r.w_ids[kw++] = d; });
         }
-        e += total;
+        eu += tu;
+        ew += tw;
     }
-    if (KIND == kListU || KIND == kListX) {
-        const int32_t ref = KIND == kListU ? b : t.parent[b];  // adjacency reference
-        if (ref >= 0)
-            for (int32_t anc = t.parent[b]; anc >= 0; anc = t.parent[anc]) {
-                const int32_t c = lane < 27 ? t.coll[(int64_t)anc * 27 + lane] : -1;
-                bool hit = c >= 0 && c != anc && t.nchild[c] == 0 && adjacent(t, ref, c);
-                if (KIND == kListX && hit) hit = !adjacent(t, b, c);
-                const unsigned bal = __ballot_sync(0xffffffffu, hit);
-                if (FILL && hit) ids[e + __popc(bal & lt)] = c;
-                e += __popc(bal);
-            }
+    const int32_t p = t.parent[b];
+    for (int32_t anc = p; anc >= 0; anc = t.parent[anc]) {
+        const int32_t c = lane < 27 ? t.coll[(int64_t)anc * 27 + lane] : -1;
+        const bool near = c >= 0 && c != anc && t.nchild[c] == 0 && adjacent(t, p, c);
+        const bool touch = near && adjacent(t, b, c);  // touching b, a box touches b's parent too
+        const bool hu = touch && leaf, hx = near && !touch;
+        const unsigned bu = __ballot_sync(0xffffffffu, hu), bx = __ballot_sync(0xffffffffu, hx);
+        if (FILL && hu) r.u_ids[eu + __popc(bu & lt)] = c;
+        if (FILL && hx) r.x_ids[ex + __popc(bx & lt)] = c;
+        eu += __popc(bu);
+        ex += __popc(bx);
     }
-    if (!FILL && lane == 0) cnt[b] = e;
+    if (!FILL && lane == 0) {
+        r.u_cnt[b] = eu;
+        r.w_cnt[b] = ew;
+        r.x_cnt[b] = ex;
+    }
 }
 
-// The same U, W and X rows, one thread per cell (slots in sequence): on large trees the warp
-// form leaves most lanes idle while one descends, and its fill repeats the descents.
-template <int KIND, bool FILL>
-__global__ void k_alist_thread(Span cells, TreeView t, uint32_t *__restrict__ cnt, const uint32_t *__restrict__ offs,
-                               int32_t *__restrict__ ids, int *status)
+// The same rows, one thread per cell (slots in sequence): on large trees the warp form leaves
+// most lanes idle while one descends, and its fill repeats the descents.
+template <bool FILL>
+__global__ void __launch_bounds__(128) k_alist_thread(Span cells, TreeView t, ListRows r, int *status)
 {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= span_count(cells)) return;
+    if (i >= span_count(cells)) {
+        if (!FILL && i < cells.cap) r.u_cnt[i] = r.w_cnt[i] = r.x_cnt[i] = 0;
+        return;
+    }
     const int64_t bb = span_first(cells) + i;
     const int32_t b = (int32_t)bb;
-    uint32_t e = FILL ? offs[b] : 0u;
-    auto emit = [&](int32_t d) {
-        if (FILL) ids[e] = d;
-        ++e;
+    const bool leaf = t.nchild[b] == 0;
+    uint32_t eu = FILL ? r.u_offs[b] : 0u, ew = FILL ? r.w_offs[b] : 0u, ex = FILL ? r.x_offs[b] : 0u;
+    auto u = [&](int32_t d) {
+        if (FILL) r.u_ids[eu] = d;
+        ++eu;
     };
-    if (KIND == kListU || KIND == kListW) {
-        if (t.nchild[b] != 0) {
-            if (!FILL) cnt[b] = 0;
-            return;
-        }
+    auto w = [&](int32_t d) {
+        if (FILL) r.w_ids[ew] = d;
+        ++ew;
+    };
+    if (leaf) {
         bool ok = true;
-        for (int sl = 0; sl < 27; ++sl) ok &= descend<KIND == kListU>(t, b, t.coll[(int64_t)b * 27 + sl], emit);
+        for (int sl = 0; sl < 27; ++sl) ok &= descend(t, b, t.coll[(int64_t)b * 27 + sl], u, w);
         if (!FILL && !ok) atomicOr(status, kStatusTimeout);
     }
-    if (KIND == kListU || KIND == kListX) {
-        const int32_t ref = KIND == kListU ? b : t.parent[b];
-        if (ref >= 0)
-            for (int32_t anc = t.parent[b]; anc >= 0; anc = t.parent[anc])
-                for (int sl = 0; sl < 27; ++sl) {
-                    const int32_t c = t.coll[(int64_t)anc * 27 + sl];
-                    if (c < 0 || c == anc || t.nchild[c] != 0 || !adjacent(t, ref, c)) continue;
-                    if (KIND == kListX && adjacent(t, b, c)) continue;
-                    emit(c);
-                }
+    const int32_t p = t.parent[b];
+    for (int32_t anc = p; anc >= 0; anc = t.parent[anc])
+        for (int sl = 0; sl < 27; ++sl) {
+            const int32_t c = t.coll[(int64_t)anc * 27 + sl];
+            if (c < 0 || c == anc || t.nchild[c] != 0 || !adjacent(t, p, c)) continue;
+            if (!adjacent(t, b, c)) {
+                if (FILL) r.x_ids[ex] = c;
+                ++ex;
+            } else if (leaf) {
+                u(c);
+            }
+        }
+    if (!FILL) {
+        r.u_cnt[b] = eu;
+        r.w_cnt[b] = ew;
+        r.x_cnt[b] = ex;
     }
-    if (!FILL) cnt[b] = e;
 }
 
 // V list, one warp per cell: lane j takes the candidate offsets t = j, j + 32, ... of the
@@ -577,7 +624,10 @@ __global__ void k_vlist_warp(Span cells, TreeView t, uint32_t *__restrict__ cnt,
 {
     const int lane = threadIdx.x & 31;
     const int64_t w = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (w >= span_count(cells)) return;
+    if (w >= span_count(cells)) {
+        if (!FILL && w < cells.cap && lane == 0) cnt[w] = 0;  // rows past the cells stay empty
+        return;
+    }
     const int64_t b = span_first(cells) + w;
     const int l = t.level[b];
     if (l < 2) {
@@ -647,7 +697,10 @@ __global__ void k_chain_count(Span cells, const int32_t *__restrict__ nchild, co
                               uint32_t *__restrict__ cnt)
 {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= span_count(cells)) return;
+    if (i >= span_count(cells)) {
+        if (i < cells.cap) cnt[i] = 0;  // rows past the cells stay empty
+        return;
+    }
     const int64_t c = span_first(cells) + i;
     uint32_t k = 0;
     if (nchild[c] == 0) {
@@ -858,26 +911,24 @@ int treecode_adaptive(gbfmm_ctx *ctx, AdaptiveState &A, const Ranges &R, const g
     const OpsCache &ops = ctx->ops[order_slot(P)];
     ctx->stage_order_last = 0;
     // chain lists: [0] U + ancestors' X (P2P), [1] W + ancestors' V (M2P)
-    if (grow(A.tc_cnt, 4 * (ncells + 1), false, 0, s) || grow(A.tc_offs[0], 4 * (ncells + 1), false, 0, s) ||
+    if (grow(A.tc_cnt, 8 * (ncells + 1), false, 0, s) || grow(A.tc_offs[0], 4 * (ncells + 1), false, 0, s) ||
         grow(A.tc_offs[1], 4 * (ncells + 1), false, 0, s))
         return fail(ctx, GBFMM_ENOMEM, "treecode lists");
+    int32_t *info = A.info.as<int32_t>();
     const int ka[2] = {kListU, kListW}, kb[2] = {kListX, kListV};
+    ScanJobs jobs{};
     for (int j = 0; j < 2; ++j) {
-        if (R.dev) cudaMemsetAsync(A.tc_cnt.p, 0, 4 * (ncells + 1), s);
+        uint32_t *cnt = A.tc_cnt.as<uint32_t>() + j * (ncells + 1);
         k_chain_count<<<blocks_for(ncells), 256, 0, s>>>(R.cells(), A.nchild.as<int32_t>(), A.parent.as<int32_t>(),
                                                          A.loffs[ka[j]].as<uint32_t>(), A.loffs[kb[j]].as<uint32_t>(),
-                                                         A.tc_cnt.as<uint32_t>());
+                                                         cnt);
         note_launches(1);
-        launch_exclusive_scan(A.tc_cnt.as<uint32_t>(), A.tc_offs[j].as<uint32_t>(), ncells, A.scan_tmp.as<uint32_t>(),
-                              s);
+        jobs.j[j] = {cnt, A.tc_offs[j].as<uint32_t>(), info + kInfoChain + j};
     }
-    int32_t *info = A.info.as<int32_t>();
-    k_list_totals<<<1, 32, 0, s>>>(ncells, A.tc_offs[0].as<uint32_t>(), A.tc_offs[1].as<uint32_t>(),
-                                   A.tc_offs[0].as<uint32_t>(), A.tc_offs[1].as<uint32_t>(), info + kInfoChain);
-    note_launches(1);
+    launch_exclusive_scans(jobs, 2, ncells, A.scan_tmp.as<uint32_t>(), s);
     int64_t tot[2];
     if (!R.dev) {
-        int32_t h[4];
+        int32_t h[2];
         cudaMemcpyAsync(h, info + kInfoChain, sizeof(h), cudaMemcpyDeviceToHost, s);
         cudaStreamSynchronize(s);
         for (int j = 0; j < 2; ++j) A.counts.chain[j] = tot[j] = (uint32_t)h[j];
@@ -1008,9 +1059,14 @@ int evaluate_adaptive_in(gbfmm_ctx *ctx, AdaptiveState &A, const AdaptCaps *caps
             if (grow(*e.b, e.per * c, keep, e.per * used, s) != 0) return false;
         return true;
     };
+    auto cell_aux = [&](int64_t c) {
+        return grow(A.geom, 16 * (size_t)c, false, 0, s) == 0 && grow(A.anchor, 16 * (size_t)c, false, 0, s) == 0 &&
+               grow(A.coll, 4 * 27 * (size_t)c, false, 0, s) == 0;
+    };
     std::vector<int> ls;
     int64_t ncells = 0;
     int maxl = 0;
+    const int32_t *leaves_of = nullptr;  // leaf_of holds ordinals in this list (one-pass build) or cells
     if (n > 0 && window <= kTreeMaxWindow) {
         // one pass: per-particle level ranges, per-level ranks, one host read of the level sizes
         // (or, under capacities, a device check of them)
@@ -1042,7 +1098,7 @@ int evaluate_adaptive_in(gbfmm_ctx *ctx, AdaptiveState &A, const AdaptCaps *caps
             note_launches(1);
         }
         if (!cell_bufs(ncells, false, 0) || grow(A.end, 4 * ncells, false, 0, s) ||
-            grow(A.leaves, 4 * ncells + 4, false, 0, s))
+            grow(A.leaves, 4 * ncells + 4, false, 0, s) || !cell_aux(ncells))
             return fail(ctx, GBFMM_ENOMEM, "adaptive cells");
         k_tree_cells<<<(unsigned)tb, kTreeB, 0, s>>>(n, skeys, tb, range, hbase, A.level.as<int32_t>(),
                                                      A.key.as<uint64_t>(), A.begin.as<int32_t>(),
@@ -1055,9 +1111,10 @@ int evaluate_adaptive_in(gbfmm_ctx *ctx, AdaptiveState &A, const AdaptCaps *caps
                                                            A.key.as<uint64_t>(), A.begin.as<int32_t>(),
                                                            A.count.as<int32_t>(), A.end.as<int32_t>(),
                                                            A.parent.as<int32_t>(), A.child_begin.as<int32_t>(),
-                                                           A.nchild.as<int32_t>(), A.child_of.as<int32_t>());
-        k_tree_leaf_of<<<blocks_for(n), 256, 0, s>>>(n, A.leaves.as<int32_t>(), A.leaf_of.as<int32_t>(), abort);
-        note_launches(3);
+                                                           A.nchild.as<int32_t>(), A.child_of.as<int32_t>(), box,
+                                                           A.geom.as<float4>(), A.anchor.as<int4>());
+        note_launches(2);
+        leaves_of = A.leaves.as<int32_t>();
     } else {
         // level by level (leaf sizes beyond the one-pass window, or no particles): one flag /
         // scan / compact round per level, the host reading the number of new cells after each
@@ -1116,90 +1173,103 @@ int evaluate_adaptive_in(gbfmm_ctx *ctx, AdaptiveState &A, const AdaptCaps *caps
     A.max_level = maxl;
     A.level_start = ls;
     const Ranges R{dev, info, abort, ncells, A.nleaves, &A.level_start, caps};
-    if (grow(A.coll, 4 * 27 * ncells, false, 0, s)) return fail(ctx, GBFMM_ENOMEM, "adaptive cells");
-    if (grow(A.geom, 16 * (size_t)ncells, false, 0, s)) return fail(ctx, GBFMM_ENOMEM, "adaptive cells");
     const float4 *geom = A.geom.as<float4>();
-    launch_cell_geom(R.cells(), A.level.as<int32_t>(), A.key.as<uint64_t>(), box, A.geom.as<float4>(), s);
-    for (int l = 0; l <= maxl; ++l) {
-        const Span lv = R.level(l);
-        if (lv.cap <= 0) continue;
-        k_colleagues<<<blocks_for(lv.cap), 256, 0, s>>>(lv, l, A.key.as<uint64_t>(), A.parent.as<int32_t>(),
-                                                       A.child_of.as<int32_t>(), A.coll.as<int32_t>());
+    const Span cs = R.cells();
+    if (!leaves_of) {  // the one-pass build has written the geometry and boxes with the links
+        if (!cell_aux(ncells)) return fail(ctx, GBFMM_ENOMEM, "adaptive cells");
+        launch_cell_geom(cs, A.level.as<int32_t>(), A.key.as<uint64_t>(), box, A.geom.as<float4>(), s);
+        if (ncells > 0) {
+            k_cell_anchor<<<blocks_for(ncells), 256, 0, s>>>(cs, A.level.as<int32_t>(), A.key.as<uint64_t>(),
+                                                            A.anchor.as<int4>());
+            note_launches(1);
+        }
+    }
+    const unsigned g8 = blocks_for(ncells, 8);
+    if (leaves_of && ncells > 0 && ncells < kColleagueFindCells) {
+        k_colleagues_find<<<g8, 256, 0, s>>>(cs, info, A.level.as<int32_t>(), A.key.as<uint64_t>(),
+                                             A.coll.as<int32_t>());
         note_launches(1);
+    } else {
+        for (int l = 0; l <= maxl; ++l) {
+            const Span lv = R.level(l);
+            if (lv.cap <= 0) continue;
+            k_colleagues<<<blocks_for(lv.cap), 256, 0, s>>>(lv, l, A.key.as<uint64_t>(), A.parent.as<int32_t>(),
+                                                           A.child_of.as<int32_t>(), A.coll.as<int32_t>());
+            note_launches(1);
+        }
     }
 
-    // ---- lists: counts and offsets of the four kinds, one host read of their sizes (or a device
-    // check against the capacities), fills ----
-    if (grow(A.scan_tmp, 4 * (exclusive_scan_tmp_words(ncells + 1) + 64), false, 0, s))
+    // ---- lists: counts and offsets, one host read of their sizes (or a device check against the
+    // capacities), fills.  The block M2L reads no V list: V rows are built for the treecode and the
+    // M2L forms that walk them, and by gbfmm_export_lists on demand ----
+    if (grow(A.scan_tmp, 4 * (4 * exclusive_scan_tmp_words(ncells + 1) + 64), false, 0, s))
         return fail(ctx, GBFMM_ENOMEM, "adaptive scan");
-    if (grow(A.anchor, 16 * (size_t)ncells, false, 0, s)) return fail(ctx, GBFMM_ENOMEM, "adaptive lists");
-    if (ncells > 0) {
-        k_cell_anchor<<<blocks_for(ncells), 256, 0, s>>>(R.cells(), A.level.as<int32_t>(), A.key.as<uint64_t>(),
-                                                        A.anchor.as<int4>());
-        note_launches(1);
-    }
+    const bool cores = (prm->flags & GBFMM_FLAG_M2L_CUDA_CORES) != 0;
+    const bool gathered = (prm->flags & GBFMM_FLAG_M2L_GATHERED) != 0;
+    const bool vrows = prm->method == GBFMM_METHOD_TREECODE || cores || gathered;
+    A.v_rows = vrows;
     TreeView tv{A.level.as<int32_t>(), A.parent.as<int32_t>(), A.nchild.as<int32_t>(), A.child_of.as<int32_t>(),
                 A.coll.as<int32_t>(), A.key.as<uint64_t>(), A.anchor.as<int4>()};
-    const unsigned g8 = blocks_for(ncells, 8);
     // U, W, X rows: a warp per cell while the tree is small (latency: the 27 colleague slots in
     // parallel), a thread per cell on large trees (throughput)
     const bool warp_rows = ncells < kListWarpCells;
-    const Span cs = R.cells();
-    auto launch_alist = [&](int k, bool fill, uint32_t *cnt, const uint32_t *offs, int32_t *ids) {
-        const unsigned gt = blocks_for(ncells, 128);
-#define GB_ALIST(KIND, FILL)                                                                               \
-    (warp_rows ? k_alist_warp<KIND, FILL><<<g8, 256, 0, s>>>(cs, tv, cnt, offs, ids, ctx->d_status)        \
-               : k_alist_thread<KIND, FILL><<<gt, 128, 0, s>>>(cs, tv, cnt, offs, ids, ctx->d_status))
-        if (k == kListU) {
-            if (fill) GB_ALIST(kListU, true); else GB_ALIST(kListU, false);
-        } else if (k == kListW) {
-            if (fill) GB_ALIST(kListW, true); else GB_ALIST(kListW, false);
-        } else {
-            if (fill) GB_ALIST(kListX, true); else GB_ALIST(kListX, false);
-        }
-#undef GB_ALIST
-        note_launches(1);
-    };
-    for (int k = 0; k < 4; ++k) {
-        if (grow(A.lcnt[k], 4 * (ncells + 1), false, 0, s) || grow(A.loffs[k], 4 * (ncells + 1), false, 0, s))
+    for (int k = 0; k < 4; ++k)
+        if ((k != kListV || vrows) &&
+            (grow(A.lcnt[k], 4 * (ncells + 1), false, 0, s) || grow(A.loffs[k], 4 * (ncells + 1), false, 0, s)))
             return fail(ctx, GBFMM_ENOMEM, "adaptive lists");
-        uint32_t *cnt = A.lcnt[k].as<uint32_t>();
-        if (dev) cudaMemsetAsync(cnt, 0, 4 * (ncells + 1), s);  // rows past the cells stay empty
-        if (ncells > 0) {
-            if (k == kListV)
-                k_vlist_warp<false><<<g8, 256, 0, s>>>(cs, tv, cnt, nullptr, nullptr, nullptr);
-            else
-                launch_alist(k, false, cnt, nullptr, nullptr);
+    ListRows rows{A.lcnt[kListU].as<uint32_t>(),  A.lcnt[kListW].as<uint32_t>(),  A.lcnt[kListX].as<uint32_t>(),
+                  A.loffs[kListU].as<uint32_t>(), A.loffs[kListW].as<uint32_t>(), A.loffs[kListX].as<uint32_t>(),
+                  nullptr, nullptr, nullptr};
+    ScanJobs jobs{};
+    int njobs = 0;
+    for (int k : {kListU, kListW, kListX, kListV})
+        if (k != kListV || vrows)
+            jobs.j[njobs++] = {A.lcnt[k].as<uint32_t>(), A.loffs[k].as<uint32_t>(), info + kInfoLists + k};
+    if (ncells > 0) {
+        if (warp_rows)
+            k_alist_warp<false><<<g8, 256, 0, s>>>(cs, tv, rows, ctx->d_status);
+        else
+            k_alist_thread<false><<<blocks_for(ncells, 128), 128, 0, s>>>(cs, tv, rows, ctx->d_status);
+        note_launches(1);
+        if (vrows) {
+            k_vlist_warp<false><<<g8, 256, 0, s>>>(cs, tv, A.lcnt[kListV].as<uint32_t>(), nullptr, nullptr, nullptr);
+            note_launches(1);
         }
-        launch_exclusive_scan(A.lcnt[k].as<uint32_t>(), A.loffs[k].as<uint32_t>(), ncells,
-                              A.scan_tmp.as<uint32_t>(), s);
     }
-    k_list_totals<<<1, 32, 0, s>>>(ncells, A.loffs[0].as<uint32_t>(), A.loffs[1].as<uint32_t>(),
-                                   A.loffs[2].as<uint32_t>(), A.loffs[3].as<uint32_t>(), info + kInfoLists);
-    note_launches(1);
+    launch_exclusive_scans(jobs, njobs, ncells, A.scan_tmp.as<uint32_t>(), s);
     if (!dev) {
         int32_t ltot[4];
         cudaMemcpyAsync(ltot, info + kInfoLists, sizeof(ltot), cudaMemcpyDeviceToHost, s);
         cudaStreamSynchronize(s);
-        for (int k = 0; k < 4; ++k) A.entries[k] = (uint32_t)ltot[k];
+        for (int k = 0; k < 4; ++k) A.entries[k] = k != kListV || vrows ? (int64_t)(uint32_t)ltot[k] : 0;
     } else {
         GuardCaps g{};
-        for (int k = 0; k < 4; ++k) g.v[k] = A.entries[k] = caps->list[k];
+        for (int k = 0; k < 4; ++k) {
+            A.entries[k] = k != kListV || vrows ? caps->list[k] : 0;
+            g.v[k] = k != kListV || vrows ? caps->list[k] : INT64_MAX;
+        }
         k_guard<<<1, 32, 0, s>>>(info, g, 1, info + kInfoAbort, ctx->d_status);
         note_launches(1);
     }
     for (int k = 0; k < 4; ++k) {
-        const int64_t ne = A.entries[k];
-        if (grow(A.lids[k], 4 * (size_t)ne + 4, false, 0, s)) return fail(ctx, GBFMM_ENOMEM, "adaptive lists");
-        if (k == kListV && grow(A.vcode, 2 * (size_t)ne + 4, false, 0, s))
+        const size_t ne = (size_t)A.entries[k];
+        if (grow(A.lids[k], 4 * ne + 4, false, 0, s) || (k == kListV && vrows && grow(A.vcode, 2 * ne + 4, false, 0, s)))
             return fail(ctx, GBFMM_ENOMEM, "adaptive lists");
-        if (ncells == 0) continue;
-        const uint32_t *offs = A.loffs[k].as<uint32_t>();
-        int32_t *ids = A.lids[k].as<int32_t>();
-        if (k == kListV)
-            k_vlist_warp<true><<<g8, 256, 0, s>>>(cs, tv, nullptr, offs, ids, A.vcode.as<uint16_t>());
+    }
+    rows.u_ids = A.lids[kListU].as<int32_t>();
+    rows.w_ids = A.lids[kListW].as<int32_t>();
+    rows.x_ids = A.lids[kListX].as<int32_t>();
+    if (ncells > 0) {
+        if (warp_rows)
+            k_alist_warp<true><<<g8, 256, 0, s>>>(cs, tv, rows, ctx->d_status);
         else
-            launch_alist(k, true, nullptr, offs, ids);
+            k_alist_thread<true><<<blocks_for(ncells, 128), 128, 0, s>>>(cs, tv, rows, ctx->d_status);
+        note_launches(1);
+        if (vrows) {
+            k_vlist_warp<true><<<g8, 256, 0, s>>>(cs, tv, nullptr, A.loffs[kListV].as<uint32_t>(),
+                                                  A.lids[kListV].as<int32_t>(), A.vcode.as<uint16_t>());
+            note_launches(1);
+        }
     }
     mark(3);
     A.n = n;
@@ -1264,8 +1334,6 @@ int evaluate_adaptive_in(gbfmm_ctx *ctx, AdaptiveState &A, const AdaptCaps *caps
     for (int l = maxl - 1; l >= 2; --l)
         launch_translate_cells(P, true, R.level(l), A.child_of.as<int32_t>(), A.nchild.as<int32_t>(), ops.m2m, M, s);
     mark(5);
-    const bool cores = (prm->flags & GBFMM_FLAG_M2L_CUDA_CORES) != 0;
-    const bool gathered = (prm->flags & GBFMM_FLAG_M2L_GATHERED) != 0;
     if (deep && !cores && !gathered) {
         // M2L in block form: one GEMM per parent offset over the units (cells with children),
         // their colleagues' children gathered per tile; no V list is read
@@ -1359,7 +1427,7 @@ int evaluate_adaptive_in(gbfmm_ctx *ctx, AdaptiveState &A, const AdaptCaps *caps
             cudaStreamWaitEvent(s, ctx->ev_near, 0);
             if (timing) cudaEventRecord(ctx->ev_aux[2], s);
         }
-        launch_l2p_cells(P, n, A.leaf_of.as<int32_t>(), A.level.as<int32_t>(), geom, A.sx.as<float4>(), Lc, far, s,
+        launch_l2p_cells(P, n, A.leaf_of.as<int32_t>(), leaves_of, A.level.as<int32_t>(), geom, A.sx.as<float4>(), Lc, far, s,
                          near, perm, reinterpret_cast<float4 *>(d_out), abort);
         mark(9);
         if (fork) {
@@ -1368,7 +1436,7 @@ int evaluate_adaptive_in(gbfmm_ctx *ctx, AdaptiveState &A, const AdaptCaps *caps
             s = s_main;
         }
     } else {
-        launch_l2p_cells(P, n, A.leaf_of.as<int32_t>(), A.level.as<int32_t>(), geom, A.sx.as<float4>(), Lc, far, s,
+        launch_l2p_cells(P, n, A.leaf_of.as<int32_t>(), leaves_of, A.level.as<int32_t>(), geom, A.sx.as<float4>(), Lc, far, s,
                          nullptr, nullptr, nullptr, abort);
         if (deep)
             launch_m2p_cells(P, A.leaves.as<int32_t>(), R.leaves(), geom, A.begin.as<int32_t>(),
@@ -1447,8 +1515,29 @@ int export_adaptive_expansions(gbfmm_ctx *ctx, int which, double *coef)
 
 int export_adaptive_list(gbfmm_ctx *ctx, int kind, int32_t *offs, int32_t *ids, int64_t cap, int64_t *n_entries)
 {
-    const AdaptiveState &A = ctx->ad;
+    AdaptiveState &A = ctx->ad;
     const int64_t rows = A.ncells;
+    if (kind == kListV && !A.v_rows) {  // the evaluation's block M2L read no V list: build the rows now
+        const cudaStream_t s = nullptr;
+        const TreeView tv{A.level.as<int32_t>(), A.parent.as<int32_t>(), A.nchild.as<int32_t>(),
+                          A.child_of.as<int32_t>(), A.coll.as<int32_t>(), A.key.as<uint64_t>(), A.anchor.as<int4>()};
+        if (grow(A.lcnt[kListV], 4 * (rows + 1), false, 0, s) || grow(A.loffs[kListV], 4 * (rows + 1), false, 0, s))
+            return fail(ctx, GBFMM_ENOMEM, "V list export");
+        const Span cs = host_span(0, rows);
+        const unsigned g8 = blocks_for(rows, 8);
+        uint32_t *cnt = A.lcnt[kListV].as<uint32_t>(), *vo = A.loffs[kListV].as<uint32_t>();
+        if (rows > 0) k_vlist_warp<false><<<g8, 256, 0, s>>>(cs, tv, cnt, nullptr, nullptr, nullptr);
+        launch_exclusive_scan(cnt, vo, rows, A.scan_tmp.as<uint32_t>(), s);
+        const size_t ne = read1<uint32_t>(vo + rows, s);
+        if (grow(A.lids[kListV], 4 * ne + 4, false, 0, s) || grow(A.vcode, 2 * ne + 4, false, 0, s))
+            return fail(ctx, GBFMM_ENOMEM, "V list export");
+        if (rows > 0)
+            k_vlist_warp<true><<<g8, 256, 0, s>>>(cs, tv, nullptr, vo, A.lids[kListV].as<int32_t>(),
+                                                  A.vcode.as<uint16_t>());
+        const cudaError_t e = cudaDeviceSynchronize();
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "V list export");
+        A.v_rows = true;
+    }
     std::vector<uint32_t> o(rows + 1);
     cudaMemcpy(o.data(), A.loffs[kind].p, 4 * (rows + 1), cudaMemcpyDeviceToHost);
     const int64_t ne = o[rows];

@@ -251,6 +251,25 @@ GB_DEV uint32_t grid_coord21(float c, const Box &b, int d)
 constexpr int kGeoLevels = 22;
 inline size_t geo_floats(int L) { return kGeoLevels + 3 * ((size_t(2) << L) - 1); }
 
+// A cell's centre and the inverse of its side: FP64 expressions rounded once to FP32.
+struct CellGeom {
+    float cx, cy, cz, inv_h;
+};
+
+// the level-l cell with 63-bit-key prefix `key`
+GB_DEV CellGeom cell_geom63(const Box &b, int l, uint64_t key)
+{
+    int ix, iy, iz;
+    demorton63(key, ix, iy, iz);
+    double h = b.side / (double)(int64_t(1) << l);
+    CellGeom g;
+    g.cx = (float)(b.origin[0] + (ix + 0.5) * h);
+    g.cy = (float)(b.origin[1] + (iy + 0.5) * h);
+    g.cz = (float)(b.origin[2] + (iz + 0.5) * h);
+    g.inv_h = (float)(1.0 / h);
+    return g;
+}
+
 // Layout of one evaluation's workspace (byte offsets from the workspace base).
 struct Layout {
     int64_t n;
@@ -297,6 +316,17 @@ constexpr size_t sort_scratch_bytes(int64_t n, int bits)
 void launch_sort_gather(uint32_t *k0, uint32_t *k1, uint32_t *v0, uint32_t *v1, int64_t n, int bits, void *scratch,
                         int *err, const float4 *x, float4 *sx, uint32_t **keys_out, uint32_t **idx_out,
                         cudaStream_t s);
+// exclusive scans of up to four arrays of n values each: out[n] (and *total, if given) = the sum
+struct ScanJob {
+    const uint32_t *in = nullptr;
+    uint32_t *out = nullptr;
+    int32_t *total = nullptr;
+};
+struct ScanJobs {
+    ScanJob j[4];
+};
+// tmp: exclusive_scan_tmp_words(n) words per array
+void launch_exclusive_scans(const ScanJobs &jobs, int count, int64_t n, uint32_t *tmp, cudaStream_t s);
 void launch_exclusive_scan(const uint32_t *in, uint32_t *out, int64_t n, uint32_t *tmp, cudaStream_t s);
 size_t exclusive_scan_tmp_words(int64_t n);
 void launch_cells(const uint32_t *sorted_leaf_keys, int64_t n, int L, int32_t *begin, int32_t *end, cudaStream_t s);
@@ -375,7 +405,8 @@ void launch_p2l_cells(int P, Span cells, const int32_t *level, const float4 *geo
                       cudaStream_t s);
 // near != nullptr: far holds the M2P sums; the local expansion's value, those and the near-field
 // sums are added and written to out[perm[i]].  Nothing runs once *abort is nonzero.
-void launch_l2p_cells(int P, int64_t n, const int32_t *leaf_of, const int32_t *level, const float4 *geom,
+// Particle i's leaf is leaves[leaf_of[i]], or leaf_of[i] itself with leaves == nullptr.
+void launch_l2p_cells(int P, int64_t n, const int32_t *leaf_of, const int32_t *leaves, const int32_t *level, const float4 *geom,
                       const float4 *sx, const float *Lc, float4 *far, cudaStream_t s, const float4 *near = nullptr,
                       const uint32_t *perm = nullptr, float4 *out = nullptr, const int32_t *abort = nullptr);
 // long_rows: the treecode's chain rows (the warp kernel, k_m2p_warp); else the FMM's short W

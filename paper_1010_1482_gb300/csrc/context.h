@@ -64,6 +64,7 @@ struct AdaptiveState {
     AdaptCaps counts;  // the sizes the last host-counted evaluation read back
     int64_t n = 0, ncells = 0, nleaves = 0, entries[4] = {0, 0, 0, 0};
     int P = 0, max_level = 0;
+    bool v_rows = false;  // the V rows are built (the block M2L reads none)
     std::vector<int> level_start;
     uint64_t *skeys = nullptr;
     uint32_t *perm = nullptr;

@@ -437,9 +437,6 @@ int build_m2l_rot_table(int P, std::vector<float> &out)
 // ------------------------------------------------------------------------------------------
 // FP32 helpers
 // ------------------------------------------------------------------------------------------
-struct CellGeom {
-    float cx, cy, cz, inv_h;
-};
 
 // ------------------------------------------------------------------------------------------
 // Cell geometry tables.  The centre of a level-l cell with integer coordinates (ix, iy, iz) is
@@ -1354,19 +1351,6 @@ void launch_m2p(int P, int L, const float *geo, const float4 *sx, const int32_t 
 // ==========================================================================================
 // Adaptive tree: cells are given by index; each carries its level and 63-bit key prefix.
 // ==========================================================================================
-GB_DEV CellGeom cell_geom63(const Box &b, int l, uint64_t key)
-{
-    int ix, iy, iz;
-    demorton63(key, ix, iy, iz);
-    double h = b.side / (double)(int64_t(1) << l);
-    CellGeom g;
-    g.cx = (float)(b.origin[0] + (ix + 0.5) * h);
-    g.cy = (float)(b.origin[1] + (iy + 0.5) * h);
-    g.cz = (float)(b.origin[2] + (iz + 0.5) * h);
-    g.inv_h = (float)(1.0 / h);
-    return g;
-}
-
 __global__ void k_cell_geom(Span cells, const int32_t *__restrict__ level, const uint64_t *__restrict__ key,
                             const Box *__restrict__ box, float4 *__restrict__ geom)
 {
@@ -1437,6 +1421,7 @@ __global__ void __launch_bounds__(128) k_p2l_cells(Span cells, const int32_t *__
 // L2P at every particle's leaf (leaves above level 2 carry no local expansion)
 template <int P>
 __global__ void __launch_bounds__(128) k_l2p_cells(int64_t n, const int32_t *__restrict__ leaf_of,
+                                                   const int32_t *__restrict__ leaves,
                                                    const int32_t *__restrict__ level, const float4 *__restrict__ geom,
                                                    const float4 *__restrict__ sx, const float *__restrict__ Lc,
                                                    float4 *__restrict__ far, const float4 *__restrict__ near,
@@ -1445,7 +1430,7 @@ __global__ void __launch_bounds__(128) k_l2p_cells(int64_t n, const int32_t *__r
 {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n || (abort && *abort)) return;
-    const int32_t c = leaf_of[i];
+    const int32_t lo = leaf_of[i], c = leaves ? leaves[lo] : lo;
     float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
     if (level[c] >= 2) {
         const CellGeom cg = geo_cell(geom, c);
@@ -1654,13 +1639,13 @@ void launch_p2l_cells(int P, Span cells, const int32_t *level, const float4 *geo
     note_launches(1);
 }
 
-void launch_l2p_cells(int P, int64_t n, const int32_t *leaf_of, const int32_t *level, const float4 *geom,
+void launch_l2p_cells(int P, int64_t n, const int32_t *leaf_of, const int32_t *leaves, const int32_t *level, const float4 *geom,
                       const float4 *sx, const float *Lc, float4 *far, cudaStream_t s, const float4 *near,
                       const uint32_t *perm, float4 *out, const int32_t *abort)
 {
     if (n <= 0) return;
     const unsigned grid = (unsigned)((n + 127) / 128);
-    GBFMM_DISPATCH_P(P, (k_l2p_cells<PQ><<<grid, 128, 0, s>>>(n, leaf_of, level, geom, sx, Lc, far, near, perm, out,
+    GBFMM_DISPATCH_P(P, (k_l2p_cells<PQ><<<grid, 128, 0, s>>>(n, leaf_of, leaves, level, geom, sx, Lc, far, near, perm, out,
                                                               abort)));
     note_launches(1);
 }

@@ -217,9 +217,12 @@ constexpr int kScanThreads = 256, kScanItems = 8, kScanTile = kScanThreads * kSc
 
 size_t exclusive_scan_tmp_words(int64_t n) { return (size_t)((n + kScanTile - 1) / kScanTile) + 1; }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_reduce(const uint32_t *__restrict__ in, int64_t n,
-                                                              uint32_t *__restrict__ part)
+// The launches cover up to four arrays of the same length (blockIdx.y); a job's `total`, if given,
+// receives the sum as well.  tmp holds exclusive_scan_tmp_words(n) words per job.
+__global__ void __launch_bounds__(kScanThreads) k_scan_reduce(ScanJobs jobs, int64_t n, uint32_t *__restrict__ tmp,
+                                                              int64_t tmp_words)
 {
+    const uint32_t *__restrict__ in = jobs.j[blockIdx.y].in;
     int64_t base = blockIdx.x * (int64_t)kScanTile;
     uint32_t s = 0;
 #pragma unroll
@@ -235,54 +238,88 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_reduce(const uint32_t *__
     if (threadIdx.x == 0) {
         uint32_t t = 0;
         for (int w = 0; w < kScanThreads / 32; ++w) t += ws[w];
-        part[blockIdx.x] = t;
+        tmp[blockIdx.y * tmp_words + blockIdx.x] = t;
     }
 }
 
-// single block: exclusive scan of the nb block sums in place; total to *total
-__global__ void __launch_bounds__(1024) k_scan_partials(uint32_t *part, int64_t nb, uint32_t *total)
+// one CTA per job: exclusive scan of src[0, n) into dst (src == dst allowed), four values a thread
+// and round, the next round's loads in flight while the current one is scanned; the sum to
+// *sum (dst + n, or elsewhere) and *total
+GB_DEV void scan_by_block(const uint32_t *src, uint32_t *dst, int64_t n, uint32_t *sum, int32_t *total)
 {
-    __shared__ uint32_t ws[32];
-    __shared__ uint32_t carry;
-    if (threadIdx.x == 0) carry = 0;
-    __syncthreads();
+    constexpr int kRound = 4 * 1024;
+    __shared__ uint32_t ws[2][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int64_t base = 0; base < nb; base += 1024) {
-        int64_t i = base + threadIdx.x;
-        uint32_t v = (i < nb) ? part[i] : 0u;
-        uint32_t incl = v;
+    uint32_t carry = 0;
+    uint32_t v[4];
+    auto load = [&](int64_t base) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int64_t i = base + 4 * threadIdx.x + k;
+            v[k] = i < n ? src[i] : 0u;
+        }
+    };
+    load(0);
+    int buf = 0;
+    for (int64_t base = 0; base < n; base += kRound, buf ^= 1) {
+        uint32_t c[4], s = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            c[k] = s;
+            s += v[k];
+        }
+        load(base + kRound);
+        uint32_t incl = s;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+            const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
             if (lane >= o) incl += t;
         }
-        if (lane == 31) ws[warp] = incl;
+        if (lane == 31) ws[buf][warp] = incl;
         __syncthreads();
-        if (warp == 0) {
-            uint32_t w = ws[lane];
-            uint32_t wi = w;
+        const uint32_t w = ws[buf][lane];
+        uint32_t wi = w;
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                uint32_t t = __shfl_up_sync(0xffffffffu, wi, o);
-                if (lane >= o) wi += t;
-            }
-            ws[lane] = wi - w;  // exclusive prefix of warp totals
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(0xffffffffu, wi, o);
+            if (lane >= o) wi += t;
         }
-        __syncthreads();
-        uint32_t c = carry;
-        if (i < nb) part[i] = c + ws[warp] + incl - v;
-        __syncthreads();
-        if (threadIdx.x == 1023) carry = c + ws[warp] + incl;
-        __syncthreads();
+        const uint32_t before = carry + __shfl_sync(0xffffffffu, wi - w, warp) + incl - s;
+        carry += __shfl_sync(0xffffffffu, wi, 31);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int64_t i = base + 4 * threadIdx.x + k;
+            if (i < n) dst[i] = before + c[k];
+        }
     }
-    if (threadIdx.x == 0 && total) *total = carry;
+    if (threadIdx.x == 0) {
+        *sum = carry;
+        if (total) *total = (int32_t)carry;
+    }
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_apply(const uint32_t *in, uint32_t *out, int64_t n,
-                                                             const uint32_t *__restrict__ part)
+// the scan of a job's block sums; the sum to out[n]
+__global__ void __launch_bounds__(1024) k_scan_partials(ScanJobs jobs, int64_t n, uint32_t *tmp, int64_t tmp_words,
+                                                        int64_t nb)
+{
+    uint32_t *part = tmp + blockIdx.x * tmp_words;
+    scan_by_block(part, part, nb, jobs.j[blockIdx.x].out + n, jobs.j[blockIdx.x].total);
+}
+
+// a whole job by one CTA (small n)
+__global__ void __launch_bounds__(1024) k_scan_one(ScanJobs jobs, int64_t n)
+{
+    const ScanJob j = jobs.j[blockIdx.x];
+    scan_by_block(j.in, j.out, n, j.out + n, j.total);
+}
+
+__global__ void __launch_bounds__(kScanThreads) k_scan_apply(ScanJobs jobs, int64_t n, const uint32_t *__restrict__ tmp,
+                                                             int64_t tmp_words)
 {
     __shared__ uint32_t tile[kScanTile];
     __shared__ uint32_t ws[kScanThreads / 32];
+    const uint32_t *in = jobs.j[blockIdx.y].in;
+    uint32_t *out = jobs.j[blockIdx.y].out;
     int64_t base = blockIdx.x * (int64_t)kScanTile;
 #pragma unroll
     for (int r = 0; r < kScanItems; ++r) {
@@ -308,7 +345,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_apply(const uint32_t *in,
     __syncthreads();
     uint32_t wpre = 0;
     for (int w = 0; w < warp; ++w) wpre += ws[w];
-    uint32_t pre = part[blockIdx.x] + wpre + incl - s;
+    uint32_t pre = tmp[blockIdx.y * tmp_words + blockIdx.x] + wpre + incl - s;
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < kScanItems; ++k) tile[threadIdx.x * kScanItems + k] = pre + loc[k];
@@ -320,17 +357,28 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_apply(const uint32_t *in,
     }
 }
 
-void launch_exclusive_scan(const uint32_t *in, uint32_t *out, int64_t n, uint32_t *tmp, cudaStream_t s)
+// up to here one CTA scans the whole array: up to four rounds of loads in one launch instead of
+// three launches one after another (@@)
+constexpr int64_t kScanOneN = 16384;
+
+void launch_exclusive_scans(const ScanJobs &jobs, int count, int64_t n, uint32_t *tmp, cudaStream_t s)
 {
-    int64_t nb = (n + kScanTile - 1) / kScanTile;
-    if (nb == 0) {
-        cudaMemsetAsync(out, 0, sizeof(uint32_t), s);
+    if (n <= kScanOneN) {
+        k_scan_one<<<count, 1024, 0, s>>>(jobs, n);
+        note_launches(1);
         return;
     }
-    k_scan_reduce<<<(unsigned)nb, kScanThreads, 0, s>>>(in, n, tmp);
-    k_scan_partials<<<1, 1024, 0, s>>>(tmp, nb, out + n);
-    k_scan_apply<<<(unsigned)nb, kScanThreads, 0, s>>>(in, out, n, tmp);
+    const int64_t nb = (n + kScanTile - 1) / kScanTile, tw = (int64_t)exclusive_scan_tmp_words(n);
+    const dim3 grid((unsigned)nb, (unsigned)count);
+    k_scan_reduce<<<grid, kScanThreads, 0, s>>>(jobs, n, tmp, tw);
+    k_scan_partials<<<count, 1024, 0, s>>>(jobs, n, tmp, tw, nb);
+    k_scan_apply<<<grid, kScanThreads, 0, s>>>(jobs, n, tmp, tw);
     note_launches(3);
+}
+
+void launch_exclusive_scan(const uint32_t *in, uint32_t *out, int64_t n, uint32_t *tmp, cudaStream_t s)
+{
+    launch_exclusive_scans(ScanJobs{{{in, out, nullptr}}}, 1, n, tmp, s);
 }
 
 // ------------------------------------------------------------------------------------------
