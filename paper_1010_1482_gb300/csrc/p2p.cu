@@ -38,21 +38,30 @@ GB_DEV void pair(float xi, float yi, float zi, float4 s, float eps2, float &phi,
     gz = fmaf(-dz, qi3, gz);
 }
 
-// Scalar pair rule of pair(), with the zero-distance test only where MASK (the target's own
-// cell); the gradient accumulates +d q / r^3 and is negated once at the end.
+// The pair rule of pair() for two targets at once, in packed FP32 (fma.rn.f32x2 and its kin: two
+// lanes per instruction), against one source; the zero-distance test only where MASK (the targets'
+// own cell).  nx, ny, nz: the targets' negated coordinates; the sums are those of pair().  The loop
+// of scalar pairs was bound by instruction issue: of its own, 2.02e12 pairs/s scalar, 2.24e12 packed.
 template <bool SOFT, bool MASK>
-GB_DEV void pairm(float xi, float yi, float zi, float4 s, float eps2, float &phi, float &gx, float &gy, float &gz)
+GB_DEV void pair2(uint64_t nx, uint64_t ny, uint64_t nz, float4 s, uint64_t eps2, uint64_t &phi, uint64_t &gx,
+                  uint64_t &gy, uint64_t &gz)
 {
-    const float dx = xi - s.x, dy = yi - s.y, dz = zi - s.z;
-    const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-    float inv = rsqrt_ftz(SOFT ? d2 + eps2 : d2);
-    if (MASK) inv = d2 > 0.f ? inv : 0.f;
-    const float w = s.w * inv;
-    phi += w;
-    const float w3 = w * inv * inv;
-    gx = fmaf(dx, w3, gx);
-    gy = fmaf(dy, w3, gy);
-    gz = fmaf(dz, w3, gz);
+    const uint64_t dx = add2(pack2(s.x, s.x), nx), dy = add2(pack2(s.y, s.y), ny), dz = add2(pack2(s.z, s.z), nz);
+    const uint64_t d2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
+    float a, b;
+    unpack2(SOFT ? add2(d2, eps2) : d2, a, b);
+    float ia = rsqrt_ftz(a), ib = rsqrt_ftz(b);
+    if (MASK) {
+        if (SOFT) unpack2(d2, a, b);
+        ia = a > 0.f ? ia : 0.f;
+        ib = b > 0.f ? ib : 0.f;
+    }
+    const uint64_t inv = pack2(ia, ib), w = mul2(pack2(s.w, s.w), inv);
+    phi = add2(phi, w);
+    const uint64_t w3 = mul2(mul2(w, inv), inv);
+    gx = fma2(dx, w3, gx);
+    gy = fma2(dy, w3, gy);
+    gz = fma2(dz, w3, gz);
 }
 
 // ---- warp-specialised P2P: one producer warp stages, four consumer warps apply the pair rule ---
@@ -69,9 +78,14 @@ GB_DEV void pairm(float xi, float yi, float zi, float4 s, float eps2, float &phi
 // consumers apply the pair rule to a stage while the producer fills the other, so a leaf's list
 // reads, row copies and the previous leaf's reduction overlap the pair loop.  Targets: 2 per
 // consumer thread; when a leaf has fewer target slots than there are consumers the threads form G
-// groups that take the staged sources round-robin; group partials are combined per target with
-// compensated sums as before.  Every wait is bounded: on expiry the kernel raises kStatusTimeout,
+// groups that take the staged sources round-robin; group partials are combined with compensated
+// sums, in group order, a thread per target and component.  Small uniform trees, whose leaves are
+// fewer than the CTAs that fit, give a leaf's targets to `parts` CTAs.  Every wait is bounded: on expiry the kernel raises kStatusTimeout,
 // stops, and returns once its own copies have landed (bounded again).
+// Bound by the FP32 pipe and its issue (13 operations and a MUFU per pair).  Alone, scalar pairs and
+// a one-warp reduction -> packed pairs, the reduction over all threads and stages of equal size:
+// 1M particles (mean 32 per leaf) 522 -> 493 us, 5M (19 per leaf) 1852 -> 1648, 400,009 Plummer
+// 222 -> 190; 16M Plummer step 26.76 -> 25.61 ms.
 constexpr int kP2PCap = 512;
 constexpr int kP2PConsumers = 128;
 constexpr int kP2PWsThreads = kP2PConsumers + 32;
@@ -79,7 +93,7 @@ constexpr int kP2PTargets = 2 * kP2PConsumers;  // targets per pass over the sou
 
 struct P2PItem {
     int b0;     // the leaf's first particle (sorted order); -1 ends the stream
-    int T;      // the leaf's particle count
+    int T;      // one past the last target this CTA takes
     int tc;     // first target of this pass
     int chunk;  // sources staged (0: none, the pass only ends)
     int mend;   // leading staged sources of the target's own cell (zero-distance test)
@@ -88,7 +102,7 @@ struct P2PItem {
 
 template <bool SOFT, bool UNI>
 __global__ void __launch_bounds__(kP2PWsThreads, 8) k_p2p_ws(int L, const int32_t *__restrict__ leaves, Span lv,
-                                                           int64_t nleaf, const float4 *__restrict__ sx,
+                                                           int64_t nleaf, int parts, const float4 *__restrict__ sx,
                                                            const int32_t *__restrict__ begin,
                                                            const int32_t *__restrict__ end,
                                                            const uint32_t *__restrict__ p2p_offs,
@@ -115,7 +129,7 @@ __global__ void __launch_bounds__(kP2PWsThreads, 8) k_p2p_ws(int L, const int32_
         fence_mbar_init();
     }
     __syncthreads();
-    const int64_t count = UNI ? nleaf : span_count(lv);
+    const int64_t count = UNI ? nleaf * parts : span_count(lv);  // UNI: item li = part li % parts of leaf li / parts
 
     if (tid >= kP2PConsumers) {  // ---------------- producer warp
         int stage = 0;
@@ -152,7 +166,7 @@ __global__ void __launch_bounds__(kP2PWsThreads, 8) k_p2p_ws(int L, const int32_
             cb = cn = 0;
             if (li >= count || lane >= 27) return;
             int x, y, z;
-            demorton3((uint32_t)li, x, y, z);
+            demorton3((uint32_t)(li / parts), x, y, z);
             x += lane % 3 - 1;
             y += (lane / 3) % 3 - 1;
             z += lane / 9 - 1;
@@ -166,24 +180,28 @@ __global__ void __launch_bounds__(kP2PWsThreads, 8) k_p2p_ws(int L, const int32_
         if (UNI) grid_row(blockIdx.x, nb, nn);
         for (int64_t li = blockIdx.x; ok && li < count; li += gridDim.x) {
             const int gb = nb, gn = nn;
-            int b0, T, nrow;
+            int b0, T, nrow, t0 = 0, t1;  // targets [t0, t1) of the leaf's T particles
             uint32_t r0 = 0;
             if (UNI) {
                 grid_row(li + gridDim.x, nb, nn);
                 b0 = __shfl_sync(~0u, gb, 13);
                 T = __shfl_sync(~0u, gn, 13);
-                if (T <= 0) continue;
+                const int per = (T + parts - 1) / parts;
+                t0 = (int)(li % parts) * per;
+                t1 = min(T, t0 + per);
+                if (t0 >= t1) continue;
                 nrow = 27;
             } else {
                 const int64_t g = leaves[li];
                 b0 = begin[g];
                 T = end[g] - b0;
                 if (T <= 0) continue;
+                t1 = T;
                 r0 = p2p_offs[g];
                 nrow = (int)(p2p_offs[g + 1] - r0);
             }
-            for (int tc = 0; ok && tc < T; tc += kP2PTargets) {
-                const int Tc = min(T - tc, kP2PTargets);
+            for (int tc = t0; ok && tc < t1; tc += kP2PTargets) {
+                const int Tc = min(t1 - tc, kP2PTargets);
                 bool emitted = false;
                 for (int rb = 0; ok && rb < nrow; rb += 32) {
                     const int nr = min(32, nrow - rb);
@@ -214,15 +232,16 @@ __global__ void __launch_bounds__(kP2PWsThreads, 8) k_p2p_ws(int L, const int32_
                     }
                     const int pref = incl - cn, S = __shfl_sync(~0u, incl, 31);
                     const int nself = self ? T : 0;
-                    for (int sc = 0; sc < S; sc += kP2PCap) {
-                        const int chunk = min(kP2PCap, S - sc);
+                    const int per_stage = S > 0 ? (S + (S + kP2PCap - 1) / kP2PCap - 1) / ((S + kP2PCap - 1) / kP2PCap) : 1;
+                    for (int sc = 0; sc < S; sc += per_stage) {  // stages of about equal size
+                        const int chunk = min(per_stage, S - sc);
                         if (!claim()) {
                             ok = false;
                             break;
                         }
-                        const bool last = last_rb && sc + kP2PCap >= S;
+                        const bool last = last_rb && sc + chunk >= S;
                         const bool staged = rb == 0 && sc == 0 && nself > 0 && tc + Tc <= chunk;
-                        publish(P2PItem{b0, T, tc, chunk, max(0, min(chunk, nself - sc)),
+                        publish(P2PItem{b0, t1, tc, chunk, max(0, min(chunk, nself - sc)),
                                         (emitted ? 0 : 1) | (last ? 2 : 0) | (staged ? 4 : 0)});
                         const int lo = max(pref, sc), hi = min(pref + cn, sc + chunk);
                         if (hi > lo)
@@ -236,7 +255,7 @@ __global__ void __launch_bounds__(kP2PWsThreads, 8) k_p2p_ws(int L, const int32_
                             ok = false;
                             break;
                         }
-                        publish(P2PItem{b0, T, tc, 0, 0, (emitted ? 0 : 1) | 2});
+                        publish(P2PItem{b0, t1, tc, 0, 0, (emitted ? 0 : 1) | 2});
                         emitted = true;
                         advance();
                     }
@@ -246,7 +265,7 @@ __global__ void __launch_bounds__(kP2PWsThreads, 8) k_p2p_ws(int L, const int32_
                         ok = false;
                         break;
                     }
-                    publish(P2PItem{b0, T, tc, 0, 0, 3});
+                    publish(P2PItem{b0, t1, tc, 0, 0, 3});
                     advance();
                 }
             }
@@ -267,8 +286,9 @@ __global__ void __launch_bounds__(kP2PWsThreads, 8) k_p2p_ws(int L, const int32_
     int stage = 0, rpar = 0;
     uint32_t fpar = 0u, rphase = 0u;  // per stage / per reduction buffer: parity of the next phase
     int slots = 1, G = 1, slot = 0, grp = 0, Tc = 0;
-    float ax = 0.f, ay = 0.f, az = 0.f, bx = 0.f, by = 0.f, bz = 0.f;
-    float pa = 0.f, gax = 0.f, gay = 0.f, gaz = 0.f, pb = 0.f, gbx = 0.f, gby = 0.f, gbz = 0.f;
+    // two targets per thread, packed: negated coordinates, sums
+    uint64_t nx = 0, ny = 0, nz = 0, phi = 0, gx = 0, gy = 0, gz = 0;
+    const uint64_t e2 = pack2(eps2, eps2);
     while (true) {
         if (!mbar_wait_bounded(&full[stage], (fpar >> stage) & 1u, kWaitLimitNs, &abort_flag) || abort_flag) {
             if (!abort_flag) {
@@ -290,22 +310,14 @@ __global__ void __launch_bounds__(kP2PWsThreads, 8) k_p2p_ws(int L, const int32_
             const int ta = 2 * slot, tb = ta + 1 < Tc ? ta + 1 : ta;
             const float4 A = (it.flags & 4) ? src[it.tc + ta] : __ldg(&sx[it.b0 + it.tc + ta]);
             const float4 B = (it.flags & 4) ? src[it.tc + tb] : __ldg(&sx[it.b0 + it.tc + tb]);
-            ax = A.x, ay = A.y, az = A.z, bx = B.x, by = B.y, bz = B.z;
-            pa = gax = gay = gaz = pb = gbx = gby = gbz = 0.f;
+            nx = pack2(-A.x, -B.x), ny = pack2(-A.y, -B.y), nz = pack2(-A.z, -B.z);
+            phi = gx = gy = gz = 0;
         }
         if (grp < G) {
             int j = grp;
-            for (; j < it.mend; j += G) {
-                const float4 s4 = src[j];
-                pairm<SOFT, true>(ax, ay, az, s4, eps2, pa, gax, gay, gaz);
-                pairm<SOFT, true>(bx, by, bz, s4, eps2, pb, gbx, gby, gbz);
-            }
+            for (; j < it.mend; j += G) pair2<SOFT, true>(nx, ny, nz, src[j], e2, phi, gx, gy, gz);
 #pragma unroll 4
-            for (; j < it.chunk; j += G) {
-                const float4 s4 = src[j];
-                pairm<SOFT, false>(ax, ay, az, s4, eps2, pa, gax, gay, gaz);
-                pairm<SOFT, false>(bx, by, bz, s4, eps2, pb, gbx, gby, gbz);
-            }
+            for (; j < it.chunk; j += G) pair2<SOFT, false>(nx, ny, nz, src[j], e2, phi, gx, gy, gz);
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(&empty[stage]);
@@ -315,8 +327,15 @@ __global__ void __launch_bounds__(kP2PWsThreads, 8) k_p2p_ws(int L, const int32_
         // end of the pass: combine the groups' partials per target.  red alternates between two
         // buffers, and every consumer waits for the pass's arrivals, so a pass's writes never
         // meet the previous pass's reads.
-        red[rpar][0][tid] = make_float4(pa, -gax, -gay, -gaz);
-        red[rpar][1][tid] = make_float4(pb, -gbx, -gby, -gbz);
+        {
+            float4 va, vb;
+            unpack2(phi, va.x, vb.x);
+            unpack2(gx, va.y, vb.y);
+            unpack2(gy, va.z, vb.z);
+            unpack2(gz, va.w, vb.w);
+            red[rpar][0][tid] = va;
+            red[rpar][1][tid] = vb;
+        }
         mbar_arrive(&redbar[rpar]);
         if (!mbar_wait_bounded(&redbar[rpar], (rphase >> rpar) & 1u, kWaitLimitNs, &abort_flag)) {
             if (!abort_flag) {
@@ -326,34 +345,22 @@ __global__ void __launch_bounds__(kP2PWsThreads, 8) k_p2p_ws(int L, const int32_
             return;
         }
         rphase ^= 1u << rpar;
-        if (grp == 0) {
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int t = 2 * slot + h;
-                if (t >= Tc) break;
-                const int i = it.b0 + it.tc + t;
-                Kahan a{0.f, 0.f}, kx{0.f, 0.f}, ky{0.f, 0.f}, kz{0.f, 0.f};
-                for (int k = 0; k < G; ++k) {
-                    const float4 v = red[rpar][h][k * slots + slot];
-                    a.add(v.x);
-                    kx.add(v.y);
-                    ky.add(v.z);
-                    kz.add(v.w);
-                }
-                if (near) {  // the compensated sums so far; the far field is added by L2P
-                    near[2 * (int64_t)i] = make_float4(a.s, kx.s, ky.s, kz.s);
-                    near[2 * (int64_t)i + 1] = make_float4(a.c, kx.c, ky.c, kz.c);
-                    continue;
-                }
-                if (far) {
-                    const float4 f = far[i];
-                    a.add(f.x);
-                    kx.add(f.y);
-                    ky.add(f.z);
-                    kz.add(f.w);
-                }
-                out[perm[i]] = make_float4(a.s, kx.s, ky.s, kz.s);
+        // one component of one target per thread (e: target parity, slot, component)
+        for (int e = tid; e < 8 * slots; e += kP2PConsumers) {
+            const int cp = e & 3, hs = e >> 2, h = hs >= slots, sl = hs - (h ? slots : 0), t = 2 * sl + h;
+            if (t >= Tc) continue;
+            const int64_t i = it.b0 + it.tc + t;
+            const float *r = reinterpret_cast<const float *>(&red[rpar][h][sl]) + cp;
+            Kahan a{0.f, 0.f};
+            for (int k = 0; k < G; ++k) a.add(r[4 * k * slots]);
+            if (near) {  // the compensated sums so far; the far field is added by L2P
+                float *nr = reinterpret_cast<float *>(near + 2 * i) + cp;
+                nr[0] = a.s;
+                nr[4] = a.c;
+                continue;
             }
+            if (far) a.add(reinterpret_cast<const float *>(far + i)[cp]);
+            reinterpret_cast<float *>(out + perm[i])[cp] = a.s;
         }
         rpar ^= 1;
     }
@@ -383,6 +390,7 @@ static int p2p_blocks_per_sm()
 // 0.525, 0.541, 0.596 ms alone and 1.158, 1.152, 1.163, 1.189, 1.248 ms for the forked step; on
 // 16M Plummer (p = 8) P2P took 8.91, 7.97, 9.29 ms with 1, 4 and one wave.
 constexpr int kP2PLeavesPerCta = 4;
+constexpr int kP2PMaxParts = 16, kP2PWave = 152 * 8;
 // the evaluating context's choice (gbfmm_set_p2p_leaves_per_cta, gbfmm_tune), set on entry to an
 // evaluation by the thread that issues its launches; 0: kP2PLeavesPerCta
 static thread_local int tl_leaves_per_cta = 0;
@@ -394,13 +402,17 @@ static void launch_leaf(int64_t nleaf, int L, const int32_t *leaves, const float
                         Span lv = Span{})
 {
     const int64_t resident = (int64_t)sm_count() * p2p_blocks_per_sm();
+    // small uniform trees: a leaf's targets over up to kP2PMaxParts CTAs, so that the launch has one
+    // wave of CTAs (4,096 particles, 64 leaves: 39 -> 10.5 us, packed pairs included).  Fixed by the depth: the sums do not depend on
+    // the launch shape.
+    const int parts = leaves ? 1 : (int)std::max<int64_t>(1, std::min<int64_t>(kP2PMaxParts, kP2PWave / nleaf));
     const int lpc = tl_leaves_per_cta > 0 ? tl_leaves_per_cta : kP2PLeavesPerCta;
     int64_t grid = (nleaf + lpc - 1) / lpc;
-    grid = std::min<int64_t>(nleaf, std::max<int64_t>(grid, resident));
+    grid = std::min<int64_t>(nleaf * parts, std::max<int64_t>(grid, resident));
     const bool soft = eps2 > 0.f;
     auto k = leaves ? (soft ? k_p2p_ws<true, false> : k_p2p_ws<false, false>)
                     : (soft ? k_p2p_ws<true, true> : k_p2p_ws<false, true>);
-    k<<<(unsigned)grid, kP2PWsThreads, 0, s>>>(L, leaves, lv, nleaf, sx, begin, end, offs, ids, far, perm, eps2, out,
+    k<<<(unsigned)grid, kP2PWsThreads, 0, s>>>(L, leaves, lv, nleaf, parts, sx, begin, end, offs, ids, far, perm, eps2, out,
                                                near, status);
     note_launches(1);
 }
