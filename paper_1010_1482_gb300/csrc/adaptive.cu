@@ -958,11 +958,11 @@ int treecode_adaptive(gbfmm_ctx *ctx, AdaptiveState &A, const Ranges &R, const g
     for (int l = maxl - 1; l >= 2; --l)
         launch_translate_cells(P, true, R.level(l), A.child_of.as<int32_t>(), A.nchild.as<int32_t>(), ops.m2m, M, s);
     mark(5);
-    cudaMemsetAsync(far, 0, 16 * (size_t)n, s);
-    if (deep)
+    if (!deep)
+        cudaMemsetAsync(far, 0, 16 * (size_t)n, s);
+    else
         launch_m2p_cells(P, A.leaves.as<int32_t>(), R.leaves(), geom, A.begin.as<int32_t>(), A.end.as<int32_t>(),
-                         A.tc_offs[1].as<uint32_t>(), A.tc_ids[1].as<int32_t>(), A.sx.as<float4>(), M, far, s,
-                         true);
+                         A.tc_offs[1].as<uint32_t>(), A.tc_ids[1].as<int32_t>(), A.sx.as<float4>(), M, far, s);
     mark(6);  // M2P is reported with M2L; no L2L, no L2P
     mark(7);
     mark(8);
@@ -1291,14 +1291,10 @@ int evaluate_adaptive_in(gbfmm_ctx *ctx, AdaptiveState &A, const AdaptCaps *caps
     // context's low-priority stream while the expansions run on its high-priority one (unless
     // the evaluation is timed, serial or device-counted); L2P adds the far field to them and
     // writes the output
-    const bool split = p2p_near_supported();
-    const bool fork = split && (prm->flags & GBFMM_FLAG_SERIAL) == 0 && !dev;
-    ctx->stage_order_last = fork ? 2 : (split ? 1 : 0);
-    float4 *near = nullptr;
-    if (split) {
-        if (grow(A.near, 32 * (size_t)n, false, 0, s)) return fail(ctx, GBFMM_ENOMEM, "adaptive near field");
-        near = A.near.as<float4>();
-    }
+    const bool fork = (prm->flags & GBFMM_FLAG_SERIAL) == 0 && !dev;
+    ctx->stage_order_last = fork ? 2 : 1;
+    if (grow(A.near, 32 * (size_t)n, false, 0, s)) return fail(ctx, GBFMM_ENOMEM, "adaptive near field");
+    float4 *near = A.near.as<float4>();
     const cudaStream_t s_main = s;
     // an error after the fork still joins both streams back into the caller's
     auto fail_joined = [&](int code, const char *msg) {
@@ -1408,45 +1404,32 @@ int evaluate_adaptive_in(gbfmm_ctx *ctx, AdaptiveState &A, const AdaptCaps *caps
         launch_translate_cells(P, false, R.level(l - 1), A.child_of.as<int32_t>(), A.nchild.as<int32_t>(), ops.l2l,
                                Lc, s);
     mark(7);
-    if (split) {
-        // M2P into the zeroed far field, then L2P adds the local expansion's value and the
-        // near-field sums (the same rounding as L2P then M2P: one addition each)
-        if (!fork) {
-            launch_p2p_cells_near(A.leaves.as<int32_t>(), R.leaves(), n, A.sx.as<float4>(), A.begin.as<int32_t>(),
-                                  A.end.as<int32_t>(), A.loffs[kListU].as<uint32_t>(), A.lids[kListU].as<int32_t>(),
-                                  (float)prm->eps2, near, ctx->d_status, s);
-            mark(8);
-        }
-        cudaMemsetAsync(far, 0, 16 * (size_t)n, s);
-        if (deep)
-            launch_m2p_cells(P, A.leaves.as<int32_t>(), R.leaves(), geom, A.begin.as<int32_t>(),
-                             A.end.as<int32_t>(), A.loffs[kListW].as<uint32_t>(), A.lids[kListW].as<int32_t>(),
-                             A.sx.as<float4>(), M, far, s);
-        if (fork) {
-            mark(8);
-            cudaStreamWaitEvent(s, ctx->ev_near, 0);
-            if (timing) cudaEventRecord(ctx->ev_aux[2], s);
-        }
-        launch_l2p_cells(P, n, A.leaf_of.as<int32_t>(), leaves_of, A.level.as<int32_t>(), geom, A.sx.as<float4>(), Lc, far, s,
-                         near, perm, reinterpret_cast<float4 *>(d_out), abort);
-        mark(9);
-        if (fork) {
-            cudaEventRecord(ctx->ev_join, s);
-            cudaStreamWaitEvent(s_main, ctx->ev_join, 0);
-            s = s_main;
-        }
-    } else {
-        launch_l2p_cells(P, n, A.leaf_of.as<int32_t>(), leaves_of, A.level.as<int32_t>(), geom, A.sx.as<float4>(), Lc, far, s,
-                         nullptr, nullptr, nullptr, abort);
-        if (deep)
-            launch_m2p_cells(P, A.leaves.as<int32_t>(), R.leaves(), geom, A.begin.as<int32_t>(),
-                             A.end.as<int32_t>(), A.loffs[kListW].as<uint32_t>(), A.lids[kListW].as<int32_t>(),
-                             A.sx.as<float4>(), M, far, s);
+    // M2P into the far field, then L2P adds the local expansion's value and the
+    // near-field sums (the same rounding as L2P then M2P: one addition each)
+    if (!fork) {
+        launch_p2p_cells_near(A.leaves.as<int32_t>(), R.leaves(), n, A.sx.as<float4>(), A.begin.as<int32_t>(),
+                              A.end.as<int32_t>(), A.loffs[kListU].as<uint32_t>(), A.lids[kListU].as<int32_t>(),
+                              (float)prm->eps2, near, ctx->d_status, s);
         mark(8);
-        launch_p2p_cells(A.leaves.as<int32_t>(), R.leaves(), n, A.sx.as<float4>(), A.begin.as<int32_t>(),
-                         A.end.as<int32_t>(), A.loffs[kListU].as<uint32_t>(), A.lids[kListU].as<int32_t>(), far, perm,
-                         (float)prm->eps2, reinterpret_cast<float4 *>(d_out), ctx->d_status, s);
-        mark(9);
+    }
+    if (!deep)
+        cudaMemsetAsync(far, 0, 16 * (size_t)n, s);
+    else
+        launch_m2p_cells(P, A.leaves.as<int32_t>(), R.leaves(), geom, A.begin.as<int32_t>(),
+                         A.end.as<int32_t>(), A.loffs[kListW].as<uint32_t>(), A.lids[kListW].as<int32_t>(),
+                         A.sx.as<float4>(), M, far, s);
+    if (fork) {
+        mark(8);
+        cudaStreamWaitEvent(s, ctx->ev_near, 0);
+        if (timing) cudaEventRecord(ctx->ev_aux[2], s);
+    }
+    launch_l2p_cells(P, n, A.leaf_of.as<int32_t>(), leaves_of, A.level.as<int32_t>(), geom, A.sx.as<float4>(), Lc, far, s,
+                     near, perm, reinterpret_cast<float4 *>(d_out), abort);
+    mark(9);
+    if (fork) {
+        cudaEventRecord(ctx->ev_join, s);
+        cudaStreamWaitEvent(s_main, ctx->ev_join, 0);
+        s = s_main;
     }
     A.P = P;
     cudaError_t e = cudaGetLastError();

@@ -465,7 +465,7 @@ int evaluate_uniform_in(gbfmm_ctx *ctx, const gbfmm_params *prm, int64_t n, cons
     // near field beside the far field (FMM): P2P writes its compensated sums, L2P adds the far
     // field to them and writes the output; concurrently on the context's two streams unless the
     // evaluation is timed or serial
-    const bool split = L >= 2 && prm->method == GBFMM_METHOD_FMM && p2p_near_supported();
+    const bool split = L >= 2 && prm->method == GBFMM_METHOD_FMM;
     const bool fork = split && (prm->flags & GBFMM_FLAG_SERIAL) == 0;
     float4 *near = split ? far : nullptr;
     const cudaStream_t s_main = s;

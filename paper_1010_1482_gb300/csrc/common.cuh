@@ -437,11 +437,11 @@ void launch_p2l_cells(int P, Span cells, const int32_t *level, const float4 *geo
 void launch_l2p_cells(int P, int64_t n, const int32_t *leaf_of, const int32_t *leaves, const int32_t *level, const float4 *geom,
                       const float4 *sx, const float *Lc, float4 *far, cudaStream_t s, const float4 *near = nullptr,
                       const uint32_t *perm = nullptr, float4 *out = nullptr, const int32_t *abort = nullptr);
-// long_rows: the treecode's chain rows (the warp kernel, k_m2p_warp); else the FMM's short W
-// rows (one CTA of 64 per leaf, k_m2p_cells)
+// Writes far of every listed leaf's particles (0 where a row is empty): the FMM's W
+// rows or the treecode's chain rows
 void launch_m2p_cells(int P, const int32_t *leaves, Span lv, const float4 *geom, const int32_t *begin,
                       const int32_t *end, const uint32_t *w_offs, const int32_t *w_ids, const float4 *sx,
-                      const float *M, float4 *far, cudaStream_t s, bool long_rows = false);
+                      const float *M, float4 *far, cudaStream_t s);
 void launch_p2p_cells(const int32_t *leaves, Span lv, int64_t n, const float4 *sx, const int32_t *begin,
                       const int32_t *end, const uint32_t *u_offs, const int32_t *u_ids, const float4 *far,
                       const uint32_t *perm, float eps2, float4 *out, int *status, cudaStream_t s);
@@ -488,10 +488,8 @@ void launch_m2l_rot(int P, int L, const int32_t *begin, const int32_t *end, cons
 
 // p2p.cu
 // P2P without the far field: the compensated near-field sums of every particle in sorted order,
-// near[2 i] = sums (phi, dphi/dx, dphi/dy, dphi/dz), near[2 i + 1] = their compensations (the
-// warp-specialised kernel: p2p_near_supported()).  The P2P launchers take the context's status
+// near[2 i] = sums (phi, dphi/dx, dphi/dy, dphi/dz), near[2 i + 1] = their compensations.  The P2P launchers take the context's status
 // word: a bounded wait that expires raises kStatusTimeout there.
-bool p2p_near_supported();
 // P2P launch shape for the launches this thread issues next: about `leaves` target leaves per
 // CTA (0: the library's choice; at most kMaxP2PLeavesPerCta); the results do not depend on it
 constexpr int kMaxP2PLeavesPerCta = 64;

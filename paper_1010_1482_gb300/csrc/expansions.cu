@@ -44,8 +44,11 @@ __constant__ float c_ra[kMaxDeg + 1][kMaxDeg + 1];     // (2n+1) / sqrt((n+1-m)(
 __constant__ float c_rb[kMaxDeg + 1][kMaxDeg + 1];     // sqrt((n-m)(n+m)) / sqrt((n+1-m)(n+1+m))
 __constant__ float c_sq[2 * kMaxDeg + 4][2 * kMaxDeg + 4];  // sqrt(a*b)
 
+void m2p_tables();
+
 void init_expansion_constants()
 {
+    m2p_tables();
     float rmm[kMaxDeg + 1], ra[kMaxDeg + 1][kMaxDeg + 1], rb[kMaxDeg + 1][kMaxDeg + 1];
     static float sq[2 * kMaxDeg + 4][2 * kMaxDeg + 4];
     for (int m = 0; m <= kMaxDeg; ++m) rmm[m] = m ? (float)sqrt((2.0 * m - 1.0) / (2.0 * m)) : 0.f;
@@ -1061,291 +1064,332 @@ void launch_l2p(int P, int L, const float *geo, int64_t n, const float4 *sx, con
 //   dphi/dx + i dphi/dy =  (1/h^2) sum s(m) sqrt((n+m+2)(n+m+1)) M~_n^m I_{n+1}^{m+1},
 //   s(m) = +1 for m >= 0, -1 for m < 0.
 // ------------------------------------------------------------------------------------------
-// The constants of these sums are folded into the source cell's coefficients once per cell
-// (staged in shared memory), so that each (particle, cell) evaluation spends two FMAs per real
-// term: per (N, m), 0 <= m <= N <= P, two float4 (in two halves of the fold, F[q] and F[NM + q])
-//   {w M_N^m (re, im), -w sqrt((N-m)(N+m)) M_{N-1}^m (re, im)},
-//   {A - B (re, im), A + B (re, im)},  A = sqrt((N+m)(N+m-1)) M_{N-1}^{m-1},
-//                                      B = sqrt((N-m)(N-m-1)) M_{N-1}^{m+1},
-// w = 2 for m > 0; dphi/dx + i dphi/dy = sum A I - conj(B I), so its real part takes A - B
-// against (Re I, -Im I) and its imaginary part A + B against (Im I, Re I).
+// With xi = (x^ + i y^) / r^2 and u = z^ / r^2 the harmonics of one m are a power of xi times real
+// functions of one recurrence in N,
+//   I_N^m = (1/r) k_N^m xi^m g_N,   g_m = 1,  g_N = u g_{N-1} - beta_N^m (1/r^2) g_{N-2},
+// the constants k absorbing the recurrence's factors (m2p_tables).  With three complex sums per m,
+//   F_m = sum w k_N M_N^m g_N,   Z_m = -sum w k_N sqrt((N-m)(N+m)) M_{N-1}^m g_N,
+//   A_m = sum k_N sqrt((N+m)(N+m-1)) M_{N-1}^{m-1} g_N          (w = 2 for m > 0, else 1)
+// every m contributes Re(xi^m F_m) to phi, Re(xi^m Z_m) to dphi/dz and to dphi/dx + i dphi/dy
+//   xi^m A_m + conj(xi^{m-1} (m F_m / r^2 + |xi|^2 A_{m+1}))     (the second for m >= 1),
+// the lowered term following from (d/dx - i d/dy)(X^m h) = X^{m-1} (2 m h + |X|^2 2 dh/d(r^2)): 9
+// FP32-pipe operations per (N, m) instead of the 14 of complex recurrences and four sums, and half
+// their rounding error against FP64.
+//
+// Two source cells share every instruction (packed FP32, a lane each): per pair of cells the warp
+// stages both expansions (cp.async, one step ahead) and folds the constants in, so that a record
+// of three 16-byte loads per (N, m) holds {F re, F im}, {Z re, Z im}, {A re, A im}, each a (cell 0,
+// cell 1) pair.  Issue-bound before (complex recurrences, one cell at a time: 73% issue, FP32 pipe
+// 40% of active cycles).
+//
+// The four warps of a CTA take a target leaf, the sources of its rows dealt to them 2 G at a time
+// (one warp a leaf: the longest rows were the tail, and half the GPU's warps idle); targets go in
+// chunks of up to 32, and a chunk of T < 32 takes G = min(GMAX, 32 / T) pairs of cells a step (lane
+// l: target l % T, pair l / T).  The lanes' partial sums are added in warp and group order.
+// M2P alone, the earlier kernels (a warp or a CTA of 64 per leaf) -> this one: treecode, 131,072
+// uniform p = 6 1325 -> 653 us, 50,021 Plummer p = 8 2348 -> 1023; W rows, 20,011 Plummer p = 4
+// 59 -> 24, 400,009 p = 10 428 -> 286, 16M p = 8 3587 -> 2773.
 template <int P>
-struct M2PFold {
-    static constexpr int NM = (P + 1) * (P + 2) / 2;
+struct M2PW {
+    static constexpr int PP = P * P, NM = (P + 1) * (P + 2) / 2, NO = 6 * NM;
+    static constexpr int GMAX = P <= 6 ? 4 : 2;
+    static constexpr int kF = GMAX * NO * 8, kM = 2 * 2 * GMAX * PP * 4, kG = 2 * 2 * GMAX * 16;  // bytes per warp
+    static constexpr int kWarp = kF + kM + kG;
+    static_assert(kF % 16 == 0 && kM % 16 == 0 && GMAX * NO * 8 >= 32 * 16, "alignment; F also holds the lanes' sums");
 };
 
 GB_HD constexpr int nm_idx(int N, int m) { return N * (N + 1) / 2 + m; }
 
-// per (N, m) of the folded coefficients: where its four source coefficients sit in M (re and im
-// index each, -1 for none) and their factors; built once per CTA by m2p_fold_table
-template <int P>
-struct M2PFoldTab {
-    int4 re, im;   // source coefficient of {phi, dz, A, B}: real / imaginary part index, -1: zero
-    float4 c;      // factors of {phi, dz, A, B}
-};
+// from here on four leaves a CTA (most W rows of a large tree are empty); fewer leaves are spread
+// over more CTAs (4,096 leaves, four a CTA: 887 us instead of 653)
+constexpr int64_t kM2PManyLeaves = 1 << 16;
+constexpr int kM2PMaxNO = 3 * (kMaxP + 1) * (kMaxP + 2);
+// per compiled order (4, 6, 8, 10) and folded coefficient 6 nm_idx(N, m) + {F re, im, Z re, im, A re,
+// im}: its source coefficient and factor (as bits); 0, 0 where there is none
+__device__ int2 d_m2p_tab[4][kM2PMaxNO];
+__constant__ uint64_t c_nbeta[kMaxP + 1][kMaxP + 1];  // (-beta, -beta) of (N, m)
 
-template <int P>
-GB_DEV void m2p_fold_table(M2PFoldTab<P> *__restrict__ T, int t, int nt)
+void m2p_tables()
 {
-    auto root = [](int a, int b) { return sqrtf((float)(a * b)); };
-    for (int q = t; q < M2PFold<P>::NM; q += nt) {
-        int N = 0;
-        while ((N + 1) * (N + 2) / 2 <= q) ++N;
-        const int m = q - N * (N + 1) / 2;
-        const float w = m > 0 ? 2.f : 1.f;
-        M2PFoldTab<P> e;
-        e.re = make_int4(-1, -1, -1, -1);
-        e.im = make_int4(-1, -1, -1, -1);
-        e.c = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (N <= P - 1) {
-            e.re.x = re_idx(N, m);
-            e.im.x = m > 0 ? im_idx(N, m) : -1;
-            e.c.x = w;
+    static int2 tab[4][kM2PMaxNO];
+    static uint64_t nbeta[kMaxP + 1][kMaxP + 1];
+    auto ra = [](int n, int m) { return (2.0 * n + 1.0) / sqrt((double)(n + 1 - m) * (n + 1 + m)); };
+    auto rb = [](int n, int m) { return sqrt((double)(n - m) * (n + m)) / sqrt((double)(n + 1 - m) * (n + 1 + m)); };
+    const int orders[4] = {4, 6, 8, 10};
+    memset(tab, 0, sizeof(tab));
+    memset(nbeta, 0, sizeof(nbeta));
+    double gamma = 1.0;
+    for (int m = 0; m <= kMaxP; ++m) {
+        if (m > 0) gamma *= -sqrt((2.0 * m - 1.0) / (2.0 * m));
+        const double w = m > 0 ? 2.0 : 1.0;
+        double k = gamma;  // k_N^m
+        for (int N = m; N <= kMaxP; ++N) {
+            if (N > m) k *= ra(N - 1, m);
+            if (N > m + 1) {
+                const float f = (float)(-rb(N - 1, m) / (ra(N - 1, m) * ra(N - 2, m)));
+                uint32_t bits;
+                memcpy(&bits, &f, 4);
+                nbeta[N][m] = (uint64_t)bits << 32 | bits;
+            }
+            for (int o = 0; o < 4; ++o) {
+                const int P = orders[o];
+                if (N > P) continue;
+                auto put = [&](int j, int n, int mm, double c) {  // complex coefficient M_n^mm, factor c
+                    const float f = (float)c;
+                    int bits;
+                    memcpy(&bits, &f, 4);
+                    tab[o][6 * nm_idx(N, m) + 2 * j] = make_int2(re_idx(n, mm), bits);
+                    if (mm > 0) tab[o][6 * nm_idx(N, m) + 2 * j + 1] = make_int2(im_idx(n, mm), bits);
+                };
+                if (N < P) put(0, N, m, k * w);
+                if (N > m) put(1, N - 1, m, -k * w * sqrt((double)(N - m) * (N + m)));
+                if (m > 0) put(2, N - 1, m - 1, k * sqrt((double)(N + m) * (N + m - 1)));
+            }
         }
-        if (N >= 1 && m <= N - 1) {
-            e.re.y = re_idx(N - 1, m);
-            e.im.y = m > 0 ? im_idx(N - 1, m) : -1;
-            e.c.y = -w * root(N - m, N + m);
-        }
-        if (N >= 1 && m >= 1) {
-            e.re.z = re_idx(N - 1, m - 1);
-            e.im.z = m - 1 > 0 ? im_idx(N - 1, m - 1) : -1;
-            e.c.z = root(N + m, N + m - 1);
-        }
-        if (N >= 1 && m + 1 <= N - 1) {
-            e.re.w = re_idx(N - 1, m + 1);
-            e.im.w = im_idx(N - 1, m + 1);
-            e.c.w = root(N - m, N - m - 1);
-        }
-        T[q] = e;
     }
+    cudaMemcpyToSymbol(d_m2p_tab, tab, sizeof(tab));
+    cudaMemcpyToSymbol(c_nbeta, nbeta, sizeof(nbeta));
 }
 
-// the block stages the cell's coefficients M[P^2] (coalesced) in sM, then threads t, t + nt,
-// ... fill F[2 NM] through the table
-template <int P>
-GB_DEV void m2p_fold(const float *__restrict__ M, float *__restrict__ sM, const M2PFoldTab<P> *__restrict__ T,
-                     float4 *__restrict__ F, int t, int nt)
-{
-    for (int k = t; k < P * P; k += nt) sM[k] = M[k];
-    __syncthreads();
-    auto at = [&](int k) { return k >= 0 ? sM[k] : 0.f; };
-    for (int q = t; q < M2PFold<P>::NM; q += nt) {
-        const M2PFoldTab<P> e = T[q];
-        const float pr = e.c.x * at(e.re.x), pi = e.c.x * at(e.im.x);
-        const float zr = e.c.y * at(e.re.y), zi = e.c.y * at(e.im.y);
-        const float ar = e.c.z * at(e.re.z), ai = e.c.z * at(e.im.z);
-        const float br = e.c.w * at(e.re.w), bi = e.c.w * at(e.im.w);
-        F[q] = make_float4(pr, pi, zr, zi);
-        F[M2PFold<P>::NM + q] = make_float4(ar - br, ai - bi, ar + br, ai + bi);
-    }
-}
+GB_DEV uint64_t neg2(uint64_t v) { return v ^ 0x8000000080000000ull; }
 
-// The M2P sums for NT targets at once against one source cell's folded
-// coefficients (Fa[q] = {phi, dz} pair, Fb[q] = {A - B, A + B} pair of (N, m) = q), so that every
-// coefficient load serves NT targets.  x, y, z: target minus cell centre over h; ih = 1/h.  The
-// degree recurrence takes z/r^2 and the constants' products with it once per term:
-// I_N = (a z/r^2) I_{N-1} - (b / r^2) I_{N-2}.
-template <int P, int NT>
-GB_DEV void m2p_acc_n(const float4 *__restrict__ Fa, const float4 *__restrict__ Fb, const float (&x)[NT],
-                      const float (&y)[NT], const float (&z)[NT], float ih, float (&o)[NT][4])
+// o += potential and gradient at p of the two cells of geometry g0, g1 and folded coefficients R
+template <int P>
+GB_DEV void m2p_pair(const ulonglong2 *__restrict__ R, float4 p, float4 g0, float4 g1, uint64_t (&o)[4])
 {
-    float ir2[NT], zi[NT], mre[NT], mim[NT], phi[NT], gz[NT], gpr[NT], gpi[NT];
-#pragma unroll
-    for (int k = 0; k < NT; ++k) {
-        const float r2 = x[k] * x[k] + y[k] * y[k] + z[k] * z[k];
-        const float ir = rsqrt_ftz(r2);
-        ir2[k] = ir * ir;
-        zi[k] = z[k] * ir2[k];
-        mre[k] = ir;  // I_0^0 = 1/r
-        mim[k] = 0.f;
-        phi[k] = gz[k] = gpr[k] = gpi[k] = 0.f;
-    }
+    const uint64_t x = pack2((p.x - g0.x) * g0.w, (p.x - g1.x) * g1.w);
+    const uint64_t y = pack2((p.y - g0.y) * g0.w, (p.y - g1.y) * g1.w);
+    const uint64_t z = pack2((p.z - g0.z) * g0.w, (p.z - g1.z) * g1.w);
+    float a, b;
+    unpack2(fma2(x, x, fma2(y, y, mul2(z, z))), a, b);
+    const uint64_t ir = pack2(rsqrt_ftz(a), rsqrt_ftz(b)), ir2 = mul2(ir, ir);
+    const uint64_t u = mul2(z, ir2), xr = mul2(x, ir2), xi = mul2(y, ir2), nxi = neg2(xi);
+    const uint64_t q2 = fma2(xr, xr, mul2(xi, xi));
+    uint64_t er = 0, ei = 0, er1 = 0, ei1 = 0, er2, ei2;  // xi^m, xi^(m-1), xi^(m-2) (m = 0: 1, not held)
+    uint64_t fr1 = 0, fi1 = 0;                             // F_{m-1}
+    uint64_t phi = 0, gr = 0, gi = 0, gz = 0;
 #pragma unroll
     for (int m = 0; m <= P; ++m) {
-        if (m > 0) {
-#pragma unroll
-            for (int k = 0; k < NT; ++k) {
-                const float f = -c_rmm[m] * ir2[k];
-                const float tr = f * (x[k] * mre[k] - y[k] * mim[k]), ti = f * (x[k] * mim[k] + y[k] * mre[k]);
-                mre[k] = tr;
-                mim[k] = ti;
-            }
+        er2 = er1, ei2 = ei1, er1 = er, ei1 = ei;
+        if (m == 1) {
+            er = xr, ei = xi;
+        } else if (m > 1) {
+            er = fma2(xr, er1, mul2(nxi, ei1));
+            ei = fma2(xr, ei1, mul2(xi, er1));
         }
-        float are[NT], aim[NT], bre[NT], bim[NT];
-#pragma unroll
-        for (int k = 0; k < NT; ++k) {
-            are[k] = mre[k];
-            aim[k] = mim[k];
-            bre[k] = bim[k] = 0.f;
-        }
+        uint64_t fr = 0, fi = 0, zr = 0, zi = 0, ar = 0, ai = 0, g1 = 0, g2 = 0;
 #pragma unroll
         for (int N = m; N <= P; ++N) {
-            if (N > m) {
-#pragma unroll
-                for (int k = 0; k < NT; ++k) {
-                    const float A = c_ra[N - 1][m] * zi[k], B = c_rb[N - 1][m] * ir2[k];
-                    const float nre = fmaf(A, are[k], -B * bre[k]), nim = fmaf(A, aim[k], -B * bim[k]);
-                    bre[k] = are[k];
-                    bim[k] = aim[k];
-                    are[k] = nre;
-                    aim[k] = nim;
+            const int q = 3 * nm_idx(N, m);
+            if (N == m) {  // g = 1
+                if (N < P) {
+                    const ulonglong2 f = R[q];
+                    fr = f.x, fi = f.y;
                 }
-            }
-            const int q = nm_idx(N, m);
-            if (N <= P - 1 || (N >= 1 && m <= N - 1)) {
-                const float4 a = Fa[q];
-#pragma unroll
-                for (int k = 0; k < NT; ++k) {
-                    if (N <= P - 1) phi[k] = fmaf(a.x, are[k], fmaf(-a.y, aim[k], phi[k]));
-                    if (N >= 1 && m <= N - 1) gz[k] = fmaf(a.z, are[k], fmaf(-a.w, aim[k], gz[k]));
+                if (m > 0) {
+                    const ulonglong2 c = R[q + 2];
+                    ar = c.x, ai = c.y;
                 }
+                continue;
             }
-            if (N >= 1 && (m >= 1 || m + 1 <= N - 1)) {
-                const float4 bb = Fb[q];
-#pragma unroll
-                for (int k = 0; k < NT; ++k) {
-                    gpr[k] = fmaf(bb.x, are[k], fmaf(-bb.y, aim[k], gpr[k]));
-                    gpi[k] = fmaf(bb.z, aim[k], fmaf(bb.w, are[k], gpi[k]));
+            uint64_t g;
+            if (N == m + 1)
+                g = u;
+            else
+                g = fma2(c_nbeta[N][m], N == m + 2 ? ir2 : mul2(ir2, g2), mul2(u, g1));
+            g2 = g1, g1 = g;
+            if (N < P) {
+                const ulonglong2 f = R[q];
+                fr = fma2(f.x, g, fr);
+                if (m > 0) fi = fma2(f.y, g, fi);
+            }
+            const ulonglong2 c = R[q + 1];
+            if (N == m + 1) {
+                zr = mul2(c.x, g);
+                if (m > 0) zi = mul2(c.y, g);
+            } else {
+                zr = fma2(c.x, g, zr);
+                if (m > 0) zi = fma2(c.y, g, zi);
+            }
+            if (m > 0) {
+                const ulonglong2 d = R[q + 2];
+                ar = fma2(d.x, g, ar);
+                if (m > 1) ai = fma2(d.y, g, ai);
+            }
+        }
+        if (m == 0) {
+            phi = fr;
+            gz = zr;
+        } else {
+            const uint64_t nei = neg2(ei);
+            if (m < P) {
+                phi = fma2(er, fr, fma2(nei, fi, phi));
+                gz = fma2(er, zr, fma2(nei, zi, gz));
+            }
+            if (m == 1) {  // A_1 comes from the real M^0
+                gr = mul2(er, ar);
+                gi = mul2(ei, ar);
+            } else {
+                gr = fma2(er, ar, fma2(nei, ai, gr));
+                gi = fma2(er, ai, fma2(ei, ar, gi));
+                const uint64_t h = m == 2 ? ir2 : mul2(pack2((float)(m - 1), (float)(m - 1)), ir2);
+                const uint64_t tr = fma2(h, fr1, mul2(q2, ar)), ti = fma2(h, fi1, mul2(q2, ai));
+                if (m == 2) {
+                    gr = add2(gr, tr);
+                    gi = add2(gi, neg2(ti));
+                } else {
+                    gr = fma2(er2, tr, fma2(neg2(ei2), ti, gr));
+                    gi = fma2(neg2(er2), ti, fma2(neg2(ei2), tr, gi));
                 }
             }
         }
+        fr1 = fr, fi1 = fi;
     }
-    const float ih2 = ih * ih;
-#pragma unroll
-    for (int k = 0; k < NT; ++k) {
-        o[k][0] += phi[k] * ih;
-        o[k][1] += gpr[k] * ih2;
-        o[k][2] += gpi[k] * ih2;
-        o[k][3] += gz[k] * ih2;
+    const uint64_t ih = pack2(g0.w, g1.w), s1 = mul2(ir, ih), s2 = mul2(s1, ih);
+    o[0] = fma2(phi, s1, o[0]);
+    o[1] = fma2(gr, s2, o[1]);
+    o[2] = fma2(gi, s2, o[2]);
+    o[3] = fma2(gz, s2, o[3]);
+}
+
+// Sources: the M2L rows of the leaf's ancestors at levels 2..L (uniform tree, UNI) or one row
+// of a cell list (adaptive tree).  Writes far of every particle of the leaves.
+// A CTA takes lpc leaves one after another; an empty row only stores zeros.
+template <int P, bool UNI>
+__global__ void __launch_bounds__(128, 5) k_m2p(int L, const float *__restrict__ geo, const int32_t *__restrict__ leaves,
+                                             Span lv, int lpc, const float4 *__restrict__ geom,
+                                             const int32_t *__restrict__ begin, const int32_t *__restrict__ end,
+                                             const uint32_t *__restrict__ offs, const int32_t *__restrict__ ids,
+                                             const float4 *__restrict__ sx, const float *__restrict__ M,
+                                             float4 *__restrict__ far)
+{
+    using W = M2PW<P>;
+    constexpr int PP = W::PP, NO = W::NO, C4 = PP / 4;
+    extern __shared__ __align__(16) unsigned char m2p_sm[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float2 *F = reinterpret_cast<float2 *>(m2p_sm + warp * W::kWarp);
+    float *sM = reinterpret_cast<float *>(m2p_sm + warp * W::kWarp + W::kF);
+    float4 *sG = reinterpret_cast<float4 *>(m2p_sm + warp * W::kWarp + W::kF + W::kM);
+    const int2 *tab = d_m2p_tab[P / 2 - 2];
+    const int64_t w1 = min(span_count(lv), (int64_t)(blockIdx.x + 1) * lpc);
+    for (int64_t w = blockIdx.x * (int64_t)lpc; w < w1; ++w) {
+        const int64_t b = UNI ? level_offset(L) + w : (int64_t)leaves[w];
+        const int b0 = begin[b], nt = end[b] - b0;
+        if (!UNI && offs[b] == offs[b + 1]) {
+            for (int t = threadIdx.x; t < nt; t += 128) far[b0 + t] = make_float4(0.f, 0.f, 0.f, 0.f);
+            continue;
+        }
+        for (int c0 = 0; c0 < nt; c0 += 32) {
+            const int T = min(32, nt - c0);
+            const int G = min(W::GMAX, 32 / T), S = 2 * G;
+            const int t = lane % T, g = lane / T;
+            const float4 p = __ldg(&sx[b0 + c0 + t]);
+            uint64_t o[4] = {0, 0, 0, 0};
+            auto row = [&](uint32_t e0, uint32_t e1, int l) {
+                // one step's cells: lane j < S holds the id of cell j (-1: none, zero coefficients and
+                // cell 0's geometry)
+                auto id_at = [&](uint32_t e) { return lane < S && e + lane < e1 ? ids[e + lane] : -1; };
+                auto fetch = [&](int id, int buf) {
+                    float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (id >= 0) {
+                        const CellGeom cg = UNI ? geo_level_cell(geo, l, (uint32_t)(id - level_offset(l))) : geo_cell(geom, id);
+                        q = make_float4(cg.cx, cg.cy, cg.cz, cg.inv_h);
+                    }
+                    const float4 q0 = make_float4(__shfl_sync(~0u, q.x, 0), __shfl_sync(~0u, q.y, 0),
+                                                  __shfl_sync(~0u, q.z, 0), __shfl_sync(~0u, q.w, 0));
+                    if (lane < S) sG[buf * 2 * W::GMAX + lane] = id >= 0 ? q : q0;
+                    float *m = sM + buf * 2 * W::GMAX * PP;
+                    for (int k0 = 0; k0 < S * C4; k0 += 32) {
+                        const int k = k0 + lane, j = min(k / C4, S - 1);
+                        const int idj = __shfl_sync(~0u, id, j);
+                        if (k < S * C4)
+                            cp_async16_t(m + 4 * k, M + (int64_t)max(idj, 0) * PP + 4 * (k - j * C4), idj >= 0 ? 16u : 0u);
+                    }
+                    asm volatile("cp.async.commit_group;" ::: "memory");
+                };
+                const uint32_t step = 4 * S;
+                uint32_t e = e0 + warp * S;
+                if (e >= e1) return;
+                int buf = 0;
+                fetch(id_at(e), 0);
+                int next = id_at(e + step);
+                for (; e < e1; e += step, buf ^= 1) {
+                    asm volatile("cp.async.wait_group 0;" ::: "memory");
+                    __syncwarp();
+                    if (e + step < e1) {
+                        fetch(next, buf ^ 1);
+                        next = id_at(e + 2 * step);
+                    }
+                    const float *m = sM + buf * 2 * W::GMAX * PP;
+                    for (int k = lane; k < NO; k += 32) {
+                        const int2 c = __ldg(&tab[k]);
+                        const float f = __int_as_float(c.y);
+                        for (int pr = 0; pr < G; ++pr)
+                            F[pr * NO + k] = make_float2(f * m[2 * pr * PP + c.x], f * m[(2 * pr + 1) * PP + c.x]);
+                    }
+                    __syncwarp();
+                    if (g < G) {
+                        const float4 *gg = sG + buf * 2 * W::GMAX + 2 * g;
+                        m2p_pair<P>(reinterpret_cast<const ulonglong2 *>(F + g * NO), p, gg[0], gg[1], o);
+                    }
+                    __syncwarp();
+                }
+            };
+            if (UNI) {
+                for (int l = 2; l <= L; ++l) {
+                    const int64_t a = level_offset(l) + (w >> (3 * (L - l)));
+                    row(offs[a], offs[a + 1], l);
+                }
+            } else {
+                row(offs[b], offs[b + 1], 0);
+            }
+            // the partial sums of the leaf's warps and groups, added in that order
+            float4 v;
+            float h;
+            unpack2(o[0], v.x, h), v.x += h;
+            unpack2(o[1], v.y, h), v.y += h;
+            unpack2(o[2], v.z, h), v.z += h;
+            unpack2(o[3], v.w, h), v.w += h;
+            reinterpret_cast<float4 *>(F)[lane] = v;
+            __syncthreads();
+            if (warp == 0 && g == 0) {
+                float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int ww = 0; ww < 4; ++ww) {
+                    const float4 *part = reinterpret_cast<const float4 *>(m2p_sm + ww * W::kWarp);
+                    for (int gg = 0; gg < G; ++gg) {
+                        const float4 q = part[t + gg * T];
+                        r.x += q.x;
+                        r.y += q.y;
+                        r.z += q.z;
+                        r.w += q.w;
+                    }
+                }
+                far[b0 + c0 + t] = r;
+            }
+            __syncthreads();
+        }
     }
 }
 
-// M2P by warps (the treecode on both trees): two warps per target leaf and no block barrier.
-// The leaf's targets go in chunks of up to 32, warp h of the leaf taking chunks h, h + 2, ...;
-// a chunk of T targets takes G = min(4, 32 / T) source cells per step (lane l: target l % T,
-// source group l / T), so small leaves and the remainder chunk still fill the warp.  Per step the warp stages the cells' coefficients and folds them into its own
-// shared memory (the M2P constants of m2p_fold), then every active lane evaluates its target
-// against its group's cell (m2p_acc_n).  At the end of a chunk the groups' partial sums are
-// added in group order (deterministic).  Sources: the M2L rows of the leaf's ancestors at levels
-// 2..L (uniform tree, UNI) or one cell-list row (adaptive tree).  ADD: add into far (else write).
-template <int P>
-struct M2PW {
-    static constexpr int NM = M2PFold<P>::NM;
-    static constexpr int GMAX = 4;
-    static constexpr int NMP = NM % 8 == 0 ? NM + 1 : NM;  // float4 stride of the two halves (bank spread)
-    static constexpr int WARPS = 4;                         // per CTA; two per leaf
-};
-
-template <int P, bool UNI, bool ADD>
-__global__ void __launch_bounds__(128) k_m2p_warp(int L, const float *__restrict__ geo,
-                                                  const int32_t *__restrict__ leaves, Span lv,
-                                                  const float4 *__restrict__ geom, const int32_t *__restrict__ begin,
-                                                  const int32_t *__restrict__ end, const uint32_t *__restrict__ offs,
-                                                  const int32_t *__restrict__ ids, const float4 *__restrict__ sx,
-                                                  const float *__restrict__ M, float4 *__restrict__ far)
+template <int P, bool UNI>
+static void launch_m2p_t(int L, const float *geo, const int32_t *leaves, Span lv, const float4 *geom,
+                         const int32_t *begin, const int32_t *end, const uint32_t *offs, const int32_t *ids,
+                         const float4 *sx, const float *M, float4 *far, cudaStream_t s)
 {
-    using W = M2PW<P>;
-    constexpr int PP = P * P, NM = W::NM, G4 = W::GMAX, NMP = W::NMP;
-    __shared__ M2PFoldTab<P> sT[NM];
-    __shared__ float4 sF[W::WARPS][G4 * 2 * NMP];
-    __shared__ float sM[W::WARPS][G4 * PP];
-    __shared__ float4 sR[W::WARPS][32];
-    m2p_fold_table<P>(sT, threadIdx.x, blockDim.x);
-    __syncthreads();  // the only block barrier: the table
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t w = (blockIdx.x * (int64_t)W::WARPS + warp) >> 1;
-    const int half = warp & 1;
-    if (w >= span_count(lv)) return;
-    const int64_t b = UNI ? level_offset(L) + w : (int64_t)leaves[w];
-    const int b0 = begin[b], nt = end[b] - b0;
-    if (nt <= 32 * half || (!UNI && offs[b] == offs[b + 1])) return;  // no chunk, or no sources (far untouched)
-    float4 *F = sF[warp];
-    float *Ms = sM[warp];
-    for (int c0 = 32 * half; c0 < nt; c0 += 64) {
-        const int T = min(32, nt - c0);
-        const int G = min(G4, 32 / T);
-        const int t = lane % T, g = lane / T;
-        const bool act = g < G;
-        const float4 p = __ldg(&sx[b0 + c0 + (act ? t : 0)]);
-        float o[1][4] = {{0.f, 0.f, 0.f, 0.f}};
-        auto row = [&](uint32_t e0, uint32_t e1, int l) {
-            for (uint32_t e = e0; e < e1; e += G) {
-                const int ng = (int)(e1 - e < (uint32_t)G ? e1 - e : (uint32_t)G);
-                __syncwarp();
-                for (int k = lane; k < ng * PP; k += 32) {
-                    const int gg = k / PP, kk = k - gg * PP;
-                    Ms[k] = M[(int64_t)ids[e + gg] * PP + kk];
-                }
-                __syncwarp();
-                for (int q = lane; q < ng * NM; q += 32) {
-                    const int gg = q / NM, qq = q - gg * NM;
-                    const M2PFoldTab<P> en = sT[qq];
-                    const float *m = Ms + gg * PP;
-                    auto at = [&](int k) { return k >= 0 ? m[k] : 0.f; };
-                    const float pr = en.c.x * at(en.re.x), pi = en.c.x * at(en.im.x);
-                    const float zr = en.c.y * at(en.re.y), zi = en.c.y * at(en.im.y);
-                    const float ar = en.c.z * at(en.re.z), ai = en.c.z * at(en.im.z);
-                    const float br = en.c.w * at(en.re.w), bi = en.c.w * at(en.im.w);
-                    F[gg * 2 * NMP + qq] = make_float4(pr, pi, zr, zi);
-                    F[gg * 2 * NMP + NMP + qq] = make_float4(ar - br, ai - bi, ar + br, ai + bi);
-                }
-                __syncwarp();
-                if (act && g < ng) {
-                    const int64_t sc = ids[e + g];
-                    const CellGeom cg = UNI ? geo_level_cell(geo, l, (uint32_t)(sc - level_offset(l))) : geo_cell(geom, sc);
-                    const float4 *Fa = F + g * 2 * NMP;
-                    float xs[1] = {(p.x - cg.cx) * cg.inv_h}, ys[1] = {(p.y - cg.cy) * cg.inv_h};
-                    float zs[1] = {(p.z - cg.cz) * cg.inv_h};
-                    m2p_acc_n<P, 1>(Fa, Fa + NMP, xs, ys, zs, cg.inv_h, o);
-                }
-            }
-        };
-        if (UNI) {
-            for (int l = 2; l <= L; ++l) {
-                const int64_t a = level_offset(l) + (w >> (3 * (L - l)));
-                row(offs[a], offs[a + 1], l);
-            }
-        } else {
-            row(offs[b], offs[b + 1], 0);
-        }
-        // the groups' partial sums, added in group order
-        __syncwarp();
-        sR[warp][lane] = make_float4(o[0][0], o[0][1], o[0][2], o[0][3]);
-        __syncwarp();
-        if (act && g == 0) {
-            float4 r = sR[warp][t];
-            for (int gg = 1; gg < G; ++gg) {
-                const float4 v = sR[warp][t + gg * T];
-                r.x += v.x;
-                r.y += v.y;
-                r.z += v.z;
-                r.w += v.w;
-            }
-            const int64_t i = b0 + c0 + t;
-            if (ADD) {
-                float4 f = far[i];
-                f.x += r.x;
-                f.y += r.y;
-                f.z += r.z;
-                f.w += r.w;
-                far[i] = f;
-            } else {
-                far[i] = r;
-            }
-        }
-    }
+    constexpr int smem = 4 * M2PW<P>::kWarp;
+    cudaFuncSetAttribute(k_m2p<P, UNI>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    const int lpc = lv.cap > kM2PManyLeaves ? 4 : 1;
+    const unsigned grid = (unsigned)((lv.cap + lpc - 1) / lpc);
+    k_m2p<P, UNI><<<grid, 128, smem, s>>>(L, geo, leaves, lv, lpc, geom, begin, end, offs, ids, sx, M, far);
+    note_launches(1);
 }
 
 void launch_m2p(int P, int L, const float *geo, const float4 *sx, const int32_t *begin, const int32_t *end,
                 const uint32_t *m2l_offs, const int32_t *m2l_ids, const float *M, float4 *far, cudaStream_t s)
 {
-    const int64_t nl = int64_t(1) << (3 * L);
-    const unsigned grid = (unsigned)((nl + 1) / 2);  // two warps per leaf, four per CTA
-    const Span lv = host_span(0, nl);
-    GBFMM_DISPATCH_P(P, (k_m2p_warp<PQ, true, false><<<grid, 128, 0, s>>>(L, geo, nullptr, lv, nullptr, begin, end,
-                                                                          m2l_offs, m2l_ids, sx, M, far)));
-    note_launches(1);
+    const Span lv = host_span(0, int64_t(1) << (3 * L));
+    GBFMM_DISPATCH_P(P, (launch_m2p_t<PQ, true>(L, geo, nullptr, lv, nullptr, begin, end, m2l_offs, m2l_ids, sx, M,
+                                                   far, s)));
 }
 
 // ==========================================================================================
@@ -1447,55 +1491,6 @@ __global__ void __launch_bounds__(128) k_l2p_cells(int64_t n, const int32_t *__r
         out[perm[i]] = near_plus_far(near, i, f);
     } else {
         far[i] = f;
-    }
-}
-
-// M2P over the W list, one CTA per listed leaf; adds into the far-field accumulator
-template <int P>
-__global__ void __launch_bounds__(64) k_m2p_cells(const int32_t *__restrict__ leaves, Span lv,
-                                                  const float4 *__restrict__ geom, const int32_t *__restrict__ begin,
-                                                  const int32_t *__restrict__ end,
-                                                  const uint32_t *__restrict__ w_offs,
-                                                  const int32_t *__restrict__ w_ids, const float4 *__restrict__ sx,
-                                                  const float *__restrict__ M, float4 *__restrict__ far)
-{
-    __shared__ float4 sF[2 * M2PFold<P>::NM];
-    __shared__ float sM[P * P];
-    __shared__ M2PFoldTab<P> sT[M2PFold<P>::NM];
-    if (blockIdx.x >= span_count(lv)) return;
-    const int32_t b = leaves[blockIdx.x];
-    const uint32_t e0 = w_offs[b], e1 = w_offs[b + 1];
-    if (e0 == e1) return;
-    m2p_fold_table<P>(sT, threadIdx.x, blockDim.x);  // read after the first fold's barrier
-    const int b0 = begin[b], bend = end[b];
-    for (int t0 = b0; t0 < bend; t0 += blockDim.x) {
-        const int t = t0 + threadIdx.x;
-        const bool act = t < bend;
-        float4 p = act ? __ldg(&sx[t]) : make_float4(0.f, 0.f, 0.f, 0.f);
-        float o[4] = {0.f, 0.f, 0.f, 0.f};
-        for (uint32_t e = e0; e < e1; ++e) {
-            const int32_t sc = w_ids[e];
-            __syncthreads();
-            m2p_fold<P>(M + (int64_t)sc * (P * P), sM, sT, sF, threadIdx.x, blockDim.x);
-            __syncthreads();
-            const CellGeom cg = geo_cell(geom, sc);
-            if (act) {
-                float xs[1] = {(p.x - cg.cx) * cg.inv_h}, ys[1] = {(p.y - cg.cy) * cg.inv_h};
-                float zs[1] = {(p.z - cg.cz) * cg.inv_h};
-                float o1[1][4] = {{o[0], o[1], o[2], o[3]}};
-                m2p_acc_n<P, 1>(sF, sF + M2PFold<P>::NM, xs, ys, zs, cg.inv_h, o1);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) o[k] = o1[0][k];
-            }
-        }
-        if (act) {
-            float4 f = far[t];
-            f.x += o[0];
-            f.y += o[1];
-            f.z += o[2];
-            f.w += o[3];
-            far[t] = f;
-        }
     }
 }
 
@@ -1652,18 +1647,11 @@ void launch_l2p_cells(int P, int64_t n, const int32_t *leaf_of, const int32_t *l
 
 void launch_m2p_cells(int P, const int32_t *leaves, Span lv, const float4 *geom, const int32_t *begin,
                       const int32_t *end, const uint32_t *w_offs, const int32_t *w_ids, const float4 *sx,
-                      const float *M, float4 *far, cudaStream_t s, bool long_rows)
+                      const float *M, float4 *far, cudaStream_t s)
 {
     if (lv.cap <= 0) return;
-    if (long_rows) {
-        const unsigned grid = (unsigned)((lv.cap + 1) / 2);  // two warps per leaf, four per CTA
-        GBFMM_DISPATCH_P(P, (k_m2p_warp<PQ, false, true><<<grid, 128, 0, s>>>(0, nullptr, leaves, lv, geom, begin,
-                                                                              end, w_offs, w_ids, sx, M, far)));
-    } else {
-        GBFMM_DISPATCH_P(P, (k_m2p_cells<PQ><<<(unsigned)lv.cap, 64, 0, s>>>(leaves, lv, geom, begin, end, w_offs,
-                                                                             w_ids, sx, M, far)));
-    }
-    note_launches(1);
+    GBFMM_DISPATCH_P(P, (launch_m2p_t<PQ, false>(0, nullptr, leaves, lv, geom, begin, end, w_offs, w_ids, sx, M, far,
+                                                 s)));
 }
 
 template <int P, bool UP, int TN, int CN>

@@ -433,8 +433,6 @@ void launch_p2p_cells(const int32_t *leaves, Span lv, int64_t n, const float4 *s
     launch_leaf(lv.cap, 0, leaves, sx, begin, end, u_offs, u_ids, far, perm, eps2, out, nullptr, status, s, lv);
 }
 
-bool p2p_near_supported() { return true; }
-
 void launch_p2p_near(int L, int64_t n, const float4 *sx, const int32_t *begin, const int32_t *end, float eps2,
                      float4 *near, int *status, cudaStream_t s)
 {
