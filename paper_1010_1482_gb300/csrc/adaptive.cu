@@ -905,7 +905,7 @@ template <class Mark>
 int treecode_adaptive(gbfmm_ctx *ctx, AdaptiveState &A, const Ranges &R, const gbfmm_params *prm, int64_t n,
                       float *d_out, cudaStream_t s, Mark &mark)
 {
-    const int P = prm->p, PP = P * P;
+    const int P = prm->p, PP = P * P, leaf_size = prm->leaf_size;
     const int64_t ncells = R.ncells;
     const int maxl = A.max_level;
     const OpsCache &ops = ctx->ops[order_slot(P)];
@@ -952,7 +952,7 @@ int treecode_adaptive(gbfmm_ctx *ctx, AdaptiveState &A, const Ranges &R, const g
     float4 *far = A.far.as<float4>();
     const float4 *geom = A.geom.as<float4>();
     const bool deep = maxl >= 2;
-    if (deep) launch_p2m_cells(P, A.leaves.as<int32_t>(), R.leaves(), A.level.as<int32_t>(), geom,
+    if (deep) launch_p2m_cells(P, est_adaptive_leaves(n, leaf_size), A.leaves.as<int32_t>(), R.leaves(), A.level.as<int32_t>(), geom,
                                A.begin.as<int32_t>(), A.count.as<int32_t>(), A.sx.as<float4>(), M, s);
     mark(4);
     for (int l = maxl - 1; l >= 2; --l)
@@ -1324,7 +1324,7 @@ int evaluate_adaptive_in(gbfmm_ctx *ctx, AdaptiveState &A, const AdaptCaps *caps
     float *M = A.M.as<float>(), *Lc = A.Lc.as<float>();
     float4 *far = A.far.as<float4>();
     const bool deep = maxl >= 2;
-    if (deep) launch_p2m_cells(P, A.leaves.as<int32_t>(), R.leaves(), A.level.as<int32_t>(), geom,
+    if (deep) launch_p2m_cells(P, est_adaptive_leaves(n, leaf_size), A.leaves.as<int32_t>(), R.leaves(), A.level.as<int32_t>(), geom,
                                A.begin.as<int32_t>(), A.count.as<int32_t>(), A.sx.as<float4>(), M, s);
     mark(4);
     for (int l = maxl - 1; l >= 2; --l)
@@ -1356,7 +1356,7 @@ int evaluate_adaptive_in(gbfmm_ctx *ctx, AdaptiveState &A, const AdaptCaps *caps
                             fork ? sm_count() : 0) != 0)
             return fail_joined(GBFMM_ECUDA, "TMA tensor map encoding failed");
         if (ksplit > 1) launch_ablk_reduce(P, R.deep(), ksplit, part_stride, A.lpart.as<float>(), Lc, s);
-        launch_p2l_cells(P, R.cells(), A.level.as<int32_t>(), geom, A.begin.as<int32_t>(), A.count.as<int32_t>(),
+        launch_p2l_cells(P, est_adaptive_leaves(n, leaf_size), R.cells(), A.level.as<int32_t>(), geom, A.begin.as<int32_t>(), A.count.as<int32_t>(),
                          A.loffs[kListX].as<uint32_t>(), A.lids[kListX].as<int32_t>(), A.sx.as<float4>(), Lc, s);
     } else if (deep) {
         // M2L targets: every cell at levels >= 2, grouped by (level, child position) into tiles
@@ -1396,7 +1396,7 @@ int evaluate_adaptive_in(gbfmm_ctx *ctx, AdaptiveState &A, const AdaptCaps *caps
             launch_m2l_tiles(P, A.tdesc.as<int4>(), (int)tcap, A.tlist.as<int32_t>(), A.begin.as<int32_t>(),
                              A.end.as<int32_t>(), A.loffs[kListV].as<uint32_t>(), A.lids[kListV].as<int32_t>(),
                              A.vcode.as<uint16_t>(), ops.m2l, M, Lc, ctx->d_zero, ctx->d_status, s);
-        launch_p2l_cells(P, R.cells(), A.level.as<int32_t>(), geom, A.begin.as<int32_t>(), A.count.as<int32_t>(),
+        launch_p2l_cells(P, est_adaptive_leaves(n, leaf_size), R.cells(), A.level.as<int32_t>(), geom, A.begin.as<int32_t>(), A.count.as<int32_t>(),
                          A.loffs[kListX].as<uint32_t>(), A.lids[kListX].as<int32_t>(), A.sx.as<float4>(), Lc, s);
     }
     mark(6);

@@ -396,8 +396,12 @@ void launch_sort_gather64(uint64_t *k0, uint64_t *k1, uint32_t *v0, uint32_t *v1
 // launches their leaves as a Span over the leaf list (leaf ordinals i < count()).
 void launch_cell_geom(Span cells, const int32_t *level, const uint64_t *key, const Box *box, float4 *geom,
                       cudaStream_t s);
-void launch_p2m_cells(int P, const int32_t *leaves, Span lv, const int32_t *level, const float4 *geom,
-                      const int32_t *begin, const int32_t *count, const float4 *sx, float *M, cudaStream_t s);
+// est_leaves: the number of leaves expected of n and leaf_size alone (est_adaptive_leaves)
+void launch_p2m_cells(int P, int64_t est_leaves, const int32_t *leaves, Span lv, const int32_t *level,
+                      const float4 *geom, const int32_t *begin, const int32_t *count, const float4 *sx, float *M,
+                      cudaStream_t s);
+// leaves of an adaptive tree hold about 0.3 leaf_size particles
+inline int64_t est_adaptive_leaves(int64_t n, int leaf_size) { return 3 * n / (leaf_size > 0 ? leaf_size : 1); }
 // parents: the cells whose children are translated (M2M up into them, L2L down from them)
 void launch_translate_cells(int P, bool up, Span parents, const int32_t *child_of, const int32_t *nchild,
                             const float *ops, float *X, cudaStream_t s);
@@ -428,7 +432,7 @@ int sm_count();
 size_t presplit_bytes(int P, int64_t ncells);
 void launch_presplit(int P, const float *M, int64_t ncells, int8_t *scale, void *ps, cudaStream_t s,
                      Span cells = Span{});
-void launch_p2l_cells(int P, Span cells, const int32_t *level, const float4 *geom, const int32_t *begin,
+void launch_p2l_cells(int P, int64_t est_leaves, Span cells, const int32_t *level, const float4 *geom, const int32_t *begin,
                       const int32_t *count, const uint32_t *x_offs, const int32_t *x_ids, const float4 *sx, float *Lc,
                       cudaStream_t s);
 // near != nullptr: far holds the M2P sums; the local expansion's value, those and the near-field

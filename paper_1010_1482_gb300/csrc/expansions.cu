@@ -42,6 +42,8 @@ constexpr int kMaxDeg = 2 * kMaxP;  // harmonics up to degree 2P-2 (M2L) and P (
 __constant__ float c_rmm[kMaxDeg + 1];                 // sqrt((2m-1)/(2m))
 __constant__ float c_ra[kMaxDeg + 1][kMaxDeg + 1];     // (2n+1) / sqrt((n+1-m)(n+1+m))
 __constant__ float c_rb[kMaxDeg + 1][kMaxDeg + 1];     // sqrt((n-m)(n+m)) / sqrt((n+1-m)(n+1+m))
+__constant__ float c_nbeta1[kMaxP + 1][kMaxP + 1];  // -beta_n^m of the real recurrences (P2M, P2L, M2P)
+__device__ float d_kscale[kMaxP * kMaxP];           // k_n^m of the real-packed coefficient n^2 + ...
 __constant__ float c_sq[2 * kMaxDeg + 4][2 * kMaxDeg + 4];  // sqrt(a*b)
 
 void m2p_tables();
@@ -505,65 +507,69 @@ GB_DEV CellGeom geo_cell(const float4 *__restrict__ geom, int64_t c)
 }
 
 // ------------------------------------------------------------------------------------------
-// P2M: one warp per leaf; lanes stride over the leaf's particles, each accumulates the full
-// real-packed expansion in registers, then a butterfly reduction sums the lanes.
+// P2M: NL lanes per leaf; each strides over the leaf's particles and accumulates the full
+// real-packed expansion in registers, then the lanes' sums are added through shared memory.
 // ------------------------------------------------------------------------------------------
-// acc += sum over particles j = b0 + lane, b0 + lane + 32, ... < e0 of q_j conj(H_n^m(x^_j)),
+// acc += sum over particles j = b0 + lane, b0 + lane + NL, ... < e0 of q_j conj(H_n^m(x^_j)) / k_n^m,
 // x^ = (x - c) / h, with H the regular harmonics R (P2M, Eq. 2) or the irregular harmonics I
-// (P2L, Eq. 3), real-packed
-template <int P, bool IRREG>
+// (P2L, Eq. 3), real-packed.  The harmonics of one m are a power of x + iy (irregular: over r^2)
+// times real functions of one recurrence in n, H_n^m = k_n^m E_m g_n with
+//   g_m = 1, g_n = u g_{n-1} - beta_n^m v g_{n-2},   (u, v) = (z, r^2), irregular (z, 1) / r^2,
+// so a term costs 3 operations for the real recurrence and 2 sums instead of 8 or 10 with complex
+// ones; the constants k enter once per expansion (lanes_store).
+template <int P, bool IRREG, int NL>
 GB_DEV void p2x_particles(float (&acc)[P * P], const float4 *__restrict__ sx, int b0, int e0, int lane,
                           const CellGeom &cg)
 {
-    for (int j = b0 + lane; j < e0; j += 32) {
-        float4 p = __ldg(&sx[j]);
+    for (int j = b0 + lane; j < e0; j += NL) {
+        const float4 p = __ldg(&sx[j]);
         const float x = (p.x - cg.cx) * cg.inv_h, y = (p.y - cg.cy) * cg.inv_h, z = (p.z - cg.cz) * cg.inv_h;
-        const float q = p.w, r2 = x * x + y * y + z * z;
-        const float ir = IRREG ? rsqrt_ftz(r2) : 1.f;
-        const float ir2 = ir * ir;
-        float mre = ir, mim = 0.f;  // H_m^m
+        const float r2 = x * x + y * y + z * z;
+        const float ir = IRREG ? rsqrt_ftz(r2) : 1.f, v = IRREG ? ir * ir : r2;
+        const float u = IRREG ? z * v : z, xr = IRREG ? x * v : x, xi = IRREG ? y * v : y;
+        float er = IRREG ? p.w * ir : p.w, ei = 0.f;  // E_m = q (1/r) (x + iy)^m
 #pragma unroll
         for (int m = 0; m < P; ++m) {
-            if (m > 0) {
-                const float f = -c_rmm[m] * ir2;
-                const float tr = f * (x * mre - y * mim), ti = f * (x * mim + y * mre);
-                mre = tr;
-                mim = ti;
+            if (m == 1) {
+                ei = xi * er;
+                er = xr * er;
+            } else if (m > 1) {
+                const float tr = xr * er - xi * ei;
+                ei = xr * ei + xi * er;
+                er = tr;
             }
-            float are = mre, aim = mim, bre = 0.f, bim = 0.f;  // H_n^m, H_{n-1}^m
+            float g1 = 1.f, g2 = 0.f;
 #pragma unroll
             for (int n = m; n < P; ++n) {
-                if (n > m) {
-                    const float ca = c_ra[n - 1][m] * z, cb = c_rb[n - 1][m] * (IRREG ? 1.f : r2);
-                    float nre = ca * are - cb * bre, nim = ca * aim - cb * bim;
-                    if (IRREG) {
-                        nre *= ir2;
-                        nim *= ir2;
-                    }
-                    bre = are;
-                    bim = aim;
-                    are = nre;
-                    aim = nim;
+                if (n == m) {
+                    acc[re_idx(n, m)] += er;
+                    if (m > 0) acc[im_idx(n, m)] -= ei;
+                    continue;
                 }
-                acc[re_idx(n, m)] += q * are;
-                if (m > 0) acc[im_idx(n, m)] -= q * aim;
+                const float g = n == m + 1 ? u : fmaf(c_nbeta1[n][m], n == m + 2 ? v : v * g2, u * g1);
+                g2 = g1;
+                g1 = g;
+                acc[re_idx(n, m)] = fmaf(er, g, acc[re_idx(n, m)]);
+                if (m > 0) acc[im_idx(n, m)] = fmaf(-ei, g, acc[im_idx(n, m)]);
             }
         }
     }
 }
 
-// Warp-wide sum of acc over the lanes, stored to (or added into) dst: a transpose through the
-// warp's shared-memory scratch in two halves of the coefficients (each lane writes its row,
-// then lane j sums column j over the 32 rows).  scr holds 32 x (WS_H + 1) floats.
+// The sums of acc over each NL lanes of the warp, times k_n^m, stored to (or added into) the
+// lanes' dst (the same for the NL lanes; nullptr: nothing): a transpose through the warp's
+// shared-memory scratch in two halves of the coefficients (each lane writes its row, then a lane
+// per coefficient sums its column over the NL rows).  scr holds 32 x LD floats.
 template <int P>
 struct WarpSum {
     static constexpr int PP = P * P, H = (PP + 1) / 2, LD = H + 1;
 };
 
-template <int P>
-GB_DEV void warp_store(float (&acc)[P * P], float *dst, int lane, bool add, float *scr)
+template <int P, int NL>
+GB_DEV void lanes_store(float (&acc)[P * P], float *dst, int lane, bool add, float *scr)
 {
     using W = WarpSum<P>;
+    constexpr int NG = 32 / NL;
 #pragma unroll
     for (int part = 0; part < 2; ++part) {
         __syncwarp();
@@ -571,46 +577,60 @@ GB_DEV void warp_store(float (&acc)[P * P], float *dst, int lane, bool add, floa
         for (int i = 0; i < W::H; ++i)
             if (part * W::H + i < W::PP) scr[lane * W::LD + i] = acc[part * W::H + i];
         __syncwarp();
-        for (int i = lane; i < W::H && part * W::H + i < W::PP; i += 32) {
+        for (int i0 = 0; i0 < NG * W::H; i0 += 32) {
+            const int e = i0 + lane, gr = min(e / W::H, NG - 1), i = e - gr * W::H, k = part * W::H + i;
+            float *d = reinterpret_cast<float *>(
+                __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(dst), gr * NL));
+            if (i >= W::H || k >= W::PP || !d) continue;
             float v = 0.f;
 #pragma unroll 8
-            for (int r = 0; r < 32; ++r) v += scr[r * W::LD + i];
-            float *d = dst + part * W::H + i;
-            *d = add ? *d + v : v;
+            for (int r = 0; r < NL; ++r) v += scr[(gr * NL + r) * W::LD + i];
+            v *= __ldg(&d_kscale[k]);
+            d[k] = add ? d[k] + v : v;
         }
     }
 }
 
-template <int P>
+template <int P, int NL>
 __global__ void __launch_bounds__(128) k_p2m(int L, const float *__restrict__ geo, const float4 *__restrict__ sx,
                                              const int32_t *__restrict__ begin, const int32_t *__restrict__ end,
                                              float *__restrict__ M)
 {
     __shared__ float scr[4][32 * WarpSum<P>::LD];
     const int lane = threadIdx.x & 31;
-    const int64_t leaf = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (leaf >= (int64_t(1) << (3 * L))) return;
+    const int64_t leaf = (blockIdx.x * (int64_t)4 + (threadIdx.x >> 5)) * (32 / NL) + lane / NL;
     const int64_t g = level_offset(L) + leaf;
-    const int b0 = begin[g], e0 = end[g];
-    if (e0 <= b0) return;
-    const CellGeom cg = geo_level_cell(geo, L, (uint32_t)leaf);
+    int b0 = 0, e0 = 0;
+    if (leaf < (int64_t(1) << (3 * L))) b0 = begin[g], e0 = end[g];
+    if (__all_sync(0xffffffffu, e0 <= b0)) return;
     float acc[P * P];
 #pragma unroll
     for (int i = 0; i < P * P; ++i) acc[i] = 0.f;
-    p2x_particles<P, false>(acc, sx, b0, e0, lane, cg);
-    warp_store<P>(acc, M + g * (P * P), lane, false, scr[threadIdx.x >> 5]);
+    if (e0 > b0) {
+        const CellGeom cg = geo_level_cell(geo, L, (uint32_t)leaf);
+        p2x_particles<P, false, NL>(acc, sx, b0, e0, lane % NL, cg);
+    }
+    lanes_store<P, NL>(acc, e0 > b0 ? M + g * (P * P) : nullptr, lane, false, scr[threadIdx.x >> 5]);
 }
+
+// Lanes per leaf of P2M, by the expected number of leaves and not the counted one (a captured
+// batch lays its trees out for more): 8 where the leaves fill the GPU at four to a warp (rounds of
+// 8 waste fewer lanes than rounds of 32 on 15 to 40 particles, and 8 rows are added instead of
+// 32), else 32, a leaf's particles in as few rounds as possible.  P2M, 32 lanes and complex
+// recurrences -> 8 lanes and real ones: 1M uniform p = 10 64 -> 32 us, 5M p = 6 149 -> 62, 16M
+// Plummer p = 8 1122 -> 407; P2L there 2036 -> 1305.
+constexpr int64_t kP2MManyLeaves = 8 * 1024;
 
 void launch_p2m(int P, int L, const float *geo, const float4 *sx, const int32_t *begin, const int32_t *end, float *M,
                 cudaStream_t s)
 {
-    int64_t nl = int64_t(1) << (3 * L);
-    unsigned grid = (unsigned)((nl + 3) / 4);
-    switch (P) {
-    case 4: k_p2m<4><<<grid, 128, 0, s>>>(L, geo, sx, begin, end, M); break;
-    case 6: k_p2m<6><<<grid, 128, 0, s>>>(L, geo, sx, begin, end, M); break;
-    case 8: k_p2m<8><<<grid, 128, 0, s>>>(L, geo, sx, begin, end, M); break;
-    case 10: k_p2m<10><<<grid, 128, 0, s>>>(L, geo, sx, begin, end, M); break;
+    const int64_t nl = int64_t(1) << (3 * L);
+    if (nl >= kP2MManyLeaves) {
+        const unsigned grid = (unsigned)((nl + 15) / 16);
+        GBFMM_DISPATCH_P(P, (k_p2m<PQ, 8><<<grid, 128, 0, s>>>(L, geo, sx, begin, end, M)));
+    } else {
+        const unsigned grid = (unsigned)((nl + 3) / 4);
+        GBFMM_DISPATCH_P(P, (k_p2m<PQ, 32><<<grid, 128, 0, s>>>(L, geo, sx, begin, end, M)));
     }
     note_launches(1);
 }
@@ -948,68 +968,101 @@ void launch_l2l(int P, int l, const int32_t *begin, const int32_t *end, const fl
 //   dphi/dx + i dphi/dy = sum_{n<P-1} sum_m s(m) sqrt((n+2-m)(n+1-m)) L_{n+1}^{m-1} R_n^m,
 //   s(m) = +1 for m >= 1, -1 for m <= 0.
 // ------------------------------------------------------------------------------------------
+// With R_n^m = E_m g_n, E_m a constant times (x^ + i y^)^m and g_n real, every m needs three complex
+// sums, F_m = sum L_n^m g_n, Z_m = sum sqrt((n+1-m)(n+1+m)) L_{n+1}^m g_n and
+// A_m = sum sqrt((n+2-m)(n+1-m)) L_{n+1}^{m-1} g_n; the lowered term of dphi/dx + i dphi/dy follows
+// from F_m and A_{m+1} as in M2P (there in powers of xi), with the constants' ratios
+// E_m / (x^ + i y^) E_{m-1} = -c_rmm[m].  Half the operations of complex recurrences and four sums,
+// and each coefficient is read once, a column of L at a time, instead of five times.
+template <int P>
+struct L2PState {
+    float x, y, z, r2, rho2;
+    float phi = 0.f, gz = 0.f, gr = 0.f, gi = 0.f;
+    float er = 1.f, ei = 0.f, er1 = 0.f, ei1 = 0.f;  // E_m, E_{m-1}
+    float fr1 = 0.f, fi1 = 0.f;                      // F_{m-1}
+    float pr[P], pi[P];                              // L_n^{m-1}
+};
+
+// orders M, M + 1, ..., P (P: the last lowered term only)
+template <int P, int M>
+GB_DEV void l2p_orders(L2PState<P> &s, const float *__restrict__ Lg)
+{
+    float fr = 0.f, fi = 0.f, zr = 0.f, zi = 0.f, ar = 0.f, ai = 0.f;
+    const float er2 = s.er1, ei2 = s.ei1;  // E_{m-2}
+    if constexpr (M > 0 && M < P) {
+        s.er1 = s.er, s.ei1 = s.ei;
+        const float f = -c_rmm[M];
+        s.er = f * (s.x * s.er1 - s.y * s.ei1);
+        s.ei = f * (s.x * s.ei1 + s.y * s.er1);
+    }
+    if constexpr (M < P) {
+        float cr[P], ci[P];
+#pragma unroll
+        for (int n = M; n < P; ++n) {
+            cr[n] = __ldg(&Lg[re_idx(n, M)]);
+            ci[n] = M > 0 ? __ldg(&Lg[im_idx(n, M)]) : 0.f;
+        }
+        float g1 = 1.f, g2 = 0.f;
+#pragma unroll
+        for (int n = M; n < P; ++n) {
+            float g = 1.f;
+            if (n > M) {
+                g = c_ra[n - 1][M] * (s.z * g1);
+                if (n > M + 1) g = fmaf(-c_rb[n - 1][M], s.r2 * g2, g);
+                g2 = g1;
+                g1 = g;
+            }
+            fr = fmaf(cr[n], g, fr);
+            if (M > 0) fi = fmaf(ci[n], g, fi);
+            if (n + 1 < P) {
+                const float gs = c_sq[n + 1 - M][n + 1 + M] * g;
+                zr = fmaf(cr[n + 1], gs, zr);
+                if (M > 0) {
+                    zi = fmaf(ci[n + 1], gs, zi);
+                    const float ga = c_sq[n + 2 - M][n + 1 - M] * g;
+                    ar = fmaf(s.pr[n + 1], ga, ar);
+                    if (M > 1) ai = fmaf(s.pi[n + 1], ga, ai);
+                }
+            }
+        }
+        if (M == 0) {
+            s.phi = fr;
+            s.gz = zr;
+        } else {
+            s.phi = fmaf(2.f, s.er * fr - s.ei * fi, s.phi);
+            s.gz = fmaf(2.f, s.er * zr - s.ei * zi, s.gz);
+            s.gr += s.er * ar - s.ei * ai;
+            s.gi += s.er * ai + s.ei * ar;
+        }
+#pragma unroll
+        for (int n = M; n < P; ++n) {
+            s.pr[n] = cr[n];
+            s.pi[n] = ci[n];
+        }
+    }
+    if constexpr (M >= 2) {  // the lowered term of order M - 1, with E_{M-2}
+        const float e0 = M < P ? er2 : s.er1, e1 = M < P ? ei2 : s.ei1;
+        const float cf = -2.f * (M - 1) * c_rmm[M - 1], ca = M < P ? c_rmm[M] * c_rmm[M - 1] * s.rho2 : 0.f;
+        const float tr = fmaf(cf, s.fr1, ca * ar), ti = fmaf(cf, s.fi1, ca * ai);
+        s.gr += e0 * tr - e1 * ti;
+        s.gi -= e0 * ti + e1 * tr;
+    }
+    s.fr1 = fr;
+    s.fi1 = fi;
+    if constexpr (M < P) l2p_orders<P, M + 1>(s, Lg);
+}
+
 // value and gradient of the scaled local expansion Lg at x^ (multiplied by 1/h and 1/h^2)
 template <int P>
 GB_DEV float4 l2p_eval(const float *__restrict__ Lg, float x, float y, float z, float ih)
 {
-    const float r2 = x * x + y * y + z * z;
-    float phi = 0.f, gz = 0.f, gpr = 0.f, gpi = 0.f;
-    float mre = 1.f, mim = 0.f;
-#pragma unroll
-    for (int m = 0; m < P; ++m) {
-        if (m > 0) {
-            const float f = -c_rmm[m];
-            const float tr = f * (x * mre - y * mim), ti = f * (x * mim + y * mre);
-            mre = tr;
-            mim = ti;
-        }
-        float are = mre, aim = mim, bre = 0.f, bim = 0.f;
-#pragma unroll
-        for (int nn = m; nn < P; ++nn) {
-            if (nn > m) {
-                const float ca = c_ra[nn - 1][m] * z, cb = c_rb[nn - 1][m] * r2;
-                const float nre = ca * are - cb * bre, nim = ca * aim - cb * bim;
-                bre = are;
-                bim = aim;
-                are = nre;
-                aim = nim;
-            }
-            // phi: L_nn^m R_nn^m
-            {
-                const float lre = __ldg(&Lg[re_idx(nn, m)]);
-                const float lim = (m > 0) ? __ldg(&Lg[im_idx(nn, m)]) : 0.f;
-                const float w = (m > 0) ? 2.f : 1.f;
-                phi += w * (lre * are - lim * aim);
-            }
-            if (nn + 1 < P) {
-                // d/dz: L_{nn+1}^m R_nn^m
-                {
-                    const float lre = __ldg(&Lg[re_idx(nn + 1, m)]);
-                    const float lim = (m > 0) ? __ldg(&Lg[im_idx(nn + 1, m)]) : 0.f;
-                    const float w = (m > 0) ? 2.f : 1.f;
-                    gz += w * c_sq[nn + 1 - m][nn + 1 + m] * (lre * are - lim * aim);
-                }
-                // d/dx + i d/dy, term mu = m >= 1: + sqrt((nn+2-m)(nn+1-m)) L_{nn+1}^{m-1} R_nn^m
-                if (m >= 1) {
-                    const float lre = __ldg(&Lg[re_idx(nn + 1, m - 1)]);
-                    const float lim = (m - 1 > 0) ? __ldg(&Lg[im_idx(nn + 1, m - 1)]) : 0.f;
-                    const float c = c_sq[nn + 2 - m][nn + 1 - m];
-                    gpr += c * (lre * are - lim * aim);
-                    gpi += c * (lre * aim + lim * are);
-                }
-                // term mu = -m <= 0: - sqrt((nn+2+m)(nn+1+m)) conj(L_{nn+1}^{m+1} R_nn^m)
-                {
-                    const float lre = __ldg(&Lg[re_idx(nn + 1, m + 1)]);
-                    const float lim = __ldg(&Lg[im_idx(nn + 1, m + 1)]);
-                    const float c = c_sq[nn + 2 + m][nn + 1 + m];
-                    gpr -= c * (lre * are - lim * aim);
-                    gpi += c * (lre * aim + lim * are);
-                }
-            }
-        }
-    }
+    L2PState<P> s;
+    s.x = x, s.y = y, s.z = z;
+    s.rho2 = x * x + y * y;
+    s.r2 = s.rho2 + z * z;
+    l2p_orders<P, 0>(s, Lg);
     const float ih2 = ih * ih;
-    return make_float4(phi * ih, gpr * ih2, gpi * ih2, gz * ih2);
+    return make_float4(s.phi * ih, s.gr * ih2, s.gi * ih2, s.gz * ih2);
 }
 
 // the near-field compensated sums of particle i (sorted order: the sums, then their
@@ -1113,6 +1166,7 @@ void m2p_tables()
 {
     static int2 tab[4][kM2PMaxNO];
     static uint64_t nbeta[kMaxP + 1][kMaxP + 1];
+    static float nbeta1[kMaxP + 1][kMaxP + 1], kscale[kMaxP * kMaxP];
     auto ra = [](int n, int m) { return (2.0 * n + 1.0) / sqrt((double)(n + 1 - m) * (n + 1 + m)); };
     auto rb = [](int n, int m) { return sqrt((double)(n - m) * (n + m)) / sqrt((double)(n + 1 - m) * (n + 1 + m)); };
     const int orders[4] = {4, 6, 8, 10};
@@ -1130,6 +1184,11 @@ void m2p_tables()
                 uint32_t bits;
                 memcpy(&bits, &f, 4);
                 nbeta[N][m] = (uint64_t)bits << 32 | bits;
+                nbeta1[N][m] = f;
+            }
+            if (N < kMaxP) {
+                kscale[re_idx(N, m)] = (float)k;
+                if (m > 0) kscale[im_idx(N, m)] = (float)k;
             }
             for (int o = 0; o < 4; ++o) {
                 const int P = orders[o];
@@ -1149,6 +1208,8 @@ void m2p_tables()
     }
     cudaMemcpyToSymbol(d_m2p_tab, tab, sizeof(tab));
     cudaMemcpyToSymbol(c_nbeta, nbeta, sizeof(nbeta));
+    cudaMemcpyToSymbol(c_nbeta1, nbeta1, sizeof(nbeta1));
+    cudaMemcpyToSymbol(d_kscale, kscale, sizeof(kscale));
 }
 
 GB_DEV uint64_t neg2(uint64_t v) { return v ^ 0x8000000080000000ull; }
@@ -1413,8 +1474,8 @@ void launch_cell_geom(Span cells, const int32_t *level, const uint64_t *key, con
     note_launches(1);
 }
 
-// P2M at the listed leaves (levels >= 2), one warp per leaf
-template <int P>
+// P2M at the listed leaves (levels >= 2), NL lanes per leaf
+template <int P, int NL>
 __global__ void __launch_bounds__(128) k_p2m_cells(const int32_t *__restrict__ leaves, Span lv,
                                                    const int32_t *__restrict__ level, const float4 *__restrict__ geom,
                                                    const int32_t *__restrict__ begin, const int32_t *__restrict__ count,
@@ -1422,21 +1483,20 @@ __global__ void __launch_bounds__(128) k_p2m_cells(const int32_t *__restrict__ l
 {
     __shared__ float scr[4][32 * WarpSum<P>::LD];
     const int lane = threadIdx.x & 31;
-    const int64_t w = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (w >= span_count(lv)) return;
-    const int32_t c = leaves[w];
-    if (level[c] < 2) return;
-    const CellGeom cg = geo_cell(geom, c);
+    const int64_t w = (blockIdx.x * (int64_t)4 + (threadIdx.x >> 5)) * (32 / NL) + lane / NL;
+    int32_t c = w < span_count(lv) ? leaves[w] : -1;
+    if (c >= 0 && level[c] < 2) c = -1;
+    if (__all_sync(0xffffffffu, c < 0)) return;
     float acc[P * P];
 #pragma unroll
     for (int i = 0; i < P * P; ++i) acc[i] = 0.f;
-    p2x_particles<P, false>(acc, sx, begin[c], begin[c] + count[c], lane, cg);
-    warp_store<P>(acc, M + (int64_t)c * (P * P), lane, false, scr[threadIdx.x >> 5]);
+    if (c >= 0) p2x_particles<P, false, NL>(acc, sx, begin[c], begin[c] + count[c], lane % NL, geo_cell(geom, c));
+    lanes_store<P, NL>(acc, c >= 0 ? M + (int64_t)c * (P * P) : nullptr, lane, false, scr[threadIdx.x >> 5]);
 }
 
-// P2L over the X list (Eq. 3's L from the particles of each X leaf), one warp per cell; adds
+// P2L over the X list (Eq. 3's L from the particles of each X leaf), NL lanes per cell; adds
 // into the cell's local expansion
-template <int P>
+template <int P, int NL>
 __global__ void __launch_bounds__(128) k_p2l_cells(Span cells, const int32_t *__restrict__ level,
                                                    const float4 *__restrict__ geom, const int32_t *__restrict__ begin,
                                                    const int32_t *__restrict__ count,
@@ -1446,20 +1506,22 @@ __global__ void __launch_bounds__(128) k_p2l_cells(Span cells, const int32_t *__
 {
     __shared__ float scr[4][32 * WarpSum<P>::LD];
     const int lane = threadIdx.x & 31;
-    const int64_t w = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (w >= span_count(cells)) return;
+    const int64_t w = (blockIdx.x * (int64_t)4 + (threadIdx.x >> 5)) * (32 / NL) + lane / NL;
     const int64_t b = span_first(cells) + w;
-    const uint32_t e0 = x_offs[b], e1 = x_offs[b + 1];
-    if (e0 == e1 || level[b] < 2) return;
-    const CellGeom cg = geo_cell(geom, b);
+    uint32_t e0 = 0, e1 = 0;
+    if (w < span_count(cells) && level[b] >= 2) e0 = x_offs[b], e1 = x_offs[b + 1];
+    if (__all_sync(0xffffffffu, e0 == e1)) return;
     float acc[P * P];
 #pragma unroll
     for (int i = 0; i < P * P; ++i) acc[i] = 0.f;
-    for (uint32_t e = e0; e < e1; ++e) {
-        const int32_t c = x_ids[e];
-        p2x_particles<P, true>(acc, sx, begin[c], begin[c] + count[c], lane, cg);
+    if (e0 < e1) {
+        const CellGeom cg = geo_cell(geom, b);
+        for (uint32_t e = e0; e < e1; ++e) {
+            const int32_t c = x_ids[e];
+            p2x_particles<P, true, NL>(acc, sx, begin[c], begin[c] + count[c], lane % NL, cg);
+        }
     }
-    warp_store<P>(acc, Lc + b * (P * P), lane, true, scr[threadIdx.x >> 5]);
+    lanes_store<P, NL>(acc, e0 < e1 ? Lc + b * (P * P) : nullptr, lane, true, scr[threadIdx.x >> 5]);
 }
 
 // L2P at every particle's leaf (leaves above level 2 carry no local expansion)
@@ -1614,23 +1676,37 @@ __global__ void __launch_bounds__(TransCfg<P, UP, TN, CN>::NT) k_translate_cells
     }
 }
 
-void launch_p2m_cells(int P, const int32_t *leaves, Span lv, const int32_t *level, const float4 *geom,
-                      const int32_t *begin, const int32_t *count, const float4 *sx, float *M, cudaStream_t s)
+void launch_p2m_cells(int P, int64_t est_leaves, const int32_t *leaves, Span lv, const int32_t *level,
+                      const float4 *geom, const int32_t *begin, const int32_t *count, const float4 *sx, float *M,
+                      cudaStream_t s)
 {
     if (lv.cap <= 0) return;
-    const unsigned grid = (unsigned)((lv.cap + 3) / 4);
-    GBFMM_DISPATCH_P(P, (k_p2m_cells<PQ><<<grid, 128, 0, s>>>(leaves, lv, level, geom, begin, count, sx, M)));
+    if (est_leaves >= kP2MManyLeaves) {
+        const unsigned grid = (unsigned)((lv.cap + 15) / 16);
+        GBFMM_DISPATCH_P(P, (k_p2m_cells<PQ, 8><<<grid, 128, 0, s>>>(leaves, lv, level, geom, begin, count, sx, M)));
+    } else {
+        const unsigned grid = (unsigned)((lv.cap + 3) / 4);
+        GBFMM_DISPATCH_P(P, (k_p2m_cells<PQ, 32><<<grid, 128, 0, s>>>(leaves, lv, level, geom, begin, count, sx, M)));
+    }
     note_launches(1);
 }
 
-void launch_p2l_cells(int P, Span cells, const int32_t *level, const float4 *geom, const int32_t *begin,
+void launch_p2l_cells(int P, int64_t est_leaves, Span cells, const int32_t *level, const float4 *geom, const int32_t *begin,
                       const int32_t *count, const uint32_t *x_offs, const int32_t *x_ids, const float4 *sx, float *Lc,
                       cudaStream_t s)
 {
     if (cells.cap <= 0) return;
-    const unsigned grid = (unsigned)((cells.cap + 3) / 4);
-    GBFMM_DISPATCH_P(P, (k_p2l_cells<PQ><<<grid, 128, 0, s>>>(cells, level, geom, begin, count, x_offs, x_ids, sx,
-                                                              Lc)));
+    // an X leaf of 30 to 60 particles wastes fewer lanes in rounds of 16 (16M Plummer step 23.35 ->
+    // 23.15 ms, 400,009 1696 -> 1686 us); few cells want them in few rounds (20,011: 386 against 389)
+    if (est_leaves >= kP2MManyLeaves) {
+        const unsigned grid = (unsigned)((cells.cap + 7) / 8);
+        GBFMM_DISPATCH_P(P, (k_p2l_cells<PQ, 16><<<grid, 128, 0, s>>>(cells, level, geom, begin, count, x_offs, x_ids,
+                                                                      sx, Lc)));
+    } else {
+        const unsigned grid = (unsigned)((cells.cap + 3) / 4);
+        GBFMM_DISPATCH_P(P, (k_p2l_cells<PQ, 32><<<grid, 128, 0, s>>>(cells, level, geom, begin, count, x_offs, x_ids,
+                                                                      sx, Lc)));
+    }
     note_launches(1);
 }
 
