@@ -19,28 +19,15 @@
 #include "common.cuh"
 #include "ptx.cuh"
 
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 namespace gbfmm {
 
-template <bool SOFT>
-GB_DEV void pair(float xi, float yi, float zi, float4 s, float eps2, float &phi, float &gx, float &gy, float &gz)
-{
-    const float dx = xi - s.x, dy = yi - s.y, dz = zi - s.z;
-    const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-    float inv = rsqrt_ftz(SOFT ? d2 + eps2 : d2);
-    inv = d2 > 0.f ? inv : 0.f;
-    const float qi = s.w * inv;
-    phi += qi;
-    const float qi3 = qi * inv * inv;
-    gx = fmaf(-dx, qi3, gx);
-    gy = fmaf(-dy, qi3, gy);
-    gz = fmaf(-dz, qi3, gz);
-}
-
-// The pair rule of pair() for two targets at once, in packed FP32 (fma.rn.f32x2 and its kin: two
-// lanes per instruction), against one source; the zero-distance test only where MASK (the targets'
-// own cell).  nx, ny, nz: the targets' negated coordinates; the sums are those of pair().  The loop
+// The pair rule for two targets at once, in packed FP32 (fma.rn.f32x2 and its kin: two lanes per
+// instruction), against one source; the zero-distance test only where MASK (the targets' own cell).
+// nx, ny, nz: the targets' negated coordinates; gx, gy, gz: the gradient's sums.  The loop
 // of scalar pairs was bound by instruction issue: of its own, 2.02e12 pairs/s scalar, 2.24e12 packed.
 template <bool SOFT, bool MASK>
 GB_DEV void pair2(uint64_t nx, uint64_t ny, uint64_t nz, float4 s, uint64_t eps2, uint64_t &phi, uint64_t &gx,
@@ -449,36 +436,118 @@ void launch_p2p_cells_near(const int32_t *leaves, Span lv, int64_t n, const floa
     launch_leaf(lv.cap, 0, leaves, sx, begin, end, u_offs, u_ids, nullptr, nullptr, eps2, nullptr, near, status, s, lv);
 }
 
-// Direct all-pairs sum: one thread per target, sources streamed through shared memory in
-// tiles of the block size (the tile model of the GPU Gems 3 all-pairs kernel the paper builds on).
-constexpr int kDirectThreads = 256;
+// Direct all-pairs sum.  A CTA takes 64 targets, two per lane in packed pairs, and its four warps
+// share the sources staged in shared memory (cp.async, the next tile in flight), four sources at a
+// time; a cluster of 8 CTAs splits the sources of the same targets, and the sums are added through
+// distributed shared memory, warps then CTAs in order.  So a call has 8 x 4 x n_tgt / 64 warps: with
+// a thread per target (256 to a CTA, every source in turn) 16,411 targets filled 65 of 152 SMs:
+// 442 -> 144 us.  Bound by the FP32 pipe.
+// Any two particles may coincide; the zero-distance test is made on the least of four sources' d2
+// (NaN included) and only a group that fails it takes the masked rule.
+constexpr int kDirectThreads = 128, kDirectTargets = 64, kDirectTile = 512, kDirectSplit = 8;
+
+// the least of four packed pairs; NaN if any of them is
+GB_DEV float least8(const uint64_t (&d2)[4])
+{
+    float v[8], m;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) unpack2(d2[u], v[2 * u], v[2 * u + 1]);
+    asm("min.NaN.f32 %0, %1, %2, %3;" : "=f"(m) : "f"(v[0]), "f"(v[1]), "f"(v[2]));
+    asm("min.NaN.f32 %0, %1, %2, %3;" : "=f"(m) : "f"(m), "f"(v[3]), "f"(v[4]));
+    asm("min.NaN.f32 %0, %1, %2, %3;" : "=f"(m) : "f"(m), "f"(v[5]), "f"(v[6]));
+    asm("min.NaN.f32 %0, %1, %2;" : "=f"(m) : "f"(m), "f"(v[7]));
+    return m;
+}
 
 template <bool SOFT>
-__global__ void __launch_bounds__(kDirectThreads) k_direct(int64_t ns, const float4 *__restrict__ src, int64_t nt,
-                                                           const float4 *__restrict__ tgt, float eps2,
-                                                           float4 *__restrict__ out)
+__global__ void __cluster_dims__(kDirectSplit, 1, 1) __launch_bounds__(kDirectThreads)
+    k_direct(int64_t ns, const float4 *__restrict__ src, int64_t nt, const float4 *__restrict__ tgt, float eps2,
+             float4 *__restrict__ out)
 {
-    __shared__ float4 tile[kDirectThreads];
-    const int64_t i = blockIdx.x * (int64_t)kDirectThreads + threadIdx.x;
-    const float4 xi = i < nt ? __ldg(&tgt[i]) : make_float4(0.f, 0.f, 0.f, 0.f);
-    float phi = 0.f, gx = 0.f, gy = 0.f, gz = 0.f;
-    for (int64_t b = 0; b < ns; b += kDirectThreads) {
-        const int64_t j = b + threadIdx.x;
-        tile[threadIdx.x] = j < ns ? __ldg(&src[j]) : make_float4(0.f, 0.f, 0.f, 0.f);
-        __syncthreads();
-        const int cnt = (int)(ns - b < kDirectThreads ? ns - b : kDirectThreads);
-#pragma unroll 8
-        for (int k = 0; k < cnt; ++k) pair<SOFT>(xi.x, xi.y, xi.z, tile[k], eps2, phi, gx, gy, gz);
-        __syncthreads();
+    namespace cg = cooperative_groups;
+    __shared__ __align__(16) float4 tile[2][kDirectTile];
+    __shared__ float4 red[kDirectThreads / 32][kDirectTargets];
+    __shared__ float4 sum[kDirectTargets];
+    const cg::cluster_group cl = cg::this_cluster();
+    const int rank = (int)cl.block_rank(), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t t0 = (int64_t)(blockIdx.x / kDirectSplit) * kDirectTargets;
+    const int64_t per = (ns + kDirectSplit - 1) / kDirectSplit, s0 = rank * per, s1 = min(ns, s0 + per);
+    auto target = [&](int k) { return t0 + k < nt ? __ldg(&tgt[t0 + k]) : make_float4(0.f, 0.f, 0.f, 0.f); };
+    const float4 A = target(lane), B = target(lane + 32);
+    const uint64_t nx = pack2(-A.x, -B.x), ny = pack2(-A.y, -B.y), nz = pack2(-A.z, -B.z), e2 = pack2(eps2, eps2);
+    uint64_t phi = 0, gx = 0, gy = 0, gz = 0;
+    auto stage = [&](int64_t b, int buf) {
+        for (int k = tid; k < kDirectTile; k += kDirectThreads)
+            if (b + k < s1) cp_async16(&tile[buf][k], &src[b + k], 16u);
+        cp_async_commit();
+    };
+    if (s0 < s1) stage(s0, 0);
+    int buf = 0;
+    for (int64_t b = s0; b < s1; b += kDirectTile, buf ^= 1) {
+        cp_async_wait<0>();
+        __syncthreads();  // the tile is there, and the other buffer's readers are done
+        if (b + kDirectTile < s1) stage(b + kDirectTile, buf ^ 1);
+        const int cnt = (int)min((int64_t)kDirectTile, s1 - b);
+        const float4 *S = tile[buf];
+        int j = 4 * warp;
+        for (; j + 4 <= cnt; j += kDirectThreads / 8) {
+            uint64_t dx[4], dy[4], dz[4], d2[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const float4 q = S[j + u];
+                dx[u] = add2(pack2(q.x, q.x), nx), dy[u] = add2(pack2(q.y, q.y), ny), dz[u] = add2(pack2(q.z, q.z), nz);
+                d2[u] = fma2(dx[u], dx[u], fma2(dy[u], dy[u], mul2(dz[u], dz[u])));
+            }
+            if (least8(d2) > 0.f) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const float qw = S[j + u].w;
+                    float a, c;
+                    unpack2(SOFT ? add2(d2[u], e2) : d2[u], a, c);
+                    const uint64_t inv = pack2(rsqrt_ftz(a), rsqrt_ftz(c)), w = mul2(pack2(qw, qw), inv);
+                    phi = add2(phi, w);
+                    const uint64_t w3 = mul2(mul2(w, inv), inv);
+                    gx = fma2(dx[u], w3, gx);
+                    gy = fma2(dy[u], w3, gy);
+                    gz = fma2(dz[u], w3, gz);
+                }
+            } else {
+                for (int u = 0; u < 4; ++u) pair2<SOFT, true>(nx, ny, nz, S[j + u], e2, phi, gx, gy, gz);
+            }
+        }
+        for (; j < cnt; ++j) pair2<SOFT, true>(nx, ny, nz, S[j], e2, phi, gx, gy, gz);  // at most three, of one warp
     }
-    if (i < nt) out[i] = make_float4(phi, gx, gy, gz);
+    float4 va, vb;
+    unpack2(phi, va.x, vb.x);
+    unpack2(gx, va.y, vb.y);
+    unpack2(gy, va.z, vb.z);
+    unpack2(gz, va.w, vb.w);
+    red[warp][lane] = va;
+    red[warp][lane + 32] = vb;
+    __syncthreads();
+    auto add = [](float4 &r, const float4 &v) { r.x += v.x, r.y += v.y, r.z += v.z, r.w += v.w; };
+    if (tid < kDirectTargets) {
+        float4 r = red[0][tid];
+#pragma unroll
+        for (int w = 1; w < kDirectThreads / 32; ++w) add(r, red[w][tid]);
+        sum[tid] = r;
+    }
+    cl.sync();
+    // CTA `rank` adds the 8 CTAs' sums of its eighth of the targets
+    const int k = rank * (kDirectTargets / kDirectSplit) + tid;
+    if (tid < kDirectTargets / kDirectSplit && t0 + k < nt) {
+        float4 r = *cl.map_shared_rank(&sum[k], 0);
+        for (int c = 1; c < kDirectSplit; ++c) add(r, *cl.map_shared_rank(&sum[k], c));
+        out[t0 + k] = r;
+    }
+    cl.sync();  // no CTA leaves while its sums may be read
 }
 
 void launch_direct(int64_t n_src, const float4 *src, int64_t n_tgt, const float4 *tgt, float eps2, float4 *out,
                    cudaStream_t s)
 {
     if (n_tgt <= 0) return;
-    unsigned grid = (unsigned)((n_tgt + kDirectThreads - 1) / kDirectThreads);
+    const unsigned grid = (unsigned)((n_tgt + kDirectTargets - 1) / kDirectTargets * kDirectSplit);
     if (eps2 > 0.f)
         k_direct<true><<<grid, kDirectThreads, 0, s>>>(n_src, src, n_tgt, tgt, eps2, out);
     else
