@@ -155,21 +155,22 @@ GB_DEV float blk_pow2(int e) { return __int_as_float((127 + e) << 23); }
 // coefficients of its children (child sigma at [sigma p^2, (sigma + 1) p^2)) scaled by 2^s_S and
 // split into FP16 hi (plane 0) and lo (plane 1); s_S = 10 - e with max |M~| = f 2^e, f in
 // [0.5, 1) over the parent's nonempty children (empty children and empty parents: zeros, s = 0).
-// One warp per parent.
+// One warp per parent; the launch covers the parents of every level 1..L - 1 (A and scale hold the
+// levels one after another).
 template <int P>
-__global__ void __launch_bounds__(256) k_blk_presplit(int l, const int32_t *__restrict__ begin,
+__global__ void __launch_bounds__(256) k_blk_presplit(int L, const int32_t *__restrict__ begin,
                                                       const int32_t *__restrict__ end, const float *__restrict__ M,
                                                       __half *__restrict__ A, int8_t *__restrict__ scale)
 {
     constexpr int PP = P * P, KD = 8 * PP, PER = (KD + 31) / 32;
     const int lane = threadIdx.x & 31;
-    const int lp = l - 1;
-    const int64_t np = int64_t(1) << (3 * lp);
-    const int64_t i = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (i >= np) return;
-    const int pg = 1 << lp;
-    const int x = (int)(i % pg), y = (int)((i / pg) % pg), z = (int)(i / ((int64_t)pg * pg));
-    const int64_t c0 = level_offset(l) + 8 * (int64_t)morton3((uint32_t)x, (uint32_t)y, (uint32_t)z);
+    const int64_t i = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);  // parent 1 + i of all levels
+    if (i >= level_offset(L) - 1) return;
+    int lp = 1;
+    while (i + 1 >= level_offset(lp + 1)) ++lp;
+    const uint32_t il = (uint32_t)(i + 1 - level_offset(lp)), pg = 1u << lp;  // grid order, x fastest
+    const uint32_t x = il & (pg - 1), y = (il >> lp) & (pg - 1), z = il >> (2 * lp);
+    const int64_t c0 = level_offset(lp + 1) + 8 * (int64_t)morton3(x, y, z);
     float v[PER];
     float m = 0.f;
 #pragma unroll
@@ -919,17 +920,27 @@ static int blk_tiles_p(int P, int L)
     return 0;
 }
 
-// offset ranges per tile: 1 when there are at least kBlkFillCtas tiles (one per SM of a
-// 152-SM GB300), else enough ranges for about twice that many CTAs (each range a whole number of
-// offsets, at most 26).  A fixed rule, so that the workspace size does not depend on the device.
+// Offset ranges per tile: 1 when there are at least kBlkFillCtas tiles (one per SM of a 152-SM
+// GB300), else the number of ranges k with the least time in waves of kBlkFillCtas CTAs, a CTA of
+// ceil(26 / k) offsets costing that many plus two for its start, first copies and last drain (and
+// the sum of the ranges, half an offset).  12 tiles (100,000 particles, p = 8): 26 ranges took three
+// launches, the last of 8 CTAs, 75 us and 10 for the sum; 12 ranges one, and the step 244 -> 193 us.  A fixed rule, so that the workspace
+// size does not depend on the device.
 constexpr int kBlkFillCtas = 152;
-int m2l_blk_ksplit(int P, int L)
+static int blk_ranges(int64_t tiles)
 {
-    const int t = blk_tiles_p(P, L);
-    if (L < 2 || t <= 0 || t >= kBlkFillCtas) return 1;
-    const int k = (2 * kBlkFillCtas + t - 1) / t;
-    return k < 26 ? k : 26;
+    if (tiles <= 0 || tiles >= kBlkFillCtas) return 1;
+    int best = 1;
+    int64_t least = INT64_MAX;
+    for (int k = 1; k <= 26; ++k) {
+        const int64_t waves = (tiles * k + kBlkFillCtas - 1) / kBlkFillCtas;
+        const int64_t cost = 2 * waves * ((26 + k - 1) / k + 2) + (k > 1 ? 1 : 0);
+        if (cost < least) least = cost, best = k;
+    }
+    return best;
 }
+
+int m2l_blk_ksplit(int P, int L) { return L < 2 ? 1 : blk_ranges(blk_tiles_p(P, L)); }
 
 // partial sums of the offset ranges: ksplit x (cells of levels 0..L) x p^2 floats (0 if not split)
 size_t m2l_blk_part_bytes(int P, int L)
@@ -977,20 +988,16 @@ void launch_build_m2l_blk(int P, const float *ops, void *table, cudaStream_t s)
 void launch_blk_presplit(int P, int L, const int32_t *begin, const int32_t *end, const float *M, void *presplit,
                          int8_t *pscale, cudaStream_t s)
 {
-    const size_t KD = 8 * (size_t)P * P;
-    for (int l = 2; l <= L; ++l) {
-        const int64_t np = int64_t(1) << (3 * (l - 1));
-        __half *A = static_cast<__half *>(presplit) + (size_t)blk_parents_before(l - 1) * 2 * KD;
-        int8_t *sc = pscale + blk_parents_before(l - 1);
-        const unsigned grid = (unsigned)((np + 7) / 8);
-        switch (P) {
-        case 4: k_blk_presplit<4><<<grid, 256, 0, s>>>(l, begin, end, M, A, sc); break;
-        case 6: k_blk_presplit<6><<<grid, 256, 0, s>>>(l, begin, end, M, A, sc); break;
-        case 8: k_blk_presplit<8><<<grid, 256, 0, s>>>(l, begin, end, M, A, sc); break;
-        case 10: k_blk_presplit<10><<<grid, 256, 0, s>>>(l, begin, end, M, A, sc); break;
-        }
-        note_launches(1);
+    if (L < 2) return;
+    const unsigned grid = (unsigned)((blk_parents_before(L) + 7) / 8);
+    __half *A = static_cast<__half *>(presplit);
+    switch (P) {
+    case 4: k_blk_presplit<4><<<grid, 256, 0, s>>>(L, begin, end, M, A, pscale); break;
+    case 6: k_blk_presplit<6><<<grid, 256, 0, s>>>(L, begin, end, M, A, pscale); break;
+    case 8: k_blk_presplit<8><<<grid, 256, 0, s>>>(L, begin, end, M, A, pscale); break;
+    case 10: k_blk_presplit<10><<<grid, 256, 0, s>>>(L, begin, end, M, A, pscale); break;
     }
+    note_launches(1);
 }
 
 template <int P, int CH>
@@ -1084,17 +1091,15 @@ int64_t m2l_ablk_tiles_units(int64_t ucap) { return (ucap + kBlkRows - 1) / kBlk
 size_t m2l_ablk_src_bytes(int64_t ucap) { return (size_t)m2l_ablk_tiles_units(ucap) * 26 * sizeof(int32_t); }
 
 // offset ranges per tile from the particle count and leaf size alone (an estimate of the units:
-// a quarter of n / leaf_size), so that evaluations of the same count split alike whatever their
-// trees (a captured batch and the same instance alone sum in the same order)
+// half of n / leaf_size, as on Plummer spheres; 400,009 particles, leaf 64: 3,077), so that
+// evaluations of the same count split alike whatever their trees (a captured batch and the same
+// instance alone sum in the same order)
 int m2l_ablk_ksplit(int P, int64_t n, int leaf_size)
 {
     const int nt = P == 4 ? BlkCfg<4, 64>::NTILES : P == 6 ? BlkCfg<6, 64>::NTILES : P == 8 ? BlkCfg<8, 32>::NTILES
                                                                                             : BlkCfg<10, 32>::NTILES;
-    const int64_t units = n / (4 * (int64_t)(leaf_size > 0 ? leaf_size : 1)) + 1;
-    const int64_t t = (units + kBlkRows - 1) / kBlkRows * nt;
-    if (t <= 0 || t >= kBlkFillCtas) return 1;
-    const int64_t k = (2 * kBlkFillCtas + t - 1) / t;
-    return k < 26 ? (int)k : 26;
+    const int64_t units = n / (2 * (int64_t)(leaf_size > 0 ? leaf_size : 1)) + 1;
+    return blk_ranges((units + kBlkRows - 1) / kBlkRows * nt);
 }
 
 void launch_ablk_prep(int P, Span cells, int64_t ucap, const int32_t *level, const int32_t *nchild,
