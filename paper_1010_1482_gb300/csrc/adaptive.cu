@@ -34,19 +34,37 @@ constexpr int64_t kColleagueFindCells = 1 << 17;  // below this many cells one l
 constexpr int64_t kListWarpCells = 1 << 17;  // below this many cells the U/W/X rows take a warp per cell
 
 // ---- keys ---------------------------------------------------------------------------------
-__global__ void k_keys64(const float4 *__restrict__ x, int64_t n, const Box *__restrict__ box,
-                         uint64_t *__restrict__ keys, uint32_t *__restrict__ idx)
+__global__ void __launch_bounds__(kKeyThreads) k_keys64(const float4 *__restrict__ x, int64_t n,
+                                                        const Box *__restrict__ box, uint64_t *__restrict__ keys,
+                                                        uint32_t *__restrict__ idx, int passes,
+                                                        uint32_t *__restrict__ ghist)
 {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
+    __shared__ uint32_t h[8][256];
+    for (int d = 0; d < passes; ++d) h[d][threadIdx.x] = 0;
+    __syncthreads();
     const Box b = *box;
-    float4 p = __ldg(&x[i]);
-    float c[3] = {p.x, p.y, p.z};
-    uint64_t k[3];
+    const int64_t step = (int64_t)gridDim.x * kKeyThreads;
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    int64_t base = blockIdx.x * (int64_t)kKeyThreads;
+    float4 next = base + threadIdx.x < n ? __ldg(&x[base + threadIdx.x]) : zero;
+    for (; base < n; base += step) {
+        const int64_t i = base + threadIdx.x;
+        const float4 p = next;  // the next particle's load in flight while this key is made and counted
+        next = i + step < n ? __ldg(&x[i + step]) : zero;
+        uint64_t key = 0;
+        if (i < n) {
+            const float c[3] = {p.x, p.y, p.z};
+            uint64_t k[3];
 #pragma unroll
-    for (int d = 0; d < 3; ++d) k[d] = grid_coord21(c[d], b, d);  // the FP64 steps' result
-    keys[i] = morton63(k[0], k[1], k[2]);
-    idx[i] = (uint32_t)i;
+            for (int d = 0; d < 3; ++d) k[d] = grid_coord21(c[d], b, d);  // the FP64 steps' result
+            key = morton63(k[0], k[1], k[2]);
+            keys[i] = key;
+            idx[i] = (uint32_t)i;
+        }
+        digit_hist_add(h, key, passes, i < n);
+    }
+    __syncthreads();
+    digit_hist_flush(h, passes, ghist);
 }
 
 // ---- tree construction --------------------------------------------------------------------
@@ -1036,8 +1054,10 @@ int evaluate_adaptive_in(gbfmm_ctx *ctx, AdaptiveState &A, const AdaptCaps *caps
     mark(0);
     const float4 *x = reinterpret_cast<const float4 *>(d_xyzq);
     Box *box = A.box.as<Box>();
+    launch_sort_clear(A.hist.p, n, 63, s);
     launch_bbox(x, n, prm->has_box, prm->box_origin, prm->box_side, box, partials, counter, ctx->d_status, s);
-    k_keys64<<<blocks_for(n), 256, 0, s>>>(x, n, box, A.keys0.as<uint64_t>(), A.idx0.as<uint32_t>());
+    k_keys64<<<key_ctas(n), kKeyThreads, 0, s>>>(x, n, box, A.keys0.as<uint64_t>(), A.idx0.as<uint32_t>(),
+                                                 sort_passes(n, 63), sort_hist(A.hist.p));
     note_launches(1);
     mark(1);
     uint64_t *skeys = nullptr;

@@ -440,9 +440,9 @@ int evaluate_uniform_in(gbfmm_ctx *ctx, const gbfmm_params *prm, int64_t n, cons
 
     const int64_t launches0 = tl_launches;
     mark(0);
+    launch_sort_clear(hist, n, 3 * L, s);
     launch_bbox(x, n, prm->has_box, prm->box_origin, prm->box_side, box, partials, counter, ctx->d_status, s);
-    launch_keys(x, n, box, L, k0, v0, s);
-    if (L >= 2) launch_geo_levels(box, L, geo, s);
+    launch_keys(x, n, box, L, k0, v0, hist, L >= 2 ? geo : nullptr, s);
     mark(1);
     uint32_t *skeys = nullptr, *perm = nullptr;
     launch_sort_gather(k0, k1, v0, v1, n, 3 * L, hist, ctx->d_status, x, sx, &skeys, &perm, s);

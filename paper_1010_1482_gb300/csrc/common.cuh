@@ -274,10 +274,10 @@ GB_DEV uint32_t grid_coord21(float c, const Box &b, int d)
     return grid_coord_fp64(c, b.origin[d], b.key_scale);
 }
 
-// Cell geometry table of the uniform tree (expansions.cu, k_geo_levels): 1/h_l for
+// Cell geometry table of the uniform tree (tree.cu, k_keys): 1/h_l for
 // l < kGeoLevels, then the 2^l cell-centre coordinates of every level l = 0..L along x, y, z.
 constexpr int kGeoLevels = 22;
-inline size_t geo_floats(int L) { return kGeoLevels + 3 * ((size_t(2) << L) - 1); }
+GB_HD size_t geo_floats(int L) { return kGeoLevels + 3 * ((size_t(2) << L) - 1); }
 
 // A cell's centre and the inverse of its side: FP64 expressions rounded once to FP32.
 struct CellGeom {
@@ -329,14 +329,57 @@ void note_launches(int k);
 // tree.cu
 void launch_bbox(const float4 *x, int64_t n, int has_box, const double *box_origin, double box_side, Box *box_out,
                  float *partials, unsigned *counter, int *status, cudaStream_t s);
-void launch_keys(const float4 *x, int64_t n, const Box *box, int L, uint32_t *leafkey, uint32_t *idx, cudaStream_t s);
 // Radix-sort scratch (tree.cu): per-pass tile counters, the histograms of every 8-bit digit
-// position, and one 64-bit look-back word per (pass, tile of 4096 keys, digit).
+// position, and one 64-bit look-back word per (pass, tile, digit).  The key kernels count the
+// histograms: launch_sort_clear before them, launch_sort_gather after.
 constexpr size_t kRsCounterBytes = 256, kRsHistBytes = 8 * 256 * 4;
+// keys per tile: 1024 and 2048 while 4096 would leave most SMs without a tile (a pass over 20,011
+// 63-bit keys 13.5 -> 8 us, with eight look-back words in flight; 400,009: 19.5 -> 13.5)
+constexpr int sort_tile(int64_t n) { return n <= (1 << 17) ? 1024 : n <= (1 << 19) ? 2048 : 4096; }
+constexpr int sort_passes(int64_t n, int bits) { return bits <= 0 || n <= 1 ? 0 : (bits + 7) / 8; }
+constexpr bool sort_reduce_then_scan(int64_t n, int passes) { return passes >= 2 && n >= (int64_t(1) << 22); }
 constexpr size_t sort_scratch_bytes(int64_t n, int bits)
 {
-    return kRsCounterBytes + kRsHistBytes + 8 * 256 * (size_t)((bits + 7) / 8) * (size_t)((n + 4095) / 4096);
+    return kRsCounterBytes + kRsHistBytes +
+           8 * 256 * (size_t)((bits + 7) / 8) * (size_t)((n + sort_tile(n) - 1) / sort_tile(n));
 }
+inline uint32_t *sort_hist(void *scratch)
+{
+    return reinterpret_cast<uint32_t *>(static_cast<unsigned char *>(scratch) + kRsCounterBytes);
+}
+void launch_sort_clear(void *scratch, int64_t n, int bits, cudaStream_t s);
+
+// The key kernels' CTAs: kKeyThreads keys at a time, at most four CTAs per SM (each adds its digit
+// histograms to the global ones once), eight on large inputs
+constexpr int kKeyThreads = 256;
+inline unsigned key_ctas(int64_t n)
+{
+    const int64_t c = (n + kKeyThreads - 1) / kKeyThreads, most = n >= (int64_t(1) << 22) ? 8 * 152 : 4 * 152;
+    return (unsigned)(c < most ? c : most);
+}
+// counts the digits of one key per thread (a whole warp calls it; valid: this thread has a key): one
+// shared-memory add a key and digit, or one for the warp when its keys agree in the digit
+template <class KeyT, int D>
+GB_DEV void digit_hist_add(uint32_t (&h)[D][256], KeyT key, int passes, bool valid)
+{
+    for (int d = 0; d < passes; ++d) {
+        const uint32_t v = valid ? (uint32_t)(key >> (8 * d)) & 0xffu : 256u, v0 = __shfl_sync(0xffffffffu, v, 0);
+        if (__all_sync(0xffffffffu, v == v0)) {
+            if ((threadIdx.x & 31) == 0 && v0 < 256u) atomicAdd(&h[d][v0], 32u);
+        } else if (v < 256u) {
+            atomicAdd(&h[d][v], 1u);
+        }
+    }
+}
+template <int D>
+GB_DEV void digit_hist_flush(const uint32_t (&h)[D][256], int passes, uint32_t *ghist)
+{
+    for (int e = threadIdx.x; e < 256 * passes; e += blockDim.x)
+        if (h[e >> 8][e & 255]) atomicAdd(&ghist[e], h[e >> 8][e & 255]);
+}
+// leaf keys and indices; the digit histograms into scratch; with geo given, the cell-centre table
+void launch_keys(const float4 *x, int64_t n, const Box *box, int L, uint32_t *leafkey, uint32_t *idx, void *scratch,
+                 float *geo, cudaStream_t s);
 // sorts (keys, idx) by key (stable) over `bits` low bits (keys < 2^bits); on return the sorted
 // pair is in (*keys_out, *idx_out) (one of the two buffers); also gathers sx[i] = x[idx[i]].
 // `scratch` holds sort_scratch_bytes(n, bits); a look-back wait that runs out raises
@@ -367,7 +410,6 @@ void launch_list_fill(int L, const int32_t *begin, const int32_t *end, const uin
 
 // expansions.cu
 void launch_build_operators(int P, float *m2l_ops, float *m2m_ops, float *l2l_ops, cudaStream_t s);
-void launch_geo_levels(const Box *box, int L, float *geo, cudaStream_t s);
 void launch_p2m(int P, int L, const float *geo, const float4 *sx, const int32_t *begin, const int32_t *end, float *M,
                 cudaStream_t s);
 void launch_m2m(int P, int l, const int32_t *begin, const int32_t *end, const float *ops, float *M, cudaStream_t s);

@@ -454,34 +454,6 @@ int build_m2l_rot_table(int P, std::vector<float> &out)
 //            along x, then y, then z, at offset kGeoLevels + 3 (2^l - 1)
 //   adaptive: geom[c] = (cx, cy, cz, 1/h) of cell c
 // ------------------------------------------------------------------------------------------
-__global__ void k_geo_levels(const Box *__restrict__ box, int L, float *__restrict__ geo)
-{
-    const Box b = *box;
-    const int64_t total = kGeoLevels + 3 * ((int64_t(2) << L) - 1);
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        if (t < kGeoLevels) {
-            const double h = b.side / (double)(int64_t(1) << t);
-            geo[t] = (float)(1.0 / h);
-            continue;
-        }
-        const int64_t u = t - kGeoLevels;
-        int l = 0;
-        while (3 * ((int64_t(2) << l) - 1) <= u) ++l;
-        const int64_t r = u - 3 * ((int64_t(1) << l) - 1);
-        const int d = (int)(r >> l);
-        const int i = (int)(r - ((int64_t)d << l));
-        const double h = b.side / (double)(int64_t(1) << l);
-        geo[t] = (float)(b.origin[d] + (i + 0.5) * h);
-    }
-}
-
-void launch_geo_levels(const Box *box, int L, float *geo, cudaStream_t s)
-{
-    const int64_t total = kGeoLevels + 3 * ((int64_t(2) << L) - 1);
-    k_geo_levels<<<(unsigned)std::min<int64_t>((total + 255) / 256, 1024), 256, 0, s>>>(box, L, geo);
-    note_launches(1);
-}
-
 GB_DEV CellGeom geo_level_cell(const float *__restrict__ geo, int l, uint32_t key)
 {
     int ix, iy, iz;

@@ -924,8 +924,8 @@ static int blk_tiles_p(int P, int L)
 // GB300), else the number of ranges k with the least time in waves of kBlkFillCtas CTAs, a CTA of
 // ceil(26 / k) offsets costing that many plus two for its start, first copies and last drain (and
 // the sum of the ranges, half an offset).  12 tiles (100,000 particles, p = 8): 26 ranges took three
-// launches, the last of 8 CTAs, 75 us and 10 for the sum; 12 ranges one, and the step 244 -> 193 us.  A fixed rule, so that the workspace
-// size does not depend on the device.
+// launches, the last of 8 CTAs, 75 us and 10 for the sum; 12 ranges one, and the step 244 -> 193 us.
+// A fixed rule, so that the workspace size does not depend on the device.
 constexpr int kBlkFillCtas = 152;
 static int blk_ranges(int64_t tiles)
 {

@@ -114,9 +114,10 @@ extern "C" int gbfmm_sort_static(const gbfmm_params *prm, int64_t n, const float
     uint32_t *k0 = (passes % 2 == 0) ? k_caller : k_tmp, *v0 = (passes % 2 == 0) ? v_caller : v_tmp;
     uint32_t *k1 = (passes % 2 == 0) ? k_tmp : k_caller, *v1 = (passes % 2 == 0) ? v_tmp : v_caller;
     const float4 *x = reinterpret_cast<const float4 *>(d_xyzq);
+    launch_sort_clear(base + kSsHist, n, 3 * L, s);
     launch_bbox(x, n, prm->has_box, prm->box_origin, prm->box_side, box,
                 reinterpret_cast<float *>(base + kSsPartials), counter, status, s);
-    launch_keys(x, n, box, L, k0, v0, s);
+    launch_keys(x, n, box, L, k0, v0, base + kSsHist, nullptr, s);
     uint32_t *kout = nullptr, *vout = nullptr;
     launch_sort_gather(k0, k1, v0, v1, n, 3 * L, base + kSsHist, status, x, reinterpret_cast<float4 *>(d_sorted_xyzq),
                        &kout, &vout, s);

@@ -182,31 +182,72 @@ GB_DEV uint32_t leaf_coord_f(float v, int sh)
 }
 
 
-__global__ void k_keys(const float4 *__restrict__ x, int64_t n, const Box *__restrict__ box, int L,
-                       uint32_t *__restrict__ leafkey, uint32_t *__restrict__ idx)
+// The CTAs past key_ctas write the cell-centre table instead (geo, kGeoLevels; it needs the box and
+// nothing else).  The digit histograms of the sort are counted on the way (digit_hist_add).
+__global__ void __launch_bounds__(kKeyThreads) k_keys(const float4 *__restrict__ x, int64_t n, const Box *__restrict__ box,
+                                                      int L, uint32_t *__restrict__ leafkey, uint32_t *__restrict__ idx,
+                                                      int passes, uint32_t *__restrict__ ghist, unsigned key_ctas,
+                                                      float *__restrict__ geo)
 {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const Box b = *box;
-    float4 p = __ldg(&x[i]);
-    float c[3] = {p.x, p.y, p.z};
-    const int sh = 21 - L;
-    uint32_t k[3];
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        const float vf = __fmul_rn(__fsub_rn(c[d], b.origin_f[d]), b.key_scale_f);
-        const float e = __fadd_ru(__fmul_ru(fabsf(vf), 0x1p-21f), b.key_slack);
-        const uint32_t lo = leaf_coord_f(__fsub_rd(vf, e), sh), hi = leaf_coord_f(__fadd_ru(vf, e), sh);
-        k[d] = lo == hi ? lo : grid_coord_fp64(c[d], b.origin[d], b.key_scale) >> sh;
+    __shared__ uint32_t h[4][256];
+    if (blockIdx.x >= key_ctas) {
+        const double side = box->side;
+        const int64_t total = (int64_t)geo_floats(L);
+        for (int64_t t = (blockIdx.x - key_ctas) * (int64_t)kKeyThreads + threadIdx.x; t < total;
+             t += (int64_t)(gridDim.x - key_ctas) * kKeyThreads) {
+            if (t < kGeoLevels) {
+                geo[t] = (float)__ddiv_rn(1.0, __ddiv_rn(side, (double)(int64_t(1) << t)));
+                continue;
+            }
+            const int64_t u = t - kGeoLevels;
+            int l = 0;
+            while (3 * ((int64_t(2) << l) - 1) <= u) ++l;
+            const int64_t r = u - 3 * ((int64_t(1) << l) - 1);
+            const int d = (int)(r >> l), i = (int)(r - ((int64_t)d << l));
+            geo[t] = (float)__fma_rn(i + 0.5, __ddiv_rn(side, (double)(int64_t(1) << l)), box->origin[d]);
+        }
+        return;
     }
-    leafkey[i] = morton3(k[0], k[1], k[2]);
-    idx[i] = (uint32_t)i;
+    for (int d = 0; d < passes; ++d) h[d][threadIdx.x] = 0;
+    __syncthreads();
+    const Box b = *box;
+    const int sh = 21 - L;
+    const int64_t step = (int64_t)key_ctas * kKeyThreads;
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    int64_t base = blockIdx.x * (int64_t)kKeyThreads;
+    float4 next = base + threadIdx.x < n ? __ldg(&x[base + threadIdx.x]) : zero;
+    for (; base < n; base += step) {
+        const int64_t i = base + threadIdx.x;
+        const float4 p = next;  // the next particle's load in flight while this key is made and counted
+        next = i + step < n ? __ldg(&x[i + step]) : zero;
+        uint32_t key = 0;
+        if (i < n) {
+            const float c[3] = {p.x, p.y, p.z};
+            uint32_t k[3];
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                const float vf = __fmul_rn(__fsub_rn(c[d], b.origin_f[d]), b.key_scale_f);
+                const float e = __fadd_ru(__fmul_ru(fabsf(vf), 0x1p-21f), b.key_slack);
+                const uint32_t lo = leaf_coord_f(__fsub_rd(vf, e), sh), hi = leaf_coord_f(__fadd_ru(vf, e), sh);
+                k[d] = lo == hi ? lo : grid_coord_fp64(c[d], b.origin[d], b.key_scale) >> sh;
+            }
+            key = morton3(k[0], k[1], k[2]);
+            leafkey[i] = key;
+            idx[i] = (uint32_t)i;
+        }
+        digit_hist_add(h, key, passes, i < n);
+    }
+    __syncthreads();
+    digit_hist_flush(h, passes, ghist);
 }
 
-void launch_keys(const float4 *x, int64_t n, const Box *box, int L, uint32_t *leafkey, uint32_t *idx, cudaStream_t s)
+void launch_keys(const float4 *x, int64_t n, const Box *box, int L, uint32_t *leafkey, uint32_t *idx, void *scratch,
+                 float *geo, cudaStream_t s)
 {
     if (n <= 0) return;
-    k_keys<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(x, n, box, L, leafkey, idx);
+    const unsigned kc = key_ctas(n);
+    const unsigned gc = geo ? (unsigned)std::min<size_t>((geo_floats(L) + kKeyThreads - 1) / kKeyThreads, 16) : 0u;
+    k_keys<<<kc + gc, kKeyThreads, 0, s>>>(x, n, box, L, leafkey, idx, sort_passes(n, 3 * L), sort_hist(scratch), kc, geo);
     note_launches(1);
 }
 
@@ -382,9 +423,9 @@ void launch_exclusive_scan(const uint32_t *in, uint32_t *out, int64_t n, uint32_
 }
 
 // ------------------------------------------------------------------------------------------
-// Stable LSD radix sort of (key, index) pairs, 8-bit digits: one kernel counts every digit
+// Stable LSD radix sort of (key, index) pairs, 8-bit digits: the key kernels count every digit
 // position's histogram, then one kernel per digit position ranks and scatters the keys.
-// Tiles of 4096 keys are taken in launch order (a counter), each ranks its keys stably in
+// Tiles of 1024 to 4096 keys (sort_tile) are taken in launch order (a counter), each ranks its keys stably in
 // shared memory (per-warp counts over a blocked layout, warp match within a round), publishes
 // its per-digit count and looks back over the earlier tiles' counts (decoupled look-back: an
 // earlier tile publishes its count at once and its inclusive prefix when it has one) to find
@@ -393,24 +434,24 @@ void launch_exclusive_scan(const uint32_t *in, uint32_t *out, int64_t n, uint32_
 // Scratch: per-pass tile counters, the digit histograms, and one 64-bit status word per
 // (pass, tile, digit): flag (bits 62-63: 1 = count, 2 = inclusive prefix) | value.
 // ------------------------------------------------------------------------------------------
-constexpr int kRsThreads = 512, kRsItems = 8, kRsTile = kRsThreads * kRsItems;  // tile of 4096 keys
-constexpr int kRsWarps = kRsThreads / 32, kRsWarpKeys = kRsTile / kRsWarps;
-constexpr int kRsHistThreads = 256;  // one per digit
+constexpr int kRsThreads = 512, kRsWarps = kRsThreads / 32;
+constexpr int kRsTile = 4096;  // the reduce-then-scan form's tile, and the largest of the look-back form
 constexpr int64_t kRsScanMinN = int64_t(1) << 22;  // from here on the passes take the reduce-then-scan form
 constexpr uint64_t kRsAgg = 1ull << 62, kRsInc = 2ull << 62, kRsFlags = 3ull << 62;
 
-static_assert(kRsWarpKeys == 32 * kRsItems, "blocked layout: a warp owns kRsItems rounds of 32 keys");
 static_assert(kRsTile <= 65535, "16-bit per-warp digit counts and offsets");
 
-GB_DEV void st_release_u64(uint64_t *p, uint64_t v)
+// A look-back word carries its count beside its flag, so relaxed accesses suffice, and several
+// loads can be in flight at once.
+GB_DEV void st_relaxed_u64(uint64_t *p, uint64_t v)
 {
-    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
-GB_DEV uint64_t ld_acquire_u64(const uint64_t *p)
+GB_DEV uint64_t ld_relaxed_u64(const uint64_t *p)
 {
     uint64_t v;
-    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
     return v;
 }
 
@@ -439,27 +480,10 @@ GB_DEV uint32_t block_excl_scan(uint32_t v, uint32_t *wsum)
     return off + x - v;
 }
 
-template <class KeyT>
-__global__ void __launch_bounds__(kRsHistThreads) k_rs_ghist(const KeyT *__restrict__ keys, int64_t n, int passes,
-                                                             uint32_t *__restrict__ ghist)
-{
-    __shared__ uint32_t h[sizeof(KeyT)][256];
-    for (int d = 0; d < passes; ++d) h[d][threadIdx.x] = 0;
-    __syncthreads();
-    for (int64_t i = blockIdx.x * (int64_t)kRsHistThreads + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * kRsHistThreads) {
-        const KeyT k = keys[i];
-        for (int d = 0; d < passes; ++d) atomicAdd(&h[d][(uint32_t)(k >> (8 * d)) & 0xffu], 1u);
-    }
-    __syncthreads();
-    for (int d = 0; d < passes; ++d)
-        if (h[d][threadIdx.x]) atomicAdd(&ghist[d * 256 + threadIdx.x], h[d][threadIdx.x]);
-}
-
 // LB: the tile's digit starts by decoupled look-back over the earlier tiles (tiles taken in
 // launch order from a counter); else read from `starts` (tile_starts of the reduce-then-scan
 // form: starts[d * nblk + tile]), tile = blockIdx.x
-template <class KeyT, bool LB>
+template <class KeyT, bool LB, int ITEMS>
 __global__ void __launch_bounds__(kRsThreads, 3) k_rs_pass(const KeyT *__restrict__ kin, const uint32_t *__restrict__ vin,
                                                         KeyT *__restrict__ kout, uint32_t *__restrict__ vout,
                                                         int64_t n, int pass, int64_t nblk,
@@ -468,10 +492,11 @@ __global__ void __launch_bounds__(kRsThreads, 3) k_rs_pass(const KeyT *__restric
                                                         float4 *__restrict__ gsx, int *err,
                                                         const uint32_t *__restrict__ starts)
 {
+    constexpr int kTile = kRsThreads * ITEMS, kWarpKeys = 32 * ITEMS;  // blocked: a warp owns ITEMS rounds of 32 keys
     extern __shared__ __align__(16) unsigned char rs_smem[];
     KeyT *skey = reinterpret_cast<KeyT *>(rs_smem);
-    uint32_t *sval = reinterpret_cast<uint32_t *>(skey + kRsTile);
-    __shared__ uint16_t wcnt[kRsWarps][256];  // per-warp digit counts, then offsets (< kRsTile)
+    uint32_t *sval = reinterpret_cast<uint32_t *>(skey + kTile);
+    __shared__ __align__(4) uint16_t wcnt[kRsWarps][256];  // per-warp digit counts, then offsets (< kRsTile)
     __shared__ uint32_t dstart[256], gbase[256], wsum[kRsWarps];
     __shared__ uint32_t tile_sh;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -479,20 +504,20 @@ __global__ void __launch_bounds__(kRsThreads, 3) k_rs_pass(const KeyT *__restric
     const int shift = 8 * pass;
     const bool dig = tid < 256;  // the per-digit work: thread tid, digit tid
     if (tid == 0) tile_sh = LB ? atomicAdd(&counter[pass], 1u) : blockIdx.x;
-    for (int e = tid; e < kRsWarps * 256; e += kRsThreads) (&wcnt[0][0])[e] = 0;
+    for (int e = tid; e < kRsWarps * 128; e += kRsThreads) reinterpret_cast<uint32_t *>(&wcnt[0][0])[e] = 0;
     __syncthreads();
     const int64_t tile = tile_sh;
-    const int64_t base = tile * kRsTile + (int64_t)warp * kRsWarpKeys;
+    const int64_t base = tile * kTile + (int64_t)warp * kWarpKeys;
     // only the ranks stay in registers across the scans: the keys and indices are read again
     // (from L1 / L2) when they are staged, which leaves room for three CTAs per SM
-    uint32_t rk[kRsItems];
+    uint32_t rk[ITEMS];
 #pragma unroll
-    for (int r = 0; r < kRsItems; ++r) {  // the digits first: all the warp's loads in flight at once
+    for (int r = 0; r < ITEMS; ++r) {  // the digits first: all the warp's loads in flight at once
         const int64_t i = base + 32 * r + lane;
         rk[r] = i < n ? ((uint32_t)(kin[i] >> shift) & 0xffu) : 256u;
     }
 #pragma unroll
-    for (int r = 0; r < kRsItems; ++r) {
+    for (int r = 0; r < ITEMS; ++r) {
         const uint32_t d = rk[r];
         const bool valid = d < 256u;
         // the lanes holding the same digit (invalid lanes: digit 256, a class of their own),
@@ -531,25 +556,34 @@ __global__ void __launch_bounds__(kRsThreads, 3) k_rs_pass(const KeyT *__restric
     uint32_t excl = 0;
     if (!dig) {
     } else if (tile == 0) {
-        st_release_u64(&st[tid], kRsInc | cnt);
+        st_relaxed_u64(&st[tid], kRsInc | cnt);
     } else {
-        st_release_u64(&st[tile * 256 + tid], kRsAgg | cnt);
+        st_relaxed_u64(&st[tile * 256 + tid], kRsAgg | cnt);
         const uint64_t t0 = timer_ns();
-        for (int64_t t = tile - 1; t >= 0;) {
-            const uint64_t w = ld_acquire_u64(&st[t * 256 + tid]);
-            if ((w & kRsFlags) == 0) {
+        constexpr int kAhead = 8;  // predecessors read at once: a chain of loads per eight tiles
+        bool done = false;
+        for (int64_t t = tile - 1; !done && t >= 0;) {
+            uint64_t w[kAhead];
+#pragma unroll
+            for (int k = 0; k < kAhead; ++k) w[k] = t - k >= 0 ? ld_relaxed_u64(&st[(t - k) * 256 + tid]) : kRsInc;
+            int seen = 0;
+#pragma unroll
+            for (int k = 0; k < kAhead; ++k) {
+                if (done || seen < k || (w[k] & kRsFlags) == 0) continue;
+                ++seen;
+                excl += (uint32_t)w[k];
+                done = (w[k] & kRsFlags) == kRsInc;
+            }
+            t -= seen;
+            if (!done && seen < kAhead) {
                 if (timer_ns() - t0 > 1000000000ull) {  // 1 s: report and give up
                     atomicOr(err, kStatusTimeout);
                     break;
                 }
                 __nanosleep(32);
-                continue;
             }
-            excl += (uint32_t)w;
-            if ((w & kRsFlags) == kRsInc) break;
-            --t;
         }
-        st_release_u64(&st[tile * 256 + tid], kRsInc | (excl + cnt));
+        st_relaxed_u64(&st[tile * 256 + tid], kRsInc | (excl + cnt));
     }
     const uint32_t gb = block_excl_scan(dig ? ghist[pass * 256 + tid] : 0u, wsum);
     if (dig) gbase[tid] = gb + excl;
@@ -557,7 +591,7 @@ __global__ void __launch_bounds__(kRsThreads, 3) k_rs_pass(const KeyT *__restric
     __syncthreads();
     // stage in tile-sorted order, then write the runs of each digit
 #pragma unroll
-    for (int r = 0; r < kRsItems; ++r) {
+    for (int r = 0; r < ITEMS; ++r) {
         const int64_t i = base + 32 * r + lane;
         if (i < n) {
             const KeyT key = kin[i];
@@ -568,8 +602,8 @@ __global__ void __launch_bounds__(kRsThreads, 3) k_rs_pass(const KeyT *__restric
         }
     }
     __syncthreads();
-    const int64_t t0 = tile * kRsTile;
-    const int tn = (int)(n - t0 < kRsTile ? n - t0 : kRsTile);
+    const int64_t t0 = tile * kTile;
+    const int tn = (int)(n - t0 < kTile ? n - t0 : kTile);
     for (int jj = tid; jj < tn; jj += kRsThreads) {
         const KeyT key = skey[jj];
         const uint32_t val = sval[jj];
@@ -675,7 +709,8 @@ static void sort_gather_t(KeyT *k0, KeyT *k1, uint32_t *v0, uint32_t *v1, int64_
 {
     KeyT *kin = k0, *kout = k1;
     uint32_t *vin = v0, *vout = v1;
-    if (bits <= 0 || n <= 1) {
+    const int passes = sort_passes(n, bits);
+    if (passes == 0) {
         if (n > 0) {
             k_gather_identity<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(x, sx, n);
             note_launches(1);
@@ -684,33 +719,31 @@ static void sort_gather_t(KeyT *k0, KeyT *k1, uint32_t *v0, uint32_t *v1, int64_
         *idx_out = v0;
         return;
     }
-    const int passes = (bits + 7) / 8;
-    const int64_t nblk = (n + kRsTile - 1) / kRsTile;
+    const int tile = sort_tile(n);
+    const int64_t nblk = (n + tile - 1) / tile;
     unsigned char *sc = static_cast<unsigned char *>(scratch);
     uint32_t *counter = reinterpret_cast<uint32_t *>(sc);
-    uint32_t *ghist = reinterpret_cast<uint32_t *>(sc + kRsCounterBytes);
+    uint32_t *ghist = sort_hist(scratch);
     uint64_t *status = reinterpret_cast<uint64_t *>(sc + kRsCounterBytes + kRsHistBytes);
     // large inputs of several passes take the reduce-then-scan form; its tile counts and starts
     // (4 bytes each per tile and digit) use the look-back words' space of the first two passes
-    const bool rts = passes >= 2 && n >= kRsScanMinN;
+    const bool rts = sort_reduce_then_scan(n, passes);
     uint32_t *counts = reinterpret_cast<uint32_t *>(status);
     uint32_t *starts = counts + 256 * nblk;
-    cudaMemsetAsync(scratch, 0, rts ? kRsCounterBytes + kRsHistBytes : sort_scratch_bytes(n, bits), s);
-    const unsigned hgrid = (unsigned)std::min<int64_t>(nblk * (kRsTile / kRsHistThreads) / 4 + 1, 1216);
-    k_rs_ghist<KeyT><<<hgrid, kRsHistThreads, 0, s>>>(kin, n, passes, ghist);
-    const int smem = kRsTile * (int)(sizeof(KeyT) + sizeof(uint32_t));
-    cudaFuncSetAttribute(k_rs_pass<KeyT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    cudaFuncSetAttribute(k_rs_pass<KeyT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    const int smem = tile * (int)(sizeof(KeyT) + sizeof(uint32_t));
+    auto lookback = tile == 1024 ? k_rs_pass<KeyT, true, 2> : tile == 2048 ? k_rs_pass<KeyT, true, 4> : k_rs_pass<KeyT, true, 8>;
+    cudaFuncSetAttribute(lookback, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaFuncSetAttribute(k_rs_pass<KeyT, false, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     for (int pass = 0; pass < passes; ++pass) {
         const bool last = pass + 1 == passes;
         if (rts) {
             k_rs_upsweep<KeyT><<<(unsigned)nblk, 256, 0, s>>>(kin, n, pass, nblk, counts);
             k_rs_tile_starts<<<256, 1024, 0, s>>>(counts, starts, nblk, ghist, pass);
-            k_rs_pass<KeyT, false><<<(unsigned)nblk, kRsThreads, smem, s>>>(
+            k_rs_pass<KeyT, false, 8><<<(unsigned)nblk, kRsThreads, smem, s>>>(
                 kin, vin, kout, vout, n, pass, nblk, ghist, status, counter, x, last ? sx : nullptr, err, starts);
             note_launches(2);
         } else {
-            k_rs_pass<KeyT, true><<<(unsigned)nblk, kRsThreads, smem, s>>>(
+            lookback<<<(unsigned)nblk, kRsThreads, smem, s>>>(
                 kin, vin, kout, vout, n, pass, nblk, ghist, status, counter, x, last ? sx : nullptr, err, nullptr);
         }
         KeyT *t = kin;
@@ -720,9 +753,16 @@ static void sort_gather_t(KeyT *k0, KeyT *k1, uint32_t *v0, uint32_t *v1, int64_
         vin = vout;
         vout = u;
     }
-    note_launches(1 + passes);
+    note_launches(passes);
     *keys_out = kin;
     *idx_out = vin;
+}
+
+void launch_sort_clear(void *scratch, int64_t n, int bits, cudaStream_t s)
+{
+    const int passes = sort_passes(n, bits);
+    if (passes == 0) return;
+    cudaMemsetAsync(scratch, 0, sort_reduce_then_scan(n, passes) ? kRsCounterBytes + kRsHistBytes : sort_scratch_bytes(n, bits), s);
 }
 
 void launch_sort_gather(uint32_t *k0, uint32_t *k1, uint32_t *v0, uint32_t *v1, int64_t n, int bits, void *scratch,
@@ -741,7 +781,8 @@ void launch_sort_gather64(uint64_t *k0, uint64_t *k1, uint32_t *v0, uint32_t *v1
 
 // ------------------------------------------------------------------------------------------
 // Cells: for every level, the first and one-past-last sorted position of each nonempty cell
-// (arrays zeroed beforehand, so empty cells read begin == end == 0).
+// (arrays zeroed beforehand, so empty cells read begin == end == 0; `end` follows `begin` in the
+// same buffer, with less than 256 bytes between).
 // ------------------------------------------------------------------------------------------
 __global__ void k_cells(const uint32_t *__restrict__ sk, int64_t n, int L, int32_t *__restrict__ begin,
                         int32_t *__restrict__ end)
@@ -761,9 +802,8 @@ __global__ void k_cells(const uint32_t *__restrict__ sk, int64_t n, int L, int32
 
 void launch_cells(const uint32_t *sk, int64_t n, int L, int32_t *begin, int32_t *end, cudaStream_t s)
 {
-    size_t C = (size_t)level_offset(L + 1);
-    cudaMemsetAsync(begin, 0, C * sizeof(int32_t), s);
-    cudaMemsetAsync(end, 0, C * sizeof(int32_t), s);
+    const size_t C = (size_t)level_offset(L + 1);
+    cudaMemsetAsync(begin, 0, (size_t)(end + C - begin) * sizeof(int32_t), s);
     if (n > 0) {
         k_cells<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(sk, n, L, begin, end);
         note_launches(1);
