@@ -51,17 +51,16 @@ __global__ void __launch_bounds__(kKeyThreads) k_keys64(const float4 *__restrict
         const int64_t i = base + threadIdx.x;
         const float4 p = next;  // the next particle's load in flight while this key is made and counted
         next = i + step < n ? __ldg(&x[i + step]) : zero;
-        uint64_t key = 0;
         if (i < n) {
             const float c[3] = {p.x, p.y, p.z};
             uint64_t k[3];
 #pragma unroll
             for (int d = 0; d < 3; ++d) k[d] = grid_coord21(c[d], b, d);  // the FP64 steps' result
-            key = morton63(k[0], k[1], k[2]);
+            const uint64_t key = morton63(k[0], k[1], k[2]);
             keys[i] = key;
             idx[i] = (uint32_t)i;
+            digit_hist_add(h, key, passes);
         }
-        digit_hist_add(h, key, passes, i < n);
     }
     __syncthreads();
     digit_hist_flush(h, passes, ghist);

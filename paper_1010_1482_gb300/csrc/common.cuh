@@ -357,19 +357,11 @@ inline unsigned key_ctas(int64_t n)
     const int64_t c = (n + kKeyThreads - 1) / kKeyThreads, most = n >= (int64_t(1) << 22) ? 8 * 152 : 4 * 152;
     return (unsigned)(c < most ? c : most);
 }
-// counts the digits of one key per thread (a whole warp calls it; valid: this thread has a key): one
-// shared-memory add a key and digit, or one for the warp when its keys agree in the digit
+// counts the digits of one key, a shared-memory increment each
 template <class KeyT, int D>
-GB_DEV void digit_hist_add(uint32_t (&h)[D][256], KeyT key, int passes, bool valid)
+GB_DEV void digit_hist_add(uint32_t (&h)[D][256], KeyT key, int passes)
 {
-    for (int d = 0; d < passes; ++d) {
-        const uint32_t v = valid ? (uint32_t)(key >> (8 * d)) & 0xffu : 256u, v0 = __shfl_sync(0xffffffffu, v, 0);
-        if (__all_sync(0xffffffffu, v == v0)) {
-            if ((threadIdx.x & 31) == 0 && v0 < 256u) atomicAdd(&h[d][v0], 32u);
-        } else if (v < 256u) {
-            atomicAdd(&h[d][v], 1u);
-        }
-    }
+    for (int d = 0; d < passes; ++d) atomicAdd(&h[d][(uint32_t)(key >> (8 * d)) & 0xffu], 1u);
 }
 template <int D>
 GB_DEV void digit_hist_flush(const uint32_t (&h)[D][256], int passes, uint32_t *ghist)

@@ -220,7 +220,6 @@ __global__ void __launch_bounds__(kKeyThreads) k_keys(const float4 *__restrict__
         const int64_t i = base + threadIdx.x;
         const float4 p = next;  // the next particle's load in flight while this key is made and counted
         next = i + step < n ? __ldg(&x[i + step]) : zero;
-        uint32_t key = 0;
         if (i < n) {
             const float c[3] = {p.x, p.y, p.z};
             uint32_t k[3];
@@ -231,11 +230,11 @@ __global__ void __launch_bounds__(kKeyThreads) k_keys(const float4 *__restrict__
                 const uint32_t lo = leaf_coord_f(__fsub_rd(vf, e), sh), hi = leaf_coord_f(__fadd_ru(vf, e), sh);
                 k[d] = lo == hi ? lo : grid_coord_fp64(c[d], b.origin[d], b.key_scale) >> sh;
             }
-            key = morton3(k[0], k[1], k[2]);
+            const uint32_t key = morton3(k[0], k[1], k[2]);
             leafkey[i] = key;
             idx[i] = (uint32_t)i;
+            digit_hist_add(h, key, passes);
         }
-        digit_hist_add(h, key, passes, i < n);
     }
     __syncthreads();
     digit_hist_flush(h, passes, ghist);
