@@ -55,6 +55,7 @@ AdaptCaps with_margin(const AdaptCaps &c)
     AdaptCaps r = c;
     r.cells = 2 * c.cells + 64;
     r.leaves = 2 * c.leaves + 64;
+    r.units = 2 * (c.cells - c.leaves) + 64;
     r.maxl = std::min(gbfmm::kAdaptiveMaxLevel, c.maxl + 3);
     for (int l = 0; l <= gbfmm::kAdaptiveMaxLevel; ++l) r.level[l] = l <= r.maxl ? r.cells : 0;
     for (int k = 0; k < 4; ++k) r.list[k] = k == 1 ? 189 * r.cells : per_cell(c.list[k], r.cells);

@@ -40,6 +40,7 @@ struct DevBuf {
 // W, X entries; chain: the treecode's two chain-list totals; maxl: deepest level.
 struct AdaptCaps {
     int64_t cells = 0, leaves = 0;
+    int64_t units = 0;  // capacities only: cells with children
     int64_t level[kAdaptiveMaxLevel + 1] = {};
     int64_t list[4] = {}, chain[2] = {};
     int32_t maxl = 0;
@@ -58,7 +59,7 @@ struct AdaptiveState {
     DevBuf near;                                                   // P2P's compensated sums, 2 float4 per particle
     DevBuf tc_cnt, tc_offs[2], tc_ids[2];  // treecode rows: [0] U + ancestors' X, [1] W + ancestors' V
     // block-form M2L: unit flags and their scan, unit of every cell, the units, their count, the
-    // pre-split rows and scales, the colleague rows per (tile, offset), the offset ranges' partial sums
+    // pre-split rows and scales, the colleague rows per (tile, offset), the classes per (range, unit)
     DevBuf ab_flag, ab_scan, ab_unit_of, ab_units, ab_nu, ab_pre, ab_scale, ab_src, lpart;
     DevBuf partials;  // root-box reduction scratch of evaluations that do not use the context's
     AdaptCaps counts;  // the sizes the last host-counted evaluation read back

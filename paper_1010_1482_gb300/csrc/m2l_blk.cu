@@ -13,6 +13,22 @@
 // for S outside the level).  K = N = 8 p^2 (800 at p = 10): no padding, and the zero blocks of
 // B_D (near pairs) are 9% of its entries.  No interaction lists are read.
 //
+// Parity classes.  Mirroring an axis maps child sigma to its mirror image and multiplies every
+// real-packed coefficient by a sign s(n, m, re/im) (T_{R o} = S_R T_o S_R), so with the children's
+// coefficients combined into sums and differences over each axis,
+//     U_c[k] = sum_sigma (-1)^{c . sigma} s(k)^sigma M~_sigma[k],   c in {0, 1}^3,
+// class c has a definite parity in every axis, and B'_D = H B_D H^T / 8 couples class c' of the
+// targets with class c of the sources only where they agree in every axis along which D is 0.  H is
+// orthogonal up to the factor 8, so nothing is lost: L~ = H^T V / 8.  A CTA's N-tile is one unit of
+// classes (all of them agree in the axes that distinguish units), and per D it walks only the
+// units of K that its own couples with: at p = 10 (units of two classes) 148 of 208 class products
+// over the 26 offsets, at p = 6 and 8 (four classes) 176.  The pre-split kernels form U, the drains
+// write V, and a last kernel (k_blk_finish, k_ablk_finish) adds the offset ranges and applies H^T.
+// Against the untransformed blocks: M2L kernel of 1M uniform, p = 10 321 -> 266 us (the step 1022 ->
+// 969), of 400,009 Plummer, p = 10 549 -> 398; 16M Plummer, p = 8 step 23.21 -> 22.56 ms, a batch of
+// 96 instances 7.05 -> 6.62 ms.  Bound by shared memory: a K step of 16 at p = 10 reads 31 KB of
+// operands and takes 21 KB of copies in 312 cycles of MMA, 167 bytes a cycle of 128.
+//
 // Tiles: one CTA takes 128 target parents (a box of 8 x 4 x 4 in the parent grid; smaller on
 // levels 2 and 3) as the MMA's M and one N-tile of the 8 p^2 outputs, and walks the 26 offsets
 // D in chunks of 32 or 64 K values.  Operands stream through shared memory by TMA tiled loads
@@ -21,7 +37,7 @@
 // gathered kernel: x = hi + lo in FP16, D += A_lo B_hi + A_hi B_lo + A_hi B_hi with FP32
 // accumulation in TMEM.  Scales: every source parent's coefficients by 2^s_S (max -> 2^10), the
 // operators by one power of two 2^g (max over all offsets -> 2^12).  Each D's partial is drained
-// from TMEM (in DS pieces along K, bounding the truncating accumulation chain) to FP32 registers
+// from TMEM (DPU pieces a unit, bounding the truncating accumulation chain) to FP32 registers
 // and multiplied by 2^-(s_(Q+D) + g) per row before the sum; two TMEM accumulators alternate so
 // the MMAs of the next piece overlap the drain.
 #include "common.cuh"
@@ -40,9 +56,6 @@ namespace {
 
 constexpr int kBlkRows = 128;  // target parents per CTA (MMA M)
 constexpr int kBlkDrainWarps = 8;
-// drains per offset: each offset's K range (8 p^2) is accumulated in TMEM in two pieces, so no
-// truncating accumulation chain is longer than about half an offset (75 MMAs at p = 10)
-constexpr int kBlkDrainsPerOffset = 2;
 constexpr int kBlkThreads = 32 * (kBlkDrainWarps + 2);  // drain warps, TMA producer, MMA issuer
 
 // the 26 parent offsets D in {-1, 0, 1}^3 \ {0}: index d -> D
@@ -63,9 +76,18 @@ struct BlkCfg {
     static constexpr int PP = P * P, KD = 8 * PP;
     // N-tile: rows of B_D per CTA (the MMA's N, a multiple of 16) and the stride between tiles
     static constexpr int NT = P == 4 ? 128 : P == 6 ? 144 : P == 8 ? 256 : 208;
-    static constexpr int NSTRIDE = P == 10 ? 200 : NT;
-    static constexpr int NTILES = (KD + NSTRIDE - 1) / NSTRIDE;
-    static constexpr int NKC = (KD + CH - 1) / CH;
+    // units of classes: CU classes, UNIT K values (padded to the MMA's 16); K rows hold the units in
+    // order (class c, coefficient k at (c / CU) UNIT + (c % CU) PP + k), an N-tile is one unit
+    static constexpr int CU = P == 10 ? 2 : P == 4 ? 8 : 4, NUNIT = 8 / CU;
+    static constexpr int UNIT = (CU * PP + 15) / 16 * 16, KW = NUNIT * UNIT;
+    static constexpr int NSTRIDE = CU * PP, NTILES = NUNIT;
+    static constexpr int UC = (UNIT + CH - 1) / CH;  // chunks of a unit
+    // drains per unit: the MMA's accumulation truncates, and a class sums eight children.  Chains of
+    // 6, 18, 24 and 39 MMAs at p = 4, 6, 8, 10 leave the outputs as close to the FP64 FMM as, or
+    // closer than, the untransformed blocks with chains of 12, 27, 48 and 75 did (phi, 30,000 uniform
+    // particles: 1.7, 3.5, 3.5, 3.7e-7 against 1.9, 3.7, 4.3, 5.3e-7); twice as long at p = 4: 2.4e-7
+    static constexpr int DPU = P == 10 ? 1 : P == 4 ? 4 : 2;
+    static constexpr int MAX_STEPS = 26 * NUNIT * UC, MAX_DRAINS = 26 * NUNIT * DPU;
     static constexpr int A_BYTES = kBlkRows * CH * 2;  // one of hi / lo
     static constexpr int B_BYTES = NT * CH * 2;
     static constexpr int STAGE_BYTES = 2 * A_BYTES + 2 * B_BYTES;
@@ -76,12 +98,105 @@ struct BlkCfg {
     static constexpr int TMEM_COLS = 2 * NT <= 256 ? 256 : 512;
     static_assert(NT % 16 == 0 && NT <= 256, "MMA N");
     static_assert(NH % 8 == 0 && NSTRIDE % 4 == 0 && PP % 4 == 0, "drain / store granularity");
-    static_assert(NSTRIDE <= NT && NTILES * NSTRIDE >= KD, "N tiling");
+    static_assert(NSTRIDE <= NT && NTILES * NSTRIDE == KD, "N tiling");
+    static_assert(UNIT % 16 == 0 && KW % 8 == 0 && UC >= DPU && MAX_DRAINS < 1024, "steps");
     static_assert(A_BYTES % 1024 == 0 && B_BYTES % 1024 == 0, "swizzle atoms");
     static_assert(CH == 64 || CH == 32, "swizzled row of 128 or 64 bytes");
     static_assert(NSTAGE >= 2, "pipeline stages");
     static_assert(kSmemBytes <= 227 * 1024, "shared memory");
 };
+
+// the axes' signs of coefficient k (real-packed, degree n at n^2: m = 0, then re, im of m = 1, 2, ...)
+// under a mirror in x, y, z, as a bit mask of the negative ones
+GB_HD int blk_signs(int k)
+{
+    int n = 0;
+#pragma unroll
+    for (int j = 1; j < 10; ++j) n += k >= j * j;
+    const int r = k - n * n, m = (r + 1) / 2, sy = (r > 0 && r % 2 == 0) ? 1 : 0;
+    return ((m & 1) ^ sy) | sy << 1 | ((n + m) & 1) << 2;
+}
+
+// v[sigma] -> sum_sigma (-1)^{c . sigma} v[sigma], c = 0..7
+GB_DEV void blk_hadamard(float (&v)[8])
+{
+#pragma unroll
+    for (int b = 1; b < 8; b <<= 1)
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (!(i & b)) {
+                const float x = v[i], y = v[i | b];
+                v[i] = x + y;
+                v[i | b] = x - y;
+            }
+}
+
+// v[sigma] *= s^sigma
+GB_DEV void blk_sign_children(float (&v)[8], int signs)
+{
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+        if (__popc(i & signs) & 1) v[i] = -v[i];
+}
+
+// One CTA's pipeline: per step (K chunk) the offset, first K value, width and whether it opens or
+// closes a drain unit; the units' offsets.  Built by one warp before the roles part.
+template <class C, int CH>
+struct BlkSteps {
+    uint32_t step[C::MAX_STEPS];  // d | k0 / 8 << 5 | kw / 16 << 13 | first << 16 | last << 17 | drain << 18
+    uint8_t drain_d[C::MAX_DRAINS];
+    int nsteps, ndrains;
+};
+GB_DEV int step_d(uint32_t v) { return v & 31; }
+GB_DEV int step_k0(uint32_t v) { return (int)(v >> 5 & 255) * 8; }
+GB_DEV int step_kw(uint32_t v) { return (int)(v >> 13 & 7) * 16; }
+GB_DEV bool step_first(uint32_t v) { return v >> 16 & 1; }
+GB_DEV bool step_last(uint32_t v) { return v >> 17 & 1; }
+GB_DEV int step_drain(uint32_t v) { return (int)(v >> 18); }
+
+// one warp; nt: the CTA's unit of classes, offsets [d_lo, d_hi)
+template <class C, int CH>
+GB_DEV void blk_steps(BlkSteps<C, CH> &t, int nt, int d_lo, int d_hi, int lane)
+{
+    constexpr int UB = C::NUNIT == 4 ? 2 : C::NUNIT == 2 ? 1 : 0;  // axes that distinguish units: the last UB
+    const int d = d_lo + lane;
+    int dx = 0, dy = 0, dz = 0, free = 0;
+    if (d < d_hi) {
+        blk_delta(d, dx, dy, dz);
+        free = UB == 2 ? (dy != 0) | (dz != 0) << 1 : UB == 1 ? (dz != 0) : 0;
+    }
+    const int nun = d < d_hi ? 1 << __popc(free) : 0;
+    int su = nun;  // inclusive scan
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int a = __shfl_up_sync(~0u, su, o);
+        if (lane >= o) su += a;
+    }
+    int i = su - nun;  // units before, of all the CTA's offsets
+    for (int e = 0; e < C::NUNIT; ++e) {
+        if (nun == 0 || (e & ~free)) continue;
+        const int ku = nt ^ e;
+        for (int c = 0; c < C::UC; ++c) {
+            const int kw = min(CH, C::UNIT - c * CH), piece = c * C::DPU / C::UC, dr = i * C::DPU + piece;
+            const bool first = c == 0 || (c - 1) * C::DPU / C::UC != piece;
+            const bool last = c == C::UC - 1 || (c + 1) * C::DPU / C::UC != piece;
+            if (first) t.drain_d[dr] = (uint8_t)d;
+            t.step[i * C::UC + c] = (uint32_t)d | (uint32_t)((ku * C::UNIT + c * CH) / 8) << 5 | (uint32_t)(kw / 16) << 13 |
+                                    (uint32_t)first << 16 | (uint32_t)last << 17 | (uint32_t)dr << 18;
+        }
+        ++i;
+    }
+    if (lane == 31) t.nsteps = su * C::UC, t.ndrains = su * C::DPU;
+}
+
+// K values per chunk: four stages of 32 (64-byte swizzle) cover the TMA latency better than two or
+// three of 64 (1M, p = 10: 0.343 against 0.372 ms)
+constexpr int blk_ch(int) { return 32; }
+constexpr size_t blk_kw(int P)  // K row width
+{
+    return P == 4 ? BlkCfg<4, blk_ch(4)>::KW : P == 6 ? BlkCfg<6, blk_ch(6)>::KW : P == 8 ? BlkCfg<8, blk_ch(8)>::KW
+                                                                                  : BlkCfg<10, blk_ch(10)>::KW;
+}
 
 // tensor maps and tiling of one launch (kernel parameter, read by the TMA unit in place)
 struct BlkParams {
@@ -151,18 +266,17 @@ GB_DEV void blk_ld8(uint32_t taddr, uint32_t *v)
 // 2^e as a float (e within the normal range)
 GB_DEV float blk_pow2(int e) { return __int_as_float((127 + e) << 23); }
 
-// ---- pre-split sources: per parent S of level l - 1, in grid order (x fastest), the 8 p^2
-// coefficients of its children (child sigma at [sigma p^2, (sigma + 1) p^2)) scaled by 2^s_S and
-// split into FP16 hi (plane 0) and lo (plane 1); s_S = 10 - e with max |M~| = f 2^e, f in
-// [0.5, 1) over the parent's nonempty children (empty children and empty parents: zeros, s = 0).
-// One warp per parent; the launch covers the parents of every level 1..L - 1 (A and scale hold the
-// levels one after another).
-template <int P>
+// ---- pre-split sources: per parent S of levels 1 .. L - 1, in grid order (x fastest), the classes
+// U of its children's coefficients (K rows of KW values) scaled by 2^s_S and split into FP16 hi (plane
+// 0) and lo (plane 1); s_S = 10 - e with max |U| = f 2^e, f in [0.5, 1) (empty parents: zeros,
+// s = 0).  One warp per parent; A and scale hold the levels one after another.
+template <int P, int CH>
 __global__ void __launch_bounds__(256) k_blk_presplit(int L, const int32_t *__restrict__ begin,
                                                       const int32_t *__restrict__ end, const float *__restrict__ M,
                                                       __half *__restrict__ A, int8_t *__restrict__ scale)
 {
-    constexpr int PP = P * P, KD = 8 * PP, PER = (KD + 31) / 32;
+    using C = BlkCfg<P, CH>;
+    constexpr int PP = P * P;
     const int lane = threadIdx.x & 31;
     const int64_t i = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);  // parent 1 + i of all levels
     if (i >= level_offset(L) - 1) return;
@@ -171,18 +285,22 @@ __global__ void __launch_bounds__(256) k_blk_presplit(int L, const int32_t *__re
     const uint32_t il = (uint32_t)(i + 1 - level_offset(lp)), pg = 1u << lp;  // grid order, x fastest
     const uint32_t x = il & (pg - 1), y = (il >> lp) & (pg - 1), z = il >> (2 * lp);
     const int64_t c0 = level_offset(lp + 1) + 8 * (int64_t)morton3(x, y, z);
-    float v[PER];
+    bool has[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) has[q] = end[c0 + q] > begin[c0 + q];
+    __half *row = A + i * (2 * C::KW);
+    constexpr int NJ = (PP + 31) / 32;
+    float v[NJ][8];
     float m = 0.f;
 #pragma unroll
-    for (int j = 0; j < PER; ++j) {
+    for (int j = 0; j < NJ; ++j) {
         const int k = lane + 32 * j;
-        float a = 0.f;
-        if (k < KD) {
-            const int64_t c = c0 + k / PP;
-            if (end[c] > begin[c]) a = M[c0 * PP + k];
-        }
-        v[j] = a;
-        m = fmaxf(m, fabsf(a));
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[j][q] = k < PP && has[q] ? M[(c0 + q) * PP + k] : 0.f;
+        blk_sign_children(v[j], blk_signs(min(k, PP - 1)));
+        blk_hadamard(v[j]);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) m = fmaxf(m, fabsf(v[j][q]));
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
@@ -193,82 +311,130 @@ __global__ void __launch_bounds__(256) k_blk_presplit(int L, const int32_t *__re
     sc = sc < -100 ? -100 : (sc > 100 ? 100 : sc);
     if (lane == 0) scale[i] = (int8_t)sc;
     const float up = blk_pow2(sc);
-    __half *row = A + i * (2 * KD);
 #pragma unroll
-    for (int j = 0; j < PER; ++j) {
+    for (int j = 0; j < NJ; ++j) {
         const int k = lane + 32 * j;
-        if (k < KD) {
-            const float xs = v[j] * up;
+        if (k >= PP) continue;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const float xs = v[j][q] * up;
             const __half hi = __float2half_rn(xs);
-            row[k] = hi;
-            row[KD + k] = __float2half_rn(xs - __half2float(hi));
+            __half *at = row + (q / C::CU) * C::UNIT + (q % C::CU) * PP + k;
+            at[0] = hi;
+            at[C::KW] = __float2half_rn(xs - __half2float(hi));
         }
     }
+    // the units' padding, read by the MMA against zero columns
+    constexpr int PAD = C::UNIT - C::CU * PP;
+    if constexpr (PAD > 0)
+        for (int e = lane; e < 2 * C::NUNIT * PAD; e += 32)
+            row[(e / PAD) * C::UNIT + C::CU * PP + e % PAD] = __float2half_rn(0.f);
 }
 
-// ---- operator blocks B_D (FP16 hi | lo, scaled by 2^g) -----------------------------------------
-// largest |entry| over the admissible offsets' operators, as float bits (non-negative floats
-// order like their bit patterns)
-template <int P>
-__global__ void __launch_bounds__(256) k_blk_opmax(const float *__restrict__ ops, unsigned *__restrict__ mbits)
+// ---- operator blocks B'_D (FP16 hi | lo, scaled by 2^g) ----------------------------------------
+// The 64 class products of one offset, target coefficient n and source coefficient k, in FP64: the
+// 27 operators T_{2D + sigma - tau} (0 for near offsets) as a 2 x 2 Toeplitz block per axis, and per
+// axis B'[c'][c] = 1/2 sum_{tau, sigma} (-1)^{c' tau + c sigma} s(n)^tau s(k)^sigma t_{sigma - tau}.
+template <int P, class F>
+GB_DEV void blk_class_products(const float *__restrict__ ops, int d, int n, int k, F put)
 {
     constexpr int PP = P * P, PR = ops_rows_padded(P);
-    const int code = blockIdx.x;
-    const int ox = code % 7 - 3, oy = (code / 7) % 7 - 3, oz = code / 49 - 3;
-    if (max(abs(ox), max(abs(oy), abs(oz))) < 2) return;  // near offsets have no M2L operator
-    const float *src = ops + (size_t)code * PP * PR;
+    int dx, dy, dz;
+    blk_delta(d, dx, dy, dz);
+    const int sn = blk_signs(n), sk = blk_signs(k);
+    double z[2][2][9], y[2][2][2][2][3];
+    auto axis = [](double tm, double t0, double tp, bool fn, bool fk, double (&o)[2][2]) {
+        const double a = fk ? -tp : tp, b = fn ? -tm : tm, c = fn != fk ? -t0 : t0;  // (tau, sigma) = (0,1), (1,0), (1,1)
+        o[0][0] = 0.5 * (t0 + a + b + c);
+        o[0][1] = 0.5 * (t0 - a + b - c);
+        o[1][0] = 0.5 * (t0 + a - b - c);
+        o[1][1] = 0.5 * (t0 - a - b + c);
+    };
+    for (int e = 0; e < 9; ++e) {  // z axis, for every (x, y) difference
+        const int ox = 2 * dx + e % 3 - 1, oy = 2 * dy + e / 3 - 1;
+        double t[3];
+        for (int w = 0; w < 3; ++w) {
+            const int oz = 2 * dz + w - 1;
+            t[w] = max(abs(ox), max(abs(oy), abs(oz))) < 2 ? 0.0
+                       : (double)ops[(size_t)m2l_code(ox, oy, oz) * PP * PR + (size_t)k * PR + n];
+        }
+        double o[2][2];
+        axis(t[0], t[1], t[2], sn >> 2 & 1, sk >> 2 & 1, o);
+        for (int q = 0; q < 4; ++q) z[q >> 1][q & 1][e] = o[q >> 1][q & 1];
+    }
+    for (int q = 0; q < 4; ++q)
+        for (int e = 0; e < 3; ++e) {  // y axis, for every x difference
+            double o[2][2];
+            const double *t = z[q >> 1][q & 1];
+            axis(t[e], t[3 + e], t[6 + e], sn >> 1 & 1, sk >> 1 & 1, o);
+            for (int r = 0; r < 4; ++r) y[q >> 1][q & 1][r >> 1][r & 1][e] = o[r >> 1][r & 1];
+        }
+    for (int q = 0; q < 4; ++q)
+        for (int r = 0; r < 4; ++r) {
+            double o[2][2];
+            const double *t = y[q >> 1][q & 1][r >> 1][r & 1];
+            axis(t[0], t[1], t[2], sn & 1, sk & 1, o);
+            for (int w = 0; w < 4; ++w)
+                put((q >> 1) << 2 | (r >> 1) << 1 | w >> 1, (q & 1) << 2 | (r & 1) << 1 | (w & 1), o[w >> 1][w & 1]);
+        }
+}
+
+// largest |B'| over all offsets, as float bits (non-negative floats order like their bit patterns);
+// a block per (d, k), threads over n
+template <int P>
+__global__ void __launch_bounds__(128) k_blk_opmax(const float *__restrict__ ops, unsigned *__restrict__ mbits)
+{
+    constexpr int PP = P * P;
     float m = 0.f;
-    for (int e = threadIdx.x; e < PP * PP; e += blockDim.x) m = fmaxf(m, fabsf(src[(e / PP) * PR + e % PP]));
+    for (int n = threadIdx.x; n < PP; n += blockDim.x)
+        blk_class_products<P>(ops, blockIdx.x / PP, n, blockIdx.x % PP,
+                              [&](int, int, double v) { m = fmaxf(m, fabsf((float)v)); });
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     if ((threadIdx.x & 31) == 0) atomicMax(mbits, __float_as_uint(m));
 }
 
-// B[d][plane][row (tau, n)][col (sigma, k)], one block per (d, row); g stored after the table
-template <int P>
-__global__ void __launch_bounds__(256) k_blk_build(const float *__restrict__ ops, const unsigned *__restrict__ mbits,
+// B[d][plane][row: class c', n][K column of class c, k] (the columns' padding zeroed beforehand); g
+// stored after the table
+template <int P, int CH>
+__global__ void __launch_bounds__(128) k_blk_build(const float *__restrict__ ops, const unsigned *__restrict__ mbits,
                                                    __half *__restrict__ B, int *__restrict__ gout)
 {
-    constexpr int PP = P * P, PR = ops_rows_padded(P), KD = 8 * PP;
-    const int d = blockIdx.x / KD, row = blockIdx.x % KD;
-    const int tau = row / PP, n = row % PP;
-    int dx, dy, dz;
-    blk_delta(d, dx, dy, dz);
+    using C = BlkCfg<P, CH>;
+    constexpr int PP = P * P;
+    const int d = blockIdx.x / PP, n = blockIdx.x % PP;
     int ex = 0;
     const float m = __uint_as_float(*mbits);
     if (m > 0.f) frexpf(m, &ex);
     const int g = m > 0.f ? 12 - ex : 0;
     if (blockIdx.x == 0 && threadIdx.x == 0) *gout = g;
-    const float sc = blk_pow2(g);
-    __half *hi = B + ((size_t)d * 2 * KD + row) * KD;
-    __half *lo = hi + (size_t)KD * KD;
-    for (int col = threadIdx.x; col < KD; col += blockDim.x) {
-        const int sigma = col / PP, k = col % PP;
-        const int ox = 2 * dx + (sigma & 1) - (tau & 1), oy = 2 * dy + ((sigma >> 1) & 1) - ((tau >> 1) & 1),
-                  oz = 2 * dz + (sigma >> 2) - (tau >> 2);
-        float v = 0.f;
-        if (max(abs(ox), max(abs(oy), abs(oz))) >= 2)
-            v = ops[(size_t)m2l_code(ox, oy, oz) * PP * PR + (size_t)k * PR + n] * sc;
-        const __half h = __float2half_rn(v);
-        hi[col] = h;
-        lo[col] = __float2half_rn(v - __half2float(h));
-    }
+    const double sc = ldexp(1.0, g);
+    __half *hi = B + (size_t)d * 2 * C::KD * C::KW, *lo = hi + (size_t)C::KD * C::KW;
+    for (int k = threadIdx.x; k < PP; k += blockDim.x)
+        blk_class_products<P>(ops, d, n, k, [&](int ct, int cs, double v) {
+            const size_t at = (size_t)(ct * PP + n) * C::KW + (cs / C::CU) * C::UNIT + (cs % C::CU) * PP + k;
+            const float f = (float)(v * sc);
+            const __half h = __float2half_rn(f);
+            hi[at] = h;
+            lo[at] = __float2half_rn(f - __half2float(h));
+        });
 }
 
 // ---- the kernel -------------------------------------------------------------------------------
-template <int P, int DS, int CH>
+template <int P, int CH>
 __global__ void __launch_bounds__(kBlkThreads, 1)
     k_m2l_blk(const __grid_constant__ BlkParams prm, const int32_t *__restrict__ begin,
               const int32_t *__restrict__ end, const int8_t *__restrict__ pscale, const int *__restrict__ gexp,
               float *__restrict__ Lc, float *__restrict__ Lpart, int *status)
 {
     using C = BlkCfg<P, CH>;
-    constexpr int PP = C::PP, KD = C::KD, NT = C::NT, NH = C::NH, NKC = C::NKC, NSTAGE = C::NSTAGE;
+    constexpr int PP = C::PP, NT = C::NT, NH = C::NH, NSTAGE = C::NSTAGE;
     constexpr uint32_t kIdesc = (1u << 4) | ((uint32_t)(NT >> 3) << 17) | ((uint32_t)(kBlkRows >> 4) << 24);
     constexpr int kProdWarp = kBlkDrainWarps, kMmaWarp = kBlkDrainWarps + 1;
 
     extern __shared__ unsigned char blk_smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[NSTAGE], empty_bar[NSTAGE], dfull[2], dempty[2], done_bar;
     __shared__ int s_issued[NSTAGE];
+    __shared__ BlkSteps<C, CH> s_steps;
     __shared__ uint32_t s_tmem;
     __shared__ volatile int s_abort;
 
@@ -276,7 +442,6 @@ __global__ void __launch_bounds__(kBlkThreads, 1)
     const int ks = (prm.tile0 + (int)blockIdx.x) % prm.ksplit;
     const int tile = (prm.tile0 + (int)blockIdx.x) / prm.ksplit;
     const int d_lo = (26 * ks) / prm.ksplit, d_hi = (26 * (ks + 1)) / prm.ksplit;
-    const int S = (d_hi - d_lo) * NKC, NU = (d_hi - d_lo) * DS;
     int l = 2;
     while (l < prm.L && tile >= prm.tile_lo[l + 1]) ++l;
     const int pg = 1 << (l - 1);
@@ -316,16 +481,17 @@ __global__ void __launch_bounds__(kBlkThreads, 1)
         blk_prefetch_tmap(&prm.tmB);
     }
     if (warp == kMmaWarp) tmem_alloc(&s_tmem, C::TMEM_COLS);
+    if (warp == 0) blk_steps<C, CH>(s_steps, nt, d_lo, d_hi, lane);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = s_tmem;
+    const int S = s_steps.nsteps, NU = s_steps.ndrains;
 
-    // pipeline step s: offset d = s / NKC, K-chunk c = s % NKC; drain unit u = d DS + c DS / NKC
     if (warp == kProdWarp) {
         if (lane == 0) {
             for (int s = 0; s < S; ++s) {
-                const int st = s % NSTAGE, d = d_lo + s / NKC, c = s % NKC;
+                const int st = s % NSTAGE, d = step_d(s_steps.step[s]), k0 = step_k0(s_steps.step[s]);
                 if (s >= NSTAGE &&
                     !mbar_wait_bounded(&empty_bar[st], ((s / NSTAGE) - 1) & 1, kWaitLimitNs, &s_abort)) {
                     s_abort = 1;
@@ -335,7 +501,6 @@ __global__ void __launch_bounds__(kBlkThreads, 1)
                 int dx, dy, dz;
                 blk_delta(d, dx, dy, dz);
                 mbar_expect_tx(&full_bar[st], 2u * a_bytes + 2u * (uint32_t)C::B_BYTES);
-                const int k0 = c * CH;
                 blk_tma5(a_hi(st), &prm.tmA[l], k0, 0, x0 + dx, y0 + dy, z0 + dz, &full_bar[st]);
                 blk_tma5(a_lo(st), &prm.tmA[l], k0, 1, x0 + dx, y0 + dy, z0 + dz, &full_bar[st]);
                 blk_tma4(b_hi(st), &prm.tmB, k0, nt * C::NSTRIDE, 0, d, &full_bar[st]);
@@ -346,10 +511,9 @@ __global__ void __launch_bounds__(kBlkThreads, 1)
     } else if (warp == kMmaWarp) {
         if (lane == 0) {
             for (int s = 0; s < S; ++s) {
-                const int st = s % NSTAGE, c = s % NKC;
-                const int uc = (c * DS) / NKC, u = (s / NKC) * DS + uc, b = u & 1;
-                const bool first = c == 0 || ((c - 1) * DS) / NKC != uc;
-                const bool last = c == NKC - 1 || ((c + 1) * DS) / NKC != uc;
+                const uint32_t sv = s_steps.step[s];
+                const int st = s % NSTAGE, u = step_drain(sv), b = u & 1;
+                const bool first = step_first(sv), last = step_last(sv);
                 if (first && u >= 2 &&
                     !mbar_wait_bounded(&dempty[b], ((u - 2) >> 1) & 1, kWaitLimitNs, &s_abort)) {
                     s_abort = 1;
@@ -360,11 +524,10 @@ __global__ void __launch_bounds__(kBlkThreads, 1)
                     break;
                 }
                 tc_fence_after();
-                const int kw = KD - c * CH < CH ? KD - c * CH : CH;
                 const uint32_t ah = smem_u32(a_hi(st)), al = smem_u32(a_lo(st));
                 const uint32_t bh = smem_u32(b_hi(st)), bl = smem_u32(b_lo(st));
                 const uint32_t dt = tmem + (uint32_t)(b * NT);
-                for (int j = 0; j < (kw + 15) / 16; ++j) {
+                for (int j = 0; j < step_kw(sv) / 16; ++j) {
                     const uint32_t o = 32u * j;
                     blk_mma_ss(dt, blk_desc<CH>(al + o), blk_desc<CH>(bh + o), kIdesc, (first && j == 0) ? 0u : 1u);
                     blk_mma_ss(dt, blk_desc<CH>(ah + o), blk_desc<CH>(bl + o), kIdesc, 1u);
@@ -389,7 +552,7 @@ __global__ void __launch_bounds__(kBlkThreads, 1)
         for (int i = 0; i < NH; ++i) acc[i] = 0.f;
         bool alive = true;
         for (int u = 0; u < NU && alive; ++u) {
-            const int d = d_lo + u / DS, b = u & 1;
+            const int d = s_steps.drain_d[u], b = u & 1;
             int dx, dy, dz;
             blk_delta(d, dx, dy, dz);
             const int sx = qx + dx, sy = qy + dy, sz = qz + dz;
@@ -428,17 +591,15 @@ __global__ void __launch_bounds__(kBlkThreads, 1)
         __syncwarp();
         if (ok && alive && !s_abort && rok) {
             float *dst = prm.ksplit > 1 ? Lpart + (int64_t)ks * prm.part_stride : Lc;
-            const int64_t cell0 = level_offset(l) + 8 * (int64_t)morton3((uint32_t)qx, (uint32_t)qy, (uint32_t)qz);
+            // the classes V of a nonempty parent, in its children's places
+            const int64_t key = (int64_t)morton3((uint32_t)qx, (uint32_t)qy, (uint32_t)qz), par = level_offset(l - 1) + key;
+            float *row = dst + (level_offset(l) + 8 * key) * PP + nt * C::NSTRIDE;
+            if (end[par] > begin[par])
 #pragma unroll
-            for (int i = 0; i < NH; i += 4) {
-                const int col = h * NH + i;
-                const int gc = nt * C::NSTRIDE + col;
-                if (col >= C::NSTRIDE || gc >= KD) continue;
-                const int tau = gc / PP, n = gc % PP;
-                const int64_t cell = cell0 + tau;
-                if (end[cell] <= begin[cell]) continue;
-                *reinterpret_cast<float4 *>(dst + cell * PP + n) = make_float4(acc[i], acc[i + 1], acc[i + 2], acc[i + 3]);
-            }
+                for (int i = 0; i < NH; i += 4)
+                    if (h * NH + i < C::NSTRIDE)
+                        *reinterpret_cast<float4 *>(row + h * NH + i) =
+                            make_float4(acc[i], acc[i + 1], acc[i + 2], acc[i + 3]);
         }
     }
 
@@ -502,40 +663,47 @@ __global__ void k_ablk_units(Span cells, const uint32_t *__restrict__ flag, cons
     }
 }
 
-// pre-split rows: unit u (one warp): its children's scaled coefficients 2^s_u M~ in FP16 hi | lo,
-// s_u = 10 - e with max |M~| = f 2^e over its children (0 and zeros for none); row Z and its scale
-// are zero
-template <int P>
+// pre-split rows: unit u (one warp): the classes U of its children's coefficients, scaled by 2^s_u, in
+// FP16 hi | lo, s_u = 10 - e with max |U| = f 2^e (0 and zeros for none); row Z and its scale are zero
+template <int P, int CH>
 __global__ void __launch_bounds__(256) k_ablk_presplit(const int32_t *__restrict__ n_units, int64_t zrow,
                                                        const int32_t *__restrict__ units,
                                                        const int32_t *__restrict__ child_of,
                                                        const float *__restrict__ M, __half *__restrict__ A,
                                                        int8_t *__restrict__ scale)
 {
-    constexpr int PP = P * P, KD = 8 * PP, PER = (KD + 31) / 32;
+    using C = BlkCfg<P, CH>;
+    constexpr int PP = P * P;
     const int lane = threadIdx.x & 31;
     const int64_t u = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
     const int64_t nu = *n_units;
     if (u > zrow || (u >= nu && u != zrow)) return;
-    __half *row = A + u * (2 * KD);
+    __half *row = A + u * (2 * C::KW);
     if (u == zrow || u >= nu) {
-        for (int k = lane; k < 2 * KD; k += 32) row[k] = __float2half_rn(0.f);
+        for (int k = lane; k < 2 * C::KW; k += 32) row[k] = __float2half_rn(0.f);
         if (lane == 0) scale[u] = 0;
         return;
     }
-    const int64_t q = units[u];
-    float v[PER];
+    const int64_t cell = units[u];
+    bool has[8];
+    int64_t child[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        child[q] = child_of[cell * 8 + q];
+        has[q] = child[q] >= 0;
+    }
+    constexpr int NJ = (PP + 31) / 32;
+    float v[NJ][8];
     float m = 0.f;
 #pragma unroll
-    for (int j = 0; j < PER; ++j) {
+    for (int j = 0; j < NJ; ++j) {
         const int k = lane + 32 * j;
-        float a = 0.f;
-        if (k < KD) {
-            const int32_t c = child_of[q * 8 + k / PP];
-            if (c >= 0) a = M[(int64_t)c * PP + k % PP];
-        }
-        v[j] = a;
-        m = fmaxf(m, fabsf(a));
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[j][q] = k < PP && has[q] ? M[child[q] * PP + k] : 0.f;
+        blk_sign_children(v[j], blk_signs(min(k, PP - 1)));
+        blk_hadamard(v[j]);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) m = fmaxf(m, fabsf(v[j][q]));
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
@@ -547,15 +715,23 @@ __global__ void __launch_bounds__(256) k_ablk_presplit(const int32_t *__restrict
     if (lane == 0) scale[u] = (int8_t)sc;
     const float up = blk_pow2(sc);
 #pragma unroll
-    for (int j = 0; j < PER; ++j) {
+    for (int j = 0; j < NJ; ++j) {
         const int k = lane + 32 * j;
-        if (k < KD) {
-            const float xs = v[j] * up;
+        if (k >= PP) continue;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const float xs = v[j][q] * up;
             const __half hi = __float2half_rn(xs);
-            row[k] = hi;
-            row[KD + k] = __float2half_rn(xs - __half2float(hi));
+            __half *at = row + (q / C::CU) * C::UNIT + (q % C::CU) * PP + k;
+            at[0] = hi;
+            at[C::KW] = __float2half_rn(xs - __half2float(hi));
         }
     }
+    // the units' padding, read by the MMA against zero columns
+    constexpr int PAD = C::UNIT - C::CU * PP;
+    if constexpr (PAD > 0)
+        for (int e = lane; e < 2 * C::NUNIT * PAD; e += 32)
+            row[(e / PAD) * C::UNIT + C::CU * PP + e % PAD] = __float2half_rn(0.f);
 }
 
 // src[(tile 26 + d) 128 + r] = the row of unit tile 128 + r's colleague at offset d (Z if none);
@@ -589,21 +765,21 @@ struct AblkParams {
     int64_t zrow;
 };
 
-template <int P, int DS, int CH>
+template <int P, int CH>
 __global__ void __launch_bounds__(kAblkThreads, 1)
     k_m2l_ablk(const __grid_constant__ AblkParams prm, const int32_t *__restrict__ n_units,
-               const int32_t *__restrict__ units, const int32_t *__restrict__ child_of,
                const int32_t *__restrict__ src, const __half *__restrict__ Apre, const int8_t *__restrict__ uscale,
-               const int *__restrict__ gexp, float *__restrict__ Lc, float *__restrict__ Lpart, int *status)
+               const int *__restrict__ gexp, float *__restrict__ V, int *status)
 {
     using C = BlkCfg<P, CH>;
-    constexpr int PP = C::PP, KD = C::KD, NT = C::NT, NH = C::NH, NKC = C::NKC, NSTAGE = C::NSTAGE;
+    constexpr int KD = C::KD, NT = C::NT, NH = C::NH, NSTAGE = C::NSTAGE;
     constexpr uint32_t kIdesc = (1u << 4) | ((uint32_t)(NT >> 3) << 17) | ((uint32_t)(kBlkRows >> 4) << 24);
     constexpr int kLoad0 = kBlkDrainWarps, kProdWarp = kLoad0 + kAblkLoadWarps, kMmaWarp = kProdWarp + 1;
 
     extern __shared__ unsigned char blk_smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[NSTAGE], empty_bar[NSTAGE], dfull[2], dempty[2], done_bar;
     __shared__ int s_issued[NSTAGE];
+    __shared__ BlkSteps<C, CH> s_steps;
     __shared__ uint32_t s_tmem;
     __shared__ volatile int s_abort;
 
@@ -615,7 +791,6 @@ __global__ void __launch_bounds__(kAblkThreads, 1)
     const int64_t nu = *n_units;
     if (ut * kBlkRows >= nu) return;  // the whole CTA: past the units (before any barrier or TMEM)
     const int d_lo = (26 * ks) / prm.ksplit, d_hi = (26 * (ks + 1)) / prm.ksplit;
-    const int S = (d_hi - d_lo) * NKC, NU = (d_hi - d_lo) * DS;
     const int32_t *tsrc = src + ut * 26 * kBlkRows;
 
     unsigned char *smem =
@@ -641,10 +816,12 @@ __global__ void __launch_bounds__(kAblkThreads, 1)
     }
     if (warp == kProdWarp && lane == 0) blk_prefetch_tmap(&prm.tmB);
     if (warp == kMmaWarp) tmem_alloc(&s_tmem, C::TMEM_COLS);
+    if (warp == 0) blk_steps<C, CH>(s_steps, nt, d_lo, d_hi, lane);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = s_tmem;
+    const int S = s_steps.nsteps, NU = s_steps.ndrains;
 
     if (warp >= kLoad0 && warp < kProdWarp) {
         // ===== loader warps: rows 64 w + lane and 64 w + 32 + lane of A (hi and lo planes) =====
@@ -655,21 +832,21 @@ __global__ void __launch_bounds__(kAblkThreads, 1)
         constexpr int NB = RPW * 2 * CPR;                    // chunks per lane and stage
         const int r0 = (kBlkRows / kAblkLoadWarps) * (warp - kLoad0) + lane;
         auto fetch = [&](int s, int4(&v)[NB]) {
-            const int d = d_lo + s / NKC, c = s % NKC;
-            const int kw = KD - c * CH < CH ? KD - c * CH : CH;
+            const uint32_t sv = s_steps.step[s];
+            const int d = step_d(sv), kw = step_kw(sv);
 #pragma unroll
             for (int rr = 0; rr < RPW; ++rr) {
                 const int64_t row = tsrc[d * kBlkRows + r0 + 32 * rr];
 #pragma unroll
                 for (int pl = 0; pl < 2; ++pl) {
-                    const int4 *g = reinterpret_cast<const int4 *>(Apre + (row * 2 + pl) * KD + (int64_t)c * CH);
+                    const int4 *g = reinterpret_cast<const int4 *>(Apre + (row * 2 + pl) * C::KW + step_k0(sv));
 #pragma unroll
                     for (int q = 0; q < CPR; ++q) v[(rr * 2 + pl) * CPR + q] = 8 * q < kw ? __ldg(g + q) : int4{0, 0, 0, 0};
                 }
             }
         };
         auto put = [&](int s, const int4(&v)[NB]) {
-            const int st = s % NSTAGE, c = s % NKC;
+            const int st = s % NSTAGE, kw = step_kw(s_steps.step[s]);
             int ok = 1;
             if (s >= NSTAGE && lane == 0)
                 ok = mbar_wait_bounded(&empty_bar[st], ((s / NSTAGE) - 1) & 1, kWaitLimitNs, &s_abort) ? 1 : 0;
@@ -678,7 +855,6 @@ __global__ void __launch_bounds__(kAblkThreads, 1)
                 if (lane == 0) s_abort = 1;
                 return false;
             }
-            const int kw = KD - c * CH < CH ? KD - c * CH : CH;
 #pragma unroll
             for (int rr = 0; rr < RPW; ++rr) {
                 const int r = r0 + 32 * rr;
@@ -718,7 +894,7 @@ __global__ void __launch_bounds__(kAblkThreads, 1)
     } else if (warp == kProdWarp) {
         if (lane == 0) {
             for (int s = 0; s < S; ++s) {
-                const int st = s % NSTAGE, d = d_lo + s / NKC, c = s % NKC;
+                const int st = s % NSTAGE, d = step_d(s_steps.step[s]), k0 = step_k0(s_steps.step[s]);
                 if (s >= NSTAGE &&
                     !mbar_wait_bounded(&empty_bar[st], ((s / NSTAGE) - 1) & 1, kWaitLimitNs, &s_abort)) {
                     s_abort = 1;
@@ -726,7 +902,6 @@ __global__ void __launch_bounds__(kAblkThreads, 1)
                 }
                 if (s_abort) break;
                 mbar_expect_tx(&full_bar[st], 2u * (uint32_t)C::B_BYTES);
-                const int k0 = c * CH;
                 blk_tma4(b_hi(st), &prm.tmB, k0, nt * C::NSTRIDE, 0, d, &full_bar[st]);
                 blk_tma4(b_lo(st), &prm.tmB, k0, nt * C::NSTRIDE, 1, d, &full_bar[st]);
                 s_issued[st] += 1;
@@ -735,10 +910,9 @@ __global__ void __launch_bounds__(kAblkThreads, 1)
     } else if (warp == kMmaWarp) {
         if (lane == 0) {
             for (int s = 0; s < S; ++s) {
-                const int st = s % NSTAGE, c = s % NKC;
-                const int uc = (c * DS) / NKC, u = (s / NKC) * DS + uc, b = u & 1;
-                const bool first = c == 0 || ((c - 1) * DS) / NKC != uc;
-                const bool last = c == NKC - 1 || ((c + 1) * DS) / NKC != uc;
+                const uint32_t sv = s_steps.step[s];
+                const int st = s % NSTAGE, u = step_drain(sv), b = u & 1;
+                const bool first = step_first(sv), last = step_last(sv);
                 if (first && u >= 2 &&
                     !mbar_wait_bounded(&dempty[b], ((u - 2) >> 1) & 1, kWaitLimitNs, &s_abort)) {
                     s_abort = 1;
@@ -749,11 +923,10 @@ __global__ void __launch_bounds__(kAblkThreads, 1)
                     break;
                 }
                 tc_fence_after();
-                const int kw = KD - c * CH < CH ? KD - c * CH : CH;
                 const uint32_t ah = smem_u32(a_pl(st, 0)), al = smem_u32(a_pl(st, 1));
                 const uint32_t bh = smem_u32(b_hi(st)), bl = smem_u32(b_lo(st));
                 const uint32_t dt = tmem + (uint32_t)(b * NT);
-                for (int j = 0; j < (kw + 15) / 16; ++j) {
+                for (int j = 0; j < step_kw(sv) / 16; ++j) {
                     const uint32_t o = 32u * j;
                     blk_mma_ss(dt, blk_desc<CH>(al + o), blk_desc<CH>(bh + o), kIdesc, (first && j == 0) ? 0u : 1u);
                     blk_mma_ss(dt, blk_desc<CH>(ah + o), blk_desc<CH>(bl + o), kIdesc, 1u);
@@ -777,7 +950,7 @@ __global__ void __launch_bounds__(kAblkThreads, 1)
         for (int i = 0; i < NH; ++i) acc[i] = 0.f;
         bool alive = true;
         for (int u = 0; u < NU && alive; ++u) {
-            const int d = d_lo + u / DS, b = u & 1;
+            const int d = s_steps.drain_d[u], b = u & 1;
             const int64_t row = tsrc[d * kBlkRows + r];
             const float f = row == prm.zrow ? 0.f : blk_pow2(-((int)uscale[row] + g));
             int ok = 1;
@@ -811,19 +984,11 @@ __global__ void __launch_bounds__(kAblkThreads, 1)
         if (!ok && lane == 0) s_abort = 1;
         __syncwarp();
         if (ok && alive && !s_abort && rok) {
-            float *dst = prm.ksplit > 1 ? Lpart + (int64_t)ks * prm.part_stride : Lc;
-            const int64_t q = units[unit];
+            float *row = V + (int64_t)ks * prm.part_stride + unit * KD + nt * C::NSTRIDE;
 #pragma unroll
-            for (int i = 0; i < NH; i += 4) {
-                const int col = h * NH + i;
-                const int gc = nt * C::NSTRIDE + col;
-                if (col >= C::NSTRIDE || gc >= KD) continue;
-                const int tau = gc / PP, n = gc % PP;
-                const int32_t cell = child_of[q * 8 + tau];
-                if (cell < 0) continue;
-                *reinterpret_cast<float4 *>(dst + (int64_t)cell * PP + n) =
-                    make_float4(acc[i], acc[i + 1], acc[i + 2], acc[i + 3]);
-            }
+            for (int i = 0; i < NH; i += 4)
+                if (h * NH + i < C::NSTRIDE)
+                    *reinterpret_cast<float4 *>(row + h * NH + i) = make_float4(acc[i], acc[i + 1], acc[i + 2], acc[i + 3]);
         }
     }
 
@@ -843,25 +1008,64 @@ __global__ void __launch_bounds__(kAblkThreads, 1)
     }
 }
 
-// ---- sum of the offset ranges' partial sums (fixed order, so the result does not depend on
-// which CTA finished first): Lc = sum_k Lpart[k] over the nonempty cells of levels 2..L
-__global__ void __launch_bounds__(256) k_blk_reduce(int64_t c0, int64_t c1, int PP4, int ksplit, int64_t stride4,
-                                                    const int32_t *__restrict__ begin, const int32_t *__restrict__ end,
-                                                    const float4 *__restrict__ part, float4 *__restrict__ Lc)
+// ---- the classes back to the children: V = sum over the offset ranges (fixed order, so the result does
+// not depend on which CTA finished first), L~_tau = s^tau / 8 sum_c (-1)^{c . tau} V_c.  Eight lanes
+// per parent and four coefficients, one a class: each adds its class over the ranges (a thread for
+// all eight took 36 us on the 208 loads of 26 ranges), then three exchanges form the children.
+// Lane: item (4 to a warp) + 4 class.  In place where there is one range (uniform tree).
+GB_DEV float4 blk_child(const float4 *src, int64_t stride4, int ksplit, int n4, int c, bool valid)
 {
-    const int64_t i = c0 * PP4 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= c1 * PP4) return;
-    const int64_t cell = i / PP4;
-    if (end[cell] <= begin[cell]) return;
-    float4 a = part[i];
-    for (int k = 1; k < ksplit; ++k) {
-        const float4 b = part[i + k * stride4];
-        a.x += b.x;
-        a.y += b.y;
-        a.z += b.z;
-        a.w += b.w;
+    float v[4] = {0.f, 0.f, 0.f, 0.f};
+    if (valid) {
+        const float4 a = *src;
+        v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
+#pragma unroll 8
+        for (int k = 1; k < ksplit; ++k) {
+            const float4 t = src[k * stride4];
+            v[0] += t.x, v[1] += t.y, v[2] += t.z, v[3] += t.w;
+        }
     }
-    Lc[i] = a;
+#pragma unroll
+    for (int b = 1; b < 8; b <<= 1)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float o = __shfl_xor_sync(0xffffffffu, v[j], 4 * b);
+            v[j] = (c & b) ? o - v[j] : v[j] + o;
+        }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] *= (__popc(c & blk_signs(4 * n4 + j)) & 1) ? -0.125f : 0.125f;
+    return make_float4(v[0], v[1], v[2], v[3]);
+}
+
+// uniform tree: parents of levels 1 .. L - 1
+template <int P>
+__global__ void __launch_bounds__(256) k_blk_finish(int npar, int ksplit, int64_t stride4,
+                                                    const int32_t *__restrict__ begin, const int32_t *__restrict__ end,
+                                                    const float4 *src, float4 *Lc)
+{
+    const int lane = threadIdx.x & 31, c = lane >> 2;
+    constexpr int PP4 = P * P / 4;
+    const uint32_t i = (blockIdx.x * 8 + (threadIdx.x >> 5)) * 4 + (lane & 3), q = i / PP4, n4 = i % PP4;
+    const int64_t par = 1 + (int64_t)q, at = (8 * par + 1 + c) * PP4 + n4;  // children of cell par: 8 par + 1 ..
+    const bool ok = q < (uint32_t)npar && end[par] > begin[par];
+    const float4 v = blk_child(src + at, stride4, ksplit, (int)n4, c, ok);
+    if (ok && end[8 * par + 1 + c] > begin[8 * par + 1 + c]) Lc[at] = v;
+}
+
+// adaptive tree: units
+template <int P>
+__global__ void __launch_bounds__(256) k_ablk_finish(const int32_t *__restrict__ n_units, int ksplit, int64_t stride4,
+                                                     const int32_t *__restrict__ units,
+                                                     const int32_t *__restrict__ child_of,
+                                                     const float4 *__restrict__ V, float4 *__restrict__ Lc)
+{
+    const int lane = threadIdx.x & 31, c = lane >> 2;
+    constexpr int PP4 = P * P / 4;
+    const uint32_t i = (blockIdx.x * 8 + (threadIdx.x >> 5)) * 4 + (lane & 3), u = i / PP4, n4 = i % PP4;
+    const bool ok = u < (uint32_t)*n_units;
+    const float4 v = blk_child(V + ((int64_t)u * 8 + c) * PP4 + n4, stride4, ksplit, (int)n4, c, ok);
+    const int64_t g = ok ? child_of[(int64_t)units[u] * 8 + c] : -1;
+    if (g >= 0) Lc[g * PP4 + n4] = v;
 }
 
 // ---- host side ----------------------------------------------------------------------------------
@@ -891,7 +1095,7 @@ int64_t blk_parents_before(int lp) { return level_offset(lp) - 1; }
 size_t m2l_blk_presplit_bytes(int P, int L)
 {
     if (L < 2) return 0;
-    return (size_t)blk_parents_before(L) * 2 * 8 * P * P * sizeof(__half);
+    return (size_t)blk_parents_before(L) * 2 * blk_kw(P) * sizeof(__half);
 }
 
 size_t m2l_blk_scale_bytes(int L) { return L < 2 ? 0 : (size_t)blk_parents_before(L); }
@@ -904,7 +1108,7 @@ static int blk_tiles(int L)
     for (int l = 2; l <= L; ++l) {
         const int pg = 1 << (l - 1);
         const int bx = pg < 8 ? pg : 8, by = pg < 4 ? pg : 4;
-        n += (pg / bx) * (pg / by) * (pg / by) * BlkCfg<P, 64>::NTILES;
+        n += (pg / bx) * (pg / by) * (pg / by) * BlkCfg<P, blk_ch(P)>::NTILES;
     }
     return n;
 }
@@ -949,41 +1153,31 @@ size_t m2l_blk_part_bytes(int P, int L)
     return k > 1 ? (size_t)k * level_offset(L + 1) * P * P * sizeof(float) : 0;
 }
 
-size_t m2l_blk_table_bytes(int P)
-{
-    const size_t KD = 8 * (size_t)P * P;
-    return 26 * 2 * KD * KD * sizeof(__half) + 256;
-}
+size_t m2l_blk_table_bytes(int P) { return 26 * 2 * 8 * (size_t)P * P * blk_kw(P) * sizeof(__half) + 256; }
 
-// the table: B (hi | lo per d) then, 256-aligned, the exponent g and the max-bits scratch word
-void launch_build_m2l_blk(int P, const float *ops, void *table, cudaStream_t s)
+// the table: B' (hi | lo per d), then the exponent g and the max-bits scratch word
+template <int P>
+static void launch_build_t(const float *ops, void *table, cudaStream_t s)
 {
-    const size_t KD = 8 * (size_t)P * P;
+    using C = BlkCfg<P, blk_ch(P)>;
     __half *B = static_cast<__half *>(table);
-    int *g = reinterpret_cast<int *>(B + 26 * 2 * KD * KD);
+    int *g = reinterpret_cast<int *>(B + 26 * 2 * (size_t)C::KD * C::KW);
     unsigned *mbits = reinterpret_cast<unsigned *>(g + 1);
-    cudaMemsetAsync(mbits, 0, sizeof(unsigned), s);
-    switch (P) {
-    case 4:
-        k_blk_opmax<4><<<kM2LCodes, 256, 0, s>>>(ops, mbits);
-        k_blk_build<4><<<(unsigned)(26 * KD), 256, 0, s>>>(ops, mbits, B, g);
-        break;
-    case 6:
-        k_blk_opmax<6><<<kM2LCodes, 256, 0, s>>>(ops, mbits);
-        k_blk_build<6><<<(unsigned)(26 * KD), 256, 0, s>>>(ops, mbits, B, g);
-        break;
-    case 8:
-        k_blk_opmax<8><<<kM2LCodes, 256, 0, s>>>(ops, mbits);
-        k_blk_build<8><<<(unsigned)(26 * KD), 256, 0, s>>>(ops, mbits, B, g);
-        break;
-    case 10:
-        k_blk_opmax<10><<<kM2LCodes, 256, 0, s>>>(ops, mbits);
-        k_blk_build<10><<<(unsigned)(26 * KD), 256, 0, s>>>(ops, mbits, B, g);
-        break;
-    }
+    cudaMemsetAsync(table, 0, m2l_blk_table_bytes(P), s);
+    k_blk_opmax<P><<<26 * P * P, 128, 0, s>>>(ops, mbits);
+    k_blk_build<P, blk_ch(P)><<<26 * P * P, 128, 0, s>>>(ops, mbits, B, g);
     note_launches(2);
 }
 
+void launch_build_m2l_blk(int P, const float *ops, void *table, cudaStream_t s)
+{
+    switch (P) {
+    case 4: launch_build_t<4>(ops, table, s); break;
+    case 6: launch_build_t<6>(ops, table, s); break;
+    case 8: launch_build_t<8>(ops, table, s); break;
+    case 10: launch_build_t<10>(ops, table, s); break;
+    }
+}
 
 void launch_blk_presplit(int P, int L, const int32_t *begin, const int32_t *end, const float *M, void *presplit,
                          int8_t *pscale, cudaStream_t s)
@@ -992,10 +1186,10 @@ void launch_blk_presplit(int P, int L, const int32_t *begin, const int32_t *end,
     const unsigned grid = (unsigned)((blk_parents_before(L) + 7) / 8);
     __half *A = static_cast<__half *>(presplit);
     switch (P) {
-    case 4: k_blk_presplit<4><<<grid, 256, 0, s>>>(L, begin, end, M, A, pscale); break;
-    case 6: k_blk_presplit<6><<<grid, 256, 0, s>>>(L, begin, end, M, A, pscale); break;
-    case 8: k_blk_presplit<8><<<grid, 256, 0, s>>>(L, begin, end, M, A, pscale); break;
-    case 10: k_blk_presplit<10><<<grid, 256, 0, s>>>(L, begin, end, M, A, pscale); break;
+    case 4: k_blk_presplit<4, blk_ch(4)><<<grid, 256, 0, s>>>(L, begin, end, M, A, pscale); break;
+    case 6: k_blk_presplit<6, blk_ch(6)><<<grid, 256, 0, s>>>(L, begin, end, M, A, pscale); break;
+    case 8: k_blk_presplit<8, blk_ch(8)><<<grid, 256, 0, s>>>(L, begin, end, M, A, pscale); break;
+    case 10: k_blk_presplit<10, blk_ch(10)><<<grid, 256, 0, s>>>(L, begin, end, M, A, pscale); break;
     }
     note_launches(1);
 }
@@ -1012,17 +1206,17 @@ static int launch_blk_t(int L, const int32_t *begin, const int32_t *end, const v
     BlkParams prm;  // the kernel parameter (copied at launch)
     memset(&prm, 0, sizeof(prm));
     prm.L = L;
-    const cuuint64_t KD = C::KD;
-    const int *gexp = reinterpret_cast<const int *>(static_cast<const __half *>(table) + 26 * 2 * KD * KD);
+    const cuuint64_t KD = C::KD, KW = C::KW;
+    const int *gexp = reinterpret_cast<const int *>(static_cast<const __half *>(table) + 26 * 2 * KD * KW);
     int ntiles = 0;
     for (int l = 2; l <= L; ++l) {
         const int pg = 1 << (l - 1);
         const int bx = pg < 8 ? pg : 8, by = pg < 4 ? pg : 4, bz = by;
         prm.tile_lo[l] = ntiles;
         ntiles += (pg / bx) * (pg / by) * (pg / bz) * C::NTILES;
-        void *A = const_cast<__half *>(static_cast<const __half *>(presplit) + (size_t)blk_parents_before(l - 1) * 2 * KD);
-        const cuuint64_t dims[5] = {KD, 2, (cuuint64_t)pg, (cuuint64_t)pg, (cuuint64_t)pg};
-        const cuuint64_t strides[4] = {KD * 2, KD * 4, KD * 4 * pg, KD * 4 * pg * pg};
+        void *A = const_cast<__half *>(static_cast<const __half *>(presplit) + (size_t)blk_parents_before(l - 1) * 2 * KW);
+        const cuuint64_t dims[5] = {KW, 2, (cuuint64_t)pg, (cuuint64_t)pg, (cuuint64_t)pg};
+        const cuuint64_t strides[4] = {KW * 2, KW * 4, KW * 4 * pg, KW * 4 * pg * pg};
         const cuuint32_t box[5] = {(cuuint32_t)CH, 1, (cuuint32_t)bx, (cuuint32_t)by, (cuuint32_t)bz};
         const cuuint32_t es[5] = {1, 1, 1, 1, 1};
         if (enc(&prm.tmA[l], CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 5, A, dims, strides, box, es,
@@ -1035,8 +1229,8 @@ static int launch_blk_t(int L, const int32_t *begin, const int32_t *end, const v
     prm.part_stride = level_offset(L + 1) * C::PP;
     if (prm.ksplit > 1 && !Lpart) return -1;
     {
-        const cuuint64_t dims[4] = {KD, KD, 2, 26};
-        const cuuint64_t strides[3] = {KD * 2, KD * KD * 2, KD * KD * 4};
+        const cuuint64_t dims[4] = {KW, KD, 2, 26};
+        const cuuint64_t strides[3] = {KW * 2, KD * KW * 2, KD * KW * 4};
         const cuuint32_t box[4] = {(cuuint32_t)CH, (cuuint32_t)C::NT, 1, 1};
         const cuuint32_t es[4] = {1, 1, 1, 1};
         if (enc(&prm.tmB, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, const_cast<void *>(table), dims, strides, box, es,
@@ -1044,7 +1238,7 @@ static int launch_blk_t(int L, const int32_t *begin, const int32_t *end, const v
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return -1;
     }
-    auto kern = k_m2l_blk<P, kBlkDrainsPerOffset, CH>;
+    auto kern = k_m2l_blk<P, CH>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::kSmemBytes);
     const int nctas = ntiles * prm.ksplit;
     const int step = max_ctas > 0 ? max_ctas : nctas;
@@ -1054,14 +1248,11 @@ static int launch_blk_t(int L, const int32_t *begin, const int32_t *end, const v
         kern<<<gsz, kBlkThreads, C::kSmemBytes, s>>>(prm, begin, end, pscale, gexp, Lc, Lpart, status);
         note_launches(1);
     }
-    if (prm.ksplit > 1) {
-        const int64_t c0 = level_offset(2), c1 = level_offset(L + 1), PP4 = C::PP / 4;
-        const int64_t nthr = (c1 - c0) * PP4;
-        k_blk_reduce<<<(unsigned)((nthr + 255) / 256), 256, 0, s>>>(
-            c0, c1, (int)PP4, prm.ksplit, prm.part_stride / 4, begin, end, reinterpret_cast<const float4 *>(Lpart),
-            reinterpret_cast<float4 *>(Lc));
-        note_launches(1);
-    }
+    const int64_t npar = blk_parents_before(L), PP4 = C::PP / 4;
+    k_blk_finish<P><<<(unsigned)((npar * PP4 + 31) / 32), 256, 0, s>>>(
+        (int)npar, prm.ksplit, prm.part_stride / 4, begin, end,
+        reinterpret_cast<const float4 *>(prm.ksplit > 1 ? Lpart : Lc), reinterpret_cast<float4 *>(Lc));
+    note_launches(1);
     return 0;
 }
 
@@ -1072,19 +1263,17 @@ int launch_m2l_blk(int P, int L, const int32_t *begin, const int32_t *end, const
                    int max_ctas)
 {
     if (L < 2) return 0;
-    // p = 8, 10: four stages of 32-wide K chunks (64-byte swizzle) cover the TMA latency better
-    // than two of 64 (1M, p = 10: 0.343 against 0.372 ms); p = 4, 6 fit three 64-wide stages
     switch (P) {
-    case 4: return launch_blk_t<4, 64>(L, begin, end, presplit, pscale, table, Lc, Lpart, status, s, max_ctas);
-    case 6: return launch_blk_t<6, 64>(L, begin, end, presplit, pscale, table, Lc, Lpart, status, s, max_ctas);
-    case 8: return launch_blk_t<8, 32>(L, begin, end, presplit, pscale, table, Lc, Lpart, status, s, max_ctas);
-    case 10: return launch_blk_t<10, 32>(L, begin, end, presplit, pscale, table, Lc, Lpart, status, s, max_ctas);
+    case 4: return launch_blk_t<4, blk_ch(4)>(L, begin, end, presplit, pscale, table, Lc, Lpart, status, s, max_ctas);
+    case 6: return launch_blk_t<6, blk_ch(6)>(L, begin, end, presplit, pscale, table, Lc, Lpart, status, s, max_ctas);
+    case 8: return launch_blk_t<8, blk_ch(8)>(L, begin, end, presplit, pscale, table, Lc, Lpart, status, s, max_ctas);
+    case 10: return launch_blk_t<10, blk_ch(10)>(L, begin, end, presplit, pscale, table, Lc, Lpart, status, s, max_ctas);
     }
     return -1;
 }
 
 // ---- adaptive tree ----------------------------------------------------------------------------
-size_t m2l_ablk_presplit_bytes(int P, int64_t ucap) { return (size_t)(ucap + 1) * 2 * 8 * P * P * sizeof(__half); }
+size_t m2l_ablk_presplit_bytes(int P, int64_t ucap) { return (size_t)(ucap + 1) * 2 * blk_kw(P) * sizeof(__half); }
 
 int64_t m2l_ablk_tiles_units(int64_t ucap) { return (ucap + kBlkRows - 1) / kBlkRows * kBlkRows; }
 
@@ -1096,8 +1285,8 @@ size_t m2l_ablk_src_bytes(int64_t ucap) { return (size_t)m2l_ablk_tiles_units(uc
 // instance alone sum in the same order)
 int m2l_ablk_ksplit(int P, int64_t n, int leaf_size)
 {
-    const int nt = P == 4 ? BlkCfg<4, 64>::NTILES : P == 6 ? BlkCfg<6, 64>::NTILES : P == 8 ? BlkCfg<8, 32>::NTILES
-                                                                                            : BlkCfg<10, 32>::NTILES;
+    const int nt = P == 4 ? BlkCfg<4, blk_ch(4)>::NTILES : P == 6 ? BlkCfg<6, blk_ch(6)>::NTILES
+                 : P == 8 ? BlkCfg<8, blk_ch(8)>::NTILES : BlkCfg<10, blk_ch(10)>::NTILES;
     const int64_t units = n / (2 * (int64_t)(leaf_size > 0 ? leaf_size : 1)) + 1;
     return blk_ranges((units + kBlkRows - 1) / kBlkRows * nt);
 }
@@ -1115,10 +1304,10 @@ void launch_ablk_prep(int P, Span cells, int64_t ucap, const int32_t *level, con
     const unsigned gp = (unsigned)((ucap + 1 + 7) / 8);
     __half *A = static_cast<__half *>(Apre);
     switch (P) {
-    case 4: k_ablk_presplit<4><<<gp, 256, 0, s>>>(n_units, zrow, units, child_of, M, A, uscale); break;
-    case 6: k_ablk_presplit<6><<<gp, 256, 0, s>>>(n_units, zrow, units, child_of, M, A, uscale); break;
-    case 8: k_ablk_presplit<8><<<gp, 256, 0, s>>>(n_units, zrow, units, child_of, M, A, uscale); break;
-    case 10: k_ablk_presplit<10><<<gp, 256, 0, s>>>(n_units, zrow, units, child_of, M, A, uscale); break;
+    case 4: k_ablk_presplit<4, blk_ch(4)><<<gp, 256, 0, s>>>(n_units, zrow, units, child_of, M, A, uscale); break;
+    case 6: k_ablk_presplit<6, blk_ch(6)><<<gp, 256, 0, s>>>(n_units, zrow, units, child_of, M, A, uscale); break;
+    case 8: k_ablk_presplit<8, blk_ch(8)><<<gp, 256, 0, s>>>(n_units, zrow, units, child_of, M, A, uscale); break;
+    case 10: k_ablk_presplit<10, blk_ch(10)><<<gp, 256, 0, s>>>(n_units, zrow, units, child_of, M, A, uscale); break;
     }
     const int64_t up = m2l_ablk_tiles_units(ucap);
     k_ablk_src<<<(unsigned)((up * 26 + 255) / 256), 256, 0, s>>>(n_units, up, zrow, units, coll, unit_of, src);
@@ -1128,7 +1317,7 @@ void launch_ablk_prep(int P, Span cells, int64_t ucap, const int32_t *level, con
 template <int P, int CH>
 static int launch_ablk_t(int64_t ucap, const int32_t *n_units, const int32_t *units, const int32_t *child_of,
                          const int32_t *src, const void *Apre, const int8_t *uscale, const void *table, float *Lc,
-                         float *Lpart, int ksplit, int64_t part_stride, int *status, cudaStream_t s, int max_ctas)
+                         float *V, int ksplit, int *status, cudaStream_t s, int max_ctas)
 {
     using C = BlkCfg<P, CH>;
     constexpr CUtensorMapSwizzle kSw = CH == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
@@ -1136,11 +1325,11 @@ static int launch_ablk_t(int64_t ucap, const int32_t *n_units, const int32_t *un
     if (!enc) return -1;
     AblkParams prm;
     memset(&prm, 0, sizeof(prm));
-    const cuuint64_t KD = C::KD;
-    const int *gexp = reinterpret_cast<const int *>(static_cast<const __half *>(table) + 26 * 2 * KD * KD);
+    const cuuint64_t KD = C::KD, KW = C::KW;
+    const int *gexp = reinterpret_cast<const int *>(static_cast<const __half *>(table) + 26 * 2 * KD * KW);
     {
-        const cuuint64_t dims[4] = {KD, KD, 2, 26};
-        const cuuint64_t strides[3] = {KD * 2, KD * KD * 2, KD * KD * 4};
+        const cuuint64_t dims[4] = {KW, KD, 2, 26};
+        const cuuint64_t strides[3] = {KW * 2, KD * KW * 2, KD * KW * 4};
         const cuuint32_t box[4] = {(cuuint32_t)CH, (cuuint32_t)C::NT, 1, 1};
         const cuuint32_t es[4] = {1, 1, 1, 1};
         if (enc(&prm.tmB, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, const_cast<void *>(table), dims, strides, box, es,
@@ -1149,10 +1338,9 @@ static int launch_ablk_t(int64_t ucap, const int32_t *n_units, const int32_t *un
             return -1;
     }
     prm.ksplit = ksplit;
-    prm.part_stride = part_stride;
+    prm.part_stride = ucap * C::KD;
     prm.zrow = ucap;
-    if (ksplit > 1 && !Lpart) return -1;
-    auto kern = k_m2l_ablk<P, kBlkDrainsPerOffset, CH>;
+    auto kern = k_m2l_ablk<P, CH>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::kSmemBytes);
     const int64_t nctas64 = (ucap + kBlkRows - 1) / kBlkRows * C::NTILES * ksplit;
     const int nctas = (int)nctas64;
@@ -1160,56 +1348,35 @@ static int launch_ablk_t(int64_t ucap, const int32_t *n_units, const int32_t *un
     for (int t0 = 0; t0 < nctas; t0 += step) {
         prm.tile0 = t0;
         const int gsz = nctas - t0 < step ? nctas - t0 : step;
-        kern<<<gsz, kAblkThreads, C::kSmemBytes, s>>>(prm, n_units, units, child_of, src,
-                                                      static_cast<const __half *>(Apre), uscale, gexp, Lc, Lpart,
-                                                      status);
+        kern<<<gsz, kAblkThreads, C::kSmemBytes, s>>>(prm, n_units, src, static_cast<const __half *>(Apre), uscale,
+                                                      gexp, V, status);
         note_launches(1);
     }
+    const int64_t PP4 = C::PP / 4;
+    k_ablk_finish<P><<<(unsigned)((ucap * PP4 + 31) / 32), 256, 0, s>>>(
+        n_units, ksplit, prm.part_stride / 4, units, child_of, reinterpret_cast<const float4 *>(V),
+        reinterpret_cast<float4 *>(Lc));
+    note_launches(1);
     return 0;
+}
+
+size_t m2l_ablk_class_bytes(int P, int64_t ucap, int ksplit)
+{
+    return (size_t)ksplit * (size_t)ucap * 8 * P * P * sizeof(float);
 }
 
 int launch_m2l_ablk(int P, int64_t ucap, const int32_t *n_units, const int32_t *units, const int32_t *child_of,
                     const int32_t *src, const void *Apre, const int8_t *uscale, const void *table, float *Lc,
-                    float *Lpart, int ksplit, int64_t part_stride, int *status, cudaStream_t s, int max_ctas)
+                    float *V, int ksplit, int *status, cudaStream_t s, int max_ctas)
 {
     if (ucap <= 0) return 0;
     switch (P) {
-    case 4: return launch_ablk_t<4, 64>(ucap, n_units, units, child_of, src, Apre, uscale, table, Lc, Lpart, ksplit, part_stride, status, s, max_ctas);
-    case 6: return launch_ablk_t<6, 64>(ucap, n_units, units, child_of, src, Apre, uscale, table, Lc, Lpart, ksplit, part_stride, status, s, max_ctas);
-    case 8: return launch_ablk_t<8, 32>(ucap, n_units, units, child_of, src, Apre, uscale, table, Lc, Lpart, ksplit, part_stride, status, s, max_ctas);
-    case 10: return launch_ablk_t<10, 32>(ucap, n_units, units, child_of, src, Apre, uscale, table, Lc, Lpart, ksplit, part_stride, status, s, max_ctas);
+    case 4: return launch_ablk_t<4, blk_ch(4)>(ucap, n_units, units, child_of, src, Apre, uscale, table, Lc, V, ksplit, status, s, max_ctas);
+    case 6: return launch_ablk_t<6, blk_ch(6)>(ucap, n_units, units, child_of, src, Apre, uscale, table, Lc, V, ksplit, status, s, max_ctas);
+    case 8: return launch_ablk_t<8, blk_ch(8)>(ucap, n_units, units, child_of, src, Apre, uscale, table, Lc, V, ksplit, status, s, max_ctas);
+    case 10: return launch_ablk_t<10, blk_ch(10)>(ucap, n_units, units, child_of, src, Apre, uscale, table, Lc, V, ksplit, status, s, max_ctas);
     }
     return -1;
-}
-
-// Lc = the sum of the offset ranges' partial sums, in range order, over the cells of `deep`
-__global__ void __launch_bounds__(256) k_ablk_reduce(Span deep, int PP4, int ksplit, int64_t stride4,
-                                                     const float4 *__restrict__ part, float4 *__restrict__ Lc)
-{
-    const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (j >= span_count(deep) * PP4) return;
-    const int64_t i = span_first(deep) * PP4 + j;
-    float4 a = part[i];
-    for (int k = 1; k < ksplit; ++k) {
-        const float4 b = part[i + k * stride4];
-        a.x += b.x;
-        a.y += b.y;
-        a.z += b.z;
-        a.w += b.w;
-    }
-    Lc[i] = a;
-}
-
-void launch_ablk_reduce(int P, Span deep, int ksplit, int64_t part_stride, const float *Lpart, float *Lc,
-                        cudaStream_t s)
-{
-    const int64_t PP4 = (int64_t)P * P / 4;
-    const int64_t nthr = deep.cap * PP4;
-    if (nthr <= 0) return;
-    k_ablk_reduce<<<(unsigned)((nthr + 255) / 256), 256, 0, s>>>(deep, (int)PP4, ksplit, part_stride / 4,
-                                                                 reinterpret_cast<const float4 *>(Lpart),
-                                                                 reinterpret_cast<float4 *>(Lc));
-    note_launches(1);
 }
 
 }  // namespace gbfmm
