@@ -906,7 +906,7 @@ struct Ranges {
     }
     Span level(int l) const
     {
-        return dev ? Span{0, caps->level[l], info + l, info + l + 1, abort}
+        return dev ? Span{0, caps->level[l], info + l, info + l + 1, abort, caps->expect[l]}
                    : host_span((*ls)[l], (*ls)[l + 1] - (*ls)[l]);
     }
     // the cells of levels >= 2
@@ -973,8 +973,12 @@ int treecode_adaptive(gbfmm_ctx *ctx, AdaptiveState &A, const Ranges &R, const g
     if (deep) launch_p2m_cells(P, est_adaptive_leaves(n, leaf_size), A.leaves.as<int32_t>(), R.leaves(), A.level.as<int32_t>(), geom,
                                A.begin.as<int32_t>(), A.count.as<int32_t>(), A.sx.as<float4>(), M, s);
     mark(4);
-    for (int l = maxl - 1; l >= 2; --l)
-        launch_translate_cells(P, true, R.level(l), A.child_of.as<int32_t>(), A.nchild.as<int32_t>(), ops.m2m, M, s);
+    {
+        Span up[kAdaptMaxLevel];
+        int nl = 0;
+        for (int l = maxl - 1; l >= 2; --l) up[nl++] = R.level(l);
+        launch_translate_levels(P, true, up, nl, A.child_of.as<int32_t>(), A.nchild.as<int32_t>(), ops.m2m, M, s);
+    }
     mark(5);
     if (!deep)
         cudaMemsetAsync(far, 0, 16 * (size_t)n, s);
@@ -1348,8 +1352,12 @@ int evaluate_adaptive_in(gbfmm_ctx *ctx, AdaptiveState &A, const AdaptCaps *caps
     if (deep) launch_p2m_cells(P, est_adaptive_leaves(n, leaf_size), A.leaves.as<int32_t>(), R.leaves(), A.level.as<int32_t>(), geom,
                                A.begin.as<int32_t>(), A.count.as<int32_t>(), A.sx.as<float4>(), M, s);
     mark(4);
-    for (int l = maxl - 1; l >= 2; --l)
-        launch_translate_cells(P, true, R.level(l), A.child_of.as<int32_t>(), A.nchild.as<int32_t>(), ops.m2m, M, s);
+    {
+        Span up[kAdaptMaxLevel];
+        int nl = 0;
+        for (int l = maxl - 1; l >= 2; --l) up[nl++] = R.level(l);
+        launch_translate_levels(P, true, up, nl, A.child_of.as<int32_t>(), A.nchild.as<int32_t>(), ops.m2m, M, s);
+    }
     mark(5);
     if (deep && !cores && !gathered) {
         // M2L in block form: one GEMM per parent offset over the units (cells with children),
@@ -1418,9 +1426,12 @@ int evaluate_adaptive_in(gbfmm_ctx *ctx, AdaptiveState &A, const AdaptCaps *caps
                          A.loffs[kListX].as<uint32_t>(), A.lids[kListX].as<int32_t>(), A.sx.as<float4>(), Lc, s);
     }
     mark(6);
-    for (int l = 3; l <= maxl; ++l)
-        launch_translate_cells(P, false, R.level(l - 1), A.child_of.as<int32_t>(), A.nchild.as<int32_t>(), ops.l2l,
-                               Lc, s);
+    {
+        Span down[kAdaptMaxLevel];
+        int nl = 0;
+        for (int l = 3; l <= maxl; ++l) down[nl++] = R.level(l - 1);
+        launch_translate_levels(P, false, down, nl, A.child_of.as<int32_t>(), A.nchild.as<int32_t>(), ops.l2l, Lc, s);
+    }
     mark(7);
     // M2P into the far field, then L2P adds the local expansion's value and the
     // near-field sums (the same rounding as L2P then M2P: one addition each)

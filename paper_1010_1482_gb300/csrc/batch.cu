@@ -41,8 +41,8 @@ size_t align256(size_t b) { return (b + 255) / 256 * 256; }
 // 119 against 237 cells for two samples of 3981 Plummer particles at leaf size 256), moves cells
 // between levels and may reach a few levels deeper; so the cells and leaves get twice the count
 // plus a constant, and every level down to three below the deepest may hold as many cells as
-// the whole tree (the per-level launches cover the whole capacity, their CTAs past the level's
-// cells idle).  The lists grow with the cells, and by more than the cells on small trees (their
+// the whole tree (runs of small levels share a launch that loops over what there is; a large
+// level's launch covers the whole capacity, its CTAs past the level's cells idle).  The lists grow with the cells, and by more than the cells on small trees (their
 // rows fill as the tree deepens): the V rows are bounded by 189 per cell, the others take their
 // entries per cell times the cell capacity, with half again as margin.
 AdaptCaps with_margin(const AdaptCaps &c)
@@ -57,7 +57,10 @@ AdaptCaps with_margin(const AdaptCaps &c)
     r.leaves = 2 * c.leaves + 64;
     r.units = 2 * (c.cells - c.leaves) + 64;
     r.maxl = std::min(gbfmm::kAdaptiveMaxLevel, c.maxl + 3);
-    for (int l = 0; l <= gbfmm::kAdaptiveMaxLevel; ++l) r.level[l] = l <= r.maxl ? r.cells : 0;
+    for (int l = 0; l <= gbfmm::kAdaptiveMaxLevel; ++l) {
+        r.level[l] = l <= r.maxl ? r.cells : 0;
+        r.expect[l] = c.level[l];
+    }
     for (int k = 0; k < 4; ++k) r.list[k] = k == 1 ? 189 * r.cells : per_cell(c.list[k], r.cells);
     for (int j = 0; j < 2; ++j) r.chain[j] = per_cell(c.chain[j], r.cells);
     return r;

@@ -142,10 +142,13 @@ constexpr int kStatusCapacity = 4;  // a captured adaptive evaluation outgrew it
 // The items one launch covers.  The grid spans `cap` items; the kernel takes count() of them,
 // starting at first().  With no device pointers this is [lo, lo + cap) as launched (counts the
 // host knows); with them, the range [*dlo, *dhi) is read on the device and clamped to cap, and
-// it is empty once *abort is nonzero (counts only the device knows: captured evaluations).
+// it is empty once *abort is nonzero (counts only the device knows: captured evaluations).  expect,
+// if set, is the count to choose a kernel by (every kernel covers cap whatever it is).
 struct Span {
     int64_t lo = 0, cap = 0;
     const int32_t *dlo = nullptr, *dhi = nullptr, *abort = nullptr;
+    int64_t expect = -1;
+    int64_t likely() const { return expect >= 0 ? expect : cap; }
 };
 inline Span host_span(int64_t lo, int64_t n) { return Span{lo, n < 0 ? 0 : n, nullptr, nullptr, nullptr}; }
 GB_DEV int64_t span_first(const Span &s) { return s.dlo ? (int64_t)*s.dlo : s.lo; }
@@ -437,8 +440,9 @@ void launch_p2m_cells(int P, int64_t est_leaves, const int32_t *leaves, Span lv,
 // leaves of an adaptive tree hold about 0.3 leaf_size particles
 inline int64_t est_adaptive_leaves(int64_t n, int leaf_size) { return 3 * n / (leaf_size > 0 ? leaf_size : 1); }
 // parents: the cells whose children are translated (M2M up into them, L2L down from them)
-void launch_translate_cells(int P, bool up, Span parents, const int32_t *child_of, const int32_t *nchild,
-                            const float *ops, float *X, cudaStream_t s);
+// one level, or the levels parents[0 .. n) one after another (upward: each after the level below it)
+void launch_translate_levels(int P, bool up, const Span *parents, int n, const int32_t *child_of,
+                             const int32_t *nchild, const float *ops, float *X, cudaStream_t s);
 // tile lists (tdesc: level, child position, first target in tlist, target count): tiles with a
 // count of 0 are empty and return at once
 void launch_m2l_tiles(int P, const int4 *tdesc, int ntiles, const int32_t *tlist, const int32_t *begin,

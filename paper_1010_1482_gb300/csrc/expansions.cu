@@ -19,6 +19,7 @@
 // dense p^2 x p^2 FP32 matrix computed once per order in FP64.
 #include "common.cuh"
 
+#include <cooperative_groups.h>
 #include <math.h>
 #include <string.h>
 
@@ -775,8 +776,7 @@ struct TransSmall {
     static constexpr int RGS = (NRG + SL - 1) / SL;         // row groups of a slice
     static constexpr int GT = RGS * NCG, NT = 8 * GT;       // threads of a child position, of the CTA
     static constexpr int LDA = 4 * RGS;
-    static constexpr size_t kSmem = sizeof(float) * 8 * ((size_t)PP * LDA + (size_t)TN * SB);
-    static_assert(NT * CN * 4 <= 8 * PP * LDA, "the child sums reuse the operators' space");
+    static constexpr size_t kSmem = sizeof(float) * (8 * ((size_t)PP * LDA + (size_t)TN * SB) + (size_t)NT * CN * 4);
 };
 
 struct LevelCells {  // uniform tree: parents of level l, children of level l + 1
@@ -809,63 +809,65 @@ __global__ void __launch_bounds__(TransSmall<P>::NT) k_m2m_small(Cells cells, co
     constexpr int GT = Cfg::GT, LDA = Cfg::LDA, RGS = Cfg::RGS, NRG = Cfg::NRG;
     extern __shared__ __align__(16) float tsm[];
     __shared__ int64_t s_par[TN], s_child[8][TN];
-    const int64_t q0 = blockIdx.x * (int64_t)TN, np = cells.np();
-    if (q0 >= np) return;
+    const int64_t np = cells.np();
+    if (blockIdx.x * (int64_t)TN >= np) return;
     const int tid = threadIdx.x, rg0 = blockIdx.y * RGS, rg1 = min(rg0 + RGS, NRG);
     // the columns k that rows of degree d read: those of degrees <= d
     auto k_end = [](int r) { const int d = degree_of(min(r, PP - 1)); return min(PP, ((d + 1) * (d + 1) + 3) / 4 * 4); };
     const int ke = k_end(4 * rg1 - 1);
-    float *B = tsm + 8 * PP * LDA;
+    float *B = tsm + 8 * PP * LDA, *red = B + 8 * TN * SB;
     for (int e = tid; e < 8 * PP * RGS; e += Cfg::NT) {
         const int r = e % RGS, k = (e / RGS) % PP, c = e / (RGS * PP);
         if (k < ke && rg0 + r < rg1)
             cp_async16_t(tsm + (c * PP + k) * LDA + 4 * r, ops + ((size_t)c * PP + k) * PR + 4 * (rg0 + r), 16u);
     }
-    for (int e = tid; e < 9 * TN; e += Cfg::NT) {
-        const int i = e % TN, c = e / TN - 1;
-        const int64_t g = q0 + i >= np ? -1 : c < 0 ? cells.parent(q0 + i) : cells.child(q0 + i, c);
-        (c < 0 ? s_par[i] : s_child[c][i]) = g;
-    }
-    __syncthreads();
-    for (int e = tid; e < 8 * TN * (PP / 4); e += Cfg::NT) {
-        const int k = 4 * (e % (PP / 4)), i = (e / (PP / 4)) % TN, c = e / (PP / 4 * TN);
-        const int64_t g = s_child[c][i];
-        if (k < ke) cp_async16_t(B + (c * TN + i) * SB + k, g >= 0 ? M + g * PP + k : M, g >= 0 ? 16u : 0u);
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    __syncthreads();
-    const int c = tid / GT, t = tid % GT, cg = t % NCG, rl = t / NCG, rg = rg0 + rl;
-    float acc[4][CN];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < CN; ++j) acc[i][j] = 0.f;
-    if (rg < rg1) {
-        const int kn = k_end(4 * rg + 3);
-        const float *Ar = tsm + c * PP * LDA + 4 * rl, *Bc = B + (c * TN + cg) * SB;
-#pragma unroll 2
-        for (int k = 0; k < kn; k += 4) {
-            Frag<CN, 4> f;
-            f.load(Ar, Bc, k, LDA, NCG * SB);
-            f.fma(acc);
+    for (int64_t q0 = blockIdx.x * (int64_t)TN; q0 < np; q0 += (int64_t)gridDim.x * TN) {
+        for (int e = tid; e < 9 * TN; e += Cfg::NT) {
+            const int i = e % TN, c = e / TN - 1;
+            const int64_t g = q0 + i >= np ? -1 : c < 0 ? cells.parent(q0 + i) : cells.child(q0 + i, c);
+            (c < 0 ? s_par[i] : s_child[c][i]) = g;
         }
-    }
-    __syncthreads();
+        __syncthreads();
+        for (int e = tid; e < 8 * TN * (PP / 4); e += Cfg::NT) {
+            const int k = 4 * (e % (PP / 4)), i = (e / (PP / 4)) % TN, c = e / (PP / 4 * TN);
+            const int64_t g = s_child[c][i];
+            if (k < ke) cp_async16_t(B + (c * TN + i) * SB + k, g >= 0 ? M + g * PP + k : M, g >= 0 ? 16u : 0u);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
+        const int c = tid / GT, t = tid % GT, cg = t % NCG, rl = t / NCG, rg = rg0 + rl;
+        float acc[4][CN];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < CN; ++j) tsm[(i * CN + j) * Cfg::NT + tid] = acc[i][j];
-    __syncthreads();
-    for (int e = tid; e < 4 * CN * GT; e += Cfg::NT) {
-        const int i = e % 4, tt = (e / 4) % GT, j = e / (4 * GT);
-        const int r = 4 * (rg0 + tt / NCG) + i;
-        const int64_t g = s_par[tt % NCG + j * NCG];
-        if (g < 0 || rg0 + tt / NCG >= rg1 || r >= PP) continue;
-        float v = 0.f;
+            for (int j = 0; j < CN; ++j) acc[i][j] = 0.f;
+        if (rg < rg1) {
+            const int kn = k_end(4 * rg + 3);
+            const float *Ar = tsm + c * PP * LDA + 4 * rl, *Bc = B + (c * TN + cg) * SB;
+#pragma unroll 2
+            for (int k = 0; k < kn; k += 4) {
+                Frag<CN, 4> f;
+                f.load(Ar, Bc, k, LDA, NCG * SB);
+                f.fma(acc);
+            }
+        }
 #pragma unroll
-        for (int k = 0; k < 8; ++k) v += tsm[(i * CN + j) * Cfg::NT + k * GT + tt];
-        M[g * PP + r] = v;
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < CN; ++j) red[(i * CN + j) * Cfg::NT + tid] = acc[i][j];
+        __syncthreads();
+        for (int e = tid; e < 4 * CN * GT; e += Cfg::NT) {
+            const int i = e % 4, tt = (e / 4) % GT, j = e / (4 * GT);
+            const int r = 4 * (rg0 + tt / NCG) + i;
+            const int64_t g = s_par[tt % NCG + j * NCG];
+            if (g < 0 || rg0 + tt / NCG >= rg1 || r >= PP) continue;
+            float v = 0.f;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v += red[(i * CN + j) * Cfg::NT + k * GT + tt];
+            M[g * PP + r] = v;
+        }
+        __syncthreads();  // the columns and the sums are read: the next parents may be staged
     }
 }
 
@@ -1715,16 +1717,16 @@ static void translate_cells_tn(Span par, const int32_t *child_of, const int32_t 
 }
 
 // the cells-per-CTA choice of the uniform tree's translations (launch_translate_t), on the
-// launch's capacity
+// expected count
 template <int P, bool UP>
 static void translate_cells_t(Span par, const int32_t *child_of, const int32_t *nchild, const float *ops, float *X,
                               cudaStream_t s)
 {
     if constexpr (UP)
-        if (launch_m2m_small<P>(par.cap, SpanCells{par, child_of, nchild}, ops, X, s)) return;
-    const int64_t ctas32 = (par.cap + 31) / 32 * (UP ? 1 : 8), ctas64 = (par.cap + 63) / 64 * (UP ? 1 : 8);
+        if (launch_m2m_small<P>(std::max<int64_t>(par.likely(), 1), SpanCells{par, child_of, nchild}, ops, X, s)) return;
+    const int64_t np = par.likely(), ctas32 = (np + 31) / 32 * (UP ? 1 : 8), ctas64 = (np + 63) / 64 * (UP ? 1 : 8);
     if constexpr (UP) {  // large levels: 128 (upward) or 64 cells per CTA share each staged operator
-        if ((par.cap + 127) / 128 >= 4 * 152) return translate_cells_tn<P, UP, 128, 8>(par, child_of, nchild, ops, X, s);
+        if ((np + 127) / 128 >= 4 * 152) return translate_cells_tn<P, UP, 128, 8>(par, child_of, nchild, ops, X, s);
     }
     if (ctas64 >= 4 * 152)
         translate_cells_tn<P, UP, 64, 8>(par, child_of, nchild, ops, X, s);
@@ -1734,14 +1736,146 @@ static void translate_cells_t(Span par, const int32_t *child_of, const int32_t *
         translate_cells_tn<P, UP, 16, 2>(par, child_of, nchild, ops, X, s);
 }
 
-void launch_translate_cells(int P, bool up, Span parents, const int32_t *child_of, const int32_t *nchild,
-                            const float *ops, float *X, cudaStream_t s)
+// ---- several small levels in one launch ---------------------------------------------------------
+// A tree of 20,000 particles has six levels of 50 to 500 parents, each a launch of 5 us up and 5 us
+// down for a microsecond of work.  One cluster of 8 CTAs takes a run of such levels: a CTA keeps its
+// row slice of the eight operators in shared memory throughout, takes every (8 / SL)-th eight
+// parents of a level, and a cluster barrier parts the levels.  Each sum is formed as in
+// k_m2m_small and k_translate_cells.  20,011 Plummer particles, p = 4: the four top levels 19 -> 15.5 us
+// up and 21 -> 16.5 down, the step 346 -> 332; a captured batch of 96 instances, whose launches cover
+// three levels more than there are, 6.62 -> 6.28 ms.
+constexpr int kChainCtas = 8;
+struct ChainLevels {
+    Span s[kGeoLevels];
+    int n;
+};
+
+template <int P, bool UP>
+__global__ void __cluster_dims__(kChainCtas, 1, 1) __launch_bounds__(TransSmall<P>::NT)
+    k_translate_chain(const __grid_constant__ ChainLevels lv, const int32_t *__restrict__ child_of,
+                      const int32_t *__restrict__ nchild, const float *__restrict__ ops, float *X)
 {
-    if (parents.cap <= 0) return;
+    using Cfg = TransSmall<P>;
+    constexpr int PP = Cfg::PP, PR = Cfg::PR, SB = Cfg::SB, TN = Cfg::TN, GT = Cfg::GT, LDA = Cfg::LDA;
+    constexpr int RGS = Cfg::RGS, NRG = Cfg::NRG, SL = Cfg::SL, PER = kChainCtas / SL;
+    static_assert(Cfg::CN == 1 && Cfg::NCG == TN, "a thread holds one parent's four rows");
+    namespace cg = cooperative_groups;
+    const cg::cluster_group cl = cg::this_cluster();
+    extern __shared__ __align__(16) float tsm[];
+    __shared__ int64_t s_par[TN], s_child[8][TN];
+    const int rank = (int)cl.block_rank(), tid = threadIdx.x;
+    const int rg0 = (rank % SL) * RGS, rg1 = min(rg0 + RGS, NRG);
+    auto k_end = [](int r) { const int d = degree_of(min(r, PP - 1)); return min(PP, ((d + 1) * (d + 1) + 3) / 4 * 4); };
+    auto k_beg = [](int r) { const int d = degree_of(min(r, PP - 1)); return (d * d) / 4 * 4; };
+    const int ks = UP ? 0 : k_beg(4 * rg0), ke = UP ? k_end(4 * rg1 - 1) : PP;  // the columns the slice reads
+    float *B = tsm + 8 * PP * LDA, *red = B + 8 * TN * SB;
+    const bool active = rank < SL * PER;
+    if (active) {
+        for (int e = tid; e < 8 * PP * RGS; e += Cfg::NT) {
+            const int r = e % RGS, k = (e / RGS) % PP, c = e / (RGS * PP);
+            if (k >= ks && k < ke && rg0 + r < rg1)
+                cp_async16_t(tsm + (c * PP + k) * LDA + 4 * r, ops + ((size_t)c * PP + k) * PR + 4 * (rg0 + r), 16u);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    const int c = tid / GT, t = tid % GT, col = t % TN, rl = t / TN, rg = rg0 + rl;
+    const int kb = UP ? 0 : k_beg(4 * rg), kn = UP ? k_end(4 * rg + 3) : PP;
+    for (int li = 0; li < lv.n; ++li) {
+        const int64_t np = span_count(lv.s[li]), lo = span_first(lv.s[li]);
+        for (int64_t q0 = (int64_t)(rank / SL) * TN; active && q0 < np; q0 += (int64_t)PER * TN) {
+            for (int e = tid; e < 9 * TN; e += Cfg::NT) {
+                const int i = e % TN, ch = e / TN - 1;
+                int64_t g = -1;
+                if (q0 + i < np) g = ch >= 0 ? child_of[(lo + q0 + i) * 8 + ch] : nchild[lo + q0 + i] != 0 ? lo + q0 + i : -1;
+                (ch < 0 ? s_par[i] : s_child[ch][i]) = g;
+            }
+            __syncthreads();
+            for (int e = tid; e < (UP ? 8 : 1) * TN * (PP / 4); e += Cfg::NT) {
+                const int k = 4 * (e % (PP / 4)), i = (e / (PP / 4)) % TN, ch = e / (PP / 4 * TN);
+                const int64_t g = UP ? s_child[ch][i] : s_par[i];
+                if (k >= ks && k < ke) cp_async16_t(B + (ch * TN + i) * SB + k, g >= 0 ? X + g * PP + k : X, g >= 0 ? 16u : 0u);
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            __syncthreads();
+            float acc[4][1] = {{0.f}, {0.f}, {0.f}, {0.f}};
+            if (rg < rg1) {
+                const float *Ar = tsm + c * PP * LDA + 4 * rl, *Bc = B + ((UP ? c * TN : 0) + col) * SB;
+#pragma unroll 2
+                for (int k = kb; k < kn; k += 4) {
+                    Frag<1, 4> f;
+                    f.load(Ar, Bc, k, LDA, 0);
+                    f.fma(acc);
+                }
+            }
+            if (UP) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) red[i * Cfg::NT + tid] = acc[i][0];
+                __syncthreads();
+                for (int e = tid; e < 4 * GT; e += Cfg::NT) {
+                    const int i = e % 4, tt = e / 4, r = 4 * (rg0 + tt / TN) + i;
+                    const int64_t g = s_par[tt % TN];
+                    if (g < 0 || rg0 + tt / TN >= rg1 || r >= PP) continue;
+                    float v = 0.f;
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) v += red[i * Cfg::NT + k * GT + tt];
+                    X[g * PP + r] = v;
+                }
+            } else if (rg < rg1 && 4 * rg < PP && s_child[c][col] >= 0) {
+                float4 *dst = reinterpret_cast<float4 *>(X + s_child[c][col] * PP + 4 * rg);
+                float4 v = *dst;
+                v.x += acc[0][0];
+                v.y += acc[1][0];
+                v.z += acc[2][0];
+                v.w += acc[3][0];
+                *dst = v;
+            }
+            __syncthreads();  // the columns and the sums are read: the next parents may be staged
+        }
+        __threadfence();
+        cl.sync();  // the level is written before the next one's columns are read (cp.async.cg: from L2)
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");  // a CTA that had no parents: its operators
+}
+
+// levels of up to this many parents may share a launch: four rounds of eight parents a CTA
+template <int P>
+static constexpr int64_t chain_parents()
+{
+    return 4 * TransSmall<P>::TN * (kChainCtas / TransSmall<P>::SL);
+}
+
+template <int P, bool UP>
+static void translate_levels_t(const Span *par, int n, const int32_t *child_of, const int32_t *nchild,
+                               const float *ops, float *X, cudaStream_t s)
+{
+    for (int i = 0; i < n;) {
+        ChainLevels lv;
+        lv.n = 0;
+        while (i + lv.n < n && par[i + lv.n].likely() <= chain_parents<P>()) {
+            lv.s[lv.n] = par[i + lv.n];
+            ++lv.n;
+        }
+        if (lv.n >= 2) {
+            constexpr int smem = (int)TransSmall<P>::kSmem;
+            cudaFuncSetAttribute(k_translate_chain<P, UP>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            k_translate_chain<P, UP><<<kChainCtas, TransSmall<P>::NT, smem, s>>>(lv, child_of, nchild, ops, X);
+            note_launches(1);
+            i += lv.n;
+        } else {
+            if (par[i].cap > 0) translate_cells_t<P, UP>(par[i], child_of, nchild, ops, X, s);
+            ++i;
+        }
+    }
+}
+
+void launch_translate_levels(int P, bool up, const Span *parents, int n, const int32_t *child_of,
+                             const int32_t *nchild, const float *ops, float *X, cudaStream_t s)
+{
     if (up) {
-        GBFMM_DISPATCH_P(P, (translate_cells_t<PQ, true>(parents, child_of, nchild, ops, X, s)));
+        GBFMM_DISPATCH_P(P, (translate_levels_t<PQ, true>(parents, n, child_of, nchild, ops, X, s)));
     } else {
-        GBFMM_DISPATCH_P(P, (translate_cells_t<PQ, false>(parents, child_of, nchild, ops, X, s)));
+        GBFMM_DISPATCH_P(P, (translate_levels_t<PQ, false>(parents, n, child_of, nchild, ops, X, s)));
     }
 }
 #undef GBFMM_DISPATCH_P
