@@ -284,7 +284,7 @@ int gbfmm_create(gbfmm_ctx **out, int device)
         ok = cudaDeviceGetStreamPriorityRange(&least, &greatest) == cudaSuccess &&
              cudaStreamCreateWithPriority(&ctx->s_far, cudaStreamNonBlocking, greatest) == cudaSuccess &&
              cudaStreamCreateWithPriority(&ctx->s_near, cudaStreamNonBlocking, least) == cudaSuccess;
-        for (cudaEvent_t *e : {&ctx->ev_fork, &ctx->ev_near, &ctx->ev_join})
+        for (cudaEvent_t *e : {&ctx->ev_fork, &ctx->ev_near, &ctx->ev_join, &ctx->ev_m2m})
             ok = ok && cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess;
     }
     if (ok) {
@@ -326,7 +326,7 @@ int gbfmm_destroy(gbfmm_ctx *ctx)
     free_adaptive(ctx->ad);
     for (int i = 0; i <= kStages; ++i)
         if (ctx->ev[i]) cudaEventDestroy(ctx->ev[i]);
-    for (cudaEvent_t e : {ctx->ev_fork, ctx->ev_near, ctx->ev_join, ctx->ev_aux[0], ctx->ev_aux[1], ctx->ev_aux[2]})
+    for (cudaEvent_t e : {ctx->ev_fork, ctx->ev_near, ctx->ev_join, ctx->ev_m2m, ctx->ev_aux[0], ctx->ev_aux[1], ctx->ev_aux[2]})
         if (e) cudaEventDestroy(e);
     if (ctx->s_far) cudaStreamDestroy(ctx->s_far);
     if (ctx->s_near) cudaStreamDestroy(ctx->s_near);

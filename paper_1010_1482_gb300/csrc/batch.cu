@@ -41,8 +41,7 @@ size_t align256(size_t b) { return (b + 255) / 256 * 256; }
 // 119 against 237 cells for two samples of 3981 Plummer particles at leaf size 256), moves cells
 // between levels and may reach a few levels deeper; so the cells and leaves get twice the count
 // plus a constant, and every level down to three below the deepest may hold as many cells as
-// the whole tree (runs of small levels share a launch that loops over what there is; a large
-// level's launch covers the whole capacity, its CTAs past the level's cells idle).  The lists grow with the cells, and by more than the cells on small trees (their
+// the whole tree (the per-level launches are sized by the counts and loop over what there is).  The lists grow with the cells, and by more than the cells on small trees (their
 // rows fill as the tree deepens): the V rows are bounded by 189 per cell, the others take their
 // entries per cell times the cell capacity, with half again as margin.
 AdaptCaps with_margin(const AdaptCaps &c)

@@ -107,7 +107,7 @@ struct gbfmm_ctx {
     // the near field runs beside the far field: P2P on s_near (lowest priority), M2L .. L2P on
     // s_far (highest), forked from and joined into the caller's stream by events
     cudaStream_t s_far = nullptr, s_near = nullptr;
-    cudaEvent_t ev_fork = nullptr, ev_near = nullptr, ev_join = nullptr;
+    cudaEvent_t ev_fork = nullptr, ev_near = nullptr, ev_join = nullptr, ev_m2m = nullptr;
     cudaEvent_t ev_aux[3] = {};
     bool ops_built_last = false;
     int64_t launches_last = 0;

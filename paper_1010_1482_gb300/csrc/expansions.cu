@@ -1534,7 +1534,9 @@ __global__ void __launch_bounds__(128) k_l2p_cells(int64_t n, const int32_t *__r
 // As k_translate: the operator of each child position and the TN source columns are copied into
 // shared memory with cp.async (zero-filled for missing children), the next child position's
 // copies in flight while the current one is applied.
-template <int P, bool UP, int TN, int CN>
+// LOOP: the CTAs take TN parents after TN (a captured level, whose count only the device knows: a
+// launch over its whole capacity, most of it idle, cost a batch of 96 instances 3%).
+template <int P, bool UP, int TN, int CN, bool LOOP>
 __global__ void __launch_bounds__(TransCfg<P, UP, TN, CN>::NT) k_translate_cells(Span par,
                                                                          const int32_t *__restrict__ child_of,
                                                                          const int32_t *__restrict__ nchild,
@@ -1544,7 +1546,7 @@ __global__ void __launch_bounds__(TransCfg<P, UP, TN, CN>::NT) k_translate_cells
     using Cfg = TransCfg<P, UP, TN, CN>;
     constexpr int PP = Cfg::PP, PR = Cfg::PR, SB = Cfg::SB, NCG = Cfg::NCG, NRG = Cfg::NRG;
     extern __shared__ __align__(16) float tsm[];
-    const int64_t q0 = blockIdx.x * (int64_t)TN;
+    int64_t q0 = blockIdx.x * (int64_t)TN;
     const int64_t lo = span_first(par), np = span_count(par);
     if (q0 >= np) return;  // the whole CTA: beyond the parents
     const int tid = threadIdx.x;
@@ -1583,71 +1585,75 @@ __global__ void __launch_bounds__(TransCfg<P, UP, TN, CN>::NT) k_translate_cells
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    float tot[4][CN];  // M2M: the child positions' sums, added in order (as k_m2m_small adds them)
+    do {
+        float tot[4][CN];  // M2M: the child positions' sums, added in order (as k_m2m_small adds them)
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < CN; ++j) tot[i][j] = 0.f;
-    const int c_first = UP ? 0 : blockIdx.y, c_last = UP ? 7 : blockIdx.y;
-    stage(c_first, 0);
-    for (int c = c_first; c <= c_last; ++c) {
-        const int buf = UP ? (c - c_first) & 1 : 0;
-        if (c < c_last) {
-            stage(c + 1, buf ^ 1);
-            asm volatile("cp.async.wait_group 1;" ::: "memory");
-        } else {
-            asm volatile("cp.async.wait_group 0;" ::: "memory");
-        }
-        __syncthreads();
-        if (work) {
-            const float *Ar = tsm + buf * (Cfg::AF + Cfg::BF) + rg * 4;
-            const float *Bc = tsm + buf * (Cfg::AF + Cfg::BF) + Cfg::AF + cg * SB;
-            float acc[4][CN];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < CN; ++j) acc[i][j] = 0.f;
-#pragma unroll 2
-            for (int k = kbeg; k < kend; k += 4) {
-                Frag<CN, 4> f;
-                f.load(Ar, Bc, k, PR, NCG * SB);
-                f.fma(acc);
+            for (int j = 0; j < CN; ++j) tot[i][j] = 0.f;
+        const int c_first = UP ? 0 : blockIdx.y, c_last = UP ? 7 : blockIdx.y;
+        stage(c_first, 0);
+        for (int c = c_first; c <= c_last; ++c) {
+            const int buf = UP ? (c - c_first) & 1 : 0;
+            if (c < c_last) {
+                stage(c + 1, buf ^ 1);
+                asm volatile("cp.async.wait_group 1;" ::: "memory");
+            } else {
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
             }
+            __syncthreads();
+            if (work) {
+                const float *Ar = tsm + buf * (Cfg::AF + Cfg::BF) + rg * 4;
+                const float *Bc = tsm + buf * (Cfg::AF + Cfg::BF) + Cfg::AF + cg * SB;
+                float acc[4][CN];
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+                for (int i = 0; i < 4; ++i)
 #pragma unroll
-                for (int j = 0; j < CN; ++j) tot[i][j] += acc[i][j];
-        }
-        __syncthreads();  // the buffer is refilled two positions later
-    }
-    if (!work) return;
+                    for (int j = 0; j < CN; ++j) acc[i][j] = 0.f;
+#pragma unroll 2
+                for (int k = kbeg; k < kend; k += 4) {
+                    Frag<CN, 4> f;
+                    f.load(Ar, Bc, k, PR, NCG * SB);
+                    f.fma(acc);
+                }
 #pragma unroll
-    for (int j = 0; j < CN; ++j) {
-        const int64_t q = q0 + cg + j * NCG;
-        if (q >= np) continue;
-        const int r = rg * 4;
-        if (r >= PP) continue;
-        const int64_t pcell = lo + q;
-        int64_t g;
-        if (UP) {
-            if (nchild[pcell] == 0) continue;  // a leaf keeps its P2M expansion
-            g = pcell;
-        } else {
-            g = child_of[pcell * 8 + blockIdx.y];
-            if (g < 0) continue;
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int j = 0; j < CN; ++j) tot[i][j] += acc[i][j];
+            }
+            __syncthreads();  // the buffer is refilled two positions later
         }
-        float4 *dst = reinterpret_cast<float4 *>(X + g * PP + r);
-        if (UP) {
-            *dst = make_float4(tot[0][j], tot[1][j], tot[2][j], tot[3][j]);
-        } else {
-            float4 v = *dst;
-            v.x += tot[0][j];
-            v.y += tot[1][j];
-            v.z += tot[2][j];
-            v.w += tot[3][j];
-            *dst = v;
+        if (work) {
+#pragma unroll
+            for (int j = 0; j < CN; ++j) {
+                const int64_t q = q0 + cg + j * NCG;
+                if (q >= np) continue;
+                const int r = rg * 4;
+                if (r >= PP) continue;
+                const int64_t pcell = lo + q;
+                int64_t g;
+                if (UP) {
+                    if (nchild[pcell] == 0) continue;  // a leaf keeps its P2M expansion
+                    g = pcell;
+                } else {
+                    g = child_of[pcell * 8 + blockIdx.y];
+                    if (g < 0) continue;
+                }
+                float4 *dst = reinterpret_cast<float4 *>(X + g * PP + r);
+                if (UP) {
+                    *dst = make_float4(tot[0][j], tot[1][j], tot[2][j], tot[3][j]);
+                } else {
+                    float4 v = *dst;
+                    v.x += tot[0][j];
+                    v.y += tot[1][j];
+                    v.z += tot[2][j];
+                    v.w += tot[3][j];
+                    *dst = v;
+                }
+            }
         }
-    }
+        q0 += (int64_t)gridDim.x * TN;
+    } while (LOOP && q0 < np);
 }
 
 void launch_p2m_cells(int P, int64_t est_leaves, const int32_t *leaves, Span lv, const int32_t *level,
@@ -1704,15 +1710,16 @@ void launch_m2p_cells(int P, const int32_t *leaves, Span lv, const float4 *geom,
                                                  s)));
 }
 
-template <int P, bool UP, int TN, int CN>
+template <int P, bool UP, int TN, int CN, bool LOOP = false>
 static void translate_cells_tn(Span par, const int32_t *child_of, const int32_t *nchild, const float *ops, float *X,
                                cudaStream_t s)
 {
     using Cfg = TransCfg<P, UP, TN, CN>;
     const int smem = (int)Cfg::kSmem;  // operator + column block, double-buffered for M2M
-    cudaFuncSetAttribute(k_translate_cells<P, UP, TN, CN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    dim3 grid((unsigned)((par.cap + TN - 1) / TN), UP ? 1 : 8);
-    k_translate_cells<P, UP, TN, CN><<<grid, Cfg::NT, smem, s>>>(par, child_of, nchild, ops, X);
+    cudaFuncSetAttribute(k_translate_cells<P, UP, TN, CN, LOOP>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    const int64_t items = LOOP ? std::max<int64_t>(1, par.likely()) : par.cap;
+    dim3 grid((unsigned)((items + TN - 1) / TN), UP ? 1 : 8);
+    k_translate_cells<P, UP, TN, CN, LOOP><<<grid, Cfg::NT, smem, s>>>(par, child_of, nchild, ops, X);
     note_launches(1);
 }
 
@@ -1724,7 +1731,8 @@ static void translate_cells_t(Span par, const int32_t *child_of, const int32_t *
 {
     if constexpr (UP)
         if (launch_m2m_small<P>(std::max<int64_t>(par.likely(), 1), SpanCells{par, child_of, nchild}, ops, X, s)) return;
-    const int64_t np = par.likely(), ctas32 = (np + 31) / 32 * (UP ? 1 : 8), ctas64 = (np + 63) / 64 * (UP ? 1 : 8);
+    if (par.expect >= 0) return translate_cells_tn<P, UP, 16, 2, true>(par, child_of, nchild, ops, X, s);
+    const int64_t np = par.cap, ctas32 = (np + 31) / 32 * (UP ? 1 : 8), ctas64 = (np + 63) / 64 * (UP ? 1 : 8);
     if constexpr (UP) {  // large levels: 128 (upward) or 64 cells per CTA share each staged operator
         if ((np + 127) / 128 >= 4 * 152) return translate_cells_tn<P, UP, 128, 8>(par, child_of, nchild, ops, X, s);
     }
