@@ -73,7 +73,11 @@ GB_DEV void pair2(uint64_t nx, uint64_t ny, uint64_t nz, float4 s, uint64_t eps2
 // a one-warp reduction -> packed pairs, the reduction over all threads and stages of equal size:
 // 1M particles (mean 32 per leaf) 522 -> 493 us, 5M (19 per leaf) 1852 -> 1648, 400,009 Plummer
 // 222 -> 190; 16M Plummer step 26.76 -> 25.61 ms.
-constexpr int kP2PCap = 512;
+// Sources per stage: the most that leaves room for 8 CTAs per SM (5M uniform, 19 per leaf, about 515
+// sources a leaf: 512 a stage gave half the leaves a second stage, step 2705 -> 2672 us; 1M 1002 -> 993).
+// The loop unrolled by 4: by 3, 2, 8 the 1M step took 1146, 1155, 1107 us; 9 CTAs of 40 registers were
+// faster at 1M (986) and slower at 5M (2753), 6 of 64 slower (1131, 3204), as were 96 or 192 consumers.
+constexpr int kP2PCap = 576;
 constexpr int kP2PConsumers = 128;
 constexpr int kP2PWsThreads = kP2PConsumers + 32;
 constexpr int kP2PTargets = 2 * kP2PConsumers;  // targets per pass over the sources
