@@ -341,10 +341,16 @@ constexpr size_t kRsCounterBytes = 256, kRsHistBytes = 8 * 256 * 4;
 constexpr int sort_tile(int64_t n) { return n <= (1 << 17) ? 1024 : n <= (1 << 19) ? 2048 : 4096; }
 constexpr int sort_passes(int64_t n, int bits) { return bits <= 0 || n <= 1 ? 0 : (bits + 7) / 8; }
 constexpr bool sort_reduce_then_scan(int64_t n, int passes) { return passes >= 2 && n >= (int64_t(1) << 22); }
+// tiles to allow for: never fewer than a smaller input needs, so that a workspace planned for n
+// particles serves fewer
+constexpr int64_t sort_tiles_max(int64_t n)
+{
+    const int64_t t = (n + sort_tile(n) - 1) / sort_tile(n), least = n > (1 << 19) ? 256 : n > (1 << 17) ? 128 : 0;
+    return t > least ? t : least;
+}
 constexpr size_t sort_scratch_bytes(int64_t n, int bits)
 {
-    return kRsCounterBytes + kRsHistBytes +
-           8 * 256 * (size_t)((bits + 7) / 8) * (size_t)((n + sort_tile(n) - 1) / sort_tile(n));
+    return kRsCounterBytes + kRsHistBytes + 8 * 256 * (size_t)((bits + 7) / 8) * (size_t)sort_tiles_max(n);
 }
 inline uint32_t *sort_hist(void *scratch)
 {
