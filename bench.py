@@ -388,7 +388,7 @@ def run_gpu(args, w):
     # keys: 32-bit leaf keys (uniform tree) or 63-bit keys at depth 21 (adaptive tree)
     kb = 8 if adaptive else 4
     sort_passes = 8 if adaptive else -(-(3 * L) // 8)
-    sort_bytes = sort_passes * 2 * (kb + 4) + kb + 32
+    sort_bytes = sort_passes * 2 * (kb + 4) + 32  # the key kernels count the histograms
     box_bytes = 16 + kb + 4
     m2l_ms = stages.get("M2L/M2P", float("nan"))
     m2l_tf = m2l_flops / (m2l_ms / 1e3) / 1e12
@@ -399,33 +399,39 @@ def run_gpu(args, w):
     except Exception:
         tpeak, tbasis = 1900.0, "fallback 1900 TFLOP/s dense FP16/BF16 (of fallback)"
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
-    nt = {4: 128, 6: 144, 8: 256, 10: 208}[P]
-    nstride = 200 if P == 10 else nt
+    # block M2L: an N-tile is one unit of parity classes; it walks the units it couples with at every
+    # parent offset (visits over the 26 offsets, kunit K values each)
+    nt, ntiles_n, visits, kunit = {4: (128, 1, 26, 128), 6: (144, 2, 44, 144), 8: (256, 2, 44, 256),
+                                   10: (208, 4, 74, 208)}[P]
     kd = 8 * P * P
-    ntiles_n = -(-kd // nstride)
+
+    def blk_ranges(t):  # offset ranges per tile (m2l_blk.cu)
+        if t >= 152:
+            return 1
+        return min(range(1, 27), key=lambda k: (2 * -(-t * k // 152) * (-(-26 // k) + 2) + (k > 1), k))
     if adaptive:
         # block kernel over units: per tile 128 units (MMA M) x NT outputs over the 26 parent
-        # offsets, K = 8 p^2 per offset (colleagues' children gathered); 3 MMAs per product;
-        # offset ranges per tile from the particle count (m2l_ablk_ksplit)
+        # offsets (colleagues' children gathered); 3 MMAs per product; offset ranges per tile from
+        # the particle count (m2l_ablk_ksplit)
         ablk_tiles = -(-units // 128) * ntiles_n
-        est = -(-(n // (4 * w["leaf_size"]) + 1) // 128) * ntiles_n
-        ksplit = 1 if est >= 152 else min(26, -(-304 // est))
+        est = -(-(n // (2 * w["leaf_size"]) + 1) // 128) * ntiles_n
+        ksplit = blk_ranges(est)
         kname, ksrc, kprof = "k_m2l_ablk", "m2l_blk.cu", f"m2l_ablk_{w['name']}.md"
-        tensor_flops = ablk_tiles * 26 * kd * 3 * 2 * 128 * nt
+        tensor_flops = ablk_tiles * visits * kunit * 3 * 2 * 128 * nt
         m2l_launches = -(-(ablk_tiles * ksplit) // sms)
-        kshape = (f"{ablk_tiles} tiles of 128 units (cells with children) x {nt} outputs (of 8p^2 = {kd}), K = {kd} "
-                  f"per parent offset, 26 offsets, offsets split over {ksplit} CTA(s) per tile; the M2L stage "
+        kshape = (f"{ablk_tiles} tiles of 128 units (cells with children) x {nt} outputs (of 8p^2 = {kd}), {visits} K "
+                  f"units of {kunit} over the 26 offsets, offsets split over {ksplit} CTA(s) per tile; the M2L stage "
                   "also holds P2L over the X lists")
     else:
         # block kernel: per tile 128 target parents (MMA M) x NT outputs (MMA N) over the 26 parent
-        # offsets, K = 8 p^2 per offset; 3 MMAs per product
+        # offsets; 3 MMAs per product
         blk_tiles = sum(max(1, 8 ** (l - 1) // 128) * ntiles_n for l in range(2, L + 1))
-        ksplit = 1 if blk_tiles >= 152 else min(26, -(-304 // blk_tiles))
+        ksplit = blk_ranges(blk_tiles)
         kname, ksrc, kprof = "k_m2l_blk", "m2l_blk.cu", f"m2l_blk_{w['name']}.md"
-        tensor_flops = blk_tiles * 26 * kd * 3 * 2 * 128 * nt
+        tensor_flops = blk_tiles * visits * kunit * 3 * 2 * 128 * nt
         m2l_launches = -(-(blk_tiles * ksplit) // sms)
-        kshape = (f"{blk_tiles} tiles of 128 target parents x {nt} outputs (of 8p^2 = {kd}), K = {kd} per parent "
-                  f"offset, 26 offsets, offsets split over {ksplit} CTA(s) per tile")
+        kshape = (f"{blk_tiles} tiles of 128 target parents x {nt} outputs (of 8p^2 = {kd}), {visits} K units of "
+                  f"{kunit} over the 26 offsets, offsets split over {ksplit} CTA(s) per tile")
     traffic = traffic_from_profile(ksrc, kprof, kname)
     m2l_roof = {"kernel": kname, "bound": "tensor", "achieved": m2l_tf, "peak": tpeak, "unit": "TFLOP/s",
                 "frac": m2l_tf / tpeak,
@@ -490,8 +496,8 @@ def run_gpu(args, w):
                                  f"({kb + 4} B); the box read is counted once"},
             "sort": {"bytes_per_particle": sort_bytes, "achieved_gbs": sort_bytes * n / (stages["sort"] / 1e3) / 1e9,
                      "peak_gbs": hbm_peak, "bound": "hbm",
-                     "note": f"one histogram read of the keys (4 B), {sort_passes} radix passes x (read key + index 8 B, "
-                             "write 8 B), gather (16 B in, 16 B out)"},
+                     "note": f"{sort_passes} radix passes x (read key + index {kb + 4} B, write {kb + 4} B), "
+                             "gather (16 B in, 16 B out)"},
         },
         "stages_ms": stages,
         "serial": {"ms_per_step": float(np.median(ser_ms)), "stages_ms": ser_stages,
@@ -689,14 +695,14 @@ def run_sort_16m(G, dev, local) -> dict:
             sts.append(G.gbfmm_stage_times(ctx))
         G.gbfmm_sync_status(ctx)
         med = {k: float(np.median([st[k] for st in sts[1:]])) for k in ("box+keys", "sort", "cells+lists")}
-        sort_bytes = kbytes + passes * 2 * (kbytes + 4) + 32
+        sort_bytes = passes * 2 * (kbytes + 4) + 32
         out_rows[name] = {"n": n, "radix_passes": passes, "sort_ms": med["sort"], "sort_bytes_per_particle": sort_bytes,
                           "sort_achieved_gbs": sort_bytes * n / (med["sort"] / 1e3) / 1e9,
                           "sort_frac": sort_bytes * n / (med["sort"] / 1e3) / 1e9 / hbm,
                           "box_keys_ms": med["box+keys"], "cells_lists_ms": med["cells+lists"]}
         del xd, out, ws
     G.gbfmm_destroy(ctx)
-    out_rows["note"] = ("algorithmic bytes: one histogram read of the keys, every pass reads and writes key + index, "
+    out_rows["note"] = ("algorithmic bytes: every pass reads and writes key + index, "
                         "the gather reads and writes 16 B; frac of the measured HBM copy rate")
     return out_rows
 
