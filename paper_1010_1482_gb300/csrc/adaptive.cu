@@ -1389,7 +1389,8 @@ int evaluate_adaptive_in(gbfmm_ctx *ctx, AdaptiveState &A, const AdaptCaps *caps
             grow(A.ab_scale, (size_t)ucap + 16, false, 0, s) || grow(A.ab_src, m2l_ablk_src_bytes(ucap), false, 0, s))
             return fail_joined(GBFMM_ENOMEM, "block M2L buffers");
         const int ksplit = m2l_ablk_ksplit(P, n, prm->leaf_size);
-        if (grow(A.lpart, m2l_ablk_class_bytes(P, ucap, ksplit), false, 0, s))
+        DevBuf &lpart = A.lane_lpart ? *A.lane_lpart : A.lpart;
+        if (grow(lpart, m2l_ablk_class_bytes(P, ucap, ksplit), false, 0, s))
             return fail_joined(GBFMM_ENOMEM, "block M2L classes");
         launch_ablk_prep(P, R.cells(), ucap, A.level.as<int32_t>(), A.nchild.as<int32_t>(), A.child_of.as<int32_t>(),
                          A.coll.as<int32_t>(), M, A.ab_flag.as<uint32_t>(), A.ab_scan.as<uint32_t>(),
@@ -1397,7 +1398,7 @@ int evaluate_adaptive_in(gbfmm_ctx *ctx, AdaptiveState &A, const AdaptCaps *caps
                          A.ab_nu.as<int32_t>(), A.ab_pre.p, A.ab_scale.as<int8_t>(), A.ab_src.as<int32_t>(), s);
         if (launch_m2l_ablk(P, ucap, A.ab_nu.as<int32_t>(), A.ab_units.as<int32_t>(), A.child_of.as<int32_t>(),
                             A.ab_src.as<int32_t>(), A.ab_pre.p, A.ab_scale.as<int8_t>(), ops.m2l_blk, Lc,
-                            A.lpart.as<float>(), ksplit, ctx->d_status, s, fork ? sm_count() : 0) != 0)
+                            lpart.as<float>(), ksplit, ctx->d_status, s, fork ? sm_count() : 0) != 0)
             return fail_joined(GBFMM_ECUDA, "TMA tensor map encoding failed");
         launch_p2l_cells(P, est_adaptive_leaves(n, leaf_size), R.cells(), A.level.as<int32_t>(), geom, A.begin.as<int32_t>(), A.count.as<int32_t>(),
                          A.loffs[kListX].as<uint32_t>(), A.lids[kListX].as<int32_t>(), A.sx.as<float4>(), Lc, s);

@@ -41,9 +41,10 @@ size_t align256(size_t b) { return (b + 255) / 256 * 256; }
 // 119 against 237 cells for two samples of 3981 Plummer particles at leaf size 256), moves cells
 // between levels and may reach a few levels deeper; so the cells and leaves get twice the count
 // plus a constant, and every level down to three below the deepest may hold as many cells as
-// the whole tree (the per-level launches are sized by the counts and loop over what there is).  The lists grow with the cells, and by more than the cells on small trees (their
-// rows fill as the tree deepens): the V rows are bounded by 189 per cell, the others take their
-// entries per cell times the cell capacity, with half again as margin.
+// the whole tree (the per-level launches are sized by the counts and loop over what there is).
+// The lists grow with the cells, and by more than the cells on small trees (their rows fill as the
+// tree deepens): the V rows are bounded by 189 per cell, the others take their entries per cell
+// times the cell capacity, with half again as margin.
 AdaptCaps with_margin(const AdaptCaps &c)
 {
     auto up = [](int64_t v, int64_t slack) { return v + v / 4 + slack; };
@@ -54,7 +55,7 @@ AdaptCaps with_margin(const AdaptCaps &c)
     AdaptCaps r = c;
     r.cells = 2 * c.cells + 64;
     r.leaves = 2 * c.leaves + 64;
-    r.units = 2 * (c.cells - c.leaves) + 64;
+    r.units = r.cells;  // a refilled sample of chains has far more cells with children per leaf
     r.maxl = std::min(gbfmm::kAdaptiveMaxLevel, c.maxl + 3);
     for (int l = 0; l <= gbfmm::kAdaptiveMaxLevel; ++l) {
         r.level[l] = l <= r.maxl ? r.cells : 0;
@@ -86,6 +87,7 @@ struct gbfmm_batch {
     void *ws = nullptr;          // uniform workspaces
     float *scratch = nullptr;    // root-box reduction scratch: kBoxPartials floats per lane
     unsigned *counters = nullptr;  // and one counter per lane
+    std::vector<gbfmm::DevBuf> lpart;  // and the block M2L's class sums of one instance per lane
     int lanes = 1;
     const float *x = nullptr;
     float *out = nullptr;
@@ -97,6 +99,7 @@ struct gbfmm_batch {
         if (graph) cudaGraphDestroy(graph);
         for (auto &s : states)
             if (s) gbfmm::free_adaptive(*s);
+        for (gbfmm::DevBuf &v : lpart) cudaFree(v.p);
         cudaFree(ws);
         cudaFree(scratch);
         cudaFree(counters);
@@ -186,6 +189,11 @@ int gbfmm_batch_create(gbfmm_batch **out, gbfmm_ctx *ctx, int32_t nb, const int6
             load[k] += b->inst[i].n;
         }
     }
+    // a class buffer holds up to 26 ranges of the unit capacity: the instances of a lane, which run
+    // one after another, share it (1,000 sets of 20,000 particles, p = 10: 10 GB instead of 150)
+    b->lpart.resize(b->lanes);
+    for (const Instance &it : b->inst)
+        if (it.state >= 0) b->states[it.state]->lane_lpart = &b->lpart[it.lane];
     if ((ws_total && cudaMalloc(&b->ws, ws_total) != cudaSuccess) ||
         cudaMalloc(&b->scratch, sizeof(float) * gbfmm::kBoxPartials * b->lanes) != cudaSuccess ||
         cudaMalloc(&b->counters, sizeof(unsigned) * b->lanes) != cudaSuccess ||

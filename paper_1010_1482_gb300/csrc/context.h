@@ -62,6 +62,7 @@ struct AdaptiveState {
     // block-form M2L: unit flags and their scan, unit of every cell, the units, their count, the
     // pre-split rows and scales, the colleague rows per (tile, offset), the classes per (range, unit)
     DevBuf ab_flag, ab_scan, ab_unit_of, ab_units, ab_nu, ab_pre, ab_scale, ab_src, lpart;
+    DevBuf *lane_lpart = nullptr;  // in place of lpart: one buffer for instances that run one after another
     DevBuf partials;  // root-box reduction scratch of evaluations that do not use the context's
     AdaptCaps counts;  // the sizes the last host-counted evaluation read back
     int64_t n = 0, ncells = 0, nleaves = 0, entries[4] = {0, 0, 0, 0};

@@ -135,6 +135,34 @@ def test_batch_capacity_overflow_is_reported(G, ctx):
         G.gbfmm_batch_destroy(b)
 
 
+def _chains(m):
+    """512 points over a 4 x 4 x 4 grid of cells: 8 in each (m = 0), or nine close ones in each of m
+    cells, where chains of cells lead to two leaves at level 5, and at most 8 in every other."""
+    g = (np.arange(4) + 0.5) / 4
+    c = np.stack(np.meshgrid(g, g, g, indexing="ij"), -1).reshape(-1, 3)
+    d = np.stack(np.meshgrid([-1, 1], [-1, 1], [-1, 1], indexing="ij"), -1).reshape(-1, 3) / 32.0
+    order, left, k = [0, 63, *range(1, 63)], 512 - 9 * m, 64 - m
+    pts = [c[i] + (d[::-1] if i == 63 else d)[: left // k + (j < left % k)] for j, i in enumerate(order[:k])]
+    pts += [c[i] + 0.025 + np.linspace(-0.02, 0.02, 9)[:, None] * np.array([1, 0, 0]) for i in order[k:]]
+    x = np.concatenate(pts)
+    return np.c_[x, np.full(len(x), 1 / 512)].astype(np.float32)
+
+
+def test_batch_refilled_with_chains(G, ctx):
+    # 9 of 73 cells have children at creation, 89 of 187 in the refilled sample (cell capacity 210)
+    prms, off = [G.gbfmm_default_params(p=6, tree=G.TREE_ADAPTIVE, leaf_size=8)], np.array([0, 512], dtype=np.int64)
+    xd = torch.from_numpy(_chains(0)).cuda()
+    out = torch.zeros_like(xd)
+    b = G.gbfmm_batch_create(ctx, off, prms, xd, out, lanes=1)
+    try:
+        xd.copy_(torch.from_numpy(_chains(34)))
+        G.gbfmm_batch_launch(ctx, b)
+        G.gbfmm_sync_status(ctx)
+        assert np.array_equal(out.cpu().numpy(), _alone(G, ctx, xd.cpu().numpy(), off, prms))
+    finally:
+        G.gbfmm_batch_destroy(b)
+
+
 def test_evaluate_batch_keeps_its_graph(G, ctx):
     inst = inputs.batch_instances(count=16, n_lo=1000, n_hi=20000)
     xs = [inputs.make_particles(r["n"], r["dist"], r["seed"]) for r in inst]
