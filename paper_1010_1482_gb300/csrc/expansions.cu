@@ -53,7 +53,7 @@ void init_expansion_constants()
 {
     m2p_tables();
     float rmm[kMaxDeg + 1], ra[kMaxDeg + 1][kMaxDeg + 1], rb[kMaxDeg + 1][kMaxDeg + 1];
-    static float sq[2 * kMaxDeg + 4][2 * kMaxDeg + 4];
+    float sq[2 * kMaxDeg + 4][2 * kMaxDeg + 4];
     for (int m = 0; m <= kMaxDeg; ++m) rmm[m] = m ? (float)sqrt((2.0 * m - 1.0) / (2.0 * m)) : 0.f;
     for (int n = 0; n <= kMaxDeg; ++n)
         for (int m = 0; m <= kMaxDeg; ++m) {
@@ -1136,16 +1136,19 @@ constexpr int kM2PMaxNO = 3 * (kMaxP + 1) * (kMaxP + 2);
 __device__ int2 d_m2p_tab[4][kM2PMaxNO];
 __constant__ uint64_t c_nbeta[kMaxP + 1][kMaxP + 1];  // (-beta, -beta) of (N, m)
 
-void m2p_tables()
+// the host copies of those tables and of c_nbeta1 and d_kscale
+struct M2PTables {
+    int2 tab[4][kM2PMaxNO] = {};
+    uint64_t nbeta[kMaxP + 1][kMaxP + 1] = {};
+    float nbeta1[kMaxP + 1][kMaxP + 1] = {}, kscale[kMaxP * kMaxP] = {};
+    M2PTables();
+};
+
+M2PTables::M2PTables()
 {
-    static int2 tab[4][kM2PMaxNO];
-    static uint64_t nbeta[kMaxP + 1][kMaxP + 1];
-    static float nbeta1[kMaxP + 1][kMaxP + 1], kscale[kMaxP * kMaxP];
     auto ra = [](int n, int m) { return (2.0 * n + 1.0) / sqrt((double)(n + 1 - m) * (n + 1 + m)); };
     auto rb = [](int n, int m) { return sqrt((double)(n - m) * (n + m)) / sqrt((double)(n + 1 - m) * (n + 1 + m)); };
     const int orders[4] = {4, 6, 8, 10};
-    memset(tab, 0, sizeof(tab));
-    memset(nbeta, 0, sizeof(nbeta));
     double gamma = 1.0;
     for (int m = 0; m <= kMaxP; ++m) {
         if (m > 0) gamma *= -sqrt((2.0 * m - 1.0) / (2.0 * m));
@@ -1180,10 +1183,15 @@ void m2p_tables()
             }
         }
     }
-    cudaMemcpyToSymbol(d_m2p_tab, tab, sizeof(tab));
-    cudaMemcpyToSymbol(c_nbeta, nbeta, sizeof(nbeta));
-    cudaMemcpyToSymbol(c_nbeta1, nbeta1, sizeof(nbeta1));
-    cudaMemcpyToSymbol(d_kscale, kscale, sizeof(kscale));
+}
+
+void m2p_tables()
+{
+    static const M2PTables t;  // built once: contexts are created from several threads
+    cudaMemcpyToSymbol(d_m2p_tab, t.tab, sizeof(t.tab));
+    cudaMemcpyToSymbol(c_nbeta, t.nbeta, sizeof(t.nbeta));
+    cudaMemcpyToSymbol(c_nbeta1, t.nbeta1, sizeof(t.nbeta1));
+    cudaMemcpyToSymbol(d_kscale, t.kscale, sizeof(t.kscale));
 }
 
 GB_DEV uint64_t neg2(uint64_t v) { return v ^ 0x8000000080000000ull; }
