@@ -546,7 +546,6 @@ int evaluate_uniform_in(gbfmm_ctx *ctx, const gbfmm_params *prm, int64_t n, cons
     ctx->last_keys = (size_t)(reinterpret_cast<unsigned char *>(skeys) - ctx->last_ws);
     ctx->last_idx = (size_t)(reinterpret_cast<unsigned char *>(perm) - ctx->last_ws);
     ctx->last_method = prm->method;
-    ctx->last_lists = false;
     ctx->timed_last = timing;
     ctx->stage_order_last = fork ? 2 : (split ? 1 : 0);
     ctx->ops_built_last = built_now;
@@ -677,8 +676,9 @@ int gbfmm_export_lists(gbfmm_ctx *ctx, int kind, int32_t *offs, int32_t *ids, in
     }
     if (kind != GBFMM_LIST_P2P && kind != GBFMM_LIST_M2L) return fail(ctx, GBFMM_EINVAL, "unknown list kind");
     const Layout &lo = ctx->last;
-    if (!ctx->last_lists) {
-        // evaluations build at most the M2L rows they walk: build both kinds now from the cells
+    {
+        // evaluations build at most the M2L rows they walk: build both kinds now from the cells, for
+        // every export, since replays of a captured evaluation change them without passing here
         unsigned char *w = ctx->last_ws;
         const int32_t *cb = reinterpret_cast<const int32_t *>(w + lo.cell_begin);
         const int32_t *ce = reinterpret_cast<const int32_t *>(w + lo.cell_end);
@@ -692,7 +692,6 @@ int gbfmm_export_lists(gbfmm_ctx *ctx, int kind, int32_t *offs, int32_t *ids, in
                          reinterpret_cast<int32_t *>(w + lo.m2l_ids), reinterpret_cast<uint16_t *>(w + lo.m2l_code), 0);
         e = cudaDeviceSynchronize();
         if (e != cudaSuccess) return cuda_fail(ctx, e, "list build");
-        ctx->last_lists = true;
     }
     const int64_t rows = kind == GBFMM_LIST_P2P ? lo.nleaves : lo.ncells;
     std::vector<uint32_t> o(rows + 1);

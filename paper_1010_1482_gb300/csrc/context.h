@@ -91,7 +91,6 @@ struct gbfmm_ctx {
     unsigned char *last_ws = nullptr;
     size_t last_keys = 0, last_idx = 0;
     int last_method = 0;
-    bool last_lists = false;  // gbfmm_export_lists has built the last uniform evaluation's P2P and M2L rows
     gbfmm::AdaptiveState ad;
     // host-buffer path
     float *h_in = nullptr, *h_out = nullptr;

@@ -57,6 +57,31 @@ def test_graph_replay_equals_eager_evaluation(G, ctx):
         G.gbfmm_graph_destroy(g)
 
 
+def test_lists_exported_between_replays(G, ctx):
+    """Each export shows the cells of the last replay (an export kept the rows of the first)."""
+    n, leaf = 3000, 64
+    prm = G.gbfmm_default_params(p=4, leaf_size=leaf)
+    ws = torch.empty(G.gbfmm_plan(prm, n)[1], dtype=torch.uint8, device="cuda")
+    xs = [inputs.uniform_cube(n, 44), inputs.plummer(n, 45)]  # all 64 leaves filled, and few of them
+    xd = torch.from_numpy(xs[0]).cuda()
+    out = torch.empty_like(xd)
+    g = G.gbfmm_graph_create(ctx, prm, xd, out, ws)
+    try:
+        for x in xs:
+            xd.copy_(torch.from_numpy(x))
+            G.gbfmm_graph_launch(g)
+            G.gbfmm_sync_status(ctx)
+            t = O.build_tree(x, leaf)
+            ref = O.build_lists(t)
+            for kind, name, rows in ((G.LIST_P2P, "p2p", 8 ** t["L"]), (G.LIST_M2L, "m2l", O.level_offset(t["L"] + 1))):
+                offs, ids = G.gbfmm_export_lists(ctx, kind, rows)
+                assert np.array_equal(offs, ref[name + "_offs"]), name
+                row = np.repeat(np.arange(rows), np.diff(offs))
+                assert np.array_equal(ids, ref[name + "_ids"][np.lexsort((ref[name + "_ids"], row))]), name
+    finally:
+        G.gbfmm_graph_destroy(g)
+
+
 def test_graph_rejects_adaptive_tree(G, ctx):
     prm = G.gbfmm_default_params(p=4, leaf_size=32, tree=G.TREE_ADAPTIVE)
     xd = torch.from_numpy(inputs.plummer(5000, 3)).cuda()
