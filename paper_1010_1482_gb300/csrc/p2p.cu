@@ -448,7 +448,19 @@ void launch_p2p_cells_near(const int32_t *leaves, Span lv, int64_t n, const floa
 // 442 -> 144 us.  Bound by the FP32 pipe.
 // Any two particles may coincide; the zero-distance test is made on the least of four sources' d2
 // (NaN included) and only a group that fails it takes the masked rule.
+//
+// Targets alone fill the GPU where they are many and the sources few, and a cluster of 8 CTAs for a
+// handful of sources is launches and sums only: 1,000,000 targets of 64 sources took 321 us, 256 of
+// 352, 1024 of 570 (a thread per target: 39, 138, 538).  So (us, cluster of 8 / CTA alone / thread
+// per target):
+//   - a thread per target up to 128 sources: 64 of 1M 321 / 47 / 39, 128 of 1M 326 / 70 / 72, 64 of
+//     10,000 8.2 / 6.1 / 4.2; for up to 1024 targets the cluster is as fast from 32 sources on
+//     (128 of 64: 4.2 / 6.1 / 6.2);
+//   - up to 1024 sources a CTA alone (SPLIT = 1) from 48 targets a source on: 256 of 10,000 8.3 / 7.2 /
+//     10.3, 512 of 20,000 12.4 / 12.4 / 16.4, 1024 of 50,000 33.0 / 32.9 / 47.2, 1024 of 1M 570 / 442 / 538;
+//   - else the cluster (4096 of 20,000: 45 / 64 / 102), which also keeps every sum short.
 constexpr int kDirectThreads = 128, kDirectTargets = 64, kDirectTile = 512, kDirectSplit = 8;
+constexpr int64_t kDirectFewSources = 128, kDirectOneSources = 1024;
 
 // the least of four packed pairs; NaN if any of them is
 GB_DEV float least8(const uint64_t (&d2)[4])
@@ -463,8 +475,43 @@ GB_DEV float least8(const uint64_t (&d2)[4])
     return m;
 }
 
+// sources S[first + step k .. + 4) of the cnt staged ones, for k = 0, 1, ...; a group cut short by cnt goes
+// one source at a time
 template <bool SOFT>
-__global__ void __cluster_dims__(kDirectSplit, 1, 1) __launch_bounds__(kDirectThreads)
+GB_DEV void direct_sources(const float4 *S, int cnt, int first, int step, uint64_t nx, uint64_t ny, uint64_t nz,
+                           uint64_t e2, uint64_t &phi, uint64_t &gx, uint64_t &gy, uint64_t &gz)
+{
+    int j = first;
+    for (; j + 4 <= cnt; j += step) {
+        uint64_t dx[4], dy[4], dz[4], d2[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const float4 q = S[j + u];
+            dx[u] = add2(pack2(q.x, q.x), nx), dy[u] = add2(pack2(q.y, q.y), ny), dz[u] = add2(pack2(q.z, q.z), nz);
+            d2[u] = fma2(dx[u], dx[u], fma2(dy[u], dy[u], mul2(dz[u], dz[u])));
+        }
+        if (least8(d2) > 0.f) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const float qw = S[j + u].w;
+                float a, c;
+                unpack2(SOFT ? add2(d2[u], e2) : d2[u], a, c);
+                const uint64_t inv = pack2(rsqrt_ftz(a), rsqrt_ftz(c)), w = mul2(pack2(qw, qw), inv);
+                phi = add2(phi, w);
+                const uint64_t w3 = mul2(mul2(w, inv), inv);
+                gx = fma2(dx[u], w3, gx);
+                gy = fma2(dy[u], w3, gy);
+                gz = fma2(dz[u], w3, gz);
+            }
+        } else {
+            for (int u = 0; u < 4; ++u) pair2<SOFT, true>(nx, ny, nz, S[j + u], e2, phi, gx, gy, gz);
+        }
+    }
+    for (; j < cnt; ++j) pair2<SOFT, true>(nx, ny, nz, S[j], e2, phi, gx, gy, gz);
+}
+
+template <bool SOFT, int SPLIT>
+__global__ void __cluster_dims__(SPLIT, 1, 1) __launch_bounds__(kDirectThreads)
     k_direct(int64_t ns, const float4 *__restrict__ src, int64_t nt, const float4 *__restrict__ tgt, float eps2,
              float4 *__restrict__ out)
 {
@@ -474,8 +521,8 @@ __global__ void __cluster_dims__(kDirectSplit, 1, 1) __launch_bounds__(kDirectTh
     __shared__ float4 sum[kDirectTargets];
     const cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank(), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int64_t t0 = (int64_t)(blockIdx.x / kDirectSplit) * kDirectTargets;
-    const int64_t per = (ns + kDirectSplit - 1) / kDirectSplit, s0 = rank * per, s1 = min(ns, s0 + per);
+    const int64_t t0 = (int64_t)(blockIdx.x / SPLIT) * kDirectTargets;
+    const int64_t per = (ns + SPLIT - 1) / SPLIT, s0 = rank * per, s1 = min(ns, s0 + per);
     auto target = [&](int k) { return t0 + k < nt ? __ldg(&tgt[t0 + k]) : make_float4(0.f, 0.f, 0.f, 0.f); };
     const float4 A = target(lane), B = target(lane + 32);
     const uint64_t nx = pack2(-A.x, -B.x), ny = pack2(-A.y, -B.y), nz = pack2(-A.z, -B.z), e2 = pack2(eps2, eps2);
@@ -493,33 +540,7 @@ __global__ void __cluster_dims__(kDirectSplit, 1, 1) __launch_bounds__(kDirectTh
         if (b + kDirectTile < s1) stage(b + kDirectTile, buf ^ 1);
         const int cnt = (int)min((int64_t)kDirectTile, s1 - b);
         const float4 *S = tile[buf];
-        int j = 4 * warp;
-        for (; j + 4 <= cnt; j += kDirectThreads / 8) {
-            uint64_t dx[4], dy[4], dz[4], d2[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const float4 q = S[j + u];
-                dx[u] = add2(pack2(q.x, q.x), nx), dy[u] = add2(pack2(q.y, q.y), ny), dz[u] = add2(pack2(q.z, q.z), nz);
-                d2[u] = fma2(dx[u], dx[u], fma2(dy[u], dy[u], mul2(dz[u], dz[u])));
-            }
-            if (least8(d2) > 0.f) {
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const float qw = S[j + u].w;
-                    float a, c;
-                    unpack2(SOFT ? add2(d2[u], e2) : d2[u], a, c);
-                    const uint64_t inv = pack2(rsqrt_ftz(a), rsqrt_ftz(c)), w = mul2(pack2(qw, qw), inv);
-                    phi = add2(phi, w);
-                    const uint64_t w3 = mul2(mul2(w, inv), inv);
-                    gx = fma2(dx[u], w3, gx);
-                    gy = fma2(dy[u], w3, gy);
-                    gz = fma2(dz[u], w3, gz);
-                }
-            } else {
-                for (int u = 0; u < 4; ++u) pair2<SOFT, true>(nx, ny, nz, S[j + u], e2, phi, gx, gy, gz);
-            }
-        }
-        for (; j < cnt; ++j) pair2<SOFT, true>(nx, ny, nz, S[j], e2, phi, gx, gy, gz);  // at most three, of one warp
+        direct_sources<SOFT>(S, cnt, 4 * warp, kDirectThreads / 8, nx, ny, nz, e2, phi, gx, gy, gz);
     }
     float4 va, vb;
     unpack2(phi, va.x, vb.x);
@@ -537,25 +558,63 @@ __global__ void __cluster_dims__(kDirectSplit, 1, 1) __launch_bounds__(kDirectTh
         sum[tid] = r;
     }
     cl.sync();
-    // CTA `rank` adds the 8 CTAs' sums of its eighth of the targets
-    const int k = rank * (kDirectTargets / kDirectSplit) + tid;
-    if (tid < kDirectTargets / kDirectSplit && t0 + k < nt) {
+    // CTA `rank` adds the CTAs' sums of its share of the targets
+    const int k = rank * (kDirectTargets / SPLIT) + tid;
+    if (tid < kDirectTargets / SPLIT && t0 + k < nt) {
         float4 r = *cl.map_shared_rank(&sum[k], 0);
-        for (int c = 1; c < kDirectSplit; ++c) add(r, *cl.map_shared_rank(&sum[k], c));
+        for (int c = 1; c < SPLIT; ++c) add(r, *cl.map_shared_rank(&sum[k], c));
         out[t0 + k] = r;
     }
     cl.sync();  // no CTA leaves while its sums may be read
+}
+
+// Few sources: a thread per target takes every source in turn, nothing is staged twice or added up.
+constexpr int kDirectFewThreads = 256;
+
+template <bool SOFT>
+__global__ void __launch_bounds__(kDirectFewThreads) k_direct_few(int ns, const float4 *__restrict__ src, int64_t nt,
+                                                                  const float4 *__restrict__ tgt, float eps2,
+                                                                  float4 *__restrict__ out)
+{
+    __shared__ float4 tile[kDirectFewSources];
+    if (threadIdx.x < ns) tile[threadIdx.x] = __ldg(&src[threadIdx.x]);
+    __syncthreads();
+    const int64_t i = blockIdx.x * (int64_t)kDirectFewThreads + threadIdx.x;
+    if (i >= nt) return;
+    const float4 t = __ldg(&tgt[i]);
+    float phi = 0.f, gx = 0.f, gy = 0.f, gz = 0.f;
+#pragma unroll 8
+    for (int j = 0; j < ns; ++j) {
+        const float4 q = tile[j];
+        const float dx = q.x - t.x, dy = q.y - t.y, dz = q.z - t.z;
+        const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+        const float inv = d2 > 0.f ? rsqrt_ftz(SOFT ? d2 + eps2 : d2) : 0.f;
+        const float w = q.w * inv, w3 = w * inv * inv;
+        phi += w;
+        gx = fmaf(dx, w3, gx);
+        gy = fmaf(dy, w3, gy);
+        gz = fmaf(dz, w3, gz);
+    }
+    out[i] = make_float4(phi, gx, gy, gz);
 }
 
 void launch_direct(int64_t n_src, const float4 *src, int64_t n_tgt, const float4 *tgt, float eps2, float4 *out,
                    cudaStream_t s)
 {
     if (n_tgt <= 0) return;
-    const unsigned grid = (unsigned)((n_tgt + kDirectTargets - 1) / kDirectTargets * kDirectSplit);
-    if (eps2 > 0.f)
-        k_direct<true><<<grid, kDirectThreads, 0, s>>>(n_src, src, n_tgt, tgt, eps2, out);
-    else
-        k_direct<false><<<grid, kDirectThreads, 0, s>>>(n_src, src, n_tgt, tgt, eps2, out);
+    const bool soft = eps2 > 0.f;
+    const int64_t ctas = (n_tgt + kDirectTargets - 1) / kDirectTargets;
+    if (n_src <= kDirectFewSources && (n_src <= 32 || n_tgt > 1024)) {
+        const unsigned grid = (unsigned)((n_tgt + kDirectFewThreads - 1) / kDirectFewThreads);
+        auto k = soft ? k_direct_few<true> : k_direct_few<false>;
+        k<<<grid, kDirectFewThreads, 0, s>>>((int)n_src, src, n_tgt, tgt, eps2, out);
+    } else if (n_src <= kDirectOneSources && n_tgt > 48 * n_src) {
+        auto k = soft ? k_direct<true, 1> : k_direct<false, 1>;
+        k<<<(unsigned)ctas, kDirectThreads, 0, s>>>(n_src, src, n_tgt, tgt, eps2, out);
+    } else {
+        auto k = soft ? k_direct<true, kDirectSplit> : k_direct<false, kDirectSplit>;
+        k<<<(unsigned)(ctas * kDirectSplit), kDirectThreads, 0, s>>>(n_src, src, n_tgt, tgt, eps2, out);
+    }
     note_launches(1);
 }
 

@@ -70,6 +70,52 @@ def test_direct_tiles(G, ctx, ns, nt, eps2):
     assert np.linalg.norm(got - ref) <= TOL_DIRECT * max(np.linalg.norm(ref), 1e-30) + (0 if ref.any() else 1e-30)
 
 
+# both sides of the rules that choose the form: 32 and 128 sources, 1024 targets, 48 targets a source
+# (up to 1024 sources), and the edges of each form's tiles beyond them
+@pytest.mark.parametrize("ns,nt", [(32, 257), (33, 1024), (33, 1025), (128, 1025), (129, 48 * 129), (129, 48 * 129 + 1),
+                                   (1023, 48 * 1023 + 1), (1024, 48 * 1024 + 1), (1025, 48 * 1025 + 1)])
+@pytest.mark.parametrize("eps2", [0.0, 1e-3])
+def test_direct_forms(G, ctx, ns, nt, eps2):
+    src = inputs.uniform_cube(ns, 110 + ns)
+    tgt = inputs.uniform_cube(nt, 210 + nt)
+    tgt[:ns] = src[:nt]
+    src[1] = src[0]
+    out = torch.full((nt, 4), float("nan"), device="cuda")
+    G.gbfmm_direct(ctx, torch.from_numpy(src).cuda(), torch.from_numpy(tgt).cuda(), out, eps2)
+    torch.cuda.synchronize()
+    got = out.cpu().numpy().astype(np.float64)
+    pick = np.unique(np.r_[: min(nt, ns + 70), max(0, nt - 130): nt])  # coincident pairs, the last CTAs
+    ref = direct64(src, tgt[pick], eps2)
+    assert np.all(np.isfinite(got))
+    assert np.linalg.norm(got[pick] - ref) <= TOL_DIRECT * np.linalg.norm(ref)
+
+
+def test_direct_many_targets_few_sources_time(G, ctx):
+    """A million targets of a few sources pay for their pairs, not for splitting the sources: at most
+    three times a copy of the targets plus the pairs at half the rate of the all-pairs sum (8e11 a second)."""
+    nt = 1 << 20
+    tgt = torch.rand((nt, 4), device="cuda")
+    out = torch.empty_like(tgt)
+
+    def us(f):
+        f()
+        best = float("inf")
+        for _ in range(5):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            for _ in range(10):
+                f()
+            b.record()
+            b.synchronize()
+            best = min(best, 100 * a.elapsed_time(b))
+        return best
+
+    copy = us(lambda: out.copy_(tgt))
+    for ns in (1, 16, 64, 256):
+        src = torch.rand((ns, 4), device="cuda")
+        assert us(lambda: G.gbfmm_direct(ctx, src, tgt, out)) <= 3 * copy + nt * ns / 8e5 + 20, ns
+
+
 def test_direct_no_sources(G, ctx):
     tgt = torch.rand((70, 4), device="cuda")
     out = torch.full((70, 4), 7.0, device="cuda")
