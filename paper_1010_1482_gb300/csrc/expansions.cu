@@ -594,16 +594,26 @@ __global__ void __launch_bounds__(128) k_p2m(int L, const float *__restrict__ ge
 // Plummer p = 8 1122 -> 407; P2L there 2036 -> 1305.
 constexpr int64_t kP2MManyLeaves = 8 * 1024;
 
+// P2M starts beside P2P, with priority.  An SM that runs it under another split of shared memory and L1
+// than P2P's takes no P2P CTA until it is idle, and P2P's CTAs crowded onto the rest, eight on 60 SMs
+// and none on 90 (100,000 Plummer particles, 465 leaves of up to 1024): so it asks for P2P's split.
+// Forked evaluations with it: that one 3.59 .. 4.59 -> 3.21 ms, 400,009 with leaves of up to 512 3.45 -> 2.5.
+template <class K>
+static void p2m_carveout(K k)
+{
+    cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+}
+
 void launch_p2m(int P, int L, const float *geo, const float4 *sx, const int32_t *begin, const int32_t *end, float *M,
                 cudaStream_t s)
 {
     const int64_t nl = int64_t(1) << (3 * L);
     if (nl >= kP2MManyLeaves) {
         const unsigned grid = (unsigned)((nl + 15) / 16);
-        GBFMM_DISPATCH_P(P, (k_p2m<PQ, 8><<<grid, 128, 0, s>>>(L, geo, sx, begin, end, M)));
+        GBFMM_DISPATCH_P(P, (p2m_carveout(k_p2m<PQ, 8>), k_p2m<PQ, 8><<<grid, 128, 0, s>>>(L, geo, sx, begin, end, M)));
     } else {
         const unsigned grid = (unsigned)((nl + 3) / 4);
-        GBFMM_DISPATCH_P(P, (k_p2m<PQ, 32><<<grid, 128, 0, s>>>(L, geo, sx, begin, end, M)));
+        GBFMM_DISPATCH_P(P, (p2m_carveout(k_p2m<PQ, 32>), k_p2m<PQ, 32><<<grid, 128, 0, s>>>(L, geo, sx, begin, end, M)));
     }
     note_launches(1);
 }
@@ -1671,10 +1681,12 @@ void launch_p2m_cells(int P, int64_t est_leaves, const int32_t *leaves, Span lv,
     if (lv.cap <= 0) return;
     if (est_leaves >= kP2MManyLeaves) {
         const unsigned grid = (unsigned)((lv.cap + 15) / 16);
-        GBFMM_DISPATCH_P(P, (k_p2m_cells<PQ, 8><<<grid, 128, 0, s>>>(leaves, lv, level, geom, begin, count, sx, M)));
+        GBFMM_DISPATCH_P(P, (p2m_carveout(k_p2m_cells<PQ, 8>),
+                             k_p2m_cells<PQ, 8><<<grid, 128, 0, s>>>(leaves, lv, level, geom, begin, count, sx, M)));
     } else {
         const unsigned grid = (unsigned)((lv.cap + 3) / 4);
-        GBFMM_DISPATCH_P(P, (k_p2m_cells<PQ, 32><<<grid, 128, 0, s>>>(leaves, lv, level, geom, begin, count, sx, M)));
+        GBFMM_DISPATCH_P(P, (p2m_carveout(k_p2m_cells<PQ, 32>),
+                             k_p2m_cells<PQ, 32><<<grid, 128, 0, s>>>(leaves, lv, level, geom, begin, count, sx, M)));
     }
     note_launches(1);
 }
