@@ -245,10 +245,11 @@ int gbfmm_export_adaptive_tree(gbfmm_ctx *ctx, double *origin_side, int64_t *nce
 /*
  * Per-stage device times (ms) of the last evaluate run with
  * GBFMM_FLAG_STAGE_TIMING, in this order: 0 box+keys, 1 sort, 2 cells+lists,
- * 3 P2M, 4 M2M, 5 M2L (or M2P), 6 L2L, 7 L2P(+output), 8 P2P, 9 operator build
- * (0 when cached).  When P2P ran on the context's second stream (the default for the FMM),
- * stage 8 is its own duration, overlapping stages 3-6, and the stages add up to more than the
- * evaluation took; with GBFMM_FLAG_SERIAL they are consecutive.  Waits for the device.
+ * 3 P2M, 4 M2M, 5 M2L (treecode: M2P), 6 L2L, 7 L2P(+output; adaptive FMM: and M2P over the
+ * W lists), 8 P2P, 9 operator build (0 when cached).  When P2P ran on the context's second
+ * stream (the default for the FMM), stage 8 and an M2P that followed it there are their own
+ * durations, overlapping stages 3-6, and the stages add up to more than the evaluation took;
+ * with GBFMM_FLAG_SERIAL they are consecutive.  Waits for the device.
  * *count = stages written (<= max).
  */
 int gbfmm_stage_times(gbfmm_ctx *ctx, float *ms, int max, int *count);

@@ -1317,7 +1317,7 @@ int evaluate_adaptive_in(gbfmm_ctx *ctx, AdaptiveState &A, const AdaptCaps *caps
     // the evaluation is timed, serial or device-counted); L2P adds the far field to them and
     // writes the output
     const bool fork = (prm->flags & GBFMM_FLAG_SERIAL) == 0 && !dev;
-    ctx->stage_order_last = fork ? 2 : 1;
+    ctx->stage_order_last = fork ? 3 : 1;
     if (grow(A.near, 32 * (size_t)n, false, 0, s)) return fail(ctx, GBFMM_ENOMEM, "adaptive near field");
     float4 *near = A.near.as<float4>();
     const cudaStream_t s_main = s;
@@ -1373,7 +1373,9 @@ int evaluate_adaptive_in(gbfmm_ctx *ctx, AdaptiveState &A, const AdaptCaps *caps
     if (fork) {
         cudaEventRecord(ctx->ev_m2m, s);
         cudaStreamWaitEvent(ctx->s_near, ctx->ev_m2m, 0);
+        if (timing) cudaEventRecord(ctx->ev_aux[3], ctx->s_near);
         far_m2p(ctx->s_near);
+        if (timing) cudaEventRecord(ctx->ev_aux[4], ctx->s_near);
         cudaEventRecord(ctx->ev_near, ctx->s_near);
     }
     if (deep && !cores && !gathered) {

@@ -278,7 +278,7 @@ int gbfmm_create(gbfmm_ctx **out, int device)
              cudaMemset(ctx->d_counter, 0, sizeof(unsigned)) == cudaSuccess &&
              cudaMemset(ctx->d_zero, 0, 128 * sizeof(float)) == cudaSuccess;
     for (int i = 0; ok && i <= kStages; ++i) ok = cudaEventCreate(&ctx->ev[i]) == cudaSuccess;
-    for (int i = 0; ok && i < 3; ++i) ok = cudaEventCreate(&ctx->ev_aux[i]) == cudaSuccess;
+    for (cudaEvent_t &e : ctx->ev_aux) ok = ok && cudaEventCreate(&e) == cudaSuccess;
     if (ok) {
         int least = 0, greatest = 0;
         ok = cudaDeviceGetStreamPriorityRange(&least, &greatest) == cudaSuccess &&
@@ -326,7 +326,9 @@ int gbfmm_destroy(gbfmm_ctx *ctx)
     free_adaptive(ctx->ad);
     for (int i = 0; i <= kStages; ++i)
         if (ctx->ev[i]) cudaEventDestroy(ctx->ev[i]);
-    for (cudaEvent_t e : {ctx->ev_fork, ctx->ev_near, ctx->ev_join, ctx->ev_m2m, ctx->ev_aux[0], ctx->ev_aux[1], ctx->ev_aux[2]})
+    for (cudaEvent_t e : {ctx->ev_fork, ctx->ev_near, ctx->ev_join, ctx->ev_m2m})
+        if (e) cudaEventDestroy(e);
+    for (cudaEvent_t e : ctx->ev_aux)
         if (e) cudaEventDestroy(e);
     if (ctx->s_far) cudaStreamDestroy(ctx->s_far);
     if (ctx->s_near) cudaStreamDestroy(ctx->s_near);
@@ -795,11 +797,12 @@ int gbfmm_stage_times(gbfmm_ctx *ctx, float *ms, int max, int *count)
         cudaEventElapsedTime(&t9[k], ctx->ev[k], ctx->ev[k + 1]);
     }
     if (ctx->stage_order_last == 1) std::swap(t9[7], t9[8]);  // reported as 7 L2P, 8 P2P
-    if (ctx->stage_order_last == 2) {
-        float l2p = 0.f, p2p = 0.f;
+    if (ctx->stage_order_last >= 2) {
+        float l2p = 0.f, p2p = 0.f, m2p = 0.f;
         cudaEventElapsedTime(&l2p, ctx->ev_aux[2], ctx->ev[9]);
         cudaEventElapsedTime(&p2p, ctx->ev_aux[0], ctx->ev_aux[1]);
-        t9[7] += l2p;  // ev 7 -> 8: what ran on the far stream before the join (adaptive: M2P)
+        if (ctx->stage_order_last == 3) cudaEventElapsedTime(&m2p, ctx->ev_aux[3], ctx->ev_aux[4]);
+        t9[7] += l2p + m2p;  // ev 7 -> 8: what ran on the far stream between L2L and the join (M2P, or nothing)
         t9[8] = p2p;
     }
     int k = 0;

@@ -102,13 +102,14 @@ struct gbfmm_ctx {
     bool timed_last = false;
     // order of the last timed evaluation's stages 7 (L2P) and 8 (P2P): 0 = L2P then P2P (ev 7, 8,
     // 9); 1 = P2P then L2P, serial; 2 = P2P on s_near between ev_aux[0] and ev_aux[1] while the
-    // far field ran on s_far, whose L2P (after the join on ev_aux[2]) ends at ev[9]
+    // far field ran on s_far, whose L2P (after the join on ev_aux[2]) ends at ev[9]; 3 = as 2, with
+    // the adaptive tree's M2P on s_near too, between ev_aux[3] and ev_aux[4]
     int stage_order_last = 0;
     // the near field runs beside the far field: P2P on s_near (lowest priority), M2L .. L2P on
     // s_far (highest), forked from and joined into the caller's stream by events
     cudaStream_t s_far = nullptr, s_near = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_near = nullptr, ev_join = nullptr, ev_m2m = nullptr;
-    cudaEvent_t ev_aux[3] = {};
+    cudaEvent_t ev_aux[5] = {};
     bool ops_built_last = false;
     int64_t launches_last = 0;
     // gbfmm_evaluate_batch: the captured batch of the last call and the arguments it was made for

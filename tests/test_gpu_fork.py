@@ -48,3 +48,12 @@ def test_fork_of_heavy_leaves(G, ctx):
     alone or a little more (crowded onto the SMs that P2M left free it took a third more)."""
     kw = dict(p=10, leaf_size=1024)
     assert timed(G, ctx, 100_000, **kw)[0] <= 1.05 * timed(G, ctx, 100_000, flags=G.FLAG_SERIAL, **kw)[0]
+
+
+@pytest.mark.parametrize("n,p,leaf", [(100_000, 10, 64), (20_000, 10, 512)])
+def test_stage_times_hold_m2p(G, ctx, n, p, leaf):
+    """M2P over the W rows is part of the reported L2P stage, serial or forked."""
+    kw = dict(p=p, leaf_size=leaf)
+    serial = timed(G, ctx, n, flags=G.FLAG_SERIAL | G.FLAG_STAGE_TIMING, **kw)[1]
+    fork = timed(G, ctx, n, flags=G.FLAG_STAGE_TIMING, **kw)[1]
+    assert fork["L2P"] >= 0.75 * serial["L2P"], (fork, serial)
