@@ -1317,7 +1317,7 @@ int evaluate_adaptive_in(gbfmm_ctx *ctx, AdaptiveState &A, const AdaptCaps *caps
     // the evaluation is timed, serial or device-counted); L2P adds the far field to them and
     // writes the output
     const bool fork = (prm->flags & GBFMM_FLAG_SERIAL) == 0 && !dev;
-    ctx->stage_order_last = fork ? 3 : 1;
+    ctx->stage_order_last = fork ? 2 : 1;
     if (grow(A.near, 32 * (size_t)n, false, 0, s)) return fail(ctx, GBFMM_ENOMEM, "adaptive near field");
     float4 *near = A.near.as<float4>();
     const cudaStream_t s_main = s;
@@ -1359,9 +1359,13 @@ int evaluate_adaptive_in(gbfmm_ctx *ctx, AdaptiveState &A, const AdaptCaps *caps
         launch_translate_levels(P, true, up, nl, A.child_of.as<int32_t>(), A.nchild.as<int32_t>(), ops.m2m, M, s);
     }
     mark(5);
-    // M2P over the W rows needs the multipoles alone: forked, it follows P2P on the near field's stream,
-    // beside the M2L and L2L (20,011 Plummer particles 334 -> 309 us, 400,009 1502 -> 1425); serial, it
-    // comes before L2P
+    // M2P over the W rows needs the multipoles alone.  Forked, it follows P2P on the near field's stream,
+    // beside the M2L and L2L, where the far field is the longer side: leaves of up to 96 + 10 p (us, this
+    // against M2P after L2L: 20,000 Plummer particles p = 4 leaf 64 324 : 348, p = 10 leaf 128 435 : 516,
+    // leaf 192 662 : 681; 400,000 p = 10 leaf 160 1398 : 1523).  Larger leaves make P2P the longer one
+    // (20,000 p = 8 leaf 512 1281 : 945, 400,000 p = 4 leaf 160 1022 : 933, p = 10 leaf 256 1883 : 1717).
+    // The CUDA-core M2L of p = 4 and 6, several of whose CTAs fit an SM, crowds onto the SMs that M2P has
+    // left (100,000 p = 6 1462 : 1047): there M2P follows L2L too.  Serial, it comes before L2P.
     auto far_m2p = [&](cudaStream_t st) {
         if (!deep)
             cudaMemsetAsync(far, 0, 16 * (size_t)n, st);
@@ -1370,7 +1374,9 @@ int evaluate_adaptive_in(gbfmm_ctx *ctx, AdaptiveState &A, const AdaptCaps *caps
                              A.loffs[kListW].as<uint32_t>(), A.lids[kListW].as<int32_t>(), A.sx.as<float4>(), M, far,
                              st);
     };
-    if (fork) {
+    const bool near_m2p = fork && leaf_size <= 96 + 10 * P && !(cores && P <= 6);
+    if (near_m2p) {
+        ctx->stage_order_last = 3;
         cudaEventRecord(ctx->ev_m2m, s);
         cudaStreamWaitEvent(ctx->s_near, ctx->ev_m2m, 0);
         if (timing) cudaEventRecord(ctx->ev_aux[3], ctx->s_near);
@@ -1461,7 +1467,7 @@ int evaluate_adaptive_in(gbfmm_ctx *ctx, AdaptiveState &A, const AdaptCaps *caps
                               (float)prm->eps2, near, ctx->d_status, s);
         mark(8);
     }
-    if (!fork) far_m2p(s);
+    if (!near_m2p) far_m2p(s);
     if (fork) {
         mark(8);
         cudaStreamWaitEvent(s, ctx->ev_near, 0);

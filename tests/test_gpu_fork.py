@@ -52,8 +52,17 @@ def test_fork_of_heavy_leaves(G, ctx):
 
 @pytest.mark.parametrize("n,p,leaf", [(100_000, 10, 64), (20_000, 10, 512)])
 def test_stage_times_hold_m2p(G, ctx, n, p, leaf):
-    """M2P over the W rows is part of the reported L2P stage, serial or forked."""
+    """M2P over the W rows is part of the reported L2P stage, serial or forked, on either stream."""
     kw = dict(p=p, leaf_size=leaf)
     serial = timed(G, ctx, n, flags=G.FLAG_SERIAL | G.FLAG_STAGE_TIMING, **kw)[1]
     fork = timed(G, ctx, n, flags=G.FLAG_STAGE_TIMING, **kw)[1]
     assert fork["L2P"] >= 0.75 * serial["L2P"], (fork, serial)
+
+
+@pytest.mark.parametrize("n,p,leaf,flags", [(20_000, 10, 512, 0), (100_000, 6, 64, 2)])
+def test_m2p_stays_off_the_longer_side(G, ctx, n, p, leaf, flags):
+    """Where P2P is the longer side (512 a leaf), or the M2L's CTAs crowd (CUDA cores, p = 6), M2P is
+    not put before the end of either: the fork keeps hiding what it can."""
+    kw = dict(p=p, leaf_size=leaf)
+    a, b = (timed(G, ctx, n, flags=flags | f, **kw)[0] for f in (0, G.FLAG_SERIAL))
+    assert a <= {512: 0.85, 64: 1.05}[leaf] * b, (a, b)
