@@ -758,10 +758,10 @@ __global__ void k_chain_fill(Span cells, const int32_t *__restrict__ nchild, con
 constexpr int kInfoLists = 32, kInfoChain = 40, kInfoAbort = 48;
 
 struct GuardCaps {
-    int64_t v[kTreeBins + 2];
+    int64_t v[kTreeBins + 1];
 };
 
-// stage 0: the tree (cells, leaves, the cells of every level, the cells with children); stage 1: the four lists;
+// stage 0: the tree (cells, leaves, the cells of every level); stage 1: the four lists;
 // stage 2: the chain lists.  A count above its capacity sets the abort word and kStatusCapacity.
 __global__ void k_guard(const int32_t *__restrict__ info, GuardCaps g, int stage, int32_t *__restrict__ abort,
                         int *__restrict__ status)
@@ -769,8 +769,7 @@ __global__ void k_guard(const int32_t *__restrict__ info, GuardCaps g, int stage
     if (threadIdx.x != 0) return;
     bool over = false;
     if (stage == 0) {
-        over = info[kTreeBins - 1] > g.v[0] || info[kTreeBins] - info[kTreeBins - 1] > g.v[1] ||
-               2 * (int64_t)info[kTreeBins - 1] - info[kTreeBins] > g.v[kTreeBins + 1];
+        over = info[kTreeBins - 1] > g.v[0] || info[kTreeBins] - info[kTreeBins - 1] > g.v[1];
         for (int l = 0; l <= kAdaptMaxLevel; ++l) over = over || (info[l + 1] - info[l] > g.v[2 + l]);
     } else {
         const int base = stage == 1 ? kInfoLists : kInfoChain, k = stage == 1 ? 4 : 2;
@@ -1118,7 +1117,6 @@ int evaluate_adaptive_in(gbfmm_ctx *ctx, AdaptiveState &A, const AdaptCaps *caps
             g.v[0] = caps->cells;
             g.v[1] = caps->leaves;
             for (int l = 0; l <= kAdaptMaxLevel; ++l) g.v[2 + l] = l <= maxl ? caps->level[l] : 0;
-            g.v[kTreeBins + 1] = caps->units;
             k_guard<<<1, 32, 0, s>>>(info, g, 0, info + kInfoAbort, ctx->d_status);
             note_launches(1);
         }
@@ -1389,7 +1387,7 @@ int evaluate_adaptive_in(gbfmm_ctx *ctx, AdaptiveState &A, const AdaptCaps *caps
         // their colleagues' children gathered per tile; no V list is read
         rc = ensure_blk(ctx, P, s);
         if (rc != GBFMM_OK) return fail_joined(rc, "block operators");
-        const int64_t ucap = dev ? caps->units : std::max<int64_t>(1, ncells - A.nleaves);
+        const int64_t ucap = dev ? ncells : std::max<int64_t>(1, ncells - A.nleaves), uexp = dev ? caps->units : ucap;
         const int64_t up = m2l_ablk_tiles_units(ucap);
         if (grow(A.ab_flag, 4 * (size_t)(ncells + 1), false, 0, s) || grow(A.ab_scan, 4 * (size_t)(ncells + 1), false, 0, s) ||
             grow(A.ab_unit_of, 4 * (size_t)ncells + 4, false, 0, s) || grow(A.ab_units, 4 * (size_t)up + 4, false, 0, s) ||
@@ -1398,13 +1396,13 @@ int evaluate_adaptive_in(gbfmm_ctx *ctx, AdaptiveState &A, const AdaptCaps *caps
             return fail_joined(GBFMM_ENOMEM, "block M2L buffers");
         const int ksplit = m2l_ablk_ksplit(P, n, prm->leaf_size);
         DevBuf &lpart = A.lane_lpart ? *A.lane_lpart : A.lpart;
-        if (grow(lpart, m2l_ablk_class_bytes(P, ucap, ksplit), false, 0, s))
+        if (grow(lpart, m2l_ablk_class_bytes(P, ucap, uexp, ksplit), false, 0, s))
             return fail_joined(GBFMM_ENOMEM, "block M2L classes");
         launch_ablk_prep(P, R.cells(), ucap, A.level.as<int32_t>(), A.nchild.as<int32_t>(), A.child_of.as<int32_t>(),
                          A.coll.as<int32_t>(), M, A.ab_flag.as<uint32_t>(), A.ab_scan.as<uint32_t>(),
                          A.scan_tmp.as<uint32_t>(), A.ab_unit_of.as<int32_t>(), A.ab_units.as<int32_t>(),
                          A.ab_nu.as<int32_t>(), A.ab_pre.p, A.ab_scale.as<int8_t>(), A.ab_src.as<int32_t>(), s);
-        if (launch_m2l_ablk(P, ucap, A.ab_nu.as<int32_t>(), A.ab_units.as<int32_t>(), A.child_of.as<int32_t>(),
+        if (launch_m2l_ablk(P, ucap, uexp, A.ab_nu.as<int32_t>(), A.ab_units.as<int32_t>(), A.child_of.as<int32_t>(),
                             A.ab_src.as<int32_t>(), A.ab_pre.p, A.ab_scale.as<int8_t>(), ops.m2l_blk, Lc,
                             lpart.as<float>(), ksplit, ctx->d_status, s, fork ? sm_count() : 0) != 0)
             return fail_joined(GBFMM_ECUDA, "TMA tensor map encoding failed");

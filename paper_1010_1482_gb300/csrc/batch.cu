@@ -55,7 +55,7 @@ AdaptCaps with_margin(const AdaptCaps &c)
     AdaptCaps r = c;
     r.cells = 2 * c.cells + 64;
     r.leaves = 2 * c.leaves + 64;
-    r.units = r.cells;  // a refilled sample of chains has far more cells with children per leaf
+    r.units = c.cells - c.leaves;  // expected; a refilled sample of chains may have up to r.cells
     r.maxl = std::min(gbfmm::kAdaptiveMaxLevel, c.maxl + 3);
     for (int l = 0; l <= gbfmm::kAdaptiveMaxLevel; ++l) {
         r.level[l] = l <= r.maxl ? r.cells : 0;
@@ -189,8 +189,8 @@ int gbfmm_batch_create(gbfmm_batch **out, gbfmm_ctx *ctx, int32_t nb, const int6
             load[k] += b->inst[i].n;
         }
     }
-    // a class buffer holds up to 26 ranges of the unit capacity: the instances of a lane, which run
-    // one after another, share it (1,000 sets of 20,000 particles, p = 10: 10 GB instead of 150)
+    // a class buffer holds up to 26 ranges of the expected units and one of the rest: the instances of a
+    // lane, which run one after another, share it
     b->lpart.resize(b->lanes);
     for (const Instance &it : b->inst)
         if (it.state >= 0) b->states[it.state]->lane_lpart = &b->lpart[it.lane];

@@ -519,10 +519,11 @@ void launch_ablk_prep(int P, Span cells, int64_t ucap, const int32_t *level, con
                       const int32_t *child_of, const int32_t *coll, const float *M, uint32_t *flag, uint32_t *scan,
                       uint32_t *scan_tmp, int32_t *unit_of, int32_t *units, int32_t *n_units, void *Apre,
                       int8_t *uscale, int32_t *src, cudaStream_t s);
-// V: the classes of every unit and offset range, m2l_ablk_class_bytes
-size_t m2l_ablk_class_bytes(int P, int64_t ucap, int ksplit);
+// uexp: the units expected of the ucap there may be.  V: the classes of the units and offset ranges,
+// m2l_ablk_class_bytes
+size_t m2l_ablk_class_bytes(int P, int64_t ucap, int64_t uexp, int ksplit);
 // -1 if the operators' tensor map cannot be encoded (nothing launched)
-int launch_m2l_ablk(int P, int64_t ucap, const int32_t *n_units, const int32_t *units, const int32_t *child_of,
+int launch_m2l_ablk(int P, int64_t ucap, int64_t uexp, const int32_t *n_units, const int32_t *units, const int32_t *child_of,
                     const int32_t *src, const void *Apre, const int8_t *uscale, const void *table, float *Lc,
                     float *V, int ksplit, int *status, cudaStream_t s, int max_ctas);
 

@@ -40,7 +40,7 @@ struct DevBuf {
 // W, X entries; chain: the treecode's two chain-list totals; maxl: deepest level.
 struct AdaptCaps {
     int64_t cells = 0, leaves = 0;
-    int64_t units = 0;  // capacities only: cells with children
+    int64_t units = 0;  // capacities only: the cells with children of the counts they were made from
     int64_t level[kAdaptiveMaxLevel + 1] = {};
     int64_t expect[kAdaptiveMaxLevel + 1] = {};  // capacities only: the counts they were made from
     int64_t list[4] = {}, chain[2] = {};

@@ -761,11 +761,19 @@ struct AblkParams {
     CUtensorMap tmB;  // B_D, FP16 hi | lo
     int tile0;        // tile of block 0 (launch in waves)
     int ksplit;
+    int64_t ut0;          // unit tile of tile 0
     int64_t part_stride;  // floats between the partial sums of two offset ranges
     int64_t zrow;
+    int seq0;  // SEQ: from this tile on a CTA takes the ranges of its tile one after another
 };
 
-template <int P, int CH>
+// Classes of unit u (from the launch's first on) and range k: V + k part_stride + u KD.  A captured
+// evaluation may meet far more units than its capacities were made from, and the classes of all of
+// them for up to 26 ranges are memory and idle CTAs that few refills use.  So there (SEQ) the units past
+// the expected ones take their ranges one after another in one CTA, which adds them in V in range
+// order, as k_ablk_finish does for the others; their V rows follow the split ones'.  64 sets of 20,000
+// particles, p = 8: 10.2 GB -> 2.0, 4.65 ms -> 4.31; a batch of 96 instances 6.54 ms -> 6.37.
+template <int P, int CH, bool SEQ>
 __global__ void __launch_bounds__(kAblkThreads, 1)
     k_m2l_ablk(const __grid_constant__ AblkParams prm, const int32_t *__restrict__ n_units,
                const int32_t *__restrict__ src, const __half *__restrict__ Apre, const int8_t *__restrict__ uscale,
@@ -784,13 +792,15 @@ __global__ void __launch_bounds__(kAblkThreads, 1)
     __shared__ volatile int s_abort;
 
     // ---- tile: unit tile, N-tile, offset range [d_lo, d_hi)
-    const int ks = (prm.tile0 + (int)blockIdx.x) % prm.ksplit;
-    const int tt = (prm.tile0 + (int)blockIdx.x) / prm.ksplit;
+    const int bid = prm.tile0 + (int)blockIdx.x;
+    const bool seq = SEQ && bid >= prm.seq0;
+    const int ks = seq ? prm.ksplit - 1 : bid % prm.ksplit;  // seq: the V rows past part_stride
+    const int tt = seq ? prm.seq0 / prm.ksplit + (bid - prm.seq0) : bid / prm.ksplit;
     const int nt = tt % C::NTILES;
-    const int64_t ut = tt / C::NTILES;
+    const int64_t ut = prm.ut0 + tt / C::NTILES;
     const int64_t nu = *n_units;
     if (ut * kBlkRows >= nu) return;  // the whole CTA: past the units (before any barrier or TMEM)
-    const int d_lo = (26 * ks) / prm.ksplit, d_hi = (26 * (ks + 1)) / prm.ksplit;
+    const int d_lo = seq ? 0 : (26 * ks) / prm.ksplit, d_hi = (26 * (ks + 1)) / prm.ksplit;
     const int32_t *tsrc = src + ut * 26 * kBlkRows;
 
     unsigned char *smem =
@@ -944,7 +954,11 @@ __global__ void __launch_bounds__(kAblkThreads, 1)
         const uint32_t lane_base = (uint32_t)(32 * quad) << 16;
         const int64_t unit = ut * kBlkRows + r;
         const bool rok = unit < nu;
+        auto vrow = [&] {
+            return V + (int64_t)ks * prm.part_stride + (unit - prm.ut0 * kBlkRows) * KD + nt * C::NSTRIDE + h * NH;
+        };
         const int g = *gexp;
+        int range = 0;  // SEQ: of the sums in acc
         float acc[NH];
 #pragma unroll
         for (int i = 0; i < NH; ++i) acc[i] = 0.f;
@@ -976,6 +990,22 @@ __global__ void __launch_bounds__(kAblkThreads, 1)
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&dempty[b]);
+            if (SEQ && seq && (u + 1 == NU || s_steps.drain_d[u + 1] >= (26 * (range + 1)) / prm.ksplit)) {
+                if (rok) {
+                    float *row = vrow();
+#pragma unroll
+                    for (int i = 0; i < NH; i += 4)
+                        if (h * NH + i < C::NSTRIDE) {
+                            float4 *at = reinterpret_cast<float4 *>(row + i);
+                            float4 t = range > 0 ? *at : make_float4(0.f, 0.f, 0.f, 0.f);
+                            t.x += acc[i], t.y += acc[i + 1], t.z += acc[i + 2], t.w += acc[i + 3];
+                            *at = t;
+                        }
+                }
+#pragma unroll
+                for (int i = 0; i < NH; ++i) acc[i] = 0.f;
+                ++range;
+            }
         }
         if (!alive && lane == 0) s_abort = 1;
         int ok = 1;
@@ -983,12 +1013,12 @@ __global__ void __launch_bounds__(kAblkThreads, 1)
         ok = __shfl_sync(0xffffffffu, ok, 0);
         if (!ok && lane == 0) s_abort = 1;
         __syncwarp();
-        if (ok && alive && !s_abort && rok) {
-            float *row = V + (int64_t)ks * prm.part_stride + unit * KD + nt * C::NSTRIDE;
+        if (ok && alive && !s_abort && rok && !seq) {
+            float *row = vrow();
 #pragma unroll
             for (int i = 0; i < NH; i += 4)
                 if (h * NH + i < C::NSTRIDE)
-                    *reinterpret_cast<float4 *>(row + h * NH + i) = make_float4(acc[i], acc[i + 1], acc[i + 2], acc[i + 3]);
+                    *reinterpret_cast<float4 *>(row + i) = make_float4(acc[i], acc[i + 1], acc[i + 2], acc[i + 3]);
         }
     }
 
@@ -1052,9 +1082,10 @@ __global__ void __launch_bounds__(256) k_blk_finish(int npar, int ksplit, int64_
     if (ok && end[8 * par + 1 + c] > begin[8 * par + 1 + c]) Lc[at] = v;
 }
 
-// adaptive tree: units
-template <int P>
-__global__ void __launch_bounds__(256) k_ablk_finish(const int32_t *__restrict__ n_units, int ksplit, int64_t stride4,
+// adaptive tree: units u0 .. u0 + n; SEQ: the first n_split have their ranges apart (else all)
+template <int P, bool SEQ>
+__global__ void __launch_bounds__(256) k_ablk_finish(const int32_t *__restrict__ n_units, int64_t u0, uint32_t n,
+                                                     uint32_t n_split, int ksplit, int64_t stride4,
                                                      const int32_t *__restrict__ units,
                                                      const int32_t *__restrict__ child_of,
                                                      const float4 *__restrict__ V, float4 *__restrict__ Lc)
@@ -1062,9 +1093,14 @@ __global__ void __launch_bounds__(256) k_ablk_finish(const int32_t *__restrict__
     const int lane = threadIdx.x & 31, c = lane >> 2;
     constexpr int PP4 = P * P / 4;
     const uint32_t i = (blockIdx.x * 8 + (threadIdx.x >> 5)) * 4 + (lane & 3), u = i / PP4, n4 = i % PP4;
-    const bool ok = u < (uint32_t)*n_units;
-    const float4 v = blk_child(V + ((int64_t)u * 8 + c) * PP4 + n4, stride4, ksplit, (int)n4, c, ok);
-    const int64_t g = ok ? child_of[(int64_t)units[u] * 8 + c] : -1;
+    const bool ok = u < n && u0 + u < *n_units;
+    const float4 *src = V + ((int64_t)u * 8 + c) * PP4 + n4;
+    if (SEQ && u >= n_split) {
+        src += (ksplit - 1) * stride4;
+        ksplit = 1;
+    }
+    const float4 v = blk_child(src, stride4, ksplit, (int)n4, c, ok);
+    const int64_t g = ok ? child_of[(int64_t)units[u0 + u] * 8 + c] : -1;
     if (g >= 0) Lc[g * PP4 + n4] = v;
 }
 
@@ -1314,8 +1350,28 @@ void launch_ablk_prep(int P, Span cells, int64_t ucap, const int32_t *level, con
     note_launches(4);
 }
 
+// How the units share V: `chunk` units at a time, the first `split` of them with their ranges apart (whole
+// tiles).  Captured evaluations (uexp < ucap) size V by a quarter more than the units expected, and
+// the others take their ranges in turn in the same launch; where there is one range, half the units
+// at a time (four sets of 1,000,000 particles, p = 10: 4.4 GB -> 3.7, 10.98 ms -> 11.02; chunks of the
+// expected units 2.9 GB and 11.18 ms).  A chunk's classes fit 1 GB: a tree of more units (at p = 10
+// 335,000, of about 20M Plummer particles) takes its tiles in turns instead of 3.2 KB a unit.
+struct AblkUnits {
+    int64_t chunk, split;
+    AblkUnits(int P, int64_t ucap, int64_t uexp, int ksplit)
+    {
+        const int64_t all = m2l_ablk_tiles_units(ucap), most = (int64_t(1) << 30) / ((int64_t)ksplit * 32 * P * P);
+        split = std::min(all, m2l_ablk_tiles_units(std::max<int64_t>(1, uexp + uexp / 4)));
+        if (ksplit > 1 && split < all)
+            chunk = all;
+        else
+            split = chunk = std::min(std::max(split, m2l_ablk_tiles_units(all / 2)),
+                                     std::max<int64_t>(kBlkRows, most / kBlkRows * kBlkRows));
+    }
+};
+
 template <int P, int CH>
-static int launch_ablk_t(int64_t ucap, const int32_t *n_units, const int32_t *units, const int32_t *child_of,
+static int launch_ablk_t(int64_t ucap, int64_t uexp, const int32_t *n_units, const int32_t *units, const int32_t *child_of,
                          const int32_t *src, const void *Apre, const int8_t *uscale, const void *table, float *Lc,
                          float *V, int ksplit, int *status, cudaStream_t s, int max_ctas)
 {
@@ -1338,43 +1394,51 @@ static int launch_ablk_t(int64_t ucap, const int32_t *n_units, const int32_t *un
             return -1;
     }
     prm.ksplit = ksplit;
-    prm.part_stride = ucap * C::KD;
     prm.zrow = ucap;
-    auto kern = k_m2l_ablk<P, CH>;
+    const AblkUnits lay(P, ucap, uexp, ksplit);
+    const bool seq = lay.split < lay.chunk;
+    auto kern = seq ? k_m2l_ablk<P, CH, true> : k_m2l_ablk<P, CH, false>;
+    auto finish = seq ? k_ablk_finish<P, true> : k_ablk_finish<P, false>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::kSmemBytes);
-    const int64_t nctas64 = (ucap + kBlkRows - 1) / kBlkRows * C::NTILES * ksplit;
-    const int nctas = (int)nctas64;
-    const int step = max_ctas > 0 ? max_ctas : nctas;
-    for (int t0 = 0; t0 < nctas; t0 += step) {
-        prm.tile0 = t0;
-        const int gsz = nctas - t0 < step ? nctas - t0 : step;
-        kern<<<gsz, kAblkThreads, C::kSmemBytes, s>>>(prm, n_units, src, static_cast<const __half *>(Apre), uscale,
-                                                      gexp, V, status);
+    for (int64_t u0 = 0; u0 < ucap; u0 += lay.chunk) {
+        const int64_t n = std::min(lay.chunk, ucap - u0), n_split = std::min(lay.split, n);
+        prm.ut0 = u0 / kBlkRows;
+        prm.part_stride = n_split * C::KD;
+        prm.seq0 = (int)((n_split + kBlkRows - 1) / kBlkRows * C::NTILES * ksplit);
+        const int nctas = prm.seq0 + (int)((n - n_split + kBlkRows - 1) / kBlkRows * C::NTILES);
+        const int step = max_ctas > 0 ? max_ctas : nctas;
+        for (int t0 = 0; t0 < nctas; t0 += step) {
+            prm.tile0 = t0;
+            const int gsz = nctas - t0 < step ? nctas - t0 : step;
+            kern<<<gsz, kAblkThreads, C::kSmemBytes, s>>>(prm, n_units, src, static_cast<const __half *>(Apre), uscale,
+                                                          gexp, V, status);
+            note_launches(1);
+        }
+        finish<<<(unsigned)((n * (C::PP / 4) + 31) / 32), 256, 0, s>>>(
+            n_units, u0, (uint32_t)n, (uint32_t)n_split, ksplit, prm.part_stride / 4, units, child_of,
+            reinterpret_cast<const float4 *>(V), reinterpret_cast<float4 *>(Lc));
         note_launches(1);
     }
-    const int64_t PP4 = C::PP / 4;
-    k_ablk_finish<P><<<(unsigned)((ucap * PP4 + 31) / 32), 256, 0, s>>>(
-        n_units, ksplit, prm.part_stride / 4, units, child_of, reinterpret_cast<const float4 *>(V),
-        reinterpret_cast<float4 *>(Lc));
-    note_launches(1);
     return 0;
 }
 
-size_t m2l_ablk_class_bytes(int P, int64_t ucap, int ksplit)
+size_t m2l_ablk_class_bytes(int P, int64_t ucap, int64_t uexp, int ksplit)
 {
-    return (size_t)ksplit * (size_t)ucap * 8 * P * P * sizeof(float);
+    const AblkUnits lay(P, ucap, uexp, ksplit);
+    const int64_t n = std::min(lay.chunk, ucap);
+    return (size_t)((ksplit - 1) * std::min(lay.split, n) + n) * 8 * P * P * sizeof(float);
 }
 
-int launch_m2l_ablk(int P, int64_t ucap, const int32_t *n_units, const int32_t *units, const int32_t *child_of,
+int launch_m2l_ablk(int P, int64_t ucap, int64_t uexp, const int32_t *n_units, const int32_t *units, const int32_t *child_of,
                     const int32_t *src, const void *Apre, const int8_t *uscale, const void *table, float *Lc,
                     float *V, int ksplit, int *status, cudaStream_t s, int max_ctas)
 {
     if (ucap <= 0) return 0;
     switch (P) {
-    case 4: return launch_ablk_t<4, blk_ch(4)>(ucap, n_units, units, child_of, src, Apre, uscale, table, Lc, V, ksplit, status, s, max_ctas);
-    case 6: return launch_ablk_t<6, blk_ch(6)>(ucap, n_units, units, child_of, src, Apre, uscale, table, Lc, V, ksplit, status, s, max_ctas);
-    case 8: return launch_ablk_t<8, blk_ch(8)>(ucap, n_units, units, child_of, src, Apre, uscale, table, Lc, V, ksplit, status, s, max_ctas);
-    case 10: return launch_ablk_t<10, blk_ch(10)>(ucap, n_units, units, child_of, src, Apre, uscale, table, Lc, V, ksplit, status, s, max_ctas);
+    case 4: return launch_ablk_t<4, blk_ch(4)>(ucap, uexp, n_units, units, child_of, src, Apre, uscale, table, Lc, V, ksplit, status, s, max_ctas);
+    case 6: return launch_ablk_t<6, blk_ch(6)>(ucap, uexp, n_units, units, child_of, src, Apre, uscale, table, Lc, V, ksplit, status, s, max_ctas);
+    case 8: return launch_ablk_t<8, blk_ch(8)>(ucap, uexp, n_units, units, child_of, src, Apre, uscale, table, Lc, V, ksplit, status, s, max_ctas);
+    case 10: return launch_ablk_t<10, blk_ch(10)>(ucap, uexp, n_units, units, child_of, src, Apre, uscale, table, Lc, V, ksplit, status, s, max_ctas);
     }
     return -1;
 }

@@ -163,6 +163,59 @@ def test_batch_refilled_with_chains(G, ctx):
         G.gbfmm_batch_destroy(b)
 
 
+def _more_chains(m, side=8):
+    """_chains with 4096 points over an 8 x 8 x 8 grid of cells."""
+    n = side**3
+    g = (np.arange(side) + 0.5) / side
+    c = np.stack(np.meshgrid(g, g, g, indexing="ij"), -1).reshape(-1, 3)
+    d = np.stack(np.meshgrid([-1, 1], [-1, 1], [-1, 1], indexing="ij"), -1).reshape(-1, 3) / (8.0 * side)
+    order, left, k = [0, n - 1, *range(1, n - 1)], 8 * n - 9 * m, n - m
+    pts = [c[i] + (d[::-1] if i == n - 1 else d)[: left // k + (j < left % k)] for j, i in enumerate(order[:k])]
+    pts += [c[i] + (0.025 + np.linspace(-0.02, 0.02, 9)[:, None] * np.array([1, 0, 0])) * 4 / side for i in order[k:]]
+    x = np.concatenate(pts)
+    return np.c_[x, np.full(len(x), 1 / len(x))].astype(np.float32)
+
+
+@pytest.mark.parametrize("p", [4, 6, 8, 10])
+def test_batch_refilled_past_the_expected_units(G, ctx, p):
+    # 163 cells with children at creation, so two tiles of 128 have their offset ranges apart; 336 in
+    # the refilled sample, whose third tile takes the ranges one after another
+    prms, n = [G.gbfmm_default_params(p=p, tree=G.TREE_ADAPTIVE, leaf_size=8)], 4096
+    off = np.array([0, n], dtype=np.int64)
+    xd = torch.from_numpy(_more_chains(34)).cuda()
+    out = torch.zeros_like(xd)
+    b = G.gbfmm_batch_create(ctx, off, prms, xd, out, lanes=1)
+    try:
+        for m in (100, 34):
+            x = _more_chains(m)
+            assert len(x) == n
+            xd.copy_(torch.from_numpy(x))
+            G.gbfmm_batch_launch(ctx, b)
+            G.gbfmm_sync_status(ctx)
+            assert np.array_equal(out.cpu().numpy(), _alone(G, ctx, x, off, prms))
+        units = [(np.asarray(O.build_adaptive_tree(_more_chains(m), 8)["nchild"]) > 0).sum() for m in (34, 100)]
+        assert 1.25 * units[0] <= 256 < units[1], units
+    finally:
+        G.gbfmm_batch_destroy(b)
+
+
+def test_batch_class_memory(G, ctx):
+    """A captured instance keeps 26 offset ranges of the units there are, not of all there may be:
+    20,000 Plummer particles, p = 8, in at most 64 MB (151 MB with every unit's)."""
+    n = 20000
+    xd = torch.from_numpy(inputs.plummer(n, 4)).cuda()
+    out = torch.zeros_like(xd)
+    prms = [G.gbfmm_default_params(p=8, tree=G.TREE_ADAPTIVE, leaf_size=64)]
+    G.gbfmm_batch_destroy(G.gbfmm_batch_create(ctx, [0, n], prms, xd, out, lanes=1))  # the context's own buffers
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    b = G.gbfmm_batch_create(ctx, [0, n], prms, xd, out, lanes=1)
+    torch.cuda.synchronize()
+    used = before - torch.cuda.mem_get_info()[0]
+    G.gbfmm_batch_destroy(b)
+    assert used <= 64e6, used
+
+
 def test_evaluate_batch_keeps_its_graph(G, ctx):
     inst = inputs.batch_instances(count=16, n_lo=1000, n_hi=20000)
     xs = [inputs.make_particles(r["n"], r["dist"], r["seed"]) for r in inst]

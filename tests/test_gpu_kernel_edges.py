@@ -226,3 +226,15 @@ def test_adaptive_tree_around_scan_sizes(G, ctx, n):
         ref, row = lists[name + "_ids"], np.repeat(np.arange(t["ncells"]), np.diff(lists[name + "_offs"]))
         assert np.array_equal(offs, lists[name + "_offs"]) and len(ids) == len(ref)
         assert np.array_equal(ids, ref[np.lexsort((ref, row))]), name
+
+
+# more units than the classes of one launch hold (1 GB: 335,000 at p = 10): the tiles in turns
+def test_block_m2l_in_turns(G, ctx):
+    x = inputs.plummer(1_000_000, 800)
+    kw = dict(p=10, leaf_size=1, tree=G.TREE_ADAPTIVE)
+    out = run(G, ctx, x, **kw)
+    t = G.gbfmm_export_adaptive_tree(ctx, len(x))
+    inner = len(np.unique(t["parent"])) - 1  # cells with children
+    assert inner > 335_544
+    ref = run(G, ctx, x, flags=G.FLAG_M2L_GATHERED, **kw)
+    assert O.rel_l2(out[:, 0], ref[:, 0]) <= TOL and O.rel_l2(out[:, 1:], ref[:, 1:]) <= TOL
