@@ -170,6 +170,25 @@ def test_expansions_on_cell_axes(G, ctx, p):
         assert O.rel_l2(free, ref) <= TOL
 
 
+# the same with the root cube [0, 1]^3 found from two particles in its corners, so that the oracle
+# builds the same cells: every other particle on a z axis of all cells it meets, or in their middle
+@pytest.mark.parametrize("p", [4, 6, 8, 10])
+def test_expansions_on_cell_axes_against_oracle(G, ctx, p):
+    n = 4096
+    g = (np.arange(16) + 0.5) / 16
+    x = np.zeros((n, 4), dtype=np.float32)
+    x[:, :3] = np.stack(np.meshgrid(g, g, g, indexing="ij"), -1).reshape(n, 3)
+    x[::2, 2] += 0.01
+    x[1234, :3], x[2345, :3] = 0.0, 1.0
+    x[:, 3] = inputs.uniform01(6, n)
+    origin, side = O.root_box(x)[:2]
+    assert not np.any(origin) and side == 1.0 and O.uniform_depth(n, 1) == 4
+    for method, om in ((G.METHOD_FMM, O.FMM), (G.METHOD_TREECODE, O.TREECODE)):
+        out = run(G, ctx, x, p=p, leaf_size=1, method=method)
+        ref = O.fmm(x, p, 1, method=om)["out"]
+        assert O.rel_l2(out[:, 0], ref[:, 0]) <= TOL and O.rel_l2(out[:, 1:], ref[:, 1:]) <= TOL
+
+
 # both sides of the rules on the expected number of leaves (8 or 32 lanes a leaf in P2M, 16 or 32
 # a cell in P2L): 8,192 leaves
 @pytest.mark.parametrize("p", [4, 8])
@@ -188,8 +207,8 @@ def test_uniform_sparse_leaves(G, ctx):
     assert O.rel_l2(out, O.fmm(x, 6, 2)["out"]) <= TOL
 
 
-# levels of 1 to 128 parents and beyond k_m2m_small's range give the same sums whichever kernel
-# takes them: the batch lays levels out for more cells than there are, and must match bit for bit
+# the same tree in a batch, whose levels beyond k_m2m_small's range take a looping form over the
+# counts of the creation, and alone: bit for bit
 @pytest.mark.parametrize("p", [4, 6, 8, 10])
 def test_m2m_forms_agree_in_batches(G, ctx, p):
     sizes = [2000, 30000]
@@ -207,6 +226,32 @@ def test_m2m_forms_agree_in_batches(G, ctx, p):
     for i, xi in enumerate(xs):
         alone = run(G, ctx, xi, p=p, leaf_size=8, tree=G.TREE_ADAPTIVE, flags=G.FLAG_SERIAL)
         assert np.array_equal(got[offs[i]:offs[i + 1]].astype(np.float64), alone)
+
+
+# A translation's sums do not depend on the kernel that takes its level.  A batch chooses by the
+# counts of the particles it was created with, an evaluation by those it has (parents of levels 2, 3, ...):
+#   600 Plummer 16, 30, 56, .. refilled with uniform 64, 339, 165, ..: runs of levels in one cluster
+#     launch against a launch a level
+#   6000: 32, 83, 184, .. with 64, 512, 3161, ..: the eight positions at once against 16 or 32 cells a CTA
+#   30000: 49, 180, 401, 950 with 64, 512, 4095, 19411: the looping form too, against up to 64 cells
+#   60000 and 160000 uniform, one a leaf, 44005 and 118411 on level 6: the looping form against 64 and
+#     128 cells a CTA
+@pytest.mark.parametrize("p", [4, 6, 8, 10])
+@pytest.mark.parametrize("n,leaf,first", [(600, 2, "plummer"), (6000, 2, "plummer"), (30000, 2, "plummer"),
+                                          (60000, 1, "uniform"), (160000, 1, "uniform")])
+def test_translation_forms_agree(G, ctx, p, n, leaf, first):
+    x = torch.from_numpy(inputs.make_particles(n, first, 600 + n)).cuda()
+    out = torch.empty_like(x)
+    b = G.gbfmm_batch_create(ctx, [0, n], [G.gbfmm_default_params(p=p, leaf_size=leaf, tree=G.TREE_ADAPTIVE)], x, out,
+                             lanes=1)
+    then = inputs.make_particles(n, "uniform", 600 + n)
+    x.copy_(torch.from_numpy(then))
+    out.fill_(0)
+    G.gbfmm_batch_launch(ctx, b)
+    G.gbfmm_sync_status(ctx)
+    got = out.cpu().numpy().astype(np.float64)
+    G.gbfmm_batch_destroy(b)
+    assert np.array_equal(got, run(G, ctx, then, p=p, leaf_size=leaf, tree=G.TREE_ADAPTIVE, flags=G.FLAG_SERIAL))
 
 
 # the scan of the level histograms by one CTA (up to 16,384 values, 23 bins x 712 blocks of 256
