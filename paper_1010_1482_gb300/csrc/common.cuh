@@ -301,6 +301,10 @@ GB_DEV CellGeom cell_geom63(const Box &b, int l, uint64_t key)
     return g;
 }
 
+// The SMs of a GB300, for rules on sizes that fix the order of sums, the workspace or a kernel's form:
+// those do not change with the device (launch shapes that may, take sm_count()).
+constexpr int kSms = 152;
+
 // Layout of one evaluation's workspace (byte offsets from the workspace base).
 struct Layout {
     int64_t n;
@@ -340,7 +344,8 @@ constexpr size_t kRsCounterBytes = 256, kRsHistBytes = 8 * 256 * 4;
 // 63-bit keys 13.5 -> 8 us, with eight look-back words in flight; 400,009: 19.5 -> 13.5)
 constexpr int sort_tile(int64_t n) { return n <= (1 << 17) ? 1024 : n <= (1 << 19) ? 2048 : 4096; }
 constexpr int sort_passes(int64_t n, int bits) { return bits <= 0 || n <= 1 ? 0 : (bits + 7) / 8; }
-constexpr bool sort_reduce_then_scan(int64_t n, int passes) { return passes >= 2 && n >= (int64_t(1) << 22); }
+constexpr int64_t kRsScanMinN = int64_t(1) << 22;  // from here on the passes take the reduce-then-scan form
+constexpr bool sort_reduce_then_scan(int64_t n, int passes) { return passes >= 2 && n >= kRsScanMinN; }
 // tiles to allow for: never fewer than a smaller input needs, so that a workspace planned for n
 // particles serves fewer
 constexpr int64_t sort_tiles_max(int64_t n)
@@ -363,7 +368,7 @@ void launch_sort_clear(void *scratch, int64_t n, int bits, cudaStream_t s);
 constexpr int kKeyThreads = 256;
 inline unsigned key_ctas(int64_t n)
 {
-    const int64_t c = (n + kKeyThreads - 1) / kKeyThreads, most = n >= (int64_t(1) << 22) ? 8 * 152 : 4 * 152;
+    const int64_t c = (n + kKeyThreads - 1) / kKeyThreads, most = n >= (int64_t(1) << 22) ? 8 * kSms : 4 * kSms;
     return (unsigned)(c < most ? c : most);
 }
 // counts the digits of one key, a shared-memory increment each

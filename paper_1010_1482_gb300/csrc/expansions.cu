@@ -630,7 +630,7 @@ void launch_p2m(int P, int L, const float *geo, const float4 *sx, const int32_t 
 constexpr int kTrTN = 32, kTrCN = 8;
 // k_m2m_small up to this many CTAs (700 parents at p = 10); beyond, k_translate's operator is staged
 // for more cells (1,040 parents: 20 us either way)
-constexpr int kTransSmallCtas = 4 * 152;
+constexpr int kTransSmallCtas = 4 * kSms;
 
 template <int P, bool UP, int TN = kTrTN, int CN = kTrCN>
 struct TransCfg {
@@ -919,7 +919,7 @@ static void launch_translate_t(int l, const int32_t *begin, const int32_t *end, 
     if constexpr (UP)
         if (launch_m2m_small<P>(np, LevelCells{level_offset(lp), level_offset(lp + 1), np, begin, end}, ops, X, s)) return;
     const int64_t ctas32 = (np + 31) / 32 * (UP ? 1 : 8);
-    if (ctas32 >= 2 * 152)
+    if (ctas32 >= 2 * kSms)
         launch_translate_tn<P, UP, 32, 8>(l, begin, end, ops, X, s);
     else
         launch_translate_tn<P, UP, 16, 2>(l, begin, end, ops, X, s);
@@ -1754,11 +1754,11 @@ static void translate_cells_t(Span par, const int32_t *child_of, const int32_t *
     if (par.expect >= 0) return translate_cells_tn<P, UP, 16, 2, true>(par, child_of, nchild, ops, X, s);
     const int64_t np = par.cap, ctas32 = (np + 31) / 32 * (UP ? 1 : 8), ctas64 = (np + 63) / 64 * (UP ? 1 : 8);
     if constexpr (UP) {  // large levels: 128 (upward) or 64 cells per CTA share each staged operator
-        if ((np + 127) / 128 >= 4 * 152) return translate_cells_tn<P, UP, 128, 8>(par, child_of, nchild, ops, X, s);
+        if ((np + 127) / 128 >= 4 * kSms) return translate_cells_tn<P, UP, 128, 8>(par, child_of, nchild, ops, X, s);
     }
-    if (ctas64 >= 4 * 152)
+    if (ctas64 >= 4 * kSms)
         translate_cells_tn<P, UP, 64, 8>(par, child_of, nchild, ops, X, s);
-    else if (ctas32 >= 2 * 152)
+    else if (ctas32 >= 2 * kSms)
         translate_cells_tn<P, UP, 32, 8>(par, child_of, nchild, ops, X, s);
     else
         translate_cells_tn<P, UP, 16, 2>(par, child_of, nchild, ops, X, s);

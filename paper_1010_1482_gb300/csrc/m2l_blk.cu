@@ -69,9 +69,16 @@ GB_HD void blk_delta(int d, int &dx, int &dy, int &dz)
 
 }  // namespace
 
-// CH: K values per pipeline stage, one swizzled shared-memory row (64: 128-byte swizzle, 32:
-// 64-byte swizzle)
-template <int P, int CH>
+// K values per pipeline stage, one shared-memory row of 64 bytes (64-byte swizzle).  Four stages of 32
+// cover the copies' latency better at p = 10 than two of 64 (M2L of 1M, 343 us against 372 before the
+// parity classes).  At p = 4 and 6 three stages of 64 run the M2L alone faster (5M: 174 us against 135
+// and 534 against 438; 400,009 Plummer 97 against 93 and 165 against 159), but take the room of a P2P
+// CTA beside them: the step gains little or loses (p = 4 1M 613 : 612, 5M 2310 : 2285; p = 6 1M 661 :
+// 670, 5M 2685 : 2689, 400,009 Plummer 790 : 785), and at p = 4 a chunk of 64 doubles the longest
+// accumulation chain, and with it the error (see DPU).
+constexpr int kBlkCh = 32;
+
+template <int P>
 struct BlkCfg {
     static constexpr int PP = P * P, KD = 8 * PP;
     // N-tile: rows of B_D per CTA (the MMA's N, a multiple of 16) and the stride between tiles
@@ -81,15 +88,15 @@ struct BlkCfg {
     static constexpr int CU = P == 10 ? 2 : P == 4 ? 8 : 4, NUNIT = 8 / CU;
     static constexpr int UNIT = (CU * PP + 15) / 16 * 16, KW = NUNIT * UNIT;
     static constexpr int NSTRIDE = CU * PP, NTILES = NUNIT;
-    static constexpr int UC = (UNIT + CH - 1) / CH;  // chunks of a unit
+    static constexpr int UC = (UNIT + kBlkCh - 1) / kBlkCh;  // chunks of a unit
     // drains per unit: the MMA's accumulation truncates, and a class sums eight children.  Chains of
     // 6, 18, 24 and 39 MMAs at p = 4, 6, 8, 10 leave the outputs as close to the FP64 FMM as, or
     // closer than, the untransformed blocks with chains of 12, 27, 48 and 75 did (phi, 30,000 uniform
     // particles: 1.7, 3.5, 3.5, 3.7e-7 against 1.9, 3.7, 4.3, 5.3e-7); twice as long at p = 4: 2.4e-7
     static constexpr int DPU = P == 10 ? 1 : P == 4 ? 4 : 2;
     static constexpr int MAX_STEPS = 26 * NUNIT * UC, MAX_DRAINS = 26 * NUNIT * DPU;
-    static constexpr int A_BYTES = kBlkRows * CH * 2;  // one of hi / lo
-    static constexpr int B_BYTES = NT * CH * 2;
+    static constexpr int A_BYTES = kBlkRows * kBlkCh * 2;  // one of hi / lo
+    static constexpr int B_BYTES = NT * kBlkCh * 2;
     static constexpr int STAGE_BYTES = 2 * A_BYTES + 2 * B_BYTES;
     static constexpr int NSTAGE_FIT = (210 * 1024) / STAGE_BYTES;
     static constexpr int NSTAGE = NSTAGE_FIT > 4 ? 4 : NSTAGE_FIT;
@@ -101,7 +108,7 @@ struct BlkCfg {
     static_assert(NSTRIDE <= NT && NTILES * NSTRIDE == KD, "N tiling");
     static_assert(UNIT % 16 == 0 && KW % 8 == 0 && UC >= DPU && MAX_DRAINS < 1024, "steps");
     static_assert(A_BYTES % 1024 == 0 && B_BYTES % 1024 == 0, "swizzle atoms");
-    static_assert(CH == 64 || CH == 32, "swizzled row of 128 or 64 bytes");
+    static_assert(2 * kBlkCh == 64, "the row of the 64-byte swizzle (descriptors, tensor maps, loaders)");
     static_assert(NSTAGE >= 2, "pipeline stages");
     static_assert(kSmemBytes <= 227 * 1024, "shared memory");
 };
@@ -141,7 +148,7 @@ GB_DEV void blk_sign_children(float (&v)[8], int signs)
 
 // One CTA's pipeline: per step (K chunk) the offset, first K value, width and whether it opens or
 // closes a drain unit; the units' offsets.  Built by one warp before the roles part.
-template <class C, int CH>
+template <class C>
 struct BlkSteps {
     uint32_t step[C::MAX_STEPS];  // d | k0 / 8 << 5 | kw / 16 << 13 | first << 16 | last << 17 | drain << 18
     uint8_t drain_d[C::MAX_DRAINS];
@@ -155,8 +162,8 @@ GB_DEV bool step_last(uint32_t v) { return v >> 17 & 1; }
 GB_DEV int step_drain(uint32_t v) { return (int)(v >> 18); }
 
 // one warp; nt: the CTA's unit of classes, offsets [d_lo, d_hi)
-template <class C, int CH>
-GB_DEV void blk_steps(BlkSteps<C, CH> &t, int nt, int d_lo, int d_hi, int lane)
+template <class C>
+GB_DEV void blk_steps(BlkSteps<C> &t, int nt, int d_lo, int d_hi, int lane)
 {
     constexpr int UB = C::NUNIT == 4 ? 2 : C::NUNIT == 2 ? 1 : 0;  // axes that distinguish units: the last UB
     const int d = d_lo + lane;
@@ -177,11 +184,11 @@ GB_DEV void blk_steps(BlkSteps<C, CH> &t, int nt, int d_lo, int d_hi, int lane)
         if (nun == 0 || (e & ~free)) continue;
         const int ku = nt ^ e;
         for (int c = 0; c < C::UC; ++c) {
-            const int kw = min(CH, C::UNIT - c * CH), piece = c * C::DPU / C::UC, dr = i * C::DPU + piece;
+            const int kw = min(kBlkCh, C::UNIT - c * kBlkCh), piece = c * C::DPU / C::UC, dr = i * C::DPU + piece;
             const bool first = c == 0 || (c - 1) * C::DPU / C::UC != piece;
             const bool last = c == C::UC - 1 || (c + 1) * C::DPU / C::UC != piece;
             if (first) t.drain_d[dr] = (uint8_t)d;
-            t.step[i * C::UC + c] = (uint32_t)d | (uint32_t)((ku * C::UNIT + c * CH) / 8) << 5 | (uint32_t)(kw / 16) << 13 |
+            t.step[i * C::UC + c] = (uint32_t)d | (uint32_t)((ku * C::UNIT + c * kBlkCh) / 8) << 5 | (uint32_t)(kw / 16) << 13 |
                                     (uint32_t)first << 16 | (uint32_t)last << 17 | (uint32_t)dr << 18;
         }
         ++i;
@@ -189,13 +196,10 @@ GB_DEV void blk_steps(BlkSteps<C, CH> &t, int nt, int d_lo, int d_hi, int lane)
     if (lane == 31) t.nsteps = su * C::UC, t.ndrains = su * C::DPU;
 }
 
-// K values per chunk: four stages of 32 (64-byte swizzle) cover the TMA latency better than two or
-// three of 64 (1M, p = 10: 0.343 against 0.372 ms)
-constexpr int blk_ch(int) { return 32; }
 constexpr size_t blk_kw(int P)  // K row width
 {
-    return P == 4 ? BlkCfg<4, blk_ch(4)>::KW : P == 6 ? BlkCfg<6, blk_ch(6)>::KW : P == 8 ? BlkCfg<8, blk_ch(8)>::KW
-                                                                                  : BlkCfg<10, blk_ch(10)>::KW;
+    return P == 4 ? BlkCfg<4>::KW : P == 6 ? BlkCfg<6>::KW : P == 8 ? BlkCfg<8>::KW
+                                                                                  : BlkCfg<10>::KW;
 }
 
 // tensor maps and tiling of one launch (kernel parameter, read by the TMA unit in place)
@@ -210,16 +214,15 @@ struct BlkParams {
 };
 
 // ---- shared-memory matrix descriptor, K-major, swizzled -----------------------------------------
-// rows of 2 CH bytes, 8-row atoms of 16 CH bytes (SBO); a K step of 16 halves advances the start
-// address by 32 bytes inside the atom.  Swizzle mode: 2 = 128-byte, 4 = 64-byte.
-template <int CH>
+// rows of 64 bytes, 8-row atoms of 512 bytes (SBO); a K step of 16 halves advances the start
+// address by 32 bytes inside the atom.  Swizzle mode: 4 = 64-byte.
 GB_DEV uint64_t blk_desc(uint32_t saddr)
 {
     uint64_t d = (uint64_t)((saddr & 0x3FFFFu) >> 4);
-    d |= (uint64_t)1 << 16;                   // LBO (unused for swizzled K-major operands)
-    d |= (uint64_t)((16 * CH) >> 4) << 32;    // SBO: 8-row atoms
-    d |= (uint64_t)1 << 46;                   // descriptor version of the 5th-generation tensor cores
-    d |= (uint64_t)(CH == 64 ? 2 : 4) << 61;  // swizzle mode
+    d |= (uint64_t)1 << 16;                     // LBO (unused for swizzled K-major operands)
+    d |= (uint64_t)((16 * kBlkCh) >> 4) << 32;  // SBO: 8-row atoms
+    d |= (uint64_t)1 << 46;                     // descriptor version of the 5th-generation tensor cores
+    d |= (uint64_t)4 << 61;                     // swizzle mode
     return d;
 }
 
@@ -270,12 +273,12 @@ GB_DEV float blk_pow2(int e) { return __int_as_float((127 + e) << 23); }
 // U of its children's coefficients (K rows of KW values) scaled by 2^s_S and split into FP16 hi (plane
 // 0) and lo (plane 1); s_S = 10 - e with max |U| = f 2^e, f in [0.5, 1) (empty parents: zeros,
 // s = 0).  One warp per parent; A and scale hold the levels one after another.
-template <int P, int CH>
+template <int P>
 __global__ void __launch_bounds__(256) k_blk_presplit(int L, const int32_t *__restrict__ begin,
                                                       const int32_t *__restrict__ end, const float *__restrict__ M,
                                                       __half *__restrict__ A, int8_t *__restrict__ scale)
 {
-    using C = BlkCfg<P, CH>;
+    using C = BlkCfg<P>;
     constexpr int PP = P * P;
     const int lane = threadIdx.x & 31;
     const int64_t i = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);  // parent 1 + i of all levels
@@ -395,11 +398,11 @@ __global__ void __launch_bounds__(128) k_blk_opmax(const float *__restrict__ ops
 
 // B[d][plane][row: class c', n][K column of class c, k] (the columns' padding zeroed beforehand); g
 // stored after the table
-template <int P, int CH>
+template <int P>
 __global__ void __launch_bounds__(128) k_blk_build(const float *__restrict__ ops, const unsigned *__restrict__ mbits,
                                                    __half *__restrict__ B, int *__restrict__ gout)
 {
-    using C = BlkCfg<P, CH>;
+    using C = BlkCfg<P>;
     constexpr int PP = P * P;
     const int d = blockIdx.x / PP, n = blockIdx.x % PP;
     int ex = 0;
@@ -420,13 +423,13 @@ __global__ void __launch_bounds__(128) k_blk_build(const float *__restrict__ ops
 }
 
 // ---- the kernel -------------------------------------------------------------------------------
-template <int P, int CH>
+template <int P>
 __global__ void __launch_bounds__(kBlkThreads, 1)
     k_m2l_blk(const __grid_constant__ BlkParams prm, const int32_t *__restrict__ begin,
               const int32_t *__restrict__ end, const int8_t *__restrict__ pscale, const int *__restrict__ gexp,
               float *__restrict__ Lc, float *__restrict__ Lpart, int *status)
 {
-    using C = BlkCfg<P, CH>;
+    using C = BlkCfg<P>;
     constexpr int PP = C::PP, NT = C::NT, NH = C::NH, NSTAGE = C::NSTAGE;
     constexpr uint32_t kIdesc = (1u << 4) | ((uint32_t)(NT >> 3) << 17) | ((uint32_t)(kBlkRows >> 4) << 24);
     constexpr int kProdWarp = kBlkDrainWarps, kMmaWarp = kBlkDrainWarps + 1;
@@ -434,7 +437,7 @@ __global__ void __launch_bounds__(kBlkThreads, 1)
     extern __shared__ unsigned char blk_smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[NSTAGE], empty_bar[NSTAGE], dfull[2], dempty[2], done_bar;
     __shared__ int s_issued[NSTAGE];
-    __shared__ BlkSteps<C, CH> s_steps;
+    __shared__ BlkSteps<C> s_steps;
     __shared__ uint32_t s_tmem;
     __shared__ volatile int s_abort;
 
@@ -452,7 +455,7 @@ __global__ void __launch_bounds__(kBlkThreads, 1)
     t /= C::NTILES;
     const int tx = t % (pg / bx), ty = (t / (pg / bx)) % (pg / by), tz = t / ((pg / bx) * (pg / by));
     const int x0 = tx * bx, y0 = ty * by, z0 = tz * bz;
-    const uint32_t a_bytes = (uint32_t)rows * CH * 2;
+    const uint32_t a_bytes = (uint32_t)rows * kBlkCh * 2;
 
     unsigned char *smem =
         blk_smem_raw + ((1024u - (smem_u32(blk_smem_raw) & 1023u)) & 1023u);  // 1024-byte aligned stages
@@ -481,7 +484,7 @@ __global__ void __launch_bounds__(kBlkThreads, 1)
         blk_prefetch_tmap(&prm.tmB);
     }
     if (warp == kMmaWarp) tmem_alloc(&s_tmem, C::TMEM_COLS);
-    if (warp == 0) blk_steps<C, CH>(s_steps, nt, d_lo, d_hi, lane);
+    if (warp == 0) blk_steps<C>(s_steps, nt, d_lo, d_hi, lane);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -529,9 +532,9 @@ __global__ void __launch_bounds__(kBlkThreads, 1)
                 const uint32_t dt = tmem + (uint32_t)(b * NT);
                 for (int j = 0; j < step_kw(sv) / 16; ++j) {
                     const uint32_t o = 32u * j;
-                    blk_mma_ss(dt, blk_desc<CH>(al + o), blk_desc<CH>(bh + o), kIdesc, (first && j == 0) ? 0u : 1u);
-                    blk_mma_ss(dt, blk_desc<CH>(ah + o), blk_desc<CH>(bl + o), kIdesc, 1u);
-                    blk_mma_ss(dt, blk_desc<CH>(ah + o), blk_desc<CH>(bh + o), kIdesc, 1u);
+                    blk_mma_ss(dt, blk_desc(al + o), blk_desc(bh + o), kIdesc, (first && j == 0) ? 0u : 1u);
+                    blk_mma_ss(dt, blk_desc(ah + o), blk_desc(bl + o), kIdesc, 1u);
+                    blk_mma_ss(dt, blk_desc(ah + o), blk_desc(bh + o), kIdesc, 1u);
                 }
                 tc_commit(&empty_bar[st]);
                 if (last) tc_commit(&dfull[b]);
@@ -665,14 +668,14 @@ __global__ void k_ablk_units(Span cells, const uint32_t *__restrict__ flag, cons
 
 // pre-split rows: unit u (one warp): the classes U of its children's coefficients, scaled by 2^s_u, in
 // FP16 hi | lo, s_u = 10 - e with max |U| = f 2^e (0 and zeros for none); row Z and its scale are zero
-template <int P, int CH>
+template <int P>
 __global__ void __launch_bounds__(256) k_ablk_presplit(const int32_t *__restrict__ n_units, int64_t zrow,
                                                        const int32_t *__restrict__ units,
                                                        const int32_t *__restrict__ child_of,
                                                        const float *__restrict__ M, __half *__restrict__ A,
                                                        int8_t *__restrict__ scale)
 {
-    using C = BlkCfg<P, CH>;
+    using C = BlkCfg<P>;
     constexpr int PP = P * P;
     const int lane = threadIdx.x & 31;
     const int64_t u = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -773,13 +776,13 @@ struct AblkParams {
 // the expected ones take their ranges one after another in one CTA, which adds them in V in range
 // order, as k_ablk_finish does for the others; their V rows follow the split ones'.  64 sets of 20,000
 // particles, p = 8: 10.2 GB -> 2.0, 4.65 ms -> 4.31; a batch of 96 instances 6.54 ms -> 6.37.
-template <int P, int CH, bool SEQ>
+template <int P, bool SEQ>
 __global__ void __launch_bounds__(kAblkThreads, 1)
     k_m2l_ablk(const __grid_constant__ AblkParams prm, const int32_t *__restrict__ n_units,
                const int32_t *__restrict__ src, const __half *__restrict__ Apre, const int8_t *__restrict__ uscale,
                const int *__restrict__ gexp, float *__restrict__ V, int *status)
 {
-    using C = BlkCfg<P, CH>;
+    using C = BlkCfg<P>;
     constexpr int KD = C::KD, NT = C::NT, NH = C::NH, NSTAGE = C::NSTAGE;
     constexpr uint32_t kIdesc = (1u << 4) | ((uint32_t)(NT >> 3) << 17) | ((uint32_t)(kBlkRows >> 4) << 24);
     constexpr int kLoad0 = kBlkDrainWarps, kProdWarp = kLoad0 + kAblkLoadWarps, kMmaWarp = kProdWarp + 1;
@@ -787,7 +790,7 @@ __global__ void __launch_bounds__(kAblkThreads, 1)
     extern __shared__ unsigned char blk_smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[NSTAGE], empty_bar[NSTAGE], dfull[2], dempty[2], done_bar;
     __shared__ int s_issued[NSTAGE];
-    __shared__ BlkSteps<C, CH> s_steps;
+    __shared__ BlkSteps<C> s_steps;
     __shared__ uint32_t s_tmem;
     __shared__ volatile int s_abort;
 
@@ -826,7 +829,7 @@ __global__ void __launch_bounds__(kAblkThreads, 1)
     }
     if (warp == kProdWarp && lane == 0) blk_prefetch_tmap(&prm.tmB);
     if (warp == kMmaWarp) tmem_alloc(&s_tmem, C::TMEM_COLS);
-    if (warp == 0) blk_steps<C, CH>(s_steps, nt, d_lo, d_hi, lane);
+    if (warp == 0) blk_steps<C>(s_steps, nt, d_lo, d_hi, lane);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -835,10 +838,10 @@ __global__ void __launch_bounds__(kAblkThreads, 1)
 
     if (warp >= kLoad0 && warp < kProdWarp) {
         // ===== loader warps: rows 64 w + lane and 64 w + 32 + lane of A (hi and lo planes) =====
-        // a stage's 16-byte chunks go through registers; where they fit twice (p = 8, 10), the
-        // next stage's loads are issued before this stage is stored, so their latency overlaps
+        // a stage's 16-byte chunks go through registers, the next stage's loads issued before this
+        // stage is stored, so their latency overlaps
         constexpr int RPW = kBlkRows / kAblkLoadWarps / 32;  // rows per lane
-        constexpr int CPR = CH / 8;                          // 16-byte chunks per row
+        constexpr int CPR = kBlkCh / 8;                      // 16-byte chunks per row
         constexpr int NB = RPW * 2 * CPR;                    // chunks per lane and stage
         const int r0 = (kBlkRows / kAblkLoadWarps) * (warp - kLoad0) + lane;
         auto fetch = [&](int s, int4(&v)[NB]) {
@@ -870,12 +873,12 @@ __global__ void __launch_bounds__(kAblkThreads, 1)
                 const int r = r0 + 32 * rr;
 #pragma unroll
                 for (int pl = 0; pl < 2; ++pl) {
-                    unsigned char *dst = a_pl(st, pl) + (size_t)r * (2 * CH);
+                    unsigned char *dst = a_pl(st, pl) + (size_t)r * (2 * kBlkCh);
 #pragma unroll
                     for (int q = 0; q < CPR; ++q) {
                         if (8 * q >= kw) break;
                         // the TMA's swizzle of this row: 16-byte chunk q at q ^ (row bits)
-                        const int qs = CH == 64 ? (q ^ (r & 7)) : (q ^ ((r >> 1) & 3));
+                        const int qs = q ^ ((r >> 1) & 3);
                         *reinterpret_cast<int4 *>(dst + 16 * qs) = v[(rr * 2 + pl) * CPR + q];
                     }
                 }
@@ -885,21 +888,13 @@ __global__ void __launch_bounds__(kAblkThreads, 1)
             if (lane == 0) mbar_arrive(&full_bar[st]);
             return true;
         };
-        if constexpr (NB <= 16) {
-            int4 va[NB], vb[NB];
-            if (S > 0) fetch(0, va);
-            for (int s = 0; s < S; s += 2) {
-                if (s + 1 < S) fetch(s + 1, vb);
-                if (!put(s, va) || s + 1 >= S) break;
-                if (s + 2 < S) fetch(s + 2, va);
-                if (!put(s + 1, vb)) break;
-            }
-        } else {
-            int4 va[NB];
-            for (int s = 0; s < S; ++s) {
-                fetch(s, va);
-                if (!put(s, va)) break;
-            }
+        int4 va[NB], vb[NB];
+        if (S > 0) fetch(0, va);
+        for (int s = 0; s < S; s += 2) {
+            if (s + 1 < S) fetch(s + 1, vb);
+            if (!put(s, va) || s + 1 >= S) break;
+            if (s + 2 < S) fetch(s + 2, va);
+            if (!put(s + 1, vb)) break;
         }
     } else if (warp == kProdWarp) {
         if (lane == 0) {
@@ -938,9 +933,9 @@ __global__ void __launch_bounds__(kAblkThreads, 1)
                 const uint32_t dt = tmem + (uint32_t)(b * NT);
                 for (int j = 0; j < step_kw(sv) / 16; ++j) {
                     const uint32_t o = 32u * j;
-                    blk_mma_ss(dt, blk_desc<CH>(al + o), blk_desc<CH>(bh + o), kIdesc, (first && j == 0) ? 0u : 1u);
-                    blk_mma_ss(dt, blk_desc<CH>(ah + o), blk_desc<CH>(bl + o), kIdesc, 1u);
-                    blk_mma_ss(dt, blk_desc<CH>(ah + o), blk_desc<CH>(bh + o), kIdesc, 1u);
+                    blk_mma_ss(dt, blk_desc(al + o), blk_desc(bh + o), kIdesc, (first && j == 0) ? 0u : 1u);
+                    blk_mma_ss(dt, blk_desc(ah + o), blk_desc(bl + o), kIdesc, 1u);
+                    blk_mma_ss(dt, blk_desc(ah + o), blk_desc(bh + o), kIdesc, 1u);
                 }
                 tc_commit(&empty_bar[st]);
                 if (last) tc_commit(&dfull[b]);
@@ -1144,7 +1139,7 @@ static int blk_tiles(int L)
     for (int l = 2; l <= L; ++l) {
         const int pg = 1 << (l - 1);
         const int bx = pg < 8 ? pg : 8, by = pg < 4 ? pg : 4;
-        n += (pg / bx) * (pg / by) * (pg / by) * BlkCfg<P, blk_ch(P)>::NTILES;
+        n += (pg / bx) * (pg / by) * (pg / by) * BlkCfg<P>::NTILES;
     }
     return n;
 }
@@ -1166,7 +1161,7 @@ static int blk_tiles_p(int P, int L)
 // the sum of the ranges, half an offset).  12 tiles (100,000 particles, p = 8): 26 ranges took three
 // launches, the last of 8 CTAs, 75 us and 10 for the sum; 12 ranges one, and the step 244 -> 193 us.
 // A fixed rule, so that the workspace size does not depend on the device.
-constexpr int kBlkFillCtas = 152;
+constexpr int kBlkFillCtas = kSms;
 static int blk_ranges(int64_t tiles)
 {
     if (tiles <= 0 || tiles >= kBlkFillCtas) return 1;
@@ -1195,13 +1190,13 @@ size_t m2l_blk_table_bytes(int P) { return 26 * 2 * 8 * (size_t)P * P * blk_kw(P
 template <int P>
 static void launch_build_t(const float *ops, void *table, cudaStream_t s)
 {
-    using C = BlkCfg<P, blk_ch(P)>;
+    using C = BlkCfg<P>;
     __half *B = static_cast<__half *>(table);
     int *g = reinterpret_cast<int *>(B + 26 * 2 * (size_t)C::KD * C::KW);
     unsigned *mbits = reinterpret_cast<unsigned *>(g + 1);
     cudaMemsetAsync(table, 0, m2l_blk_table_bytes(P), s);
     k_blk_opmax<P><<<26 * P * P, 128, 0, s>>>(ops, mbits);
-    k_blk_build<P, blk_ch(P)><<<26 * P * P, 128, 0, s>>>(ops, mbits, B, g);
+    k_blk_build<P><<<26 * P * P, 128, 0, s>>>(ops, mbits, B, g);
     note_launches(2);
 }
 
@@ -1222,21 +1217,21 @@ void launch_blk_presplit(int P, int L, const int32_t *begin, const int32_t *end,
     const unsigned grid = (unsigned)((blk_parents_before(L) + 7) / 8);
     __half *A = static_cast<__half *>(presplit);
     switch (P) {
-    case 4: k_blk_presplit<4, blk_ch(4)><<<grid, 256, 0, s>>>(L, begin, end, M, A, pscale); break;
-    case 6: k_blk_presplit<6, blk_ch(6)><<<grid, 256, 0, s>>>(L, begin, end, M, A, pscale); break;
-    case 8: k_blk_presplit<8, blk_ch(8)><<<grid, 256, 0, s>>>(L, begin, end, M, A, pscale); break;
-    case 10: k_blk_presplit<10, blk_ch(10)><<<grid, 256, 0, s>>>(L, begin, end, M, A, pscale); break;
+    case 4: k_blk_presplit<4><<<grid, 256, 0, s>>>(L, begin, end, M, A, pscale); break;
+    case 6: k_blk_presplit<6><<<grid, 256, 0, s>>>(L, begin, end, M, A, pscale); break;
+    case 8: k_blk_presplit<8><<<grid, 256, 0, s>>>(L, begin, end, M, A, pscale); break;
+    case 10: k_blk_presplit<10><<<grid, 256, 0, s>>>(L, begin, end, M, A, pscale); break;
     }
     note_launches(1);
 }
 
-template <int P, int CH>
+template <int P>
 static int launch_blk_t(int L, const int32_t *begin, const int32_t *end, const void *presplit,
                         const int8_t *pscale, const void *table, float *Lc, float *Lpart, int *status, cudaStream_t s,
                         int max_ctas)
 {
-    using C = BlkCfg<P, CH>;
-    constexpr CUtensorMapSwizzle kSw = CH == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
+    using C = BlkCfg<P>;
+    constexpr CUtensorMapSwizzle kSw = CU_TENSOR_MAP_SWIZZLE_64B;
     PFN_cuTensorMapEncodeTiled_v12000 enc = tmap_encoder();
     if (!enc) return -1;
     BlkParams prm;  // the kernel parameter (copied at launch)
@@ -1253,7 +1248,7 @@ static int launch_blk_t(int L, const int32_t *begin, const int32_t *end, const v
         void *A = const_cast<__half *>(static_cast<const __half *>(presplit) + (size_t)blk_parents_before(l - 1) * 2 * KW);
         const cuuint64_t dims[5] = {KW, 2, (cuuint64_t)pg, (cuuint64_t)pg, (cuuint64_t)pg};
         const cuuint64_t strides[4] = {KW * 2, KW * 4, KW * 4 * pg, KW * 4 * pg * pg};
-        const cuuint32_t box[5] = {(cuuint32_t)CH, 1, (cuuint32_t)bx, (cuuint32_t)by, (cuuint32_t)bz};
+        const cuuint32_t box[5] = {(cuuint32_t)kBlkCh, 1, (cuuint32_t)bx, (cuuint32_t)by, (cuuint32_t)bz};
         const cuuint32_t es[5] = {1, 1, 1, 1, 1};
         if (enc(&prm.tmA[l], CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 5, A, dims, strides, box, es,
                 CU_TENSOR_MAP_INTERLEAVE_NONE, kSw, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -1267,14 +1262,14 @@ static int launch_blk_t(int L, const int32_t *begin, const int32_t *end, const v
     {
         const cuuint64_t dims[4] = {KW, KD, 2, 26};
         const cuuint64_t strides[3] = {KW * 2, KD * KW * 2, KD * KW * 4};
-        const cuuint32_t box[4] = {(cuuint32_t)CH, (cuuint32_t)C::NT, 1, 1};
+        const cuuint32_t box[4] = {(cuuint32_t)kBlkCh, (cuuint32_t)C::NT, 1, 1};
         const cuuint32_t es[4] = {1, 1, 1, 1};
         if (enc(&prm.tmB, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, const_cast<void *>(table), dims, strides, box, es,
                 CU_TENSOR_MAP_INTERLEAVE_NONE, kSw, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return -1;
     }
-    auto kern = k_m2l_blk<P, CH>;
+    auto kern = k_m2l_blk<P>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::kSmemBytes);
     const int nctas = ntiles * prm.ksplit;
     const int step = max_ctas > 0 ? max_ctas : nctas;
@@ -1300,10 +1295,10 @@ int launch_m2l_blk(int P, int L, const int32_t *begin, const int32_t *end, const
 {
     if (L < 2) return 0;
     switch (P) {
-    case 4: return launch_blk_t<4, blk_ch(4)>(L, begin, end, presplit, pscale, table, Lc, Lpart, status, s, max_ctas);
-    case 6: return launch_blk_t<6, blk_ch(6)>(L, begin, end, presplit, pscale, table, Lc, Lpart, status, s, max_ctas);
-    case 8: return launch_blk_t<8, blk_ch(8)>(L, begin, end, presplit, pscale, table, Lc, Lpart, status, s, max_ctas);
-    case 10: return launch_blk_t<10, blk_ch(10)>(L, begin, end, presplit, pscale, table, Lc, Lpart, status, s, max_ctas);
+    case 4: return launch_blk_t<4>(L, begin, end, presplit, pscale, table, Lc, Lpart, status, s, max_ctas);
+    case 6: return launch_blk_t<6>(L, begin, end, presplit, pscale, table, Lc, Lpart, status, s, max_ctas);
+    case 8: return launch_blk_t<8>(L, begin, end, presplit, pscale, table, Lc, Lpart, status, s, max_ctas);
+    case 10: return launch_blk_t<10>(L, begin, end, presplit, pscale, table, Lc, Lpart, status, s, max_ctas);
     }
     return -1;
 }
@@ -1321,8 +1316,8 @@ size_t m2l_ablk_src_bytes(int64_t ucap) { return (size_t)m2l_ablk_tiles_units(uc
 // instance alone sum in the same order)
 int m2l_ablk_ksplit(int P, int64_t n, int leaf_size)
 {
-    const int nt = P == 4 ? BlkCfg<4, blk_ch(4)>::NTILES : P == 6 ? BlkCfg<6, blk_ch(6)>::NTILES
-                 : P == 8 ? BlkCfg<8, blk_ch(8)>::NTILES : BlkCfg<10, blk_ch(10)>::NTILES;
+    const int nt = P == 4 ? BlkCfg<4>::NTILES : P == 6 ? BlkCfg<6>::NTILES
+                 : P == 8 ? BlkCfg<8>::NTILES : BlkCfg<10>::NTILES;
     const int64_t units = n / (2 * (int64_t)(leaf_size > 0 ? leaf_size : 1)) + 1;
     return blk_ranges((units + kBlkRows - 1) / kBlkRows * nt);
 }
@@ -1340,10 +1335,10 @@ void launch_ablk_prep(int P, Span cells, int64_t ucap, const int32_t *level, con
     const unsigned gp = (unsigned)((ucap + 1 + 7) / 8);
     __half *A = static_cast<__half *>(Apre);
     switch (P) {
-    case 4: k_ablk_presplit<4, blk_ch(4)><<<gp, 256, 0, s>>>(n_units, zrow, units, child_of, M, A, uscale); break;
-    case 6: k_ablk_presplit<6, blk_ch(6)><<<gp, 256, 0, s>>>(n_units, zrow, units, child_of, M, A, uscale); break;
-    case 8: k_ablk_presplit<8, blk_ch(8)><<<gp, 256, 0, s>>>(n_units, zrow, units, child_of, M, A, uscale); break;
-    case 10: k_ablk_presplit<10, blk_ch(10)><<<gp, 256, 0, s>>>(n_units, zrow, units, child_of, M, A, uscale); break;
+    case 4: k_ablk_presplit<4><<<gp, 256, 0, s>>>(n_units, zrow, units, child_of, M, A, uscale); break;
+    case 6: k_ablk_presplit<6><<<gp, 256, 0, s>>>(n_units, zrow, units, child_of, M, A, uscale); break;
+    case 8: k_ablk_presplit<8><<<gp, 256, 0, s>>>(n_units, zrow, units, child_of, M, A, uscale); break;
+    case 10: k_ablk_presplit<10><<<gp, 256, 0, s>>>(n_units, zrow, units, child_of, M, A, uscale); break;
     }
     const int64_t up = m2l_ablk_tiles_units(ucap);
     k_ablk_src<<<(unsigned)((up * 26 + 255) / 256), 256, 0, s>>>(n_units, up, zrow, units, coll, unit_of, src);
@@ -1370,13 +1365,13 @@ struct AblkUnits {
     }
 };
 
-template <int P, int CH>
+template <int P>
 static int launch_ablk_t(int64_t ucap, int64_t uexp, const int32_t *n_units, const int32_t *units, const int32_t *child_of,
                          const int32_t *src, const void *Apre, const int8_t *uscale, const void *table, float *Lc,
                          float *V, int ksplit, int *status, cudaStream_t s, int max_ctas)
 {
-    using C = BlkCfg<P, CH>;
-    constexpr CUtensorMapSwizzle kSw = CH == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
+    using C = BlkCfg<P>;
+    constexpr CUtensorMapSwizzle kSw = CU_TENSOR_MAP_SWIZZLE_64B;
     PFN_cuTensorMapEncodeTiled_v12000 enc = tmap_encoder();
     if (!enc) return -1;
     AblkParams prm;
@@ -1386,7 +1381,7 @@ static int launch_ablk_t(int64_t ucap, int64_t uexp, const int32_t *n_units, con
     {
         const cuuint64_t dims[4] = {KW, KD, 2, 26};
         const cuuint64_t strides[3] = {KW * 2, KD * KW * 2, KD * KW * 4};
-        const cuuint32_t box[4] = {(cuuint32_t)CH, (cuuint32_t)C::NT, 1, 1};
+        const cuuint32_t box[4] = {(cuuint32_t)kBlkCh, (cuuint32_t)C::NT, 1, 1};
         const cuuint32_t es[4] = {1, 1, 1, 1};
         if (enc(&prm.tmB, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, const_cast<void *>(table), dims, strides, box, es,
                 CU_TENSOR_MAP_INTERLEAVE_NONE, kSw, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -1397,7 +1392,7 @@ static int launch_ablk_t(int64_t ucap, int64_t uexp, const int32_t *n_units, con
     prm.zrow = ucap;
     const AblkUnits lay(P, ucap, uexp, ksplit);
     const bool seq = lay.split < lay.chunk;
-    auto kern = seq ? k_m2l_ablk<P, CH, true> : k_m2l_ablk<P, CH, false>;
+    auto kern = seq ? k_m2l_ablk<P, true> : k_m2l_ablk<P, false>;
     auto finish = seq ? k_ablk_finish<P, true> : k_ablk_finish<P, false>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::kSmemBytes);
     for (int64_t u0 = 0; u0 < ucap; u0 += lay.chunk) {
@@ -1435,10 +1430,10 @@ int launch_m2l_ablk(int P, int64_t ucap, int64_t uexp, const int32_t *n_units, c
 {
     if (ucap <= 0) return 0;
     switch (P) {
-    case 4: return launch_ablk_t<4, blk_ch(4)>(ucap, uexp, n_units, units, child_of, src, Apre, uscale, table, Lc, V, ksplit, status, s, max_ctas);
-    case 6: return launch_ablk_t<6, blk_ch(6)>(ucap, uexp, n_units, units, child_of, src, Apre, uscale, table, Lc, V, ksplit, status, s, max_ctas);
-    case 8: return launch_ablk_t<8, blk_ch(8)>(ucap, uexp, n_units, units, child_of, src, Apre, uscale, table, Lc, V, ksplit, status, s, max_ctas);
-    case 10: return launch_ablk_t<10, blk_ch(10)>(ucap, uexp, n_units, units, child_of, src, Apre, uscale, table, Lc, V, ksplit, status, s, max_ctas);
+    case 4: return launch_ablk_t<4>(ucap, uexp, n_units, units, child_of, src, Apre, uscale, table, Lc, V, ksplit, status, s, max_ctas);
+    case 6: return launch_ablk_t<6>(ucap, uexp, n_units, units, child_of, src, Apre, uscale, table, Lc, V, ksplit, status, s, max_ctas);
+    case 8: return launch_ablk_t<8>(ucap, uexp, n_units, units, child_of, src, Apre, uscale, table, Lc, V, ksplit, status, s, max_ctas);
+    case 10: return launch_ablk_t<10>(ucap, uexp, n_units, units, child_of, src, Apre, uscale, table, Lc, V, ksplit, status, s, max_ctas);
     }
     return -1;
 }

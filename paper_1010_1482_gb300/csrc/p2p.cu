@@ -381,7 +381,7 @@ static int p2p_blocks_per_sm()
 // 0.525, 0.541, 0.596 ms alone and 1.158, 1.152, 1.163, 1.189, 1.248 ms for the forked step; on
 // 16M Plummer (p = 8) P2P took 8.91, 7.97, 9.29 ms with 1, 4 and one wave.
 constexpr int kP2PLeavesPerCta = 4;
-constexpr int kP2PMaxParts = 16, kP2PWave = 152 * 8;
+constexpr int kP2PMaxParts = 16, kP2PWave = kSms * 8;
 // the evaluating context's choice (gbfmm_set_p2p_leaves_per_cta, gbfmm_tune), set on entry to an
 // evaluation by the thread that issues its launches; 0: kP2PLeavesPerCta
 static thread_local int tl_leaves_per_cta = 0;

@@ -435,7 +435,6 @@ void launch_exclusive_scan(const uint32_t *in, uint32_t *out, int64_t n, uint32_
 // ------------------------------------------------------------------------------------------
 constexpr int kRsThreads = 512, kRsWarps = kRsThreads / 32;
 constexpr int kRsTile = 4096;  // the reduce-then-scan form's tile, and the largest of the look-back form
-constexpr int64_t kRsScanMinN = int64_t(1) << 22;  // from here on the passes take the reduce-then-scan form
 constexpr uint64_t kRsAgg = 1ull << 62, kRsInc = 2ull << 62, kRsFlags = 3ull << 62;
 
 static_assert(kRsTile <= 65535, "16-bit per-warp digit counts and offsets");
