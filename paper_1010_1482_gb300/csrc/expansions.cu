@@ -591,7 +591,7 @@ __global__ void __launch_bounds__(128) k_p2m(int L, const float *__restrict__ ge
 // 8 waste fewer lanes than rounds of 32 on 15 to 40 particles, and 8 rows are added instead of
 // 32), else 32, a leaf's particles in as few rounds as possible.  P2M, 32 lanes and complex
 // recurrences -> 8 lanes and real ones: 1M uniform p = 10 64 -> 32 us, 5M p = 6 149 -> 62, 16M
-// Plummer p = 8 1122 -> 407; P2L there 2036 -> 1305.
+// Plummer p = 8 1122 -> 407; P2L there 2036 -> 1108 (16 lanes a cell).
 constexpr int64_t kP2MManyLeaves = 8 * 1024;
 
 // P2M starts beside P2P, with priority.  An SM that runs it under another split of shared memory and L1
@@ -1125,7 +1125,7 @@ void launch_l2p(int P, int L, const float *geo, int64_t n, const float4 *sx, con
 // l: target l % T, pair l / T).  The lanes' partial sums are added in warp and group order.
 // M2P alone, the earlier kernels (a warp or a CTA of 64 per leaf) -> this one: treecode, 131,072
 // uniform p = 6 1325 -> 653 us, 50,021 Plummer p = 8 2348 -> 1023; W rows, 20,011 Plummer p = 4
-// 59 -> 24, 400,009 p = 10 428 -> 286, 16M p = 8 3587 -> 2773.
+// 59 -> 27, 400,009 p = 10 428 -> 234, 16M p = 8 3587 -> 2793.
 template <int P>
 struct M2PW {
     static constexpr int PP = P * P, NM = (P + 1) * (P + 2) / 2, NO = 6 * NM;
