@@ -730,8 +730,11 @@ static void sort_gather_t(KeyT *k0, KeyT *k1, uint32_t *v0, uint32_t *v1, int64_
     uint32_t *starts = counts + 256 * nblk;
     const int smem = tile * (int)(sizeof(KeyT) + sizeof(uint32_t));
     auto lookback = tile == 1024 ? k_rs_pass<KeyT, true, 2> : tile == 2048 ? k_rs_pass<KeyT, true, 4> : k_rs_pass<KeyT, true, 8>;
-    cudaFuncSetAttribute(lookback, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    cudaFuncSetAttribute(k_rs_pass<KeyT, false, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    // one size a kernel, whatever n: another thread may be about to launch it (rts: tiles of 4096)
+    if (rts)
+        cudaFuncSetAttribute(k_rs_pass<KeyT, false, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    else
+        cudaFuncSetAttribute(lookback, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     for (int pass = 0; pass < passes; ++pass) {
         const bool last = pass + 1 == passes;
         if (rts) {
